@@ -1141,12 +1141,12 @@ void part_side_layout(Carve& c, PartSide& ps, int64_t n, int b1, int b2, int pas
     const int nbuf = passes < 2 ? passes : 2;
     const int ncols = plan.gftr ? plan.ncols[side] : 0;
     for (int k = 0; k < 2; ++k) {
-        // 16 bytes of slack after each buffer: a later pass's tile loads may
+        // 16 bytes of slack after each buffer: later tile and row loads may
         // read the aligned cover of the last rows (see PartPass::src_end)
         ps.key[k] = k < nbuf ? c.take<unsigned char>((size_t)n * kb + 16) : nullptr;
         ps.idx[k] = k < nbuf ? c.take<uint32_t>((size_t)n + 4) : nullptr;
         for (int q = 0; q < kMaxCols; ++q)
-            ps.col[k][q] = (k < nbuf && q < ncols) ? c.take<unsigned char>((size_t)n * plan.col_bytes[side][q])
+            ps.col[k][q] = (k < nbuf && q < ncols) ? c.take<unsigned char>((size_t)n * plan.col_bytes[side][q] + 16)
                                                   : nullptr;
     }
     const size_t ntiles1 = (size_t)((n + kPartTile - 1) / kPartTile);

@@ -18,6 +18,7 @@
 #include "chunks.cuh"
 #include "emit.cuh"
 #include "kernels.cuh"
+#include "phj.cuh"
 
 namespace eiger {
 
@@ -26,10 +27,8 @@ size_t part_scan_blocks(size_t counts_len);
 
 namespace {
 
-constexpr int kJoinThreads = EIGER_JOIN_THREADS;
 constexpr int kMaxRows = 8;                       // rows per thread per round (at most)
 constexpr int kJoinStage = kJoinThreads * kMaxRows;  // a unique-key round never spills
-constexpr uint32_t kBuildCap = EIGER_BUILD_CAP;   // build rows per shared-memory table
 
 // Rows each thread keeps in flight per round (the current round and the next
 // one's loads) and CTAs per SM. Index pairs of 32-bit keys: 4 rows, three
@@ -45,24 +44,8 @@ struct Rows {
     static constexpr int kMinBlocks = (kLean ? 1536 : 1024) / kJoinThreads;
     static constexpr uint32_t kRound = kJoinThreads * kN;
 };
-#ifndef EIGER_PROBE_CHUNK
-#define EIGER_PROBE_CHUNK 32768
-#endif
-constexpr uint32_t kProbeChunk = EIGER_PROBE_CHUNK;  // probe rows per work item, at most
 constexpr uint32_t kTableMax = 2 * kBuildCap;
 constexpr uint32_t kEmptyRow = 0xFFFFFFFFu;
-
-template <typename KeyT>
-struct JoinIn {
-    const KeyT* bkey;
-    const uint32_t* bidx;
-    const uint32_t* bstart;
-    const KeyT* pkey;
-    const uint32_t* pidx;
-    const uint32_t* pstart;
-    const unsigned long long* item_prefix;
-    uint32_t P;
-};
 
 // Work items of partition p: build chunks x probe chunks (none if a side is empty).
 __global__ void items_count_kernel(const uint32_t* __restrict__ bstart, const uint32_t* __restrict__ pstart,
@@ -141,18 +124,9 @@ struct SmemTable;
 // Slots come in aligned pairs: the home slot is even, so a probe reads its
 // first two candidates with one 16-byte shared load (inserts are ordinary
 // linear probing from the same home slot, filling a pair's first slot first).
-__device__ __forceinline__ uint32_t slot_hash(uint32_t k) { return k * 0x9E3779B1u; }
-__device__ __forceinline__ uint32_t slot_hash(uint64_t k) {
-    return (uint32_t)((k * 0x9E3779B97F4A7C15ull) >> 32);
-}
-
 template <typename KeyT>
 __device__ __forceinline__ uint32_t home_slot(KeyT k, uint32_t tsize) {
     return 2u * (uint32_t)(((unsigned long long)slot_hash(k) * (tsize >> 1)) >> 32);
-}
-
-__device__ __forceinline__ uint32_t next_slot(uint32_t s, uint32_t tsize) {
-    return s + 1 == tsize ? 0u : s + 1;
 }
 
 // 32-bit keys: one packed 64-bit word per slot, claimed by CAS.
@@ -251,42 +225,8 @@ __device__ __forceinline__ void load_round(RoundRegs<KeyT, N>& r, const KeyT* __
     }
 }
 
-// The 128-byte lines of rows [0, n) of a partitioned side (keys, then tuple
-// IDs unless rows are identified by position) asked into L2, one line per
-// participating thread and step (thread t of `threads`). A hint: no register
-// waits on it.
-template <bool POS, typename KeyT>
-__device__ __forceinline__ void prefetch_rows_l2(const KeyT* key, const uint32_t* idx, uint32_t n, uint32_t t,
-                                                 uint32_t threads) {
-    const uint32_t klines = (uint32_t)((n * sizeof(KeyT) + 127) / 128);
-    const uint32_t ilines = POS ? 0u : (n * 4u + 127) / 128;
-    for (uint32_t l = t; l < klines + ilines; l += threads) {
-        const char* p = l < klines ? reinterpret_cast<const char*>(key) + (size_t)l * 128
-                                   : reinterpret_cast<const char*>(idx) + (size_t)(l - klines) * 128;
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-    }
-}
-
 constexpr uint32_t kHole = 0xFFFFFFFFu;  // stage position without a match
 
-// Warp-collective: the last partition p in [0, P) with prefix[p] <= item
-// (prefix is non-decreasing, prefix[0] = 0). Each step tests 32 evenly spaced
-// pivots at once, so 2^15 partitions take three dependent loads.
-__device__ __forceinline__ uint32_t find_partition(const unsigned long long* __restrict__ prefix,
-                                                   uint32_t P, unsigned long long item) {
-    const unsigned lane = lane_id();
-    uint32_t lo = 0, hi = P;
-    while (hi - lo > 1) {
-        const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
-        const uint32_t piv = lo + lane * step;
-        const bool le = piv < hi && prefix[piv] <= item;
-        const unsigned m = __ballot_sync(0xffffffffu, le);
-        const uint32_t last = 31 - __clz(m);  // lane 0 always qualifies
-        lo = lo + last * step;
-        hi = lo + step < hi ? lo + step : hi;
-    }
-    return lo;
-}
 constexpr int kJoinWarps = kJoinThreads / kWarp;
 
 // Block-collective flush of a positional stage: position j * kJoinThreads + t
@@ -404,22 +344,12 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, PAIRS>::kMinBlocks))
         unsigned long long claim = 0;
         if (threadIdx.x == 0) claim = atomicAdd(&ctrl->next_item, 1ull);
 
-        const uint32_t bs0 = a.bstart[p], bsz = a.bstart[p + 1] - bs0;
-        const uint32_t ps0 = a.pstart[p], psz = a.pstart[p + 1] - ps0;
-        const uint32_t npc = (psz + kProbeChunk - 1) / kProbeChunk;
-        const uint32_t local = (uint32_t)(item - a.item_prefix[p]);  // < items of one partition
-        const uint32_t bc = local / npc, pc = local - bc * npc;
-        // chunks of a partition are balanced (sizes differ by at most one
-        // row), so no item joins a full table with a sliver of probe rows
-        const uint32_t nbc = (bsz + kBuildCap - 1) / kBuildCap;
-        const uint32_t b_lo = (uint32_t)((unsigned long long)bc * bsz / nbc);
-        const uint32_t bn = (uint32_t)((unsigned long long)(bc + 1) * bsz / nbc) - b_lo;
-        const uint32_t p_lo = (uint32_t)((unsigned long long)pc * psz / npc);
-        const uint32_t pn = (uint32_t)((unsigned long long)(pc + 1) * psz / npc) - p_lo;
-        const KeyT* bkey = a.bkey + bs0 + b_lo;
-        const uint32_t* bidx = a.bidx + bs0 + b_lo;
-        const KeyT* pkey = a.pkey + ps0 + p_lo;
-        const uint32_t* pidx = a.pidx + ps0 + p_lo;
+        const ItemRows ir = item_rows(a, item, p);
+        const uint32_t bn = ir.bn, pn = ir.pn;
+        const KeyT* bkey = a.bkey + ir.bs0;
+        const uint32_t* bidx = a.bidx + ir.bs0;
+        const KeyT* pkey = a.pkey + ir.ps0;
+        const uint32_t* pidx = a.pidx + ir.ps0;
         // about three slots per build row (load <= 1/3), at most kTableMax
         uint32_t tsize = (3 * bn + 31) & ~31u;
         if (tsize < 64) tsize = 64;
@@ -428,7 +358,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, PAIRS>::kMinBlocks))
         // Issue the first build and probe loads before clearing the table, so
         // their latency overlaps the clear.
         RoundRegs<KeyT, kN> cur, nxt;
-        const uint32_t bpos0 = bs0 + b_lo, ppos0 = ps0 + p_lo;
+        const uint32_t bpos0 = ir.bs0, ppos0 = ir.ps0;
         load_round<POS>(nxt, bkey, bidx, 0, bn, bpos0);
         load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
         tab.clear_all(tsize);
@@ -593,20 +523,14 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     a.P = 1u << (plan.bits1 + (passes == 2 ? plan.bits2 : 0));
     const bool pairs = !out.aggregate && out.bidx && out.pidx && out.b.n == 0 && out.p.n == 0 && !out.b.rowmap &&
                        !out.p.rowmap;
-    auto kern = out.aggregate ? (plan.gftr ? phj_join_kernel<KeyT, true, false, true>
-                                           : phj_join_kernel<KeyT, true, false, false>)
+    // the sum with carried payloads has its own kernel (phj_sum.cu)
+    if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, out, ctrl, di, stream, nb, np);
+    auto kern = out.aggregate ? phj_join_kernel<KeyT, true, false, false>
                 : pairs       ? phj_join_kernel<KeyT, false, true, false>
                 : plan.gftr   ? phj_join_kernel<KeyT, false, false, true>
                               : phj_join_kernel<KeyT, false, false, false>;
-    // reads every partitioned (key', row) of both sides once, writes the matches;
-    // the positional aggregate reads keys only, each carried build payload at
-    // most once and the probe payload of every match
-    const double tuple = (double)(sizeof(KeyT) + sizeof(uint32_t));
-    const bool pos_agg = out.aggregate && plan.gftr;
-    ProfScope ps("phj_join",
-                 pos_agg ? (double)sizeof(KeyT) * (double)(nb + np) + (double)out.b.bytes[0] * (double)nb
-                         : tuple * (double)(nb + np),
-                 stream, pos_agg ? (double)out.p.bytes[0] : match_bytes(out));
+    // reads every partitioned (key', row) of both sides once, writes the matches
+    ProfScope ps("phj_join", (double)(sizeof(KeyT) + sizeof(uint32_t)) * (double)(nb + np), stream, match_bytes(out));
     const size_t smem = join_smem<KeyT>(!pairs && !out.aggregate);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

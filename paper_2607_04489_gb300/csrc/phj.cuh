@@ -1,0 +1,137 @@
+// Work items and row access shared by the partitioned join's kernels (phj.cu,
+// phj_sum.cu).
+#pragma once
+
+#include "common.cuh"
+
+#ifndef EIGER_PROBE_CHUNK
+#define EIGER_PROBE_CHUNK 32768
+#endif
+
+namespace eiger {
+
+constexpr int kJoinThreads = EIGER_JOIN_THREADS;
+constexpr uint32_t kBuildCap = EIGER_BUILD_CAP;      // build rows per shared-memory table
+constexpr uint32_t kProbeChunk = EIGER_PROBE_CHUNK;  // probe rows per work item, at most
+
+template <typename KeyT>
+struct JoinIn {
+    const KeyT* bkey;
+    const uint32_t* bidx;
+    const uint32_t* bstart;
+    const KeyT* pkey;
+    const uint32_t* pidx;
+    const uint32_t* pstart;
+    const unsigned long long* item_prefix;
+    uint32_t P;
+};
+
+// A work item's rows: partition p's build chunk [bs0, bs0 + bn) and probe chunk
+// [ps0, ps0 + pn). The chunks of a partition are balanced (sizes differ by at
+// most one row), so no item joins a full table with a sliver of probe rows.
+struct ItemRows {
+    uint32_t bs0, bn, ps0, pn;
+};
+
+template <typename KeyT>
+__device__ __forceinline__ ItemRows item_rows(const JoinIn<KeyT>& a, unsigned long long item, uint32_t p) {
+    const uint32_t b0 = a.bstart[p], bsz = a.bstart[p + 1] - b0;
+    const uint32_t p0 = a.pstart[p], psz = a.pstart[p + 1] - p0;
+    const uint32_t npc = (psz + kProbeChunk - 1) / kProbeChunk;
+    const uint32_t nbc = (bsz + kBuildCap - 1) / kBuildCap;
+    const uint32_t local = (uint32_t)(item - a.item_prefix[p]);  // < items of one partition
+    const uint32_t bc = local / npc, pc = local - bc * npc;
+    ItemRows r;
+    const uint32_t b_lo = (uint32_t)((unsigned long long)bc * bsz / nbc);
+    const uint32_t p_lo = (uint32_t)((unsigned long long)pc * psz / npc);
+    r.bs0 = b0 + b_lo;
+    r.bn = (uint32_t)((unsigned long long)(bc + 1) * bsz / nbc) - b_lo;
+    r.ps0 = p0 + p_lo;
+    r.pn = (uint32_t)((unsigned long long)(pc + 1) * psz / npc) - p_lo;
+    return r;
+}
+
+__device__ __forceinline__ uint32_t slot_hash(uint32_t k) { return k * 0x9E3779B1u; }
+__device__ __forceinline__ uint32_t slot_hash(uint64_t k) {
+    return (uint32_t)((k * 0x9E3779B97F4A7C15ull) >> 32);
+}
+
+__device__ __forceinline__ uint32_t next_slot(uint32_t s, uint32_t tsize) {
+    return s + 1 == tsize ? 0u : s + 1;
+}
+
+// Shared-memory key arrays are probed 16 bytes at a time: a group of four
+// 32-bit or two 64-bit keys per load. Home slots are group-aligned and inserts
+// fill the groups in order (linear probing), so a key's slot is preceded by no
+// empty slot from its home group on. The all-ones pattern marks an empty slot.
+template <typename KeyT>
+struct KeyGroup;
+template <>
+struct KeyGroup<uint32_t> {
+    static constexpr uint32_t kN = 4;
+    uint4 v;
+    __device__ __forceinline__ void load(const uint32_t* p) { v = *reinterpret_cast<const uint4*>(p); }
+    // index of the first key equal to k, or kN
+    __device__ __forceinline__ uint32_t first(uint32_t k) const {
+        return v.x == k ? 0u : v.y == k ? 1u : v.z == k ? 2u : v.w == k ? 3u : 4u;
+    }
+    __device__ __forceinline__ uint32_t first_or_empty(uint32_t k) const {
+        return v.x == k || v.x == ~0u ? 0u : v.y == k || v.y == ~0u ? 1u : v.z == k || v.z == ~0u ? 2u
+               : v.w == k || v.w == ~0u ? 3u : 4u;
+    }
+    __device__ __forceinline__ uint32_t last() const { return v.w; }
+};
+template <>
+struct KeyGroup<uint64_t> {
+    static constexpr uint32_t kN = 2;
+    ulonglong2 v;
+    __device__ __forceinline__ void load(const uint64_t* p) { v = *reinterpret_cast<const ulonglong2*>(p); }
+    __device__ __forceinline__ uint32_t first(uint64_t k) const { return v.x == k ? 0u : v.y == k ? 1u : 2u; }
+    __device__ __forceinline__ uint32_t first_or_empty(uint64_t k) const {
+        return v.x == k || v.x == ~0ull ? 0u : v.y == k || v.y == ~0ull ? 1u : 2u;
+    }
+    __device__ __forceinline__ uint64_t last() const { return v.y; }
+};
+
+// The 128-byte lines of rows [0, n) of a partitioned side (keys, then tuple
+// IDs unless rows are identified by position) asked into L2, one line per
+// participating thread and step (thread t of `threads`). A hint: no register
+// waits on it.
+template <bool POS, typename KeyT>
+__device__ __forceinline__ void prefetch_rows_l2(const KeyT* key, const uint32_t* idx, uint32_t n, uint32_t t,
+                                                 uint32_t threads) {
+    const uint32_t klines = (uint32_t)((n * sizeof(KeyT) + 127) / 128);
+    const uint32_t ilines = POS ? 0u : (n * 4u + 127) / 128;
+    for (uint32_t l = t; l < klines + ilines; l += threads) {
+        const char* p = l < klines ? reinterpret_cast<const char*>(key) + (size_t)l * 128
+                                   : reinterpret_cast<const char*>(idx) + (size_t)(l - klines) * 128;
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    }
+}
+
+// Warp-collective: the last partition p in [0, P) with prefix[p] <= item
+// (prefix is non-decreasing, prefix[0] = 0). Each step tests 32 evenly spaced
+// pivots at once, so 2^15 partitions take three dependent loads.
+__device__ __forceinline__ uint32_t find_partition(const unsigned long long* __restrict__ prefix,
+                                                   uint32_t P, unsigned long long item) {
+    const unsigned lane = lane_id();
+    uint32_t lo = 0, hi = P;
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
+        const uint32_t piv = lo + lane * step;
+        const bool le = piv < hi && prefix[piv] <= item;
+        const unsigned m = __ballot_sync(0xffffffffu, le);
+        const uint32_t last = 31 - __clz(m);  // lane 0 always qualifies
+        lo = lo + last * step;
+        hi = lo + step < hi ? lo + step : hi;
+    }
+    return lo;
+}
+
+// The fused sum over positions (phj_sum.cu): out.b.src[0] and out.p.src[0] are
+// the carried payload columns, indexed like the keys of `a`.
+template <typename KeyT>
+cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
+                           cudaStream_t stream, int64_t nb, int64_t np);
+
+}  // namespace eiger
