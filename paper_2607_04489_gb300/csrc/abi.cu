@@ -199,6 +199,13 @@ eiger_status run_stats(const void* keys, int64_t n, int dtype, const StatsScratc
     return EIGER_OK;
 }
 
+// Bits of the key mix of hash partitions over encoded keys 0..mx - mn.
+int mix_bits(bool key32, int64_t mn, int64_t mx) {
+    if (!key32) return 64;
+    const int b = mx >= mn ? ceil_log2_u64((uint64_t)mx - (uint64_t)mn + 1) : 0;
+    return b < 2 ? 2 : b > 32 ? 32 : b;
+}
+
 bool narrowable(int dtype, int64_t nb, int64_t mn, int64_t mx) {
     if (nb == 0) return false;
     if (dtype == EIGER_I32) return true;
@@ -226,10 +233,11 @@ PlanDev to_dev(const eiger_plan_t& p, int dtype, const eiger_stats_t* bst) {
     if (bst) {
         d.range.lo = bst->min;
         d.range.hi = bst->max;
-        // 32-bit keys are offsets from the build minimum; the sort of the
-        // sort-merge join offsets 64-bit keys too, so it orders only the span
-        d.range.offset = (d.key32 || p.variant == EIGER_SMJ) ? (uint64_t)bst->min : 0ull;
+        // partitioned and sorted keys, and 32-bit ones, are offsets from the build minimum
+        const bool raw = !d.key32 && (p.variant == EIGER_NPHJ || p.variant == EIGER_STATIC);
+        d.range.offset = raw ? 0ull : (uint64_t)bst->min;
         d.check_range = 1;
+        d.kbits = mix_bits(d.key32, bst->min, bst->max);
     } else {
         d.range.lo = INT64_MIN;
         d.range.hi = INT64_MAX;
@@ -447,7 +455,8 @@ eiger_status resolve_materialize(const JoinCall& c, const eiger_stats_t* bst, ei
 
 void set_carry(PlanDev& d, const JoinOut& out, int materialize) {
     d.gftr = materialize == EIGER_GFTR;
-    d.no_rows = d.gftr && out.aggregate;  // the positional sum needs no tuple IDs
+    // carried columns are read by position: without index outputs nothing needs tuple IDs
+    d.no_rows = d.gftr && (out.aggregate || (!out.bidx && !out.pidx));
     d.ncols[0] = d.gftr ? out.b.n : 0;
     d.ncols[1] = d.gftr ? out.p.n : 0;
     for (int q = 0; q < kMaxCols; ++q) {
@@ -1026,6 +1035,7 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
         pd.bits2 = pub.bits2;
         pd.key32 = pub.narrow;
         pd.offset = (uint64_t)kst.min;
+        pd.kbits = mix_bits(pd.key32, kst.min, kst.max);
         pd.slots = (unsigned long long)pub.table_slots;
         pd.naggs = aggs->n;
         pd.smem = pd.variant == EIGER_GB_HASH && gb_smem_table_bytes(pd.slots, aggs->n, pd.key32) <= kGbSmemBudget;

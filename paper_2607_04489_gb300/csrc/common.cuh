@@ -65,30 +65,69 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t k) {
     return k;
 }
 
-// Key encodings carried through the join.
-//  - 32-bit: key' = (uint32)(key - offset). offset = build minimum when the
+// Odd multipliers of the key mix below (2^32 / golden ratio and Appleby's
+// MurmurHash3 constants) and their inverses modulo 2^64, whose low halves are
+// the inverses modulo any smaller power of two.
+constexpr uint64_t inverse_mod_2_64(uint64_t a) {  // Newton: each step doubles the correct low bits
+    uint64_t x = a;  // 3 bits
+    for (int i = 0; i < 5; ++i) x *= 2 - a * x;
+    return x;
+}
+constexpr uint32_t kMixA32 = 0x9E3779B1u, kMixB32 = 0x85EBCA6Bu;
+constexpr uint64_t kMixA64 = 0x9E3779B97F4A7C15ull, kMixB64 = 0xFF51AFD7ED558CCDull;
+
+// Key encodings.
+//  - encode, 32-bit: (uint32)(key - offset). offset = build minimum when the
 //    build span fits 32 bits (range-offset narrowing, Sec. 4.3 frame of
 //    reference), or 0 for raw int32 keys (their bit pattern).
-//  - 64-bit: key' = the int64 bit pattern minus offset (mod 2^64): offset 0
+//  - encode, 64-bit: the int64 bit pattern minus offset (mod 2^64): offset 0
 //    for hashing; the build minimum for the sort-merge join, which then
 //    orders only the span's significant bits.
+//  - mix: what the radix partitions carry in place of the encoded key. A
+//    bijection of `kbits`-bit values (multiply, xor-shift by at least half,
+//    multiply, all modulo 2^kbits), left-aligned in the word, so that every
+//    pass takes its digit by a shift, equal mixed keys are equal keys, and the
+//    bits below the partition's spread the keys over its table. With
+//    kbits = bits of the build span, the partitions' bits and those below them
+//    name a key completely.
+//  - unmix: the inverse.
 template <typename KeyT>
 struct KeyCodec;
 
 template <>
 struct KeyCodec<uint32_t> {
     static constexpr int kBits = 32;
-    __device__ __forceinline__ static uint32_t encode(int64_t k, uint64_t offset) {
+    __host__ __device__ __forceinline__ static uint32_t encode(int64_t k, uint64_t offset) {
         return (uint32_t)((uint64_t)k - offset);
     }
     __device__ __forceinline__ static uint32_t hash(uint32_t k) { return mix32(k); }
+    __host__ __device__ __forceinline__ static uint32_t mix(uint32_t x, int kbits) {
+        const int sh = 32 - kbits, s = (kbits + 1) >> 1;
+        const uint32_t y = (x * kMixA32) << sh;
+        return (((y ^ (y >> s)) >> sh) * kMixB32) << sh;
+    }
+    __host__ __device__ __forceinline__ static uint32_t unmix(uint32_t h, int kbits) {
+        const int sh = 32 - kbits, s = (kbits + 1) >> 1;
+        const uint32_t y = ((h >> sh) * (uint32_t)inverse_mod_2_64(kMixB32)) << sh;
+        return ((((y ^ (y >> s)) >> sh) * (uint32_t)inverse_mod_2_64(kMixA32)) << sh) >> sh;
+    }
 };
 
 template <>
 struct KeyCodec<uint64_t> {
     static constexpr int kBits = 64;
-    __device__ __forceinline__ static uint64_t encode(int64_t k, uint64_t offset) { return (uint64_t)k - offset; }
+    __host__ __device__ __forceinline__ static uint64_t encode(int64_t k, uint64_t offset) {
+        return (uint64_t)k - offset;
+    }
     __device__ __forceinline__ static uint64_t hash(uint64_t k) { return mix64(k); }
+    __host__ __device__ __forceinline__ static uint64_t mix(uint64_t x, int) {  // kbits is always 64
+        const uint64_t y = x * kMixA64;
+        return (y ^ (y >> 32)) * kMixB64;
+    }
+    __host__ __device__ __forceinline__ static uint64_t unmix(uint64_t h, int) {
+        const uint64_t y = h * inverse_mod_2_64(kMixB64);
+        return (y ^ (y >> 32)) * inverse_mod_2_64(kMixA64);
+    }
 };
 
 // Probe-side range test: a key outside [lo, hi] of the build side cannot match.

@@ -332,9 +332,10 @@ __device__ __forceinline__ void write_group(const GbOut& o, unsigned long long p
     for (int a = 0; a < naggs; ++a) o.aggs[a][pos] = v[a];
 }
 
-// Occupied slots of the global table -> output, reserved per warp.
+// Occupied slots of the global table -> output, reserved per warp. mixed_bits:
+// the table holds partitioned (mixed) keys; 0: encoded keys.
 template <typename KeyT>
-__global__ void gb_compact_kernel(GbTable<KeyT> t, AggSpec s, uint64_t offset, GbOut o, Ctrl* ctrl) {
+__global__ void gb_compact_kernel(GbTable<KeyT> t, AggSpec s, uint64_t offset, int mixed_bits, GbOut o, Ctrl* ctrl) {
     resolve_slots(t);
     const unsigned long long total = t.slots + 1;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -354,7 +355,8 @@ __global__ void gb_compact_kernel(GbTable<KeyT> t, AggSpec s, uint64_t offset, G
         if ((int)lane_id() == leader) base = atomicAdd(&ctrl->cursor, (unsigned long long)__popc(m));
         base = __shfl_sync(0xffffffffu, base, leader);
         if (has) {
-            const KeyT k = i == t.slots ? Empty<KeyT>::v : t.keys[i];
+            KeyT k = i == t.slots ? Empty<KeyT>::v : t.keys[i];
+            if (mixed_bits) k = KeyCodec<KeyT>::unmix(k, mixed_bits);
             long long v[kMaxCols];
             for (int a = 0; a < s.n; ++a) v[a] = t.aggs[(size_t)a * t.stride + i];
             write_group(o, base + __popc(m & lanemask_lt()), (int64_t)((uint64_t)k + offset), v, s.n);
@@ -461,7 +463,7 @@ __device__ __forceinline__ uint32_t find_item_part(const unsigned long long* __r
 // table, which is compacted afterwards.
 template <typename KeyT>
 __global__ void __launch_bounds__(kGbThreads)
-    gb_part_kernel(GbPartIn<KeyT> a, GbTable<KeyT> spill, uint64_t offset, GbOut o, Ctrl* ctrl) {
+    gb_part_kernel(GbPartIn<KeyT> a, GbTable<KeyT> spill, uint64_t offset, int kbits, GbOut o, Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long s_scratch[kGbThreads];
     __shared__ uint32_t s_warp[kGbThreads / kWarp];
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(kGbThreads)
             if (has) {
                 long long v[kMaxCols];
                 for (int b = 0; b < a.s.n; ++b) v[b] = *tab.agg(b, i);
-                write_group(o, pos++, (int64_t)((uint64_t)k + offset), v, a.s.n);
+                write_group(o, pos++, (int64_t)((uint64_t)KeyCodec<KeyT>::unmix(k, kbits) + offset), v, a.s.n);
             }
         }
         __syncthreads();
@@ -651,7 +653,7 @@ cudaError_t gb_hash_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     ProfScope ps("gb_compact", (kb + 8.0 * s.n) * (double)(plan.slots + 1), stream,
                  (double)sizeof(InKey) + 8.0 * s.n);
     const unsigned long long blocks = (plan.slots + 1 + 255) / 256;
-    gb_compact_kernel<KeyT><<<(int)(blocks < 8192 ? blocks : 8192), 256, 0, stream>>>(t, s, plan.offset, o, ctrl);
+    gb_compact_kernel<KeyT><<<(int)(blocks < 8192 ? blocks : 8192), 256, 0, stream>>>(t, s, plan.offset, 0, o, ctrl);
     return cudaGetLastError();
 }
 
@@ -670,6 +672,7 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     pd.range.hi = INT64_MAX;
     pd.range.offset = plan.offset;
     pd.check_range = 0;
+    pd.kbits = plan.kbits;
     pd.no_rows = 1;  // groups are aggregated from the carried columns by position
     ColSide carry{};
     int nc = 0;
@@ -726,12 +729,12 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     {
         ProfScope ps("gb_part", ((double)sizeof(KeyT) + vbytes) * (double)g.n, stream,
                      (double)sizeof(InKey) + 8.0 * s.n);
-        kern<<<di.sms * per_sm, kGbThreads, smem, stream>>>(in, spill, plan.offset, o, ctrl);
+        kern<<<di.sms * per_sm, kGbThreads, smem, stream>>>(in, spill, plan.offset, plan.kbits, o, ctrl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // the groups of multi-item partitions (an empty spill table when there are none)
     ProfScope ps("gb_spill_compact", 0.0, stream);
-    gb_compact_kernel<KeyT><<<di.sms * 2, 256, 0, stream>>>(spill, s, plan.offset, o, ctrl);
+    gb_compact_kernel<KeyT><<<di.sms * 2, 256, 0, stream>>>(spill, s, plan.offset, plan.kbits, o, ctrl);
     return cudaGetLastError();
 }
 

@@ -67,6 +67,7 @@ struct PlanDev {
     int bits1, bits2; // PHJ: radix bits per pass; SMJ: digit bits per sort pass, sort passes
     int narrow;       // frame-of-reference narrowing applied (offset = build min)
     int key32;        // keys carried as 32-bit values (int32, or int64 narrowed)
+    int kbits;        // hash partitioning: bits of the key mix (key32: of the build span; else 64)
     float load_factor;
     int dtype;        // 0 int32, 1 int64
     KeyRange range;   // build range (probe range test) and encoding offset
@@ -217,6 +218,7 @@ struct GbPlanDev {
     int bits1, bits2;          // partition: radix bits per pass (bits2 = 0: one pass)
     int key32;                 // keys carried as 32-bit offsets
     uint64_t offset;           // key minimum (frame of reference)
+    int kbits;                 // bits of the key mix (key32: of the key span; else 64)
     unsigned long long slots;  // hash: global table slots (power of two)
     int smem;                  // hash: aggregate in a CTA-private shared-memory copy first
     int naggs;

@@ -2,7 +2,7 @@
 // paper adopts; partitions are taken on bits of a hash of the key so their
 // sizes are even, as Sec. 3.3 does before partitioning).
 //
-// Each pass splits every input segment by `bits` further bits of mix(key'):
+// Each pass splits every input segment by `bits` further bits of the mixed key:
 // pass 1 by the top b1 bits, pass 2 by the next b2 bits within each pass-1
 // partition. A pass runs three steps over fixed tiles of kPartTile rows:
 //   hist    per tile, a shared-memory histogram of the digits, written to a
@@ -10,15 +10,15 @@
 //   scan    one device-wide exclusive scan of that array, which turns every
 //           (tile, digit) count into the global output offset of that tile's
 //           run of the digit (segments stay contiguous and in order);
-//   scatter per tile, rank each row within its digit with a shared-memory
-//           atomic, stage the tile in shared memory grouped by digit, then
-//           write each digit run to its global offset with consecutive
-//           threads on consecutive addresses (coalesced runs instead of one
-//           scattered 8-byte store per row).
+//   scatter per tile, place each row behind its digit's run with a
+//           shared-memory atomic, staging the tile in shared memory grouped by
+//           digit, then write each digit run to its global offset with
+//           consecutive threads on consecutive addresses (coalesced runs
+//           instead of one scattered 8-byte store per row).
 // The first pass reads the raw key column (row ids are implicit), applies the
 // probe-side range test (a probe key outside [min_R, max_R] cannot match and
-// is dropped here) and the frame-of-reference narrowing; later passes read the
-// (key', row) pairs of the previous pass.
+// is dropped here), the frame-of-reference narrowing and the key mix; later
+// passes read the (mixed key', row) pairs of the previous pass.
 #include <cstdio>
 #include <type_traits>
 
@@ -56,16 +56,18 @@ struct PartPass {
     KeyT* out_key;
     uint32_t* out_idx;
     uint32_t n;              // pass 1: rows
-    KeyRange rng;
-    int check_range;
-    int dshift;              // digit = (hash >> dshift) & dmask
+    uint64_t offset;         // pass 1: key' = key - offset (modulo the key's width),
+    uint64_t span;           // rows with key' > span are dropped
+    int dshift;              // digit = (key' >> dshift) & dmask
     uint32_t dmask;
     int bits;
+    int kbits;               // hash partitioning: bits of the key mix
     uint32_t* counts;
     const Tile* tiles;       // nullptr: pass-1 tiling of [0, n)
     const uint32_t* ntiles_dev;
     uint32_t ntiles_fixed;
     ColCarry cc;
+    int col_apart;           // hash scatter: the first column batch has a stage of its own
     // Exclusive ends of the memory a tile load may read around its rows (key
     // source, tuple-ID source); the arrays' bases are the starts. A tile whose
     // 16-byte aligned cover [align_down(first), align_up(last + 1)) lies
@@ -90,14 +92,11 @@ __device__ __forceinline__ size_t count_index(const Tile& tl, uint32_t t, uint32
     return ((size_t)tl.tile_base << bits) + (size_t)d * tl.ntiles_seg + (t - tl.tile_base);
 }
 
-// Partition digit: bits of the mixed key (hash partitioning) or, for the
-// sort, bits of the encoded key itself.
-template <bool SORTM, typename KeyT>
+// Partition digit: bits of the carried key (mixed by pass 1 for hash
+// partitioning, the encoded key itself for the sort).
+template <typename KeyT>
 __device__ __forceinline__ uint32_t digit_of(KeyT k, int dshift, uint32_t dmask) {
-    if constexpr (SORTM)
-        return (uint32_t)(k >> dshift) & dmask;
-    else
-        return (uint32_t)(KeyCodec<KeyT>::hash(k) >> dshift) & dmask;
+    return (uint32_t)(k >> dshift) & dmask;
 }
 
 // Exclusive scan of in[0, n) into out[0, n), n <= kPartItems * blockDim.x.
@@ -152,7 +151,8 @@ struct PassIn {
     static constexpr uint32_t kPad = 32 / sizeof(E);  // room for the 16-byte lead and tail of a cover copy
     static constexpr size_t kKeyBytes = align_up((kPartTile + kPad) * sizeof(E), 16);
     static constexpr size_t kIdxBytes = FIRST ? 0 : align_up((kPartTile + 8) * sizeof(uint32_t), 16);
-    static constexpr size_t kBufBytes = kKeyBytes + kIdxBytes;
+    // one ring buffer, with or without the tuple IDs of a later pass
+    __host__ __device__ static constexpr size_t buf_bytes(bool rows) { return kKeyBytes + (rows ? kIdxBytes : 0); }
 };
 
 // Shared-memory tile ring: two input buffers, each filled by TMA bulk copies
@@ -268,16 +268,20 @@ __device__ __forceinline__ void issue_tile(const TileRing<InKey, KeyT, FIRST>& r
     }
 }
 
-// Decodes element e of the current tile: applies the range test and the
-// narrowing in pass 1. Returns false for a dropped row.
-template <typename InKey, typename KeyT, bool FIRST>
+// Decodes element e of the current tile: applies the range test, the narrowing
+// and (hash partitioning) the mix in pass 1. Returns false for a dropped row.
+template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
 __device__ __forceinline__ bool tile_key(const PartPass<InKey, KeyT>& a,
                                          const typename PassIn<InKey, KeyT, FIRST>::E* kbuf, uint32_t e,
                                          KeyT& k) {
     if constexpr (FIRST) {
-        const int64_t key = (int64_t)kbuf[e];
-        if (a.check_range && (key < a.rng.lo || key > a.rng.hi)) return false;
-        k = KeyCodec<KeyT>::encode(key, a.rng.offset);
+        // offset from the build minimum; a key outside [min, max] has one
+        // beyond the span (compared in the input's width)
+        using U = typename std::conditional<sizeof(InKey) == 4, uint32_t, uint64_t>::type;
+        const U d = (U)kbuf[e] - (U)a.offset;
+        if (d > (U)a.span) return false;
+        k = (KeyT)d;
+        if constexpr (!SORTM) k = KeyCodec<KeyT>::mix(k, a.kbits);
     } else {
         k = kbuf[e];
     }
@@ -285,12 +289,12 @@ __device__ __forceinline__ bool tile_key(const PartPass<InKey, KeyT>& a,
 }
 
 template <typename InKey, typename KeyT, bool FIRST>
-__device__ __forceinline__ TileRing<InKey, KeyT, FIRST> ring_setup(unsigned char* smem, size_t off) {
+__device__ __forceinline__ TileRing<InKey, KeyT, FIRST> ring_setup(unsigned char* smem, size_t off, bool rows) {
     using P = PassIn<InKey, KeyT, FIRST>;
     TileRing<InKey, KeyT, FIRST> r;
     r.bar = reinterpret_cast<uint64_t*>(smem);
     r.buf[0] = smem + off;
-    r.buf[1] = smem + off + P::kBufBytes;
+    r.buf[1] = smem + off + P::buf_bytes(rows);
     if (threadIdx.x == 0) {
         mbar_init(&r.bar[0], 1);
         mbar_init(&r.bar[1], 1);
@@ -313,7 +317,7 @@ __device__ void ring_abort(const TileRing<InKey, KeyT, FIRST>& r, int other, uin
 template <typename InKey, typename KeyT, bool FIRST>
 __host__ __device__ constexpr size_t hist_smem_bytes(int bits) {
     return align_up(16 + 2 * ((size_t)1 << bits) * sizeof(uint32_t), 16) +
-           2 * PassIn<InKey, KeyT, FIRST>::kBufBytes;
+           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(false);
 }
 
 // Two CTA barriers per tile: the digit counters are double-buffered by tile
@@ -325,7 +329,7 @@ __global__ void __launch_bounds__(kPartThreads) part_hist_kernel(PartPass<InKey,
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t nd = 1u << a.bits;
     uint32_t* s_cnt2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd]
-    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, align_up(16 + 2 * (size_t)nd * 4, 16));
+    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, align_up(16 + 2 * (size_t)nd * 4, 16), false);
     __syncthreads();
     const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
     uint32_t t = blockIdx.x;
@@ -353,8 +357,8 @@ __global__ void __launch_bounds__(kPartThreads) part_hist_kernel(PartPass<InKey,
 #pragma unroll 4
         for (uint32_t e = threadIdx.x; e < tl.len; e += kPartThreads) {
             KeyT k;
-            if (tile_key<InKey, KeyT, FIRST>(a, kbuf, e, k))
-                atomicAdd(&s_cnt[digit_of<SORTM>(k, a.dshift, a.dmask)], 1u);
+            if (tile_key<InKey, KeyT, FIRST, SORTM>(a, kbuf, e, k))
+                atomicAdd(&s_cnt[digit_of(k, a.dshift, a.dmask)], 1u);
         }
         __syncthreads();
         for (uint32_t d = threadIdx.x; d < nd; d += blockDim.x)
@@ -362,28 +366,36 @@ __global__ void __launch_bounds__(kPartThreads) part_hist_kernel(PartPass<InKey,
     }
 }
 
+// Ring and stage of the hash scatter: keys, with tuple IDs beside them (pass 1:
+// as 16-bit rows of the tile), and a batch of carried columns (8 bytes per
+// row), apart from the keys or in their place.
 template <typename InKey, typename KeyT, bool FIRST>
-__host__ __device__ constexpr size_t scatter_smem_bytes(int bits) {
+__host__ __device__ constexpr size_t scatter_smem_bytes(int bits, bool rows, bool cols, bool col_apart) {
+    const size_t key_stage = sizeof(KeyT) + (rows ? (FIRST ? 2 : 4) : 0);
+    const size_t stage = !cols ? key_stage : col_apart ? key_stage + 8 : key_stage > 8 ? key_stage : 8;
     return align_up(16 + 4 * ((size_t)1 << bits) * sizeof(uint32_t), 16) +
-           2 * PassIn<InKey, KeyT, FIRST>::kBufBytes + align_up((size_t)kPartTile * sizeof(KeyT), 16) +
-           (size_t)kPartTile * sizeof(uint32_t) + (size_t)kPartTile * sizeof(uint16_t);
+           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(rows) + (size_t)kPartTile * stage;
 }
+
+// Shared memory that lets two CTAs of a kernel share an SM.
+constexpr size_t kTwoPerSm = 113 * 1024;
 
 // Digits a thread owns in the per-tile offset table (prefetched one tile ahead).
 constexpr int kGoffPerThread = (1 << kMaxBits) / kPartThreads;
 
 constexpr int kPartWarps = kPartThreads / kWarp;
+constexpr int kDigitBits1 = 9;  // radix bits with one digit per thread
+static_assert((1 << kDigitBits1) == kPartThreads, "one digit per thread");
 constexpr int kWarpRows = kPartTile / kPartWarps;  // sort scatter: consecutive rows per warp
 static_assert(kWarpRows == kPartItems * kWarp, "sort tiles are warp-blocked");
 
-// Block-collective: moves one carried column of the current tile to the
-// output positions of its rows. Row j of this thread (tile element e_j, digit
-// and rank in dr[j]) is staged at its tile position, then every digit run is
-// written out with consecutive threads on consecutive addresses, like the
-// keys. Hash mode: e_j = j * threads + t, position = start[d] + rank. Sort
-// mode: e_j = warp * kWarpRows + j * 32 + lane, position = start[d] +
-// (rows of digit d in earlier warps) + rank.
-template <bool SORTM, typename V, typename DigT>
+// Block-collective (sort scatter): moves one carried column of the current
+// tile to the output positions of its rows. Row j of this thread (tile element
+// w * kWarpRows + j * 32 + lane, digit and rank in dr[j]) is staged at its tile
+// position start[d] + (rows of digit d in earlier warps) + rank, then every
+// digit run is written out with consecutive threads on consecutive addresses,
+// like the keys.
+template <typename V, typename DigT>
 __device__ __forceinline__ void carry_column(const V* __restrict__ src, V* __restrict__ dst,
                                              const uint32_t (&dr)[kPartItems], const uint16_t* s_wc, uint32_t nd,
                                              const uint32_t* s_start, const uint32_t* s_goff, const DigT* s_dig,
@@ -394,15 +406,8 @@ __device__ __forceinline__ void carry_column(const V* __restrict__ src, V* __res
     for (int j = 0; j < kPartItems; ++j) {
         if (dr[j] != kNoDigit) {
             const uint32_t d = dr[j] & 0xFFFu;
-            uint32_t e, pos;
-            if constexpr (SORTM) {
-                e = w * kWarpRows + j * kWarp + lane;
-                pos = s_start[d] + s_wc[w * nd + d] + (dr[j] >> 12);
-            } else {
-                e = j * kPartThreads + threadIdx.x;
-                pos = s_start[d] + (dr[j] >> 12);
-            }
-            s_col[pos] = __ldcs(src + e);
+            const uint32_t e = w * kWarpRows + j * kWarp + lane;
+            s_col[s_start[d] + s_wc[w * nd + d] + (dr[j] >> 12)] = __ldcs(src + e);
         }
     }
     __syncthreads();
@@ -413,24 +418,100 @@ __device__ __forceinline__ void carry_column(const V* __restrict__ src, V* __res
     __syncthreads();
 }
 
-// Every thread: asks L2 to fetch the carried columns of tile `tl` (one
-// 128-byte line per thread and step), a tile ahead of carry_columns reading
-// them, so the carry does not wait on DRAM. Addresses stay inside the tile.
-// Used in later passes only: measured on GB300, it cut the pass-2 scatters by
-// 0.1-0.3 ms but slowed the pass-1 scatters (which stream the caller's
-// columns beside the TMA key loads) by 0.7-1.0 ms on the wide, group-by and
-// star workloads.
-__device__ __forceinline__ void prefetch_columns(const ColCarry& cc, const Tile& tl) {
-#pragma unroll 1
-    for (int c = 0; c < cc.n; ++c) {
-        const char* base = static_cast<const char*>(cc.in[c]) + (size_t)tl.start * cc.bytes[c];
-        const uint32_t bytes = tl.len * (uint32_t)cc.bytes[c];
-        for (uint32_t off = threadIdx.x * 128u; off < bytes; off += blockDim.x * 128u)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
+// Carried columns travel in batches of at most 8 bytes per row: one 8-byte
+// column, or one or two 4-byte ones. Returns the first column after the batch
+// that starts at c.
+__device__ __forceinline__ int batch_end(const ColCarry& cc, int c) {
+    return c + 1 < cc.n && cc.bytes[c] == 4 && cc.bytes[c + 1] == 4 ? c + 2 : c + 1;
+}
+
+// Columns [c, ce) of the current tile: a thread's rows read in tile order into
+// registers (issued before the barrier that precedes their staging), staged at
+// their tile positions, and written to the output positions g of the stage
+// entries. v[0], v[1]: the halves of an 8-byte value, or two 4-byte columns.
+__device__ __forceinline__ void load_batch(const ColCarry& cc, int c, int ce, const Tile& tl,
+                                           uint32_t (&v)[2][kPartItems]) {
+    if (cc.bytes[c] == 8) {
+        const uint2* src = static_cast<const uint2*>(cc.in[c]) + tl.start + threadIdx.x;
+#pragma unroll
+        for (int j = 0; j < kPartItems; ++j)
+            if (j * kPartThreads + threadIdx.x < tl.len) {
+                const uint2 x = __ldcs(src + j * kPartThreads);
+                v[0][j] = x.x;
+                v[1][j] = x.y;
+            }
+        return;
+    }
+    const uint32_t* s0 = static_cast<const uint32_t*>(cc.in[c]) + tl.start + threadIdx.x;
+    const uint32_t* s1 = static_cast<const uint32_t*>(cc.in[ce - 1]) + tl.start + threadIdx.x;
+#pragma unroll
+    for (int j = 0; j < kPartItems; ++j)
+        if (j * kPartThreads + threadIdx.x < tl.len) v[0][j] = __ldcs(s0 + j * kPartThreads);
+    if (ce - c == 2) {
+#pragma unroll
+        for (int j = 0; j < kPartItems; ++j)
+            if (j * kPartThreads + threadIdx.x < tl.len) v[1][j] = __ldcs(s1 + j * kPartThreads);
     }
 }
 
-template <bool SORTM, typename DigT>
+__device__ __forceinline__ void stage_batch(const ColCarry& cc, int c, int ce, const uint32_t (&pos)[kPartItems],
+                                            const uint32_t (&v)[2][kPartItems], unsigned char* stage) {
+    if (cc.bytes[c] == 8) {
+        uint2* s = reinterpret_cast<uint2*>(stage);
+#pragma unroll
+        for (int j = 0; j < kPartItems; ++j)
+            if (pos[j] != kNoDigit) s[pos[j]] = make_uint2(v[0][j], v[1][j]);
+        return;
+    }
+    uint32_t* s = reinterpret_cast<uint32_t*>(stage);
+#pragma unroll
+    for (int j = 0; j < kPartItems; ++j)
+        if (pos[j] != kNoDigit) s[pos[j]] = v[0][j];
+    if (ce - c == 2) {
+        s += kPartTile;
+#pragma unroll
+        for (int j = 0; j < kPartItems; ++j)
+            if (pos[j] != kNoDigit) s[pos[j]] = v[1][j];
+    }
+}
+
+__device__ __forceinline__ void write_batch(const ColCarry& cc, int c, int ce, const uint32_t (&g)[kPartItems],
+                                            uint32_t nk, const unsigned char* stage) {
+    if (cc.bytes[c] == 8) {
+        const uint2* s = reinterpret_cast<const uint2*>(stage);
+        uint2* dst = static_cast<uint2*>(cc.out[c]);
+#pragma unroll
+        for (int i = 0; i < kPartItems; ++i) {
+            const uint32_t q = i * kPartThreads + threadIdx.x;
+            if (q < nk) dst[g[i]] = s[q];
+        }
+        return;
+    }
+    const uint32_t* s = reinterpret_cast<const uint32_t*>(stage);
+#pragma unroll 1
+    for (; c < ce; ++c, s += kPartTile) {
+        uint32_t* dst = static_cast<uint32_t*>(cc.out[c]);
+#pragma unroll
+        for (int i = 0; i < kPartItems; ++i) {
+            const uint32_t q = i * kPartThreads + threadIdx.x;
+            if (q < nk) dst[g[i]] = s[q];
+        }
+    }
+}
+
+// One thread: asks L2 to fetch the carried columns of tile `tl`, a tile ahead
+// of its loads (the 16-byte aligned part of each column's rows).
+__device__ __forceinline__ void prefetch_columns(const ColCarry& cc, const Tile& tl) {
+#pragma unroll 1
+    for (int c = 0; c < cc.n; ++c) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(cc.in[c]) + (size_t)tl.start * cc.bytes[c];
+        const uintptr_t lo = (a + 15) & ~(uintptr_t)15, hi = (a + tl.len * (uint32_t)cc.bytes[c]) & ~(uintptr_t)15;
+        if (hi > lo)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((uint32_t)(hi - lo)) : "memory");
+    }
+}
+
+template <typename DigT>
 __device__ __forceinline__ void carry_columns(const ColCarry& cc, uint32_t tstart, const uint32_t (&dr)[kPartItems],
                                               const uint16_t* s_wc, uint32_t nd, const uint32_t* s_start,
                                               const uint32_t* s_goff, const DigT* s_dig, uint32_t nk,
@@ -438,141 +519,227 @@ __device__ __forceinline__ void carry_columns(const ColCarry& cc, uint32_t tstar
 #pragma unroll 1
     for (int c = 0; c < cc.n; ++c) {
         if (cc.bytes[c] == 4)
-            carry_column<SORTM>(static_cast<const uint32_t*>(cc.in[c]) + tstart, static_cast<uint32_t*>(cc.out[c]),
-                                dr, s_wc, nd, s_start, s_goff, s_dig, nk, static_cast<uint32_t*>(s_stage));
+            carry_column(static_cast<const uint32_t*>(cc.in[c]) + tstart, static_cast<uint32_t*>(cc.out[c]), dr, s_wc,
+                         nd, s_start, s_goff, s_dig, nk, static_cast<uint32_t*>(s_stage));
         else
-            carry_column<SORTM>(static_cast<const unsigned long long*>(cc.in[c]) + tstart,
-                                static_cast<unsigned long long*>(cc.out[c]), dr, s_wc, nd, s_start, s_goff, s_dig,
-                                nk, static_cast<unsigned long long*>(s_stage));
+            carry_column(static_cast<const unsigned long long*>(cc.in[c]) + tstart,
+                         static_cast<unsigned long long*>(cc.out[c]), dr, s_wc, nd, s_start, s_goff, s_dig, nk,
+                         static_cast<unsigned long long*>(s_stage));
     }
 }
 
-// The global digit offsets are double-buffered by tile parity, so no barrier
-// follows the write-out: the next tile stores its offsets into the other
-// buffer while slower threads still write the current tile out.
-// At most 64 registers (two CTAs per SM wherever shared memory allows; 64-bit
-// keys otherwise take ~100).
-template <typename InKey, typename KeyT, bool FIRST>
+// Global offset and row count of a tile's digits, DPT consecutive groups of 32
+// digits per warp (lane l of warp w owns digits (w * DPT + q) * 32 + l). The
+// count is the distance to the next entry of the scanned counts: the next
+// tile's run of the digit, the next digit's first tile, the next segment, or
+// the total behind the last entry.
+template <int DPT>
+struct TileDigits {
+    uint32_t goff[DPT], cnt[DPT];
+    __device__ static uint32_t digit(int q) {
+        return ((threadIdx.x / kWarp) * DPT + q) * kWarp + lane_id();
+    }
+    __device__ __forceinline__ void load(const uint32_t* __restrict__ counts, const Tile& tl, uint32_t t, int bits) {
+#pragma unroll
+        for (int q = 0; q < DPT; ++q) {
+            const uint32_t d = digit(q);
+            goff[q] = cnt[q] = 0;
+            if (d >> bits) continue;
+            const uint32_t* p = counts + count_index(tl, t, d, bits);
+            goff[q] = p[0];
+            cnt[q] = p[1] - goff[q];
+        }
+    }
+    // Before the barrier: this warp's rows, for the warps behind it.
+    __device__ __forceinline__ void warp_total(uint32_t* s_wtot) const {
+        uint32_t v = 0;
+#pragma unroll
+        for (int q = 0; q < DPT; ++q) v += cnt[q];
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane_id() == 0) s_wtot[threadIdx.x / kWarp] = v;
+    }
+    // After it: the tile position of every digit's first row into s_pos, global
+    // offset minus tile position into s_goff; returns the tile's rows.
+    __device__ __forceinline__ uint32_t place(const uint32_t* s_wtot, uint32_t* s_pos, uint32_t* s_goff,
+                                              int bits) const {
+        const unsigned lane = lane_id();
+        const int w = threadIdx.x / kWarp;
+        const uint32_t v = lane < kPartWarps ? s_wtot[lane] : 0u;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, v);
+        uint32_t run = __reduce_add_sync(0xffffffffu, (int)lane < w ? v : 0u);
+#pragma unroll
+        for (int q = 0; q < DPT; ++q) {
+            uint32_t x = cnt[q];
+#pragma unroll
+            for (int o = 1; o < kWarp; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if ((int)lane >= o) x += y;
+            }
+            const uint32_t d = digit(q), pos = run + x - cnt[q];
+            if (!(d >> bits)) {
+                s_pos[d] = pos;
+                s_goff[d] = goff[q] - pos;
+            }
+            run += __shfl_sync(0xffffffffu, x, kWarp - 1);
+        }
+        return total;
+    }
+};
+
+// Scatter of one hash-partitioning pass. The scanned counts already hold every
+// tile's digit runs, so the tile positions of the runs are known before its
+// rows are read: one shared-memory atomic per row gives the row's place in the
+// digit-sorted stage, and two CTA barriers separate a tile's staging from its
+// write-out (plus two per further batch of carried columns). The positions of
+// the next tile are laid out (double-buffered) while this one is written. A
+// row's digit is read back from the staged key, whose mix already happened in
+// pass 1; the global positions of a thread's rows are computed once and serve
+// the tuple IDs and every carried column.
+//
+// What bounds it: shared-memory wavefronts (about 22 per 32 rows with one
+// 8-byte column: the rank atomics, and staging at random positions) and issue
+// slots, each near 60 %, with DRAM at 55 %; it had taken about 38 (the rank's
+// start looked up per use, a digit array beside the keys) and eight barriers
+// per tile. Measured on GB300: 20M random 64-bit keys, 5 + 6 bits, 164 + 174 ->
+// 88 + 125 us; 28M narrowed keys, 6 + 6 bits, 138 + 130 -> 105 + 106 us; 2^28
+// rows with two 4-byte columns, 6 + 6 bits, 2.13 + 1.93 -> 1.60 + 1.60 ms; 30M
+// 64-bit keys with a 4-byte column, 6 + 6 bits, 322 + 297 -> 226 + 184 us.
+//
+// At most 64 registers: two CTAs per SM wherever shared memory allows.
+template <typename InKey, typename KeyT, bool FIRST, int DPT, bool COLS>
 __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<InKey, KeyT> a, unsigned* err) {
     using Ring = TileRing<InKey, KeyT, FIRST>;
     using P = PassIn<InKey, KeyT, FIRST>;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ uint32_t s_warp[kPartThreads / kWarp];
-    __shared__ uint32_t s_kept;
+    __shared__ uint32_t s_wtot[kPartWarps];
     const uint32_t nd = 1u << a.bits;
     const bool rows = a.out_idx != nullptr;  // tuple IDs travel with the keys
-    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(smem + 16);
-    uint32_t* s_start = s_cnt + nd;
-    uint32_t* s_goff2 = s_start + nd;  // [2][nd]
+    uint32_t* s_pos2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd]
+    uint32_t* s_goff2 = s_pos2 + 2 * nd;                        // [2][nd]
     const size_t ring_off = align_up(16 + 4 * (size_t)nd * 4, 16);
-    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, ring_off);
-    KeyT* s_key = reinterpret_cast<KeyT*>(smem + ring_off + 2 * P::kBufBytes);
-    uint32_t* s_idx = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(s_key) +
-                                                  align_up((size_t)kPartTile * sizeof(KeyT), 16));
-    uint16_t* s_dig = reinterpret_cast<uint16_t*>(s_idx + kPartTile);
+    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, ring_off, rows);
+    KeyT* s_key = reinterpret_cast<KeyT*>(smem + ring_off + 2 * P::buf_bytes(rows));
+    static_assert(kPartTile <= 65536, "a row of a tile fits 16 bits");
+    using RowT = typename std::conditional<FIRST, uint16_t, uint32_t>::type;  // pass 1: row in the tile
+    RowT* s_idx = reinterpret_cast<RowT*>(s_key + kPartTile);
+    unsigned char* col_stage =
+        reinterpret_cast<unsigned char*>(s_key) + (a.col_apart ? (size_t)kPartTile * sizeof(KeyT) : 0);
     __syncthreads();
 
     const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
     uint32_t t = blockIdx.x;
-    // Global offsets of this CTA's first tile; later ones are loaded one tile
-    // ahead into registers (thread i owns digits i, i + blockDim, ...).
-    uint32_t goff[kGoffPerThread] = {};
-    Tile tl_cur;
-    if (t < ntiles) {
-        tl_cur = get_tile(a, t);
-#pragma unroll
-        for (int q = 0; q < kGoffPerThread; ++q) {
-            const uint32_t d = threadIdx.x + q * kPartThreads;
-            if (d < nd) goff[q] = a.counts[count_index(tl_cur, t, d, a.bits)];
-        }
+    if (t >= ntiles) return;
+    Tile tl = get_tile(a, t);
+    Tile tl_next{};
+    TileDigits<DPT> dg;
+    dg.load(a.counts, tl, t, a.bits);
+    if (threadIdx.x < kWarp) issue_tile(ring, a, tl, 0);
+    dg.warp_total(s_wtot);
+    __syncthreads();
+    uint32_t nk = dg.place(s_wtot, s_pos2, s_goff2, a.bits);
+    if (t + gridDim.x < ntiles) {
+        tl_next = get_tile(a, t + gridDim.x);
+        dg.load(a.counts, tl_next, t + gridDim.x, a.bits);
     }
-    Tile d_next{};  // warp 0: descriptor of the next tile to issue, loaded one tile early
-    if (threadIdx.x < kWarp) {
-        if (t < ntiles) issue_tile(ring, a, tl_cur, 0);
-        if (t + gridDim.x < ntiles) d_next = get_tile(a, t + gridDim.x);
-    }
+    __syncthreads();
+
     for (uint32_t it = 0; t < ntiles; t += gridDim.x, ++it) {
         const int b = it & 1;
         const uint32_t tn = t + gridDim.x;
-        if (threadIdx.x < kWarp && tn < ntiles) {
-            issue_tile(ring, a, d_next, b ^ 1);
-            if (tn + gridDim.x < ntiles) d_next = get_tile(a, tn + gridDim.x);
-        }
-        uint32_t* s_goff = s_goff2 + b * nd;
-        for (uint32_t d = threadIdx.x; d < nd; d += blockDim.x) s_cnt[d] = 0;
-#pragma unroll
-        for (int q = 0; q < kGoffPerThread; ++q) {
-            const uint32_t d = threadIdx.x + q * kPartThreads;
-            if (d < nd) s_goff[d] = goff[q];
+        const bool more = tn < ntiles;
+        if (threadIdx.x < kWarp && more) issue_tile(ring, a, tl_next, b ^ 1);
+        if constexpr (COLS)
+            if (threadIdx.x == kWarp && more) prefetch_columns(a.cc, tl_next);
+        uint32_t* s_pos = s_pos2 + b * nd;
+        const uint32_t* s_goff = s_goff2 + b * nd;
+        int c = 0, ce = 0;
+        uint32_t val[2][kPartItems];  // a batch of column values of this thread's tile rows
+        if constexpr (COLS) {
+            ce = batch_end(a.cc, 0);
+            if (a.col_apart) load_batch(a.cc, 0, ce, tl, val);
         }
         const bool ok = mbar_wait(&ring.bar[b], (it >> 1) & 1);
+        const auto* kbuf = ring.keys(b) + lead_of(Ring::key_src(a, tl.start));
+        uint32_t pos[kPartItems];  // tile position, or kNoDigit for a dropped row
+        if (ok) {
+            const uint32_t* rbuf = nullptr;
+            if constexpr (!FIRST)
+                if (rows) rbuf = ring.rows(b) + lead_of(a.in_idx + tl.start);
+            KeyT kk[kPartItems];
+#pragma unroll
+            for (int j = 0; j < kPartItems; ++j) {
+                const uint32_t e = j * kPartThreads + threadIdx.x;
+                pos[j] = kNoDigit;
+                if (e < tl.len && tile_key<InKey, KeyT, FIRST, false>(a, kbuf, e, kk[j])) pos[j] = 0;
+            }
+#pragma unroll
+            for (int j = 0; j < kPartItems; ++j)
+                if (pos[j] != kNoDigit) pos[j] = atomicAdd(&s_pos[digit_of(kk[j], a.dshift, a.dmask)], 1u);
+#pragma unroll
+            for (int j = 0; j < kPartItems; ++j) {
+                if (pos[j] == kNoDigit) continue;
+                s_key[pos[j]] = kk[j];
+                if (rows) {
+                    const uint32_t e = j * kPartThreads + threadIdx.x;
+                    s_idx[pos[j]] = FIRST ? (RowT)e : (RowT)rbuf[e];
+                }
+            }
+        }
+        if (more) dg.warp_total(s_wtot);
+        if constexpr (COLS) {
+            if (a.col_apart) {
+                if (ok) stage_batch(a.cc, 0, ce, pos, val, col_stage);
+            } else {
+                load_batch(a.cc, 0, ce, tl, val);
+            }
+        }
         if (__syncthreads_or(!ok)) {
-            ring_abort(ring, b ^ 1, ((it + 1) >> 1) & 1, tn < ntiles, err);
+            ring_abort(ring, b ^ 1, ((it + 1) >> 1) & 1, more, err);
             return;
         }
-        const Tile tl = tl_cur;
-        if (tn < ntiles) {  // next tile's offsets, consumed next iteration
-            tl_cur = get_tile(a, tn);
-            if constexpr (!FIRST)
-                if (a.cc.n) prefetch_columns(a.cc, tl_cur);
-#pragma unroll
-            for (int q = 0; q < kGoffPerThread; ++q) {
-                const uint32_t d = threadIdx.x + q * kPartThreads;
-                if (d < nd) goff[q] = a.counts[count_index(tl_cur, tn, d, a.bits)];
+        uint32_t nk_next = 0;
+        Tile tl_after{};
+        if (more) {
+            nk_next = dg.place(s_wtot, s_pos2 + (b ^ 1) * nd, s_goff2 + (b ^ 1) * nd, a.bits);
+            if (tn + gridDim.x < ntiles) {
+                tl_after = get_tile(a, tn + gridDim.x);
+                dg.load(a.counts, tl_after, tn + gridDim.x, a.bits);
             }
         }
-        const auto* kbuf = ring.keys(b) + lead_of(Ring::key_src(a, tl.start));
-        const uint32_t* rbuf = nullptr;
-        if constexpr (!FIRST)
-            if (rows) rbuf = ring.rows(b) + lead_of(a.in_idx + tl.start);
-
-        KeyT kk[kPartItems];
-        uint32_t dr[kPartItems];  // (rank << 12) | digit, or kNoDigit
+        uint32_t g[kPartItems];  // output positions of stage entries tid, tid + threads, ...
 #pragma unroll
-        for (int j = 0; j < kPartItems; ++j) {
-            const uint32_t e = j * kPartThreads + threadIdx.x;
-            dr[j] = kNoDigit;
-            if (e < tl.len && tile_key<InKey, KeyT, FIRST>(a, kbuf, e, kk[j]))
-                dr[j] = digit_of<false>(kk[j], a.dshift, a.dmask);
-        }
-#pragma unroll
-        for (int j = 0; j < kPartItems; ++j)
-            if (dr[j] != kNoDigit) dr[j] |= atomicAdd(&s_cnt[dr[j]], 1u) << 12;
-        __syncthreads();
-
-        // s_goff becomes (global offset - tile offset) of each digit
-        const uint32_t kept = block_scan_smem(s_cnt, s_start, nd, s_warp, s_goff);
-        if (threadIdx.x == 0) s_kept = kept;
-        __syncthreads();
-
-#pragma unroll
-        for (int j = 0; j < kPartItems; ++j) {
-            if (dr[j] != kNoDigit) {
-                const uint32_t e = j * kPartThreads + threadIdx.x;
-                const uint32_t d = dr[j] & 0xFFFu;
-                const uint32_t pos = s_start[d] + (dr[j] >> 12);
-                s_key[pos] = kk[j];
-                s_dig[pos] = (uint16_t)d;
-                if (rows) s_idx[pos] = FIRST ? tl.start + e : rbuf[e];
+        for (int i = 0; i < kPartItems; ++i) {
+            const uint32_t q = i * kPartThreads + threadIdx.x;
+            if (q < nk) {
+                const KeyT k = s_key[q];
+                g[i] = s_goff[digit_of(k, a.dshift, a.dmask)] + q;
+                a.out_key[g[i]] = k;
+                if (rows) a.out_idx[g[i]] = (FIRST ? tl.start : 0u) + s_idx[q];
             }
         }
-        __syncthreads();
-
-        // No barrier after the write-out: the next tile stores its offsets
-        // into the other s_goff buffer, and its staging writes come after
-        // three more barriers, which every thread reaches only once done here.
-        const uint32_t nk = s_kept;
-        for (uint32_t pos = threadIdx.x; pos < nk; pos += blockDim.x) {
-            const uint32_t d = s_dig[pos];
-            const uint32_t g = s_goff[d] + pos;
-            a.out_key[g] = s_key[pos];
-            if (rows) a.out_idx[g] = s_idx[pos];
+        if constexpr (COLS) {
+            if (a.col_apart) {
+                write_batch(a.cc, c, ce, g, nk, col_stage);
+                c = ce;
+                ce = c < a.cc.n ? batch_end(a.cc, c) : c;
+                if (ce > c) load_batch(a.cc, c, ce, tl, val);
+            }
+#pragma unroll 1
+            while (c < ce) {
+                __syncthreads();  // the stage's last contents are written out
+                stage_batch(a.cc, c, ce, pos, val, col_stage);
+                const int c0 = c, c1 = ce;
+                c = ce;
+                ce = c < a.cc.n ? batch_end(a.cc, c) : c;
+                if (ce > c) load_batch(a.cc, c, ce, tl, val);
+                __syncthreads();
+                write_batch(a.cc, c0, c1, g, nk, col_stage);
+            }
         }
-        // carried columns reuse the key and row staging (contiguous, >= 8 bytes per row)
-        if (a.cc.n) {
-            __syncthreads();
-            carry_columns<false>(a.cc, tl.start, dr, nullptr, nd, s_start, s_goff, s_dig, nk, s_key);
-        }
+        tl = tl_next;
+        tl_next = tl_after;
+        nk = nk_next;
+        __syncthreads();  // the stage and this tile's ring buffer are free
     }
 }
 
@@ -581,7 +748,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
 template <typename InKey, typename KeyT, bool FIRST>
 __host__ __device__ constexpr size_t sort_scatter_smem_bytes(int bits) {
     return align_up(16 + 3 * ((size_t)1 << bits) * sizeof(uint32_t), 16) +
-           2 * PassIn<InKey, KeyT, FIRST>::kBufBytes + align_up((size_t)kPartTile * sizeof(KeyT), 16) +
+           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(true) + align_up((size_t)kPartTile * sizeof(KeyT), 16) +
            (size_t)kPartTile * sizeof(uint32_t) + (size_t)kPartTile * sizeof(uint8_t) +
            (size_t)kPartWarps * ((size_t)1 << bits) * sizeof(uint16_t);
 }
@@ -606,8 +773,8 @@ __global__ void __launch_bounds__(kPartThreads, 2) sort_scatter_kernel(PartPass<
     uint32_t* s_start = s_cnt + nd;
     uint32_t* s_goff = s_start + nd;
     const size_t ring_off = align_up(16 + 3 * (size_t)nd * 4, 16);
-    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, ring_off);
-    KeyT* s_key = reinterpret_cast<KeyT*>(smem + ring_off + 2 * P::kBufBytes);
+    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, ring_off, true);
+    KeyT* s_key = reinterpret_cast<KeyT*>(smem + ring_off + 2 * P::buf_bytes(true));
     uint32_t* s_idx = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(s_key) +
                                                   align_up((size_t)kPartTile * sizeof(KeyT), 16));
     uint8_t* s_dig = reinterpret_cast<uint8_t*>(s_idx + kPartTile);
@@ -655,7 +822,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) sort_scatter_kernel(PartPass<
         if (tn < ntiles) {
             tl_cur = get_tile(a, tn);
             if constexpr (!FIRST)
-                if (a.cc.n) prefetch_columns(a.cc, tl_cur);
+                if (threadIdx.x == 0 && a.cc.n) prefetch_columns(a.cc, tl_cur);
 #pragma unroll
             for (int q = 0; q < kGoffPerThread; ++q) {
                 const uint32_t d = threadIdx.x + q * kPartThreads;
@@ -672,8 +839,8 @@ __global__ void __launch_bounds__(kPartThreads, 2) sort_scatter_kernel(PartPass<
 #pragma unroll
         for (int j = 0; j < kPartItems; ++j) {
             const uint32_t e = w * kWarpRows + j * kWarp + lane;
-            const bool v = e < tl.len && tile_key<InKey, KeyT, FIRST>(a, kbuf, e, kk[j]);
-            const uint32_t d = v ? digit_of<true>(kk[j], a.dshift, a.dmask) : kNoDigit;
+            const bool v = e < tl.len && tile_key<InKey, KeyT, FIRST, true>(a, kbuf, e, kk[j]);
+            const uint32_t d = v ? digit_of(kk[j], a.dshift, a.dmask) : kNoDigit;
             const unsigned peers = __match_any_sync(0xffffffffu, d);
             const uint32_t before = v ? s_wc[w * nd + d] : 0u;
             __syncwarp();
@@ -718,7 +885,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) sort_scatter_kernel(PartPass<
             if (rows) a.out_idx[g] = s_idx[pos];
         }
         __syncthreads();
-        if (a.cc.n) carry_columns<true>(a.cc, tl.start, dr, s_wc, nd, s_start, s_goff, s_dig, nk, s_key);
+        if (a.cc.n) carry_columns(a.cc, tl.start, dr, s_wc, nd, s_start, s_goff, s_dig, nk, s_key);
     }
 }
 
@@ -777,7 +944,8 @@ __global__ void __launch_bounds__(1024)
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-    scan_apply_kernel(uint32_t* __restrict__ data, ScanLen L, const uint32_t* __restrict__ block_sums) {
+    scan_apply_kernel(uint32_t* __restrict__ data, ScanLen L, const uint32_t* __restrict__ block_sums,
+                      const uint32_t* __restrict__ total) {
     __shared__ uint32_t s_buf[kScanChunk];
     __shared__ uint32_t s_warp[kScanThreads / kWarp];
     const size_t len = L.get();
@@ -824,6 +992,7 @@ __global__ void __launch_bounds__(kScanThreads)
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) data[beg + i] = s_buf[i];
+    if (threadIdx.x == 0 && beg + m == len) data[len] = *total;  // the end of the last run
 }
 
 // ------------------------------------------------------------ pass-2 tiling
@@ -934,7 +1103,7 @@ cudaError_t scan_counts(uint32_t* counts, ScanLen L, size_t max_len, uint32_t* b
     const uint32_t g = nblocks ? nblocks : 1;
     scan_reduce_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums);
     scan_blocksums_kernel<<<1, 1024, 0, stream>>>(block_sums, g, total);
-    scan_apply_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums);
+    scan_apply_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums, total);
     return cudaGetLastError();
 }
 
@@ -954,10 +1123,22 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
                      unsigned* err, const DevInfo& di, cudaStream_t stream, const char* side_name, int pass_no) {
     cudaError_t e;
     const size_t hsmem = hist_smem_bytes<InKey, KeyT, FIRST>(a.bits);
+    // The first batch of carried columns is staged beside the keys when no
+    // tuple IDs travel and two CTAs still fit an SM (2^28 rows, two 4-byte
+    // columns, 6 bits: 1.58 against 1.72 ms); not in a first pass of 8 bits or
+    // more, whose 2 x 256 output runs lie in as many pages at large sizes (600M
+    // rows, an 8-byte column: 5.4 against 4.7 ms; 3.3 ms with 7 bits).
+    a.col_apart = !SORTM && a.cc.n && !a.out_idx && (!FIRST || a.bits <= 7) &&
+                  scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits, false, true, true) <= kTwoPerSm;
     const size_t ssmem = SORTM ? sort_scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits)
-                               : scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits);
+                               : scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits, a.out_idx != nullptr, a.cc.n > 0, a.col_apart);
     auto hist = part_hist_kernel<InKey, KeyT, FIRST, SORTM>;
-    auto scat = SORTM ? sort_scatter_kernel<InKey, KeyT, FIRST> : part_scatter_kernel<InKey, KeyT, FIRST>;
+    auto scat = SORTM ? sort_scatter_kernel<InKey, KeyT, FIRST>
+                : a.bits <= kDigitBits1
+                    ? (a.cc.n ? part_scatter_kernel<InKey, KeyT, FIRST, 1, true>
+                              : part_scatter_kernel<InKey, KeyT, FIRST, 1, false>)
+                    : (a.cc.n ? part_scatter_kernel<InKey, KeyT, FIRST, kGoffPerThread, true>
+                              : part_scatter_kernel<InKey, KeyT, FIRST, kGoffPerThread, false>);
     if ((e = set_smem(hist, hsmem)) != cudaSuccess) return e;
     if ((e = set_smem(scat, ssmem)) != cudaSuccess) return e;
     const double n = (double)a.n;
@@ -1013,9 +1194,10 @@ cudaError_t partition_typed(const InKey* keys, uint32_t n, int side, const PlanD
     a.out_key = static_cast<KeyT*>(s.key[0]);
     a.out_idx = plan.no_rows ? nullptr : s.idx[0];
     a.n = n;
-    a.rng = plan.range;
-    a.check_range = side == 1 ? plan.check_range : 0;
+    a.offset = plan.range.offset;
+    a.span = side == 1 && plan.check_range ? (uint64_t)plan.range.hi - (uint64_t)plan.range.lo : ~0ull;
     a.dshift = KeyCodec<KeyT>::kBits - b1;
+    a.kbits = plan.kbits;
     a.dmask = (1u << b1) - 1u;
     a.bits = b1;
     a.counts = s.counts;
@@ -1042,8 +1224,6 @@ cudaError_t partition_typed(const InKey* keys, uint32_t n, int side, const PlanD
         b.out_key = static_cast<KeyT*>(s.key[1]);
         b.out_idx = plan.no_rows ? nullptr : s.idx[1];
         b.n = n;
-        b.rng = plan.range;
-        b.check_range = 0;
         b.dshift = KeyCodec<KeyT>::kBits - b1 - b2;
         b.dmask = (1u << b2) - 1u;
         b.bits = b2;
@@ -1082,8 +1262,8 @@ cudaError_t sort_typed(const InKey* keys, uint32_t n, int side, const PlanDev& p
     a.out_key = static_cast<KeyT*>(s.key[0]);
     a.out_idx = plan.no_rows ? nullptr : s.idx[0];
     a.n = n;
-    a.rng = plan.range;
-    a.check_range = side == 1 ? plan.check_range : 0;
+    a.offset = plan.range.offset;
+    a.span = side == 1 && plan.check_range ? (uint64_t)plan.range.hi - (uint64_t)plan.range.lo : ~0ull;
     a.dshift = 0;
     a.dmask = (1u << D) - 1u;
     a.bits = D;
@@ -1109,8 +1289,6 @@ cudaError_t sort_typed(const InKey* keys, uint32_t n, int side, const PlanDev& p
         b.out_key = static_cast<KeyT*>(s.key[i & 1]);
         b.out_idx = plan.no_rows ? nullptr : s.idx[i & 1];
         b.n = n;
-        b.rng = plan.range;
-        b.check_range = 0;
         b.dshift = i * D;
         b.dmask = (1u << D) - 1u;
         b.bits = D;
@@ -1141,7 +1319,7 @@ void part_side_layout(Carve& c, PartSide& ps, int64_t n, int b1, int b2, int pas
     const int nbuf = passes < 2 ? passes : 2;
     const int ncols = plan.gftr ? plan.ncols[side] : 0;
     for (int k = 0; k < 2; ++k) {
-        // 16 bytes of slack after each buffer: later tile and row loads may
+        // 16 bytes of slack after each buffer: a later pass's tile loads may
         // read the aligned cover of the last rows (see PartPass::src_end)
         ps.key[k] = k < nbuf ? c.take<unsigned char>((size_t)n * kb + 16) : nullptr;
         ps.idx[k] = k < nbuf ? c.take<uint32_t>((size_t)n + 4) : nullptr;
@@ -1151,7 +1329,7 @@ void part_side_layout(Carve& c, PartSide& ps, int64_t n, int b1, int b2, int pas
     }
     const size_t ntiles1 = (size_t)((n + kPartTile - 1) / kPartTile);
     ps.counts_len = sort ? ntiles1 << b1 : part_counts_len(n, b1, b2, passes);
-    ps.counts = c.take<uint32_t>(ps.counts_len);
+    ps.counts = c.take<uint32_t>(ps.counts_len + 1);  // and the total behind the last entry
     ps.block_sums = c.take<uint32_t>(part_scan_blocks(ps.counts_len));
     ps.total = c.take<uint32_t>(4);
     ps.segs = c.take<SegInfo>(sort ? 1 : (size_t)1 << b1);
