@@ -333,12 +333,14 @@ eiger_status eiger_groupby_workspace(int64_t n, eiger_dtype dtype, const eiger_a
  * eiger_groupby -- for every distinct key of d_keys[0, n) its aggregates.
  * Profiles the keys (min/max, HyperLogLog++; Sec. 4.1), narrows them to
  * uint32 offsets when their span allows (Sec. 4.3), then runs:
- *   EIGER_GB_AUTO: HASH when a table of 2.5x the estimated groups fits in half
- *          of the L2 cache, else PARTITION;
+ *   EIGER_GB_AUTO: HASH when a table of the estimated groups fits a CTA's
+ *          shared memory, or below 2^24 rows when a table of 2.5x the estimate
+ *          fits in half of the L2 cache; else PARTITION;
  *   EIGER_GB_HASH: slots = the power of two >= 2.5x the estimate (knobs may
  *          set table_slots);
  *   EIGER_GB_PARTITION: 2^B partitions with B = ceil(log2(estimate / 1024)),
- *          one pass up to 10 bits, else two (knobs may set bits1/bits2).
+ *          one pass up to 8 bits (10 below 2^25 rows), else two (knobs may set
+ *          bits1/bits2).
  * If a table overflows (an estimate far too low, or caller knobs too small)
  * the plan is enlarged and the group-by re-run; plan_used->attempts counts the
  * runs. Groups are written in unspecified order: d_out_keys (dtype, nullable

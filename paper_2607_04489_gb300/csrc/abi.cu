@@ -853,8 +853,8 @@ eiger_status eiger_join_wide(eiger_dtype dtype, const void* d_bkeys, int64_t nb,
 namespace {
 
 constexpr int kGbTargetGroups = 1024;          // groups per partition the PARTITION plan aims at
+constexpr int64_t kGbPartRows = 1ll << 24;      // rows from which PARTITION replaces a global HASH table
 constexpr int kGbMaxBits = 20;                  // most partition bits a retry grows to
-constexpr size_t kGbSmemBudget = 96 * 1024;     // CTA-private hash table limit
 
 unsigned long long pow2_at_least(double x) {
     unsigned long long s = 64;
@@ -866,8 +866,11 @@ unsigned long long pow2_at_least(double x) {
 // every row its own group.
 unsigned long long gb_max_slots(int64_t n) { return pow2_at_least(2.0 * (double)(n > 0 ? n : 1)); }
 
-void gb_split_bits(int B, int32_t* b1, int32_t* b2) {
-    if (B <= 10) {
+// One pass while its digits leave the tiles runs of some length and its output
+// pages stay few: always up to 8 bits, up to 10 below 2^25 rows (5M rows, 10
+// bits: one pass; 2^28 rows, 10 bits: 8.7 ms against 3.4 ms for 5 + 5), else two.
+void gb_split_bits(int B, int64_t n, int32_t* b1, int32_t* b2) {
+    if (B <= 8 || (B <= 10 && n < (1ll << 25))) {
         *b1 = B;
         *b2 = 0;
     } else {
@@ -923,7 +926,7 @@ size_t gb_workspace_bytes(int64_t n, int dtype, const eiger_aggs* aggs, int vari
         if (variant != EIGER_GB_HASH) {
             pd.variant = EIGER_GB_PARTITION;
             for (int B = 1; B <= kGbMaxBits; ++B) {
-                gb_split_bits(B, &pd.bits1, &pd.bits2);
+                gb_split_bits(B, n, &pd.bits1, &pd.bits2);
                 Carve d = c;
                 gb_layout(d, n, pd, cb, nc);
                 if (d.off > best) best = d.off;
@@ -989,10 +992,26 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
     const double est = kst.estimate > 1.0 ? kst.estimate : 1.0;
     const int keyb = pub.narrow ? 4 : 8;
     const unsigned long long hash_slots = pow2_at_least(2.5 * est);
+    GbAggs ga{};
+    ga.n = aggs->n;
+    for (int a = 0; a < aggs->n; ++a) {
+        ga.op[a] = aggs->op[a];
+        ga.vals[a] = aggs->vals[a];
+        ga.bytes[a] = aggs->bytes[a];
+        ga.out[a] = reinterpret_cast<long long*>(aggs->out[a]);
+    }
     int v = variant;
     if (v == EIGER_GB_AUTO) {
+        // HASH while its CTA tables fit shared memory. Beyond that its global
+        // table must fit half of L2, and is only the better one for fewer than
+        // kGbPartRows rows: atomics on L2 lines cost more per row than a pass
+        // over the rows, above all on hot groups, but take three launches
+        // instead of ten (int32, 25000 groups, SUM and MAX, ms HASH /
+        // PARTITION: 2M rows 0.19 / 0.24, 20M 0.63 / 0.52, 50M 1.49 / 0.93;
+        // 100M rows over 100000 skewed groups 14.4 / 2.7).
         const double table = (double)hash_slots * (keyb + 8.0 * aggs->n);
-        v = table <= (double)l2_bytes_or_default() / 2 ? EIGER_GB_HASH : EIGER_GB_PARTITION;
+        const bool in_l2 = table <= (double)l2_bytes_or_default() / 2;
+        v = gb_hash_slots(est, ga, pub.narrow != 0) || (in_l2 && n < kGbPartRows) ? EIGER_GB_HASH : EIGER_GB_PARTITION;
     }
     pub.variant = v;
     pub.selector = knobs ? 2 : 0;
@@ -1012,16 +1031,8 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
             pub.bits1 = knobs->bits1;
             pub.bits2 = knobs->bits2;
         } else {
-            gb_split_bits(B, &pub.bits1, &pub.bits2);
+            gb_split_bits(B, n, &pub.bits1, &pub.bits2);
         }
-    }
-    GbAggs ga{};
-    ga.n = aggs->n;
-    for (int a = 0; a < aggs->n; ++a) {
-        ga.op[a] = aggs->op[a];
-        ga.vals[a] = aggs->vals[a];
-        ga.bytes[a] = aggs->bytes[a];
-        ga.out[a] = reinterpret_cast<long long*>(aggs->out[a]);
     }
     int cb[kMaxCols];
     const int nc = gb_carried(aggs, cb);
@@ -1038,7 +1049,10 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
         pd.kbits = mix_bits(pd.key32, kst.min, kst.max);
         pd.slots = (unsigned long long)pub.table_slots;
         pd.naggs = aggs->n;
-        pd.smem = pd.variant == EIGER_GB_HASH && gb_smem_table_bytes(pd.slots, aggs->n, pd.key32) <= kGbSmemBudget;
+        if (pd.variant == EIGER_GB_HASH)
+            pd.smem_slots = gb_hash_slots(est, ga, pd.key32);
+        else
+            pd.part_slots = gb_part_slots(est / (double)(1ll << (pub.bits1 + pub.bits2)));
         Carve c = carve;
         const GbScratch sc = gb_layout(c, n, pd, cb, nc);
         if (c.off > ws_bytes)
@@ -1056,7 +1070,7 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
             pub.table_slots = (int64_t)(sl < max_slots ? sl : max_slots);
         } else if (pub.variant == EIGER_GB_PARTITION && pub.bits1 + pub.bits2 < kGbMaxBits) {
             int B = pub.bits1 + pub.bits2 + 2;
-            gb_split_bits(B < kGbMaxBits ? B : kGbMaxBits, &pub.bits1, &pub.bits2);
+            gb_split_bits(B < kGbMaxBits ? B : kGbMaxBits, n, &pub.bits1, &pub.bits2);
         } else {
             if (plan_used) *plan_used = pub;
             return fail(EIGER_ERR_TABLE_FULL, "group-by tables overflowed at the largest plan");

@@ -75,6 +75,8 @@ constexpr uint64_t inverse_mod_2_64(uint64_t a) {  // Newton: each step doubles 
 }
 constexpr uint32_t kMixA32 = 0x9E3779B1u, kMixB32 = 0x85EBCA6Bu;
 constexpr uint64_t kMixA64 = 0x9E3779B97F4A7C15ull, kMixB64 = 0xFF51AFD7ED558CCDull;
+constexpr uint32_t kMixA32Inv = (uint32_t)inverse_mod_2_64(kMixA32), kMixB32Inv = (uint32_t)inverse_mod_2_64(kMixB32);
+constexpr uint64_t kMixA64Inv = inverse_mod_2_64(kMixA64), kMixB64Inv = inverse_mod_2_64(kMixB64);
 
 // Key encodings.
 //  - encode, 32-bit: (uint32)(key - offset). offset = build minimum when the
@@ -108,8 +110,8 @@ struct KeyCodec<uint32_t> {
     }
     __host__ __device__ __forceinline__ static uint32_t unmix(uint32_t h, int kbits) {
         const int sh = 32 - kbits, s = (kbits + 1) >> 1;
-        const uint32_t y = ((h >> sh) * (uint32_t)inverse_mod_2_64(kMixB32)) << sh;
-        return ((((y ^ (y >> s)) >> sh) * (uint32_t)inverse_mod_2_64(kMixA32)) << sh) >> sh;
+        const uint32_t y = ((h >> sh) * kMixB32Inv) << sh;
+        return ((((y ^ (y >> s)) >> sh) * kMixA32Inv) << sh) >> sh;
     }
 };
 
@@ -125,8 +127,8 @@ struct KeyCodec<uint64_t> {
         return (y ^ (y >> 32)) * kMixB64;
     }
     __host__ __device__ __forceinline__ static uint64_t unmix(uint64_t h, int) {
-        const uint64_t y = h * inverse_mod_2_64(kMixB64);
-        return (y ^ (y >> 32)) * inverse_mod_2_64(kMixA64);
+        const uint64_t y = h * kMixB64Inv;
+        return (y ^ (y >> 32)) * kMixA64Inv;
     }
 };
 

@@ -9,11 +9,9 @@
 //
 // HASH: one global open-addressing table (linear probing, slots a power of two
 // sized from the estimate), keys claimed by CAS and aggregates updated by
-// global atomics. While the table is small enough, every CTA first aggregates
-// its rows in a private shared-memory copy of the same table (lanes of a warp
-// that hit the same slot are combined by their lowest lane before one shared
-// atomic), then merges its occupied slots into the global table; compaction
-// writes the occupied slots out.
+// global atomics. While the groups fit shared memory, every CTA first aggregates
+// its rows in a table of its own (CtaTable), then merges its groups into the
+// global table; compaction writes the occupied slots out.
 //
 // PARTITION: the keys are radix-partitioned on hash bits (Sec. 3.3 hashes
 // before partitioning so partitions are even) with the value columns carried
@@ -21,17 +19,27 @@
 // fit one shared-memory table; a persistent grid takes partitions from a
 // global counter, aggregates each in shared memory and writes its groups out.
 //
+// What bounds the CTA tables' row loop: the shared-memory latency and
+// wavefronts of a row's key group, its sums' atomics and its MIN / MAX read,
+// about 24 wavefronts per 32 rows. Measured on GB300, int32 keys, SUM and MAX of
+// int32 columns: 2^27 rows, 3000 groups, 4.27 ms (global atomics) -> 0.62 ms;
+// 2^28 rows in 4096 partitions of 1024 groups, 3.97 -> 1.30 ms (64-bit words,
+// lanes of equal slots combined by __match_any_sync and a leader's loop, one
+// row per thread per round before).
+//
 // A key whose offset equals the empty-slot pattern (all ones: only possible
 // when the key span is the whole 32- or 64-bit range) is aggregated in one
 // extra slot past the table.
 #include "kernels.cuh"
+#include "keygroup.cuh"
 
 namespace eiger {
 
 namespace {
 
 constexpr int kGbThreads = 512;
-constexpr uint32_t kPartSlots = 4096;      // shared-memory table of the partition variant
+constexpr uint32_t kPartSlots = 4096;      // most slots of a partition's shared-memory table
+constexpr size_t kGbSmemMax = 200 * 1024;   // most bytes of a CTA table of the hash variant
 constexpr int kProbeCap = 1 << 20;         // probe steps before a global insert gives up
 
 template <typename KeyT>
@@ -61,7 +69,7 @@ __device__ __forceinline__ long long agg_combine(int op, long long a, long long 
     }
 }
 
-// Adds v into *p under op (works on global and shared memory).
+// Adds v into *p (global memory) under op.
 __device__ __forceinline__ void agg_atomic(int op, long long* p, long long v) {
     switch (op) {
         case EIGER_AGG_SUM:
@@ -89,11 +97,6 @@ __device__ __forceinline__ long long agg_value(const AggSpec& s, int a, uint32_t
     if (s.op[a] == EIGER_AGG_COUNT) return 1;
     return s.bytes[a] == 4 ? (long long)__ldcs(static_cast<const int*>(s.vals[a]) + row)
                            : __ldcs(static_cast<const long long*>(s.vals[a]) + row);
-}
-
-template <typename KeyT>
-__device__ __forceinline__ uint32_t gb_hash(KeyT k) {
-    return (uint32_t)KeyCodec<KeyT>::hash(k);
 }
 
 __device__ __forceinline__ uint32_t cas_key(uint32_t* p, uint32_t expect, uint32_t v) { return atomicCAS(p, expect, v); }
@@ -169,149 +172,312 @@ __global__ void __launch_bounds__(kGbThreads)
     }
 }
 
-// Shared-memory table of one CTA: tsize slots (power of two) plus the special
-// slot at index tsize. Layout: keys[tsize + 1], then aggs[naggs][tsize + 1].
-template <typename KeyT>
-struct SmemGb {
-    KeyT* keys;
-    long long* aggs;
-    uint32_t tsize;
-    __device__ void bind(unsigned char* smem, uint32_t ts) {
-        tsize = ts;
-        keys = reinterpret_cast<KeyT*>(smem);
-        aggs = reinterpret_cast<long long*>(smem + align_up((size_t)(ts + 1) * sizeof(KeyT), 8));
-    }
-    __device__ long long* agg(int a, uint32_t slot) const { return aggs + (size_t)a * (tsize + 1) + slot; }
-    __device__ void clear(const AggSpec& s) {
-        for (uint32_t i = threadIdx.x; i <= tsize; i += blockDim.x) {
-            keys[i] = Empty<KeyT>::v;
-            for (int a = 0; a < s.n; ++a) *agg(a, i) = agg_init(s.op[a]);
-        }
-    }
-    // Slot of k (claimed if new), tsize for the all-ones key, or 0xFFFFFFFF
-    // when the table is full.
-    __device__ uint32_t slot_of(KeyT k) {
-        if (k == Empty<KeyT>::v) return tsize;
-        const uint32_t mask = tsize - 1;
-        uint32_t sl = gb_hash(k) & mask;
-        for (uint32_t step = 0; step < tsize; ++step) {
-            const KeyT cur = keys[sl];
-            if (cur == k) return sl;
-            if (cur == Empty<KeyT>::v) {
-                const KeyT prev = cas_key(keys + sl, Empty<KeyT>::v, k);
-                if (prev == Empty<KeyT>::v || prev == k) return sl;
-            }
-            sl = (sl + 1) & mask;
-        }
-        return 0xFFFFFFFFu;
-    }
+// ------------------------------------------------------------------ CTA tables
+
+// Aggregates of a CTA's shared-memory table, held in 32-bit words wherever the
+// type allows: native shared-memory atomics are 32 bits wide, and a MIN or MAX
+// is read first and updated only by a row that improves it (reads of one hot
+// group are broadcast, its atomics would be serial).
+//   kSum     two words (low, high): the low word's atomic returns the old value,
+//            the high word takes the value's high half plus the carry, when
+//            that is not zero;
+//   kCount   one word (a CTA sees fewer than 2^32 rows);
+//   kMin32.. one word: MIN and MAX of 4-byte columns;
+//   kMin64.. 8 bytes: of 8-byte columns.
+enum AggKind { kSum, kCount, kMin32, kMax32, kMin64, kMax64 };
+
+// Layout of a CTA table: keys[slots + 1] (slots a multiple of 4), then per aggregate one cell per slot
+// and copy. Every slot has 2^rlog copies of its aggregates, one per lane class,
+// so that few groups do not serialise a warp's atomics; readers combine them.
+// Slot `slots` is the special one.
+struct CtaLayout {
+    uint32_t slots;
+    int rlog;
+    int n;
+    int kind[kMaxCols];
+    uint32_t off[kMaxCols];  // bytes
+    uint32_t bytes;
 };
 
-template <typename KeyT>
-__host__ __device__ constexpr size_t smem_gb_bytes(uint32_t tsize, int naggs) {
-    return align_up((size_t)(tsize + 1) * sizeof(KeyT), 8) + (size_t)naggs * (tsize + 1) * 8;
+inline CtaLayout cta_layout(const AggSpec& s, uint32_t slots, int rlog, size_t key_bytes) {
+    CtaLayout l{};
+    l.slots = slots;
+    l.rlog = rlog;
+    l.n = s.n;
+    size_t o = align_up((size_t)(slots + 1) * key_bytes, 16);
+    const size_t cells = (size_t)(slots + 1) << rlog;
+    for (int a = 0; a < s.n; ++a) {
+        const bool wide = s.bytes[a] == 8;
+        l.kind[a] = s.op[a] == EIGER_AGG_SUM     ? kSum
+                    : s.op[a] == EIGER_AGG_COUNT ? kCount
+                    : s.op[a] == EIGER_AGG_MIN   ? (wide ? kMin64 : kMin32)
+                                                 : (wide ? kMax64 : kMax32);
+        l.off[a] = (uint32_t)o;
+        o = align_up(o + cells * (l.kind[a] == kCount || l.kind[a] == kMin32 || l.kind[a] == kMax32 ? 4 : 8), 16);
+    }
+    l.bytes = (uint32_t)o;
+    return l;
 }
 
-// Every aggregate's value of row `row` (0 where !ok), loaded together so that
-// the row costs one global-load round trip, not one per aggregate.
-__device__ __forceinline__ void agg_values(const AggSpec& s, bool ok, uint32_t row, long long (&v)[kMaxCols]) {
+template <typename KeyT>
+struct CtaTable {
+    KeyT* keys;
+    unsigned char* base;
+    const CtaLayout& l;
+    uint32_t cells;
+
+    __device__ CtaTable(unsigned char* smem, const CtaLayout& layout)
+        : keys(reinterpret_cast<KeyT*>(smem)), base(smem), l(layout), cells((layout.slots + 1) << layout.rlog) {}
+
+    __device__ void clear() {
+        for (uint32_t i = threadIdx.x; i <= l.slots; i += blockDim.x) keys[i] = Empty<KeyT>::v;
+        for (int a = 0; a < l.n; ++a) {
+            uint32_t* w = reinterpret_cast<uint32_t*>(base + l.off[a]);
+            long long* d = reinterpret_cast<long long*>(base + l.off[a]);
+            switch (l.kind[a]) {
+                case kSum:
+                    for (uint32_t i = threadIdx.x; i < 2 * cells; i += blockDim.x) w[i] = 0;
+                    break;
+                case kCount:
+                    for (uint32_t i = threadIdx.x; i < cells; i += blockDim.x) w[i] = 0;
+                    break;
+                case kMin32:
+                    for (uint32_t i = threadIdx.x; i < cells; i += blockDim.x) w[i] = 0x7FFFFFFFu;
+                    break;
+                case kMax32:
+                    for (uint32_t i = threadIdx.x; i < cells; i += blockDim.x) w[i] = 0x80000000u;
+                    break;
+                case kMin64:
+                    for (uint32_t i = threadIdx.x; i < cells; i += blockDim.x) d[i] = INT64_MAX;
+                    break;
+                default:
+                    for (uint32_t i = threadIdx.x; i < cells; i += blockDim.x) d[i] = INT64_MIN;
+            }
+        }
+    }
+    // Slots of J rows' keys (hashes h), claimed if new; the special slot for the
+    // all-ones key; ~0u for a row without one (!ok, or the table is full). The
+    // home groups of all rows are read first, which settles nearly every row;
+    // the warp is brought together after each of the others.
+    template <int J>
+    __device__ __forceinline__ void slots_of(const KeyT (&k)[J], const uint32_t (&h)[J], const bool (&ok)[J],
+                                             uint32_t (&slot)[J]) {
+        KeyGroup<KeyT> g[J];
 #pragma unroll
-    for (int a = 0; a < kMaxCols; ++a) v[a] = (ok && a < s.n) ? agg_value(s, a, row) : 0;
-}
+        for (int j = 0; j < J; ++j) {
+            slot[j] = group_home<KeyT>(h[j], l.slots);
+            g[j].load(keys + slot[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const uint32_t i = g[j].first(k[j]);
+            if (ok[j] && i < KeyGroup<KeyT>::kN && k[j] != Empty<KeyT>::v) {
+                slot[j] += i;
+            } else if (!ok[j]) {
+                slot[j] = ~0u;
+            } else if (k[j] == Empty<KeyT>::v) {
+                keys[l.slots] = 0;  // taken
+                slot[j] = l.slots;
+            } else {
+                bool fresh;
+                slot[j] = claim_slot(keys, l.slots, k[j], slot[j], fresh);
+            }
+            __syncwarp();
+        }
+    }
+    // Adds J rows' values (halves lo, hi) into the cells of aggregate a.
+    template <int J>
+    __device__ __forceinline__ void update(int a, const uint32_t (&cell)[J], const uint32_t (&lo)[J],
+                                           const uint32_t (&hi)[J]) {
+        uint32_t* w = reinterpret_cast<uint32_t*>(base + l.off[a]);
+        int* si = reinterpret_cast<int*>(w);
+        long long* d = reinterpret_cast<long long*>(w);
+        switch (l.kind[a]) {
+            case kSum:
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (cell[j] != ~0u) {
+                        const uint32_t old = atomicAdd(w + cell[j], lo[j]);
+                        const uint32_t h = hi[j] + (old + lo[j] < lo[j] ? 1u : 0u);
+                        if (h) atomicAdd(w + cells + cell[j], h);
+                    }
+                break;
+            case kCount:
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (cell[j] != ~0u) atomicAdd(w + cell[j], 1u);
+                break;
+            case kMin32:
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (cell[j] != ~0u && (int)lo[j] < *(volatile int*)(si + cell[j])) atomicMin(si + cell[j], (int)lo[j]);
+                break;
+            case kMax32:
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (cell[j] != ~0u && (int)lo[j] > *(volatile int*)(si + cell[j])) atomicMax(si + cell[j], (int)lo[j]);
+                break;
+            case kMin64:
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const long long v = (long long)(((unsigned long long)hi[j] << 32) | lo[j]);
+                    if (cell[j] != ~0u && v < *(volatile long long*)(d + cell[j])) atomicMin(d + cell[j], v);
+                }
+                break;
+            default:
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const long long v = (long long)(((unsigned long long)hi[j] << 32) | lo[j]);
+                    if (cell[j] != ~0u && v > *(volatile long long*)(d + cell[j])) atomicMax(d + cell[j], v);
+                }
+        }
+    }
+    // Aggregate a of a slot, its copies combined.
+    __device__ long long value(int a, int op, uint32_t slot) const {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(base + l.off[a]);
+        long long acc = agg_init(op);
+        for (uint32_t c = slot << l.rlog, e = c + (1u << l.rlog); c < e; ++c) {
+            long long v;
+            switch (l.kind[a]) {
+                case kSum: v = (long long)(((unsigned long long)w[cells + c] << 32) | w[c]); break;
+                case kCount: v = (long long)w[c]; break;
+                case kMin32:
+                case kMax32: v = (long long)(int)w[c]; break;
+                default: v = reinterpret_cast<const long long*>(w)[c];
+            }
+            acc = agg_combine(op, acc, v);
+        }
+        return acc;
+    }
+    __device__ bool taken(uint32_t slot) const { return keys[slot] != Empty<KeyT>::v; }
+};
 
-// Warp-collective: the lanes with `ok` add their row's aggregates `v` into
-// slot `slot` of the CTA table; lanes sharing a slot are first combined by the
-// lowest of them (values staged in the warp's scratch), so a hot group costs
-// one shared atomic per warp instead of 32.
-template <typename KeyT>
-__device__ __forceinline__ void warp_aggregate_vals(SmemGb<KeyT>& tab, const AggSpec& s, bool ok, uint32_t slot,
-                                                    const long long (&v)[kMaxCols], long long* scratch) {
+constexpr int kGbRows = 4;  // rows per thread per round
+
+// Every warp of the CTA: aggregates rows [lo, hi) into the table, in rounds of
+// kGbRows x 32 rows claimed from the counter *next (0 before): equal shares
+// instead left the warps the scheduler favours waiting a third of the time for
+// the others. key(r)
+// gives a row's key, hash(k) its 32-bit hash; a row whose key finds the table
+// full goes to full(k, r). N: aggregates held (at least s.n); W8: some value
+// column is 8 bytes wide. A round's keys and values are all loaded before the
+// first table access, so a row costs one round trip to memory.
+template <typename KeyT, int N, bool W8, typename KeyF, typename HashF, typename FullF>
+__device__ __forceinline__ void aggregate_rows(CtaTable<KeyT>& tab, const AggSpec& s, unsigned long long lo,
+                                               unsigned long long hi, uint32_t* next, KeyF key, HashF hash,
+                                               FullF full) {
+    constexpr int J = kGbRows;
     const unsigned lane = lane_id();
-    const unsigned peers = __match_any_sync(0xffffffffu, ok ? slot : 0xFFFFFFFFu);
-    const bool leader = ok && (int)lane == __ffs(peers) - 1;
+    const uint32_t copy = lane & ((1u << tab.l.rlog) - 1u);
+    for (;;) {
+        uint32_t round = 0;
+        if (lane == 0) round = atomicAdd(next, 1u);
+        round = __shfl_sync(0xffffffffu, round, 0);
+        const unsigned long long base = lo + (unsigned long long)round * (J * kWarp);
+        if (base >= hi) break;
+        KeyT k[J];
+        uint32_t v[N][J], vh[W8 ? N : 1][J];
+        bool ok[J];
 #pragma unroll
-    for (int a = 0; a < kMaxCols; ++a) {
-        if (a >= s.n) break;
-        scratch[lane] = v[a];
-        __syncwarp();
-        if (leader) {
-            long long acc = v[a];
-            unsigned m = peers & ~(1u << lane);
-            while (m) {
-                const int l = __ffs(m) - 1;
-                acc = agg_combine(s.op[a], acc, scratch[l]);
-                m &= m - 1;
+        for (int j = 0; j < J; ++j) {
+            const unsigned long long r = base + j * kWarp + lane;
+            ok[j] = r < hi;
+            if (ok[j]) k[j] = key((uint32_t)r);
+        }
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            if (a >= s.n || s.op[a] == EIGER_AGG_COUNT) continue;
+            const uint32_t r0 = (uint32_t)base + lane;
+            if (W8 && s.bytes[a] == 8) {
+                const uint2* p = static_cast<const uint2*>(s.vals[a]) + r0;
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (ok[j]) {
+                        const uint2 x = __ldcs(p + j * kWarp);
+                        v[a][j] = x.x;
+                        vh[W8 ? a : 0][j] = x.y;
+                    }
+            } else {
+                const uint32_t* p = static_cast<const uint32_t*>(s.vals[a]) + r0;
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if (ok[j]) {
+                        v[a][j] = __ldcs(p + j * kWarp);
+                        if (W8) vh[W8 ? a : 0][j] = (uint32_t)((int)v[a][j] >> 31);
+                    }
             }
-            agg_atomic(s.op[a], tab.agg(a, slot), acc);
+        }
+        // (left to itself the warp drifts apart in the searches and stays so for
+        // the rest of the round: 3 lanes per instruction, the value loads sunk
+        // into the divergent code, a fourteenth of the speed)
+        __syncwarp();
+        uint32_t h[J], cell[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) h[j] = hash(k[j]);
+        tab.template slots_of<J>(k, h, ok, cell);
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            if (cell[j] != ~0u)
+                cell[j] = (cell[j] << tab.l.rlog) + copy;
+            else if (ok[j])
+                full(k[j], (uint32_t)(base + j * kWarp + lane));
         }
         __syncwarp();
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            if (a >= s.n) continue;
+            if constexpr (W8) {
+                tab.update<J>(a, cell, v[a], vh[a]);
+            } else {
+                uint32_t sign[J];
+#pragma unroll
+                for (int j = 0; j < J; ++j) sign[j] = (uint32_t)((int)v[a][j] >> 31);
+                tab.update<J>(a, cell, v[a], sign);
+            }
+            __syncwarp();
+        }
     }
 }
 
+// Adds the CTA table's groups into a global table.
 template <typename KeyT>
-__device__ __forceinline__ void warp_aggregate(SmemGb<KeyT>& tab, const AggSpec& s, bool ok, uint32_t slot,
-                                               uint32_t row, long long* scratch) {
-    long long v[kMaxCols];
-    agg_values(s, ok, row, v);
-    warp_aggregate_vals(tab, s, ok, slot, v, scratch);
+__device__ __forceinline__ void merge_groups(const CtaTable<KeyT>& tab, const AggSpec& s, const GbTable<KeyT>& t,
+                                             unsigned* err) {
+    for (uint32_t i = threadIdx.x; i <= tab.l.slots; i += blockDim.x) {
+        if (!tab.taken(i)) continue;
+        const unsigned long long g = gb_global_slot(t, i == tab.l.slots ? KeyT(Empty<KeyT>::v) : tab.keys[i], err);
+        if (g == ~0ull) continue;
+        for (int a = 0; a < s.n; ++a) agg_atomic(s.op[a], t.aggs + (size_t)a * t.stride + g, tab.value(a, s.op[a], i));
+    }
 }
 
-template <typename InKey, typename KeyT>
-__global__ void __launch_bounds__(kGbThreads)
-    gb_hash_smem_kernel(const InKey* __restrict__ keys, uint32_t n, uint64_t offset, GbTable<KeyT> t, AggSpec s,
-                        unsigned* err) {
+// Hash variant with CTA tables: a contiguous row range per CTA; rows whose key
+// finds the CTA's table full (an estimate far too low) go to the global table.
+template <typename InKey, typename KeyT, int N, bool W8>
+__global__ void __launch_bounds__(1024, 1)
+    gb_hash_smem_kernel(const InKey* __restrict__ keys, uint32_t n, uint64_t offset, GbTable<KeyT> t,
+                        const __grid_constant__ AggSpec s, const __grid_constant__ CtaLayout layout, unsigned* err) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long s_scratch[kGbThreads];
-    __shared__ unsigned s_special;
-    SmemGb<KeyT> tab;
-    tab.bind(smem, (uint32_t)t.slots);
-    tab.clear(s);
-    if (threadIdx.x == 0) s_special = 0;
+    __shared__ uint32_t s_next;
+    CtaTable<KeyT> tab(smem, layout);
+    tab.clear();
+    if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
-    long long* scratch = s_scratch + (threadIdx.x & ~(kWarp - 1));
-    // contiguous row range per CTA, rounds of blockDim rows
     const unsigned long long per = ((unsigned long long)n + gridDim.x - 1) / gridDim.x;
-    const unsigned long long lo64 = blockIdx.x * per;
-    const uint32_t lo = (uint32_t)(lo64 < n ? lo64 : n);
-    const uint32_t hi = (uint32_t)(lo64 + per < n ? lo64 + per : n);
-    bool full = false;
-    for (unsigned long long base = lo; base < hi; base += kGbThreads) {
-        const uint32_t r = (uint32_t)(base + threadIdx.x);
-        bool ok = base + threadIdx.x < hi;
-        uint32_t slot = 0;
-        if (ok) {
-            const KeyT k = KeyCodec<KeyT>::encode((int64_t)__ldcs(keys + r), offset);
-            slot = tab.slot_of(k);
-            if (slot == tab.tsize) s_special = 1;
-            if (slot == 0xFFFFFFFFu) {  // cannot happen with the table sized from the estimate; go global
-                full = true;
-                const unsigned long long g = gb_global_slot(t, k, err);
-                if (g != ~0ull)
-                    for (int a = 0; a < s.n; ++a)
-                        agg_atomic(s.op[a], t.aggs + (size_t)a * t.stride + g, agg_value(s, a, r));
-                ok = false;
-            }
-        }
-        warp_aggregate(tab, s, ok, slot, r, scratch);
-    }
-    (void)full;
+    const unsigned long long lo = blockIdx.x * per;
+    const unsigned long long hi = lo + per < n ? lo + per : n;
+    aggregate_rows<KeyT, N, W8>(
+        tab, s, lo, hi, &s_next, [&](uint32_t r) { return KeyCodec<KeyT>::encode((int64_t)__ldcs(keys + r), offset); },
+        [&](KeyT k) {
+            return (uint32_t)(KeyCodec<KeyT>::mix(k, KeyCodec<KeyT>::kBits) >> (KeyCodec<KeyT>::kBits - 32));
+        },
+        [&](KeyT k, uint32_t r) {
+            const unsigned long long g = gb_global_slot(t, k, err);
+            if (g != ~0ull)
+                for (int a = 0; a < s.n; ++a) agg_atomic(s.op[a], t.aggs + (size_t)a * t.stride + g, agg_value(s, a, r));
+        });
     __syncthreads();
-    // merge the CTA's groups into the global table
-    const unsigned long long total = t.stride;
-    for (uint32_t i = threadIdx.x; i <= tab.tsize; i += blockDim.x) {
-        unsigned long long g;
-        if (i == tab.tsize) {
-            if (!s_special) continue;
-            atomicOr(t.special, 1u);
-            g = t.slots;
-        } else {
-            const KeyT k = tab.keys[i];
-            if (k == Empty<KeyT>::v) continue;
-            g = gb_global_slot(t, k, err);
-            if (g == ~0ull) continue;
-        }
-        for (int a = 0; a < s.n; ++a) agg_atomic(s.op[a], t.aggs + (size_t)a * total + g, *tab.agg(a, i));
-    }
+    merge_groups(tab, s, t, err);
 }
 
 // Output of a group-by: keys in the caller's dtype and one int64 column per aggregate.
@@ -366,7 +532,19 @@ __global__ void gb_compact_kernel(GbTable<KeyT> t, AggSpec s, uint64_t offset, i
 
 // ------------------------------------------------------------------ partition variant
 
-constexpr uint32_t kGbChunk = 65536;  // rows per work item of the partition variant
+// Rows per work item of the partition variant: one and a half average
+// partitions while the partitions alone fill the chip several times over, so
+// that an ordinary partition is one item and writes its groups straight out
+// (2^28 rows over 4096 partitions cut at 65536 rows each, their average: half
+// of them merged through the spill table, 0.47 ms more); else the rows over
+// eight items per SM. At least gb_min_chunk: the spill table is sized for it.
+inline uint32_t gb_min_chunk(unsigned long long n) { return n >= (1ull << 24) ? 65536u : 16384u; }
+
+inline uint32_t gb_chunk(unsigned long long n, uint32_t P, int sms) {
+    unsigned long long c = P >= (uint32_t)(8 * sms) ? 3 * n / (2ull * P) : n / (8ull * sms);
+    const unsigned long long lo = gb_min_chunk(n);
+    return (uint32_t)(c < lo ? lo : c > (1u << 20) ? (1u << 20) : c);
+}
 
 template <typename KeyT>
 struct GbPartIn {
@@ -374,16 +552,19 @@ struct GbPartIn {
     const uint32_t* start;                    // [P + 1]
     const unsigned long long* item_prefix;    // [P + 1] work items before each partition
     uint32_t P;
+    uint32_t chunk;                           // rows per work item
+    int pbits;                                // partition bits (the top bits of the mixed keys)
     AggSpec s;                                // value columns: the partitioned copies
+    CtaLayout layout;
 };
 
-// One block: work items per partition (row chunks of kGbChunk), their
+// One block: work items per partition (row chunks of `chunk`), their
 // exclusive prefix, the item total (ctrl->nitems) and the slots of the spill
 // table for the groups of partitions that span several items: at most
 // kPartSlots groups each, at load <= 1/2, capped at spill_max.
 __global__ void __launch_bounds__(1024)
     gb_items_kernel(const uint32_t* __restrict__ start, uint32_t P, unsigned long long* __restrict__ prefix,
-                    Ctrl* ctrl, unsigned long long* spill_slots, unsigned long long spill_max) {
+                    Ctrl* ctrl, unsigned long long* spill_slots, unsigned long long spill_max, uint32_t chunk) {
     __shared__ unsigned long long s_w[1024 / kWarp];
     __shared__ unsigned long long s_m[1024 / kWarp];
     const unsigned lane = lane_id();
@@ -394,7 +575,7 @@ __global__ void __launch_bounds__(1024)
         unsigned long long items = 0;
         if (p < P) {
             const uint32_t rows = start[p + 1] - start[p];
-            items = (rows + kGbChunk - 1) / kGbChunk;
+            items = (rows + (unsigned long long)chunk - 1) / chunk;
         }
         unsigned long long x = items, m = items > 1;
 #pragma unroll
@@ -456,27 +637,27 @@ __device__ __forceinline__ uint32_t find_item_part(const unsigned long long* __r
     return lo;
 }
 
-// A persistent grid takes work items (a partition's chunk of kGbChunk rows)
-// from a global counter and aggregates each in a shared-memory table. A
-// partition that is one item writes its groups out directly; the items of a
-// larger partition (few groups, many rows) merge their groups into the spill
-// table, which is compacted afterwards.
-template <typename KeyT>
-__global__ void __launch_bounds__(kGbThreads)
-    gb_part_kernel(GbPartIn<KeyT> a, GbTable<KeyT> spill, uint64_t offset, int kbits, GbOut o, Ctrl* ctrl) {
+// A persistent grid takes work items (a partition's chunk of rows) from a
+// global counter and aggregates each in a shared-memory table. A partition
+// that is one item writes its groups out directly; the items of a larger
+// partition (few groups, many rows) merge their groups into the spill table,
+// which is compacted afterwards.
+template <typename KeyT, int N, bool W8>
+__global__ void __launch_bounds__(kGbThreads, 2)
+    gb_part_kernel(const __grid_constant__ GbPartIn<KeyT> a, GbTable<KeyT> spill, uint64_t offset, int kbits,
+                   const __grid_constant__ GbOut o, Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long s_scratch[kGbThreads];
     __shared__ uint32_t s_warp[kGbThreads / kWarp];
-    __shared__ unsigned s_special;
     __shared__ unsigned long long s_item;
     __shared__ uint32_t s_part;
     __shared__ unsigned long long s_base;
     __shared__ int s_full;
+    __shared__ uint32_t s_next;
     resolve_slots(spill);
-    SmemGb<KeyT> tab;
-    tab.bind(smem, kPartSlots);
-    long long* scratch = s_scratch + (threadIdx.x & ~(kWarp - 1));
+    CtaTable<KeyT> tab(smem, a.layout);
     const unsigned long long nitems = ctrl->nitems;
+    const unsigned lane = lane_id();
+    const int w = threadIdx.x / kWarp;
     for (;;) {
         if (threadIdx.x < kWarp) {
             unsigned long long it = 0;
@@ -486,11 +667,11 @@ __global__ void __launch_bounds__(kGbThreads)
             if (threadIdx.x == 0) {
                 s_item = it;
                 s_part = p;
-                s_special = 0;
                 s_full = 0;
+                s_next = 0;
             }
         }
-        tab.clear(a.s);
+        tab.clear();
         __syncthreads();
         const unsigned long long item = s_item;
         if (item >= nitems) break;
@@ -498,38 +679,12 @@ __global__ void __launch_bounds__(kGbThreads)
         const unsigned long long c = item - a.item_prefix[p];
         const bool multi = a.item_prefix[p + 1] - a.item_prefix[p] > 1;
         const uint32_t pend = a.start[p + 1];
-        const unsigned long long beg = (unsigned long long)a.start[p] + c * kGbChunk;
-        const unsigned long long end = beg + kGbChunk < pend ? beg + kGbChunk : pend;
-        // each round's key and values are loaded one round ahead, so their
-        // round trip overlaps the previous round's table updates
-        KeyT kn{};
-        long long vn[kMaxCols];
-        {
-            const bool okn = beg + threadIdx.x < end;
-            if (okn) kn = __ldcs(a.key + (uint32_t)(beg + threadIdx.x));
-            agg_values(a.s, okn, (uint32_t)(beg + threadIdx.x), vn);
-        }
-        for (unsigned long long base = beg; base < end; base += kGbThreads) {
-            bool ok = base + threadIdx.x < end;
-            const KeyT k = kn;
-            long long v[kMaxCols];
-#pragma unroll
-            for (int q = 0; q < kMaxCols; ++q) v[q] = vn[q];
-            const unsigned long long nx = base + kGbThreads + threadIdx.x;
-            const bool okn = nx < end;
-            if (okn) kn = __ldcs(a.key + (uint32_t)nx);
-            agg_values(a.s, okn, (uint32_t)nx, vn);
-            uint32_t slot = 0;
-            if (ok) {
-                slot = tab.slot_of(k);
-                if (slot == tab.tsize) s_special = 1;
-                if (slot == 0xFFFFFFFFu) {
-                    s_full = 1;
-                    ok = false;
-                }
-            }
-            warp_aggregate_vals(tab, a.s, ok, slot, v, scratch);
-        }
+        const unsigned long long beg = (unsigned long long)a.start[p] + c * a.chunk;
+        const unsigned long long end = beg + a.chunk < pend ? beg + a.chunk : pend;
+        aggregate_rows<KeyT, N, W8>(
+            tab, a.s, beg, end, &s_next, [&](uint32_t r) { return __ldcs(a.key + r); },
+            [&](KeyT k) { return (uint32_t)((KeyT)(k << a.pbits) >> (KeyCodec<KeyT>::kBits - 32)); },
+            [&](KeyT, uint32_t) { s_full = 1; });
         __syncthreads();
         if (s_full) {  // more groups than one table: the host repartitions with more bits
             if (threadIdx.x == 0) atomicOr(&ctrl->err, kErrTableFull);
@@ -537,77 +692,71 @@ __global__ void __launch_bounds__(kGbThreads)
             continue;
         }
         if (multi) {
-            // merge this item's groups into the spill table
-            for (uint32_t i = threadIdx.x; i <= kPartSlots; i += blockDim.x) {
-                KeyT k;
-                if (i == kPartSlots) {
-                    if (!s_special) continue;
-                    k = Empty<KeyT>::v;
-                } else {
-                    k = tab.keys[i];
-                    if (k == Empty<KeyT>::v) continue;
-                }
-                const unsigned long long g = gb_global_slot(spill, k, &ctrl->err);
-                if (g == ~0ull) continue;
-                for (int b = 0; b < a.s.n; ++b)
-                    agg_atomic(a.s.op[b], spill.aggs + (size_t)b * spill.stride + g, *tab.agg(b, i));
-            }
+            merge_groups(tab, a.s, spill, &ctrl->err);
             __syncthreads();
             continue;
         }
-        // compact: block scan of occupancy, one global reservation
-        const uint32_t per = (kPartSlots + 1 + kGbThreads - 1) / kGbThreads;
+        // Compact: each warp owns a run of slots; the warps' counts are scanned,
+        // one global reservation, then the warps write their groups in slot
+        // order, lane by lane on consecutive output positions.
+        const uint32_t per = ((a.layout.slots + 1 + kGbThreads - 1) / kGbThreads) * kWarp;  // slots per warp
+        const uint32_t s0 = w * per, s1 = min(s0 + per, a.layout.slots + 1);
         uint32_t cnt = 0;
-        for (uint32_t q = 0; q < per; ++q) {
-            const uint32_t i = threadIdx.x * per + q;
-            if (i < kPartSlots) cnt += tab.keys[i] != Empty<KeyT>::v;
-            else if (i == kPartSlots) cnt += s_special != 0;
-        }
-        uint32_t x = cnt;
-        const unsigned lane = lane_id();
-        const int w = threadIdx.x / kWarp;
-#pragma unroll
-        for (int off = 1; off < kWarp; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-            if ((int)lane >= off) x += y;
-        }
-        if ((int)lane == kWarp - 1) s_warp[w] = x;
+        for (uint32_t i = s0 + lane; i < s1; i += kWarp) cnt += tab.taken(i);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) s_warp[w] = cnt;
         __syncthreads();
         if (w == 0) {
             uint32_t v = (int)lane < kGbThreads / kWarp ? s_warp[lane] : 0u;
+            const uint32_t own = v;
 #pragma unroll
             for (int off = 1; off < kWarp; off <<= 1) {
                 const uint32_t y = __shfl_up_sync(0xffffffffu, v, off);
                 if ((int)lane >= off) v += y;
             }
-            if ((int)lane < kGbThreads / kWarp) s_warp[lane] = v;
-            if (lane == kGbThreads / kWarp - 1) s_base = v ? atomicAdd(&ctrl->cursor, (unsigned long long)v) : 0ull;
+            if ((int)lane < kGbThreads / kWarp) s_warp[lane] = v - own;
+            if (lane == kWarp - 1) s_base = v ? atomicAdd(&ctrl->cursor, (unsigned long long)v) : 0ull;
         }
         __syncthreads();
-        unsigned long long pos = s_base + (w ? s_warp[w - 1] : 0u) + (x - cnt);
-        for (uint32_t q = 0; q < per; ++q) {
-            const uint32_t i = threadIdx.x * per + q;
-            bool has = false;
-            KeyT k = Empty<KeyT>::v;
-            if (i < kPartSlots) {
-                k = tab.keys[i];
-                has = k != Empty<KeyT>::v;
-            } else if (i == kPartSlots) {
-                has = s_special != 0;
-            }
+        unsigned long long pos = s_base + s_warp[w];
+        for (uint32_t i0 = s0; i0 < s1; i0 += kWarp) {
+            const uint32_t i = i0 + lane;
+            const bool has = i < s1 && tab.taken(i);
+            const unsigned m = __ballot_sync(0xffffffffu, has);
             if (has) {
+                const KeyT k = i == a.layout.slots ? Empty<KeyT>::v : tab.keys[i];
                 long long v[kMaxCols];
-                for (int b = 0; b < a.s.n; ++b) v[b] = *tab.agg(b, i);
-                write_group(o, pos++, (int64_t)((uint64_t)KeyCodec<KeyT>::unmix(k, kbits) + offset), v, a.s.n);
+                for (int b = 0; b < a.s.n; ++b) v[b] = tab.value(b, a.s.op[b], i);
+                write_group(o, pos + __popc(m & lanemask_lt()),
+                            (int64_t)((uint64_t)KeyCodec<KeyT>::unmix(k, kbits) + offset), v, a.s.n);
             }
+            pos += __popc(m);
         }
         __syncthreads();
     }
 }
 
+// Whether some value column is 8 bytes wide.
+inline bool wide_values(const AggSpec& s) {
+    for (int a = 0; a < s.n; ++a)
+        if (s.op[a] != EIGER_AGG_COUNT && s.bytes[a] == 8) return true;
+    return false;
+}
+
 template <typename KeyT>
 size_t gb_global_bytes(unsigned long long slots, int naggs) {
     return align_up((size_t)(slots + 1) * sizeof(KeyT), 256) + (size_t)naggs * (slots + 1) * 8 + 256;
+}
+
+constexpr size_t kGbHalfSm = 112 * 1024;  // table bytes that let two CTAs share an SM
+
+// CTA table of the hash variant: copies of the aggregates while they fit 48 KB
+// (several CTAs per SM), at most one per lane.
+template <typename KeyT>
+CtaLayout hash_cta_layout(const AggSpec& s, uint32_t slots) {
+    int rlog = 0;
+    while (rlog < 5 && cta_layout(s, slots, rlog + 1, sizeof(KeyT)).bytes <= 48 * 1024) ++rlog;
+    return cta_layout(s, slots, rlog, sizeof(KeyT));
 }
 
 template <typename InKey, typename KeyT>
@@ -632,18 +781,24 @@ cudaError_t gb_hash_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     double vbytes = 0;
     for (int a = 0; a < s.n; ++a) vbytes += s.op[a] == EIGER_AGG_COUNT ? 0 : s.bytes[a];
     const uint32_t n = (uint32_t)g.n;
-    const size_t smem = smem_gb_bytes<KeyT>((uint32_t)plan.slots, s.n);
-    if (plan.smem) {
-        auto kern = gb_hash_smem_kernel<InKey, KeyT>;
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if (plan.smem_slots) {
+        const bool w8 = wide_values(s);
+        auto kern = s.n <= 1   ? (w8 ? gb_hash_smem_kernel<InKey, KeyT, 1, true> : gb_hash_smem_kernel<InKey, KeyT, 1, false>)
+                    : s.n == 2 ? (w8 ? gb_hash_smem_kernel<InKey, KeyT, 2, true> : gb_hash_smem_kernel<InKey, KeyT, 2, false>)
+                               : (w8 ? gb_hash_smem_kernel<InKey, KeyT, 4, true> : gb_hash_smem_kernel<InKey, KeyT, 4, false>);
+        const CtaLayout l = hash_cta_layout<KeyT>(s, plan.smem_slots);
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes)) != cudaSuccess)
             return e;
+        // a table that leaves room for a second CTA runs 512 threads each, a
+        // larger one 1024; no more CTAs than rounds of rows
+        const int threads = l.bytes <= kGbHalfSm ? 512 : 1024;
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGbThreads, smem) != cudaSuccess ||
-            per_sm < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, l.bytes) != cudaSuccess || per_sm < 1)
             per_sm = 1;
+        const unsigned long long want = ((unsigned long long)n + threads * kGbRows - 1) / (threads * kGbRows);
+        const int grid = want < (unsigned long long)di.sms * per_sm ? (int)want : di.sms * per_sm;
         ProfScope ps("gb_hash_smem", ((double)sizeof(InKey) + vbytes) * (double)n, stream);
-        kern<<<di.sms * per_sm, kGbThreads, smem, stream>>>(static_cast<const InKey*>(g.keys), n, plan.offset, t, s,
-                                                            &ctrl->err);
+        kern<<<grid, threads, l.bytes, stream>>>(static_cast<const InKey*>(g.keys), n, plan.offset, t, s, l, &ctrl->err);
     } else {
         ProfScope ps("gb_hash_global", ((double)sizeof(InKey) + vbytes) * (double)n, stream);
         gb_hash_global_kernel<InKey, KeyT><<<di.sms * 4, kGbThreads, 0, stream>>>(
@@ -692,6 +847,7 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     if (e != cudaSuccess) return e;
     const int buf = plan.bits2 ? 1 : 0;
     const uint32_t P = 1u << (plan.bits1 + plan.bits2);
+    const uint32_t chunk = gb_chunk((unsigned long long)g.n, P, di.sms);
     GbTable<KeyT> spill;
     {
         Carve c{static_cast<char*>(sc.spill), 0};
@@ -705,7 +861,7 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     {
         ProfScope ps("gb_items", 8.0 * P, stream, 0.0, 2);
         gb_items_kernel<<<1, 1024, 0, stream>>>(sc.part.part_start, P, sc.item_prefix, ctrl, sc.spill_slots,
-                                                sc.spill_max);
+                                                sc.spill_max, chunk);
         gb_init_kernel<KeyT><<<di.sms * 2, 256, 0, stream>>>(spill, s);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
@@ -714,11 +870,17 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
     in.start = sc.part.part_start;
     in.item_prefix = sc.item_prefix;
     in.P = P;
+    in.chunk = chunk;
+    in.pbits = plan.bits1 + plan.bits2;
     in.s = s;
     for (int a = 0; a < s.n; ++a)
         if (col_of[a] >= 0) in.s.vals[a] = sc.part.col[buf][col_of[a]];
-    auto kern = gb_part_kernel<KeyT>;
-    const size_t smem = smem_gb_bytes<KeyT>(kPartSlots, s.n);
+    in.layout = cta_layout(s, plan.part_slots, 0, sizeof(KeyT));
+    const bool w8 = wide_values(s);
+    auto kern = s.n <= 1   ? (w8 ? gb_part_kernel<KeyT, 1, true> : gb_part_kernel<KeyT, 1, false>)
+                : s.n == 2 ? (w8 ? gb_part_kernel<KeyT, 2, true> : gb_part_kernel<KeyT, 2, false>)
+                           : (w8 ? gb_part_kernel<KeyT, 4, true> : gb_part_kernel<KeyT, 4, false>);
+    const size_t smem = in.layout.bytes;
     if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     int per_sm = 0;
@@ -740,9 +902,24 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
 
 }  // namespace
 
-size_t gb_smem_table_bytes(unsigned long long slots, int naggs, bool key32) {
-    if (slots > (1ull << 16)) return ~(size_t)0;  // far beyond any shared-memory budget
-    return key32 ? smem_gb_bytes<uint32_t>((uint32_t)slots, naggs) : smem_gb_bytes<uint64_t>((uint32_t)slots, naggs);
+uint32_t gb_part_slots(double groups) {
+    const double want = 3.75 * groups + 64.0;
+    return want < (double)kPartSlots ? (uint32_t)want & ~3u : kPartSlots;
+}
+
+uint32_t gb_hash_slots(double groups, const GbAggs& aggs, bool key32) {
+    AggSpec s{};
+    s.n = aggs.n;
+    for (int a = 0; a < aggs.n; ++a) {
+        s.op[a] = aggs.op[a];
+        s.bytes[a] = aggs.bytes[a];
+    }
+    const size_t kb = key32 ? 4 : 8;
+    const double per_slot = (double)cta_layout(s, 4096, 0, kb).bytes / 4097.0;
+    const double most = (double)(kGbSmemMax - 1024) / per_slot - 8.0;
+    double want = 3.5 * groups + 64.0;
+    if (want > most) want = most;
+    return want >= 1.6 * groups + 64.0 ? (uint32_t)want & ~3u : 0;
 }
 
 GbScratch gb_layout(Carve& c, int64_t n, const GbPlanDev& plan, const int* col_bytes, int ncols) {
@@ -758,10 +935,10 @@ GbScratch gb_layout(Carve& c, int64_t n, const GbPlanDev& plan, const int* col_b
         for (int q = 0; q < ncols; ++q) pd.col_bytes[0][q] = col_bytes[q];
         const int passes = plan.bits2 ? 2 : 1;
         part_side_layout(c, s.part, n, plan.bits1, plan.bits2, passes, false, plan.key32 ? 4 : 8, pd, 0);
-        // spill table: each multi-item partition has more than kGbChunk rows and at
-        // most kPartSlots groups; load <= 1/2
+        // spill table: each multi-item partition has more than a chunk's rows and
+        // at most kPartSlots groups; load <= 1/2
         const unsigned long long nn = n > 0 ? (unsigned long long)n : 1ull;
-        unsigned long long groups = (nn / kGbChunk + 1) * kPartSlots;
+        unsigned long long groups = (nn / gb_min_chunk(nn) + 1) * kPartSlots;
         if (groups > nn) groups = nn;
         unsigned long long sl = 64;
         while (sl < 2 * groups) sl <<= 1;

@@ -220,7 +220,8 @@ struct GbPlanDev {
     uint64_t offset;           // key minimum (frame of reference)
     int kbits;                 // bits of the key mix (key32: of the key span; else 64)
     unsigned long long slots;  // hash: global table slots (power of two)
-    int smem;                  // hash: aggregate in a CTA-private shared-memory copy first
+    uint32_t smem_slots;       // hash: slots of the CTA-private shared-memory tables (0: none)
+    uint32_t part_slots;       // partition: slots of a partition's shared-memory table
     int naggs;
 };
 
@@ -241,8 +242,15 @@ struct GbScratch {
     unsigned long long* item_prefix;   // [P + 1] work items per partition, prefix
 };
 
-// Shared-memory bytes of a CTA-private table of `slots` slots.
-size_t gb_smem_table_bytes(unsigned long long slots, int naggs, bool key32);
+// Slots of a CTA-private table for an estimated number of groups, or 0 when it
+// does not fit shared memory at a load of 5/8. Load 2/7 where it fits: nearly
+// every row then finds its key in its home group (2^27 rows, 3000 groups, load
+// 4/7 -> 1/3: 1.80 -> 1.36 ms).
+uint32_t gb_hash_slots(double groups, const GbAggs& aggs, bool key32);
+// Slots of a partition's table for an estimated number of groups per partition
+// (load about 1/4; 2^28 rows, 2^22 groups, load 4/9 -> 2/7: 2.06 -> 1.43 ms),
+// capped.
+uint32_t gb_part_slots(double groups);
 GbScratch gb_layout(Carve& c, int64_t n, const GbPlanDev& plan, const int* col_bytes, int ncols);
 cudaError_t gb_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch& s, const GbAggs& aggs, void* out_keys,
                    unsigned long long capacity, Ctrl* ctrl, cudaStream_t stream);

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "keygroup.cuh"
 
 #ifndef EIGER_PROBE_CHUNK
 #define EIGER_PROBE_CHUNK 32768
@@ -59,39 +60,6 @@ __device__ __forceinline__ uint32_t slot_hash(uint64_t k) {
 __device__ __forceinline__ uint32_t next_slot(uint32_t s, uint32_t tsize) {
     return s + 1 == tsize ? 0u : s + 1;
 }
-
-// Shared-memory key arrays are probed 16 bytes at a time: a group of four
-// 32-bit or two 64-bit keys per load. Home slots are group-aligned and inserts
-// fill the groups in order (linear probing), so a key's slot is preceded by no
-// empty slot from its home group on. The all-ones pattern marks an empty slot.
-template <typename KeyT>
-struct KeyGroup;
-template <>
-struct KeyGroup<uint32_t> {
-    static constexpr uint32_t kN = 4;
-    uint4 v;
-    __device__ __forceinline__ void load(const uint32_t* p) { v = *reinterpret_cast<const uint4*>(p); }
-    // index of the first key equal to k, or kN
-    __device__ __forceinline__ uint32_t first(uint32_t k) const {
-        return v.x == k ? 0u : v.y == k ? 1u : v.z == k ? 2u : v.w == k ? 3u : 4u;
-    }
-    __device__ __forceinline__ uint32_t first_or_empty(uint32_t k) const {
-        return v.x == k || v.x == ~0u ? 0u : v.y == k || v.y == ~0u ? 1u : v.z == k || v.z == ~0u ? 2u
-               : v.w == k || v.w == ~0u ? 3u : 4u;
-    }
-    __device__ __forceinline__ uint32_t last() const { return v.w; }
-};
-template <>
-struct KeyGroup<uint64_t> {
-    static constexpr uint32_t kN = 2;
-    ulonglong2 v;
-    __device__ __forceinline__ void load(const uint64_t* p) { v = *reinterpret_cast<const ulonglong2*>(p); }
-    __device__ __forceinline__ uint32_t first(uint64_t k) const { return v.x == k ? 0u : v.y == k ? 1u : 2u; }
-    __device__ __forceinline__ uint32_t first_or_empty(uint64_t k) const {
-        return v.x == k || v.x == ~0ull ? 0u : v.y == k || v.y == ~0ull ? 1u : 2u;
-    }
-    __device__ __forceinline__ uint64_t last() const { return v.y; }
-};
 
 // The 128-byte lines of rows [0, n) of a partitioned side (keys, then tuple
 // IDs unless rows are identified by position) asked into L2, one line per

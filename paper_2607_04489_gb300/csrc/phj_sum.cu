@@ -28,13 +28,6 @@ constexpr int kConsumers = kJoinThreads;
 constexpr int kSumThreads = kConsumers + kStreamWarps * kWarp;
 constexpr int kStages = 2;
 
-__device__ __forceinline__ uint32_t cas_smem(uint32_t* p, uint32_t expect, uint32_t v) {
-    return atomicCAS(p, expect, v);
-}
-__device__ __forceinline__ uint64_t cas_smem(uint64_t* p, uint64_t expect, uint64_t v) {
-    return atomicCAS(reinterpret_cast<unsigned long long*>(p), (unsigned long long)expect, (unsigned long long)v);
-}
-
 // Slots of {key, sum as two 32-bit halves, rows beyond the first}. The all-ones
 // key is the empty pattern; that key itself lives in the extra slot kSlots,
 // whose key word turns 0 when it is taken.
@@ -64,12 +57,7 @@ struct SumTable {
         if (threadIdx.x == 0) clear_slot(kSlots);
     }
     using Group = KeyGroup<KeyT>;
-    __device__ static uint32_t home(KeyT k, uint32_t tsize) {
-        return Group::kN * __umulhi(slot_hash(k), tsize / Group::kN);
-    }
-    __device__ static uint32_t next_group(uint32_t s, uint32_t tsize) {
-        return s + Group::kN == tsize ? 0u : s + Group::kN;
-    }
+    __device__ static uint32_t home(KeyT k, uint32_t tsize) { return group_home<KeyT>(slot_hash(k), tsize); }
     // Adds build row (k, v): 0 for a new key, 1 for a further row of a key, -1
     // when the table is full. 32-bit shared-memory atomics are native: the low
     // half's returns the old value, and the high half takes the addend's high
@@ -81,22 +69,10 @@ struct SumTable {
             s = kSlots;
             again = cas_smem(key + s, kEmpty, KeyT(0)) != kEmpty;
         } else {
-            uint32_t base = home(k, tsize);
-            // a lost race for a slot re-reads the group (at most tsize times)
-            for (uint32_t step = 0;;) {
-                Group g;
-                g.load(key + base);
-                const uint32_t i = g.first_or_empty(k);
-                s = base + i;
-                if (i < Group::kN) {
-                    const KeyT cur = cas_smem(key + s, kEmpty, k);
-                    again = cur == k;
-                    if (again || cur == kEmpty) break;
-                } else {
-                    base = next_group(base, tsize);
-                }
-                if (++step > 2 * tsize) return -1;
-            }
+            bool fresh = false;
+            s = claim_slot(key, tsize, k, home(k, tsize), fresh);
+            if (s == ~0u) return -1;
+            again = !fresh;
         }
         const uint32_t lo = (uint32_t)v;
         const uint32_t old = atomicAdd(&sum[s].x, lo);
@@ -115,7 +91,7 @@ struct SumTable {
             const uint32_t i = g.first(k);
             if (i < Group::kN) return s + i;
             if (g.last() == kEmpty) return ~0u;
-            s = next_group(s, tsize);
+            s = next_group<KeyT>(s, tsize);
         }
         return ~0u;
     }
