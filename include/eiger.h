@@ -173,10 +173,13 @@ eiger_status eiger_join_workspace(int64_t nb, int64_t np, eiger_dtype dtype, eig
  *          row; NULL when absent). They are read only when the matching
  *          d_out_*pay output is requested (gather by tuple ID, Sec. 3.2 GFUR).
  * variant: EIGER_AUTO runs eiger_stats on the build keys, then eiger_plan,
- *          then the chosen variant. NPHJ/PHJ1/PHJ2 also profile the build keys
- *          (narrowing and the probe range test need min/max) and take their
- *          knobs from `knobs` when non-NULL (bits1/bits2/narrow/load_factor),
- *          else from the planner. EIGER_STATIC profiles nothing.
+ *          then the chosen variant; where the build keys are dense and distinct
+ *          (32-bit keys over a span of at most 8 nb) a partitioned plan gets
+ *          fewer radix bits (tables of up to 2^14 direct-addressed slots).
+ *          NPHJ/PHJ1/PHJ2 also profile the build keys (narrowing and the probe
+ *          range test need min/max) and take their knobs from `knobs` when
+ *          non-NULL (bits1/bits2/narrow/load_factor), else from the planner.
+ *          EIGER_STATIC profiles nothing.
  * Outputs (each NULL or an array of `capacity` elements, at least one given):
  *          d_out_bidx / d_out_pidx: uint32 build / probe row of each match;
  *          d_out_bpay / d_out_ppay: the matching rows' payloads (payload_bytes

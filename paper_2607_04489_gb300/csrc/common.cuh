@@ -146,6 +146,8 @@ struct Ctrl {
     unsigned long long sum;        // aggregate mode: sum of payload pairs mod 2^64
     unsigned long long next_item;  // PHJ work-item dispenser
     unsigned long long nitems;     // PHJ work items
+    unsigned long long next_redo;  // PHJ: dispenser and number of the items a direct-addressed
+    unsigned long long nredo;      // launch left to hash tables
     unsigned int err;              // kErr* flags
     unsigned int ntiles2[2];       // pass-2 tile count per side (build, probe)
     unsigned int kept[2];          // rows kept by the range test per side

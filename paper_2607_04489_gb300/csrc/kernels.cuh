@@ -68,6 +68,7 @@ struct PlanDev {
     int narrow;       // frame-of-reference narrowing applied (offset = build min)
     int key32;        // keys carried as 32-bit values (int32, or int64 narrowed)
     int kbits;        // hash partitioning: bits of the key mix (key32: of the build span; else 64)
+    int direct;       // partitioned join: direct-addressed tables (phj.cuh)
     float load_factor;
     int dtype;        // 0 int32, 1 int64
     KeyRange range;   // build range (probe range test) and encoding offset
@@ -152,6 +153,7 @@ struct PhjScratch {
     void* rec;
     uint32_t* ovf[2];
     ChunkFix fix;
+    unsigned long long* redo;  // items a direct-addressed launch leaves to hash tables
 };
 
 PhjScratch phj_layout(Carve& c, int64_t nb, int64_t np, const PlanDev& plan);

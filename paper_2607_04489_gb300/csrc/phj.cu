@@ -11,10 +11,19 @@
 // a partition are balanced in size. A persistent grid pulls
 // items from a global counter. Per item a CTA clears a table of about three
 // slots per build row (load factor <= 1/3), inserts the build chunk with
-// shared-memory CAS, then streams the probe chunk, walking linear-probe chains.
+// shared-memory CAS, then streams the probe chunk, walking linear-probe chains;
+// or, where the build keys are dense and distinct, fills a direct-addressed
+// table (phj.cuh) that takes the whole build partition and reads one word per
+// probe row.
 // Index pairs leave through per-warp output runs (chunks.cuh), so the probe
-// loop has no CTA barrier; payloads, GFTR positions and aggregates go through
-// the CTA stage (emit.cuh).
+// loop has no CTA barrier; columns through one CTA reservation per round, column
+// by column; the matches of repeated build keys through the CTA stage
+// (emit.cuh).
+//
+// What bounds it: direct-addressed pairs read one shared word and write 8 bytes
+// per probe row (28M rows of dense keys: 0.23 ms with hash tables, 0.17 ms);
+// columns wait on the gathers of the build side's values (114M rows, two 4-byte
+// columns a side: 1.79 ms row by row through hash tables and the stage, 1.29 ms).
 #include "chunks.cuh"
 #include "emit.cuh"
 #include "kernels.cuh"
@@ -27,35 +36,36 @@ size_t part_scan_blocks(size_t counts_len);
 
 namespace {
 
-constexpr int kMaxRows = 8;                       // rows per thread per round (at most)
-constexpr int kJoinStage = kJoinThreads * kMaxRows;  // a unique-key round never spills
+// How matches leave the kernel: index pairs through per-warp output runs
+// (chunks.cuh), columns (and indices beside them) through a CTA reservation per
+// round, or summed.
+enum JoinMode { kPairs, kColumns, kSum };
 
 // Rows each thread keeps in flight per round (the current round and the next
 // one's loads) and CTAs per SM. Index pairs of 32-bit keys: 4 rows, three
 // 512-thread CTAs per SM (40 registers), so that while one CTA clears or builds
 // its table the others probe theirs (measured on GB300: 16 % faster than two
-// CTAs of 8 rows). Payload, position and aggregate outputs keep more live
-// state per match and 64-bit keys larger tables: two CTAs per SM, 8 rows for
-// 32-bit keys and 4 for 64-bit keys (64 registers).
-template <typename KeyT, bool PAIRS>
+// CTAs of 8 rows). Columns and sums keep more live state per match and 64-bit
+// keys larger tables: two CTAs per SM (64 registers), 8 rows for the sums of
+// 32-bit keys and 4 otherwise.
+template <typename KeyT, int MODE>
 struct Rows {
-    static constexpr bool kLean = sizeof(KeyT) == 4 && PAIRS;
-    static constexpr int kN = kLean || sizeof(KeyT) != 4 ? 4 : 8;
+    static constexpr bool kLean = sizeof(KeyT) == 4 && MODE == kPairs;
+    static constexpr int kN = sizeof(KeyT) == 4 && MODE == kSum ? 8 : 4;
     static constexpr int kMinBlocks = (kLean ? 1536 : 1024) / kJoinThreads;
     static constexpr uint32_t kRound = kJoinThreads * kN;
 };
+constexpr int kJoinStage = kJoinThreads * 4;  // matches staged between two flushes (duplicate build keys)
 constexpr uint32_t kTableMax = 2 * kBuildCap;
 constexpr uint32_t kEmptyRow = 0xFFFFFFFFu;
 
 // Work items of partition p: build chunks x probe chunks (none if a side is empty).
 __global__ void items_count_kernel(const uint32_t* __restrict__ bstart, const uint32_t* __restrict__ pstart,
-                                   uint32_t P, unsigned long long* __restrict__ count) {
+                                   uint32_t P, uint32_t bcap, uint32_t pcap, unsigned long long* __restrict__ count) {
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
         const uint32_t bs = bstart[p + 1] - bstart[p];
         const uint32_t ps = pstart[p + 1] - pstart[p];
-        count[p] = (bs && ps) ? (unsigned long long)((bs + kBuildCap - 1) / kBuildCap) *
-                                    ((ps + kProbeChunk - 1) / kProbeChunk)
-                              : 0ull;
+        count[p] = (bs && ps) ? (unsigned long long)chunks_of(bs, bcap) * chunks_of(ps, pcap) : 0ull;
     }
 }
 
@@ -229,34 +239,34 @@ constexpr uint32_t kHole = 0xFFFFFFFFu;  // stage position without a match
 
 constexpr int kJoinWarps = kJoinThreads / kWarp;
 
-// Block-collective flush of a positional stage: position j * kJoinThreads + t
-// holds the match of thread t's row j, or kHole. Ballots give every match its
-// rank within its (row j, warp) group, one scan over the kN x warps group
-// counts places the groups, one global atomic reserves the round's output,
-// and each warp then writes its group to consecutive output positions.
-// Thread t reads back only its own stage entries, so no barrier precedes the
-// ballots: the previous round's closing barrier already orders every read of
-// s_grp before the new counts are written.
+// Block-collective: writes a round's matches (b[j] != kHole) with their columns.
+// Ballots rank every match within its (row j, warp) group, one scan over the
+// group counts places the groups, one global atomic reserves the round's
+// output. Each column is then read for all rows of a thread before any of them
+// is written (one memory round trip per column and round; row by row the
+// gathers of 8 rows x 4 columns had waited for one another). s_grp alternates
+// between two halves by round, so no barrier follows the writes.
 template <int kN>
-__device__ __forceinline__ void flush_positional(Stage<kJoinStage>& st, uint32_t* s_grp,
-                                                 const JoinOut& out, Ctrl* ctrl) {
+__device__ __forceinline__ void flush_columns(const uint32_t (&b)[kN], const uint32_t (&p)[kN], uint32_t* s_grp,
+                                              unsigned long long* s_base, const JoinOut& out, Ctrl* ctrl) {
     const unsigned lane = lane_id();
     const int w = threadIdx.x / kWarp;
-    unsigned ball[kN];
+    constexpr int kGroups = kN * kJoinWarps;
+    unsigned rank[kN];
 #pragma unroll
     for (int j = 0; j < kN; ++j) {
-        ball[j] = __ballot_sync(0xffffffffu, st.b[j * kJoinThreads + threadIdx.x] != kHole);
-        if (lane == 0) s_grp[j * kJoinWarps + w] = __popc(ball[j]);
+        const unsigned m = __ballot_sync(0xffffffffu, b[j] != kHole);
+        rank[j] = __popc(m & lanemask_lt());
+        if (lane == 0) s_grp[j * kJoinWarps + w] = __popc(m);
     }
     __syncthreads();
     if (w == 0) {
-        // exclusive scan of kN * kJoinWarps group counts, kN * 16 / 32 per lane
-        constexpr int kPer = (kN * kJoinWarps + kWarp - 1) / kWarp;
+        constexpr int kPer = (kGroups + kWarp - 1) / kWarp;
         uint32_t v[kPer], local = 0;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int e = lane * kPer + i;
-            v[i] = e < kN * kJoinWarps ? s_grp[e] : 0u;
+            v[i] = e < kGroups ? s_grp[e] : 0u;
             local += v[i];
         }
         uint32_t x = local;
@@ -269,67 +279,95 @@ __device__ __forceinline__ void flush_positional(Stage<kJoinStage>& st, uint32_t
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
             const int e = lane * kPer + i;
-            if (e < kN * kJoinWarps) s_grp[e] = run;
+            if (e < kGroups) s_grp[e] = run;
             run += v[i];
         }
-        const uint32_t total = __shfl_sync(0xffffffffu, x, kWarp - 1);
-        if (lane == 0) {
-            st.base = total ? atomicAdd(&ctrl->cursor, (unsigned long long)total) : 0ull;
-            st.count = (unsigned)(st.base + total <= out.capacity);  // whole round fits
-        }
+        if (lane == kWarp - 1) *s_base = x ? atomicAdd(&ctrl->cursor, (unsigned long long)x) : 0ull;
     }
     __syncthreads();
-    const unsigned long long base = st.base;
-    const bool fits = st.count != 0;
-    const unsigned lt = lanemask_lt();
+    const unsigned long long base = *s_base;
+    const unsigned long long room = out.capacity > base ? out.capacity - base : 0ull;
+    uint32_t pos[kN];  // offset from base, or kHole
 #pragma unroll
     for (int j = 0; j < kN; ++j) {
-        const uint32_t i = j * kJoinThreads + threadIdx.x;
-        if (ball[j] & (1u << lane)) {
-            const unsigned long long pos = base + s_grp[j * kJoinWarps + w] + __popc(ball[j] & lt);
-            (void)fits;
-            write_match(out, pos, st.b[i], st.p[i]);
-        }
+        pos[j] = s_grp[j * kJoinWarps + w] + rank[j];
+        if (b[j] == kHole || pos[j] >= room) pos[j] = kHole;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) st.count = 0;
+    auto index = [&](uint32_t* dst, const uint32_t* map, const uint32_t(&row)[kN]) {
+        uint32_t v[kN];
+#pragma unroll
+        for (int j = 0; j < kN; ++j)
+            if (pos[j] != kHole) v[j] = map ? __ldg(map + row[j]) : row[j];
+#pragma unroll
+        for (int j = 0; j < kN; ++j)
+            if (pos[j] != kHole) __stcs(dst + base + pos[j], v[j]);
+    };
+    auto column = [&](const ColSide& cs, int c, const uint32_t(&row)[kN]) {
+        if (cs.bytes[c] == 4) {
+            index(static_cast<uint32_t*>(cs.dst[c]), static_cast<const uint32_t*>(cs.src[c]), row);
+        } else {
+            const uint2* src = static_cast<const uint2*>(cs.src[c]);
+            uint2* dst = static_cast<uint2*>(cs.dst[c]);
+            uint2 v[kN];
+#pragma unroll
+            for (int j = 0; j < kN; ++j)
+                if (pos[j] != kHole) v[j] = __ldg(src + row[j]);
+#pragma unroll
+            for (int j = 0; j < kN; ++j)
+                if (pos[j] != kHole) __stcs(dst + base + pos[j], v[j]);
+        }
+    };
+    if (out.bidx) index(out.bidx, out.b.rowmap, b);
+    if (out.pidx) index(out.pidx, out.p.rowmap, p);
+#pragma unroll 1
+    for (int c = 0; c < out.b.n; ++c) column(out.b, c, b);
+#pragma unroll 1
+    for (int c = 0; c < out.p.n; ++c) column(out.p, c, p);
 }
 
-// PAIRS: index pairs only, written through per-warp output runs (chunks.cuh)
-// without any CTA barrier in the probe loop; otherwise matches go through the
-// CTA stage (emit.cuh), which also gathers payloads, maps positions back to
-// tuple IDs (GFTR) or aggregates.
-template <typename KeyT, bool AGG, bool PAIRS, bool POS>
-__global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, PAIRS>::kMinBlocks))
-    phj_join_kernel(JoinIn<KeyT> a, JoinOut out, PairSink sink, Ctrl* ctrl) {
+// kHash: one hash table per item. kDirect: direct-addressed tables (32-bit
+// keys), slot -> build row; an item whose build keys repeat (a slot taken twice)
+// is left to a second launch. kRedo: those items, through hash tables of
+// kBuildCap build rows each.
+enum JoinKind { kHash, kDirect, kRedo };
+
+template <typename KeyT, int MODE, bool POS, int KIND>
+__global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
+    phj_join_kernel(JoinIn<KeyT> a, const __grid_constant__ JoinOut out, PairSink sink, uint32_t first_warp,
+                    Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr bool PAIRS = MODE == kPairs, AGG = MODE == kSum;
     // the stage follows the table in dynamic shared memory; index pairs and
     // aggregates use none, so none is allocated for them (shared memory left
     // unreserved serves as L1 cache, which the payload gathers of the
     // aggregate need)
-    constexpr bool kStage = !PAIRS && !AGG;
     Stage<kJoinStage>& st = *reinterpret_cast<Stage<kJoinStage>*>(smem + (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes);
-    __shared__ uint32_t s_grp[kMaxRows * kJoinWarps];
+    constexpr int kN = Rows<KeyT, MODE>::kN;
+    constexpr uint32_t kRound = Rows<KeyT, MODE>::kRound;
+    __shared__ uint32_t s_grp[2][MODE == kColumns ? kN * kJoinWarps : 1];
+    __shared__ unsigned long long s_base[2];
     __shared__ unsigned long long s_next_item;
     __shared__ uint32_t s_next_part;
-    constexpr int kN = Rows<KeyT, PAIRS>::kN;
-    constexpr uint32_t kRound = Rows<KeyT, PAIRS>::kRound;
     SmemTable<KeyT> tab;
     tab.bind(smem);
-    if (kStage && threadIdx.x == 0) st.count = 0;
+    uint32_t* dtab = reinterpret_cast<uint32_t*>(smem);
+    if (MODE == kColumns && KIND != kDirect && threadIdx.x == 0) st.count = 0;
     AggState agg{0ull, 0ull};
     WarpChunk wc;
     wc.init();
-    const unsigned long long nitems = ctrl->nitems;
+    uint32_t flushes = 0;
+    const unsigned long long nitems = KIND == kRedo ? ctrl->nredo : ctrl->nitems;
+    unsigned long long* const next = KIND == kRedo ? &ctrl->next_redo : &ctrl->next_item;
+    auto item_of = [&](unsigned long long i) { return KIND == kRedo ? a.redo[i] : i; };
 
     // Work items are claimed one ahead: the claim for the next item is issued
     // when an item starts, and its partition is looked up by warp 0 after the
     // build, so neither round trip sits between two items.
     if (threadIdx.x < kWarp) {
         unsigned long long it0 = 0;
-        if (threadIdx.x == 0) it0 = atomicAdd(&ctrl->next_item, 1ull);
+        if (threadIdx.x == 0) it0 = atomicAdd(next, 1ull);
         it0 = __shfl_sync(0xffffffffu, it0, 0);
-        const uint32_t p0 = it0 < nitems ? find_partition(a.item_prefix, a.P, it0) : 0u;
+        const uint32_t p0 = it0 < nitems ? find_partition(a.item_prefix, a.P, item_of(it0)) : 0u;
         if (threadIdx.x == 0) {
             s_next_item = it0;
             s_next_part = p0;
@@ -338,11 +376,12 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, PAIRS>::kMinBlocks))
     __syncthreads();
 
     for (;;) {
-        const unsigned long long item = s_next_item;
+        const unsigned long long cur_item = s_next_item;
         const uint32_t p = s_next_part;
-        if (item >= nitems) break;
+        if (cur_item >= nitems) break;
+        const unsigned long long item = item_of(cur_item);
         unsigned long long claim = 0;
-        if (threadIdx.x == 0) claim = atomicAdd(&ctrl->next_item, 1ull);
+        if (threadIdx.x == 0) claim = atomicAdd(next, 1ull);
 
         const ItemRows ir = item_rows(a, item, p);
         const uint32_t bn = ir.bn, pn = ir.pn;
@@ -350,162 +389,255 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, PAIRS>::kMinBlocks))
         const uint32_t* bidx = a.bidx + ir.bs0;
         const KeyT* pkey = a.pkey + ir.ps0;
         const uint32_t* pidx = a.pidx + ir.ps0;
-        // about three slots per build row (load <= 1/3), at most kTableMax
-        uint32_t tsize = (3 * bn + 31) & ~31u;
-        if (tsize < 64) tsize = 64;
-        if (tsize > kTableMax) tsize = kTableMax;
+        const uint32_t bpos0 = ir.bs0, ppos0 = ir.ps0;
 
         // Issue the first build and probe loads before clearing the table, so
         // their latency overlaps the clear.
         RoundRegs<KeyT, kN> cur, nxt;
-        const uint32_t bpos0 = ir.bs0, ppos0 = ir.ps0;
-        load_round<POS>(nxt, bkey, bidx, 0, bn, bpos0);
+        load_round<POS>(nxt, bkey, bidx, 0, KIND == kRedo ? min(bn, kBuildCap) : bn, bpos0);
         load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
-        tab.clear_all(tsize);
-        __syncthreads();
-        // Build. An insert that meets its own key proves a duplicate in this
-        // chunk; without one, every probe key has at most one match here.
-        int dup = 0;
-        for (uint32_t bb = 0; bb < bn; bb += kRound) {
-            if (bb) load_round<POS>(nxt, bkey, bidx, bb, bn, bpos0);
-#pragma unroll
-            for (int j = 0; j < kN; ++j) {
-                if (bb + j * kJoinThreads + threadIdx.x >= bn) continue;
-                uint32_t s = home_slot(nxt.k[j], tsize);
-                for (uint32_t step = 0;; ++step) {
-                    const int r = tab.insert(s, nxt.k[j], nxt.id[j]);
-                    if (r > 0) break;
-                    if (r < 0) dup = 1;
-                    if (step + 1 == tsize) {
-                        atomicOr(&ctrl->err, kErrTableFull);
-                        break;
-                    }
-                    s = next_slot(s, tsize);
-                }
-            }
-        }
-        if constexpr (sizeof(KeyT) != 4) {
-            __syncthreads();  // every key of the table is written
-            dup = tab.has_equal_keys(tsize);
-        }
-        const bool unique = __syncthreads_or(dup) == 0;
-        if (threadIdx.x < kWarp) {  // look up the next item while the probes run
-            claim = __shfl_sync(0xffffffffu, claim, 0);
-            const uint32_t pn2 = claim < nitems ? find_partition(a.item_prefix, a.P, claim) : 0u;
+
+        // Looks up the next item while the probes run, and asks L2 for the
+        // start of its partition's build rows and its first probe round, so
+        // that it starts on cache hits.
+        auto next_item = [&] {
+            if (threadIdx.x >= kWarp) return;
+            const unsigned long long cl = __shfl_sync(0xffffffffu, claim, 0);
+            const uint32_t pn2 = cl < nitems ? find_partition(a.item_prefix, a.P, item_of(cl)) : 0u;
             if (threadIdx.x == 0) {
-                s_next_item = claim;
+                s_next_item = cl;
                 s_next_part = pn2;
             }
-            // ask L2 for the start of the next partition's build rows and its
-            // first probe round, so that item starts on cache hits
-            if (claim < nitems) {
+            if (cl < nitems) {
                 const uint32_t nb0 = a.bstart[pn2], nbn = min(a.bstart[pn2 + 1] - nb0, kBuildCap);
                 const uint32_t np0 = a.pstart[pn2], npn = min(a.pstart[pn2 + 1] - np0, kRound);
                 prefetch_rows_l2<POS>(a.bkey + nb0, a.bidx + nb0, nbn, threadIdx.x, kWarp);
                 prefetch_rows_l2<POS>(a.pkey + np0, a.pidx + np0, npn, threadIdx.x, kWarp);
             }
-        }
+        };
+        // Probe rows round by round: the next round's loads are in flight while
+        // this round probes, and the round after it is on its way into L2.
+        auto probe_rounds = [&](auto&& round) {
+            for (uint32_t base = 0; base < pn; base += kRound) {
+                if (base + kRound < pn) load_round<POS>(nxt, pkey, pidx, base + kRound, pn, ppos0);
+                if (base + 2 * kRound < pn)
+                    prefetch_rows_l2<POS>(pkey + base + 2 * kRound, pidx + base + 2 * kRound,
+                                          min(pn - (base + 2 * kRound), kRound), threadIdx.x, kJoinThreads);
+                round(base);
+                cur = nxt;
+            }
+        };
+        // A round with at most one match per row: brow[j] or kHole.
+        auto emit_round = [&](const uint32_t(&brow)[kN]) {
+            if constexpr (PAIRS) {
+#pragma unroll
+                for (int j = 0; j < kN; ++j) warp_emit(wc, sink, brow[j] != kHole, brow[j], cur.id[j]);
+            } else if constexpr (AGG) {
+#pragma unroll
+                for (int j = 0; j < kN; ++j)
+                    if (brow[j] != kHole) {
+                        agg.sum += (unsigned long long)read_pay(out.b.src[0], out.b.bytes[0], brow[j]) +
+                                   (unsigned long long)read_pay(out.p.src[0], out.p.bytes[0], cur.id[j]);
+                        agg.count += 1;
+                    }
+            } else {
+                const uint32_t h = flushes++ & 1;
+                flush_columns<kN>(brow, cur.id, s_grp[h], &s_base[h], out, ctrl);
+            }
+        };
 
-        for (uint32_t base = 0; base < pn; base += kRound) {
-            // the next round's loads are in flight while this round probes,
-            // and the round after it is on its way into L2
-            if (base + kRound < pn) load_round<POS>(nxt, pkey, pidx, base + kRound, pn, ppos0);
-            if (base + 2 * kRound < pn)
-                prefetch_rows_l2<POS>(pkey + base + 2 * kRound, pidx + base + 2 * kRound,
-                                      min(pn - (base + 2 * kRound), kRound), threadIdx.x, kJoinThreads);
-            if (unique) {
-                // Fast path: stop at the first match, no collectives per step.
+        if constexpr (KIND == kDirect) {
+            const uint32_t slots = 1u << a.sbits;
+            uint4* d4 = reinterpret_cast<uint4*>(dtab);
+            for (uint32_t i = threadIdx.x; i < slots / 4 + 1; i += kJoinThreads)
+                d4[i] = make_uint4(kHole, kHole, kHole, kHole);
+            __syncthreads();
+            int dup = 0;
+            for (uint32_t bb = 0; bb < bn; bb += kRound) {
+                if (bb) load_round<POS>(nxt, bkey, bidx, bb, bn, bpos0);
+#pragma unroll
+                for (int j = 0; j < kN; ++j)
+                    if (bb + j * kJoinThreads + threadIdx.x < bn)
+                        dup |= atomicExch(dtab + direct_slot(nxt.k[j], a.pbits, a.sbits), nxt.id[j]) != kHole;
+            }
+            const bool repeats = __syncthreads_or(dup) != 0;
+            next_item();
+            if (repeats) {
+                if (threadIdx.x == 0) a.redo[atomicAdd(&ctrl->nredo, 1ull)] = item;
+            } else {
+                probe_rounds([&](uint32_t base) {
+                    uint32_t brow[kN];
+#pragma unroll
+                    for (int j = 0; j < kN; ++j)
+                        brow[j] = base + j * kJoinThreads + threadIdx.x < pn
+                                      ? dtab[direct_slot(cur.k[j], a.pbits, a.sbits)]
+                                      : kHole;
+                    emit_round(brow);
+                });
+            }
+        }
+        // hash tables: the whole build chunk, or kBuildCap of its rows at a time
+        if constexpr (KIND != kDirect) for (uint32_t b0 = 0; b0 < bn; b0 += KIND == kRedo ? kBuildCap : bn) {
+            const uint32_t hn = KIND == kRedo ? min(bn - b0, kBuildCap) : bn;
+            if (KIND == kRedo && b0) {  // the registers hold other rows by now
+                __syncthreads();
+                load_round<POS>(nxt, bkey + b0, bidx + b0, 0, hn, bpos0 + b0);
+                load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
+            }
+            // about three slots per build row (load <= 1/3), at most kTableMax
+            uint32_t tsize = (3 * hn + 31) & ~31u;
+            if (tsize < 64) tsize = 64;
+            if (tsize > kTableMax) tsize = kTableMax;
+            tab.clear_all(tsize);
+            __syncthreads();
+            // Build. An insert that meets its own key proves a duplicate in this
+            // chunk; without one, every probe key has at most one match here.
+            int dup = 0;
+            for (uint32_t bb = 0; bb < hn; bb += kRound) {
+                if (bb) load_round<POS>(nxt, bkey + b0, bidx + b0, bb, hn, bpos0 + b0);
 #pragma unroll
                 for (int j = 0; j < kN; ++j) {
-                    uint32_t brow = kHole;
-                    if (base + j * kJoinThreads + threadIdx.x < pn) {
-                        const KeyT k = cur.k[j];
-                        uint32_t s = home_slot(k, tsize);
-                        if constexpr (sizeof(KeyT) == 4) {
-                            for (uint32_t step = 0; step < tsize; step += 2) {
-                                const ulonglong2 v = tab.pair(s);
-                                if (v.x == kEmptySlot) break;
-                                if ((uint32_t)(v.x >> 32) == (uint32_t)k) {
-                                    brow = (uint32_t)v.x;
-                                    break;
-                                }
-                                if (v.y == kEmptySlot) break;
-                                if ((uint32_t)(v.y >> 32) == (uint32_t)k) {
-                                    brow = (uint32_t)v.y;
-                                    break;
-                                }
-                                s = s + 2 == tsize ? 0u : s + 2;
+                    if (bb + j * kJoinThreads + threadIdx.x < hn) {
+                        uint32_t s = home_slot(nxt.k[j], tsize);
+                        for (uint32_t step = 0;; ++step) {
+                            const int r = tab.insert(s, nxt.k[j], nxt.id[j]);
+                            if (r > 0) break;
+                            if (r < 0) dup = 1;
+                            if (step + 1 == tsize) {
+                                atomicOr(&ctrl->err, kErrTableFull);
+                                break;
                             }
-                        } else {
-                            for (uint32_t step = 0; step < tsize; ++step) {
-                                uint32_t r;
-                                const int q = tab.probe(s, k, r);
-                                if (q == 0) break;
-                                if (q == 2) {
-                                    brow = r;
-                                    break;
-                                }
-                                s = next_slot(s, tsize);
-                            }
+                            s = next_slot(s, tsize);
                         }
                     }
-                    if constexpr (PAIRS) {
-                        warp_emit(wc, sink, brow != kHole, brow, cur.id[j]);
-                    } else if constexpr (AGG) {
-                        if (brow != kHole) {
-                            agg.sum += (unsigned long long)read_pay(out.b.src[0], out.b.bytes[0], brow) +
-                                       (unsigned long long)read_pay(out.p.src[0], out.p.bytes[0], cur.id[j]);
-                            agg.count += 1;
-                        }
-                    } else {
-                        st.b[j * kJoinThreads + threadIdx.x] = brow;
-                        st.p[j * kJoinThreads + threadIdx.x] = cur.id[j];
-                    }
+                    __syncwarp();
                 }
-                if constexpr (!AGG && !PAIRS) flush_positional<kN>(st, s_grp, out, ctrl);
+            }
+            if constexpr (sizeof(KeyT) != 4) {
+                __syncthreads();  // every key of the table is written
+                dup = tab.has_equal_keys(tsize);
+            }
+            const bool unique = __syncthreads_or(dup) == 0;
+            if (b0 == 0) next_item();
+            if (unique) {
+                // Fast path: stop at the first match, no collectives per step.
+                probe_rounds([&](uint32_t base) {
+                    uint32_t brow[kN];
+#pragma unroll
+                    for (int j = 0; j < kN; ++j) {
+                        brow[j] = kHole;
+                        if (base + j * kJoinThreads + threadIdx.x < pn) {
+                            const KeyT k = cur.k[j];
+                            uint32_t s = home_slot(k, tsize);
+                            if constexpr (sizeof(KeyT) == 4) {
+                                for (uint32_t step = 0; step < tsize; step += 2) {
+                                    const ulonglong2 v = tab.pair(s);
+                                    if (v.x == kEmptySlot) break;
+                                    if ((uint32_t)(v.x >> 32) == (uint32_t)k) {
+                                        brow[j] = (uint32_t)v.x;
+                                        break;
+                                    }
+                                    if (v.y == kEmptySlot) break;
+                                    if ((uint32_t)(v.y >> 32) == (uint32_t)k) {
+                                        brow[j] = (uint32_t)v.y;
+                                        break;
+                                    }
+                                    s = s + 2 == tsize ? 0u : s + 2;
+                                }
+                            } else {
+                                for (uint32_t step = 0; step < tsize; ++step) {
+                                    uint32_t r;
+                                    const int q = tab.probe(s, k, r);
+                                    if (q == 0) break;
+                                    if (q == 2) {
+                                        brow[j] = r;
+                                        break;
+                                    }
+                                    s = next_slot(s, tsize);
+                                }
+                            }
+                        }
+                        __syncwarp();
+                    }
+                    emit_round(brow);
+                });
             } else {
                 // General path (duplicate keys): every match of every chain,
                 // emitted through the warp-aggregated stage.
+                probe_rounds([&](uint32_t base) {
 #pragma unroll 1
-                for (int j = 0; j < kN; ++j) {
-                    bool active = base + j * kJoinThreads + threadIdx.x < pn;
-                    const KeyT k = cur.k[j];
-                    const uint32_t id = cur.id[j];
-                    uint32_t s = active ? home_slot(k, tsize) : 0u;
-                    uint32_t steps = 0;
-                    while (__any_sync(0xffffffffu, active)) {
-                        bool hit = false;
-                        uint32_t brow = 0;
-                        if (active) {
-                            const int r = tab.probe(s, k, brow);
-                            if (r == 0) {
-                                active = false;
-                            } else {
-                                hit = r == 2;
-                                s = next_slot(s, tsize);
-                                if (++steps == tsize) active = false;
+                    for (int j = 0; j < kN; ++j) {
+                        bool active = base + j * kJoinThreads + threadIdx.x < pn;
+                        const KeyT k = cur.k[j];
+                        const uint32_t id = cur.id[j];
+                        uint32_t s = active ? home_slot(k, tsize) : 0u;
+                        uint32_t steps = 0;
+                        while (__any_sync(0xffffffffu, active)) {
+                            bool hit = false;
+                            uint32_t brow = 0;
+                            if (active) {
+                                const int r = tab.probe(s, k, brow);
+                                if (r == 0) {
+                                    active = false;
+                                } else {
+                                    hit = r == 2;
+                                    s = next_slot(s, tsize);
+                                    if (++steps == tsize) active = false;
+                                }
                             }
+                            if constexpr (PAIRS)
+                                warp_emit(wc, sink, hit, brow, id);
+                            else
+                                emit<AGG, kJoinStage>(st, agg, hit, brow, id, out, &ctrl->cursor);
                         }
-                        if constexpr (PAIRS)
-                            warp_emit(wc, sink, hit, brow, id);
-                        else
-                            emit<AGG, kJoinStage>(st, agg, hit, brow, id, out, &ctrl->cursor);
+                        if constexpr (MODE == kColumns) stage_flush<AGG, kJoinStage>(st, out, &ctrl->cursor);
                     }
-                }
-                if constexpr (!PAIRS) stage_flush<AGG, kJoinStage>(st, out, &ctrl->cursor);
+                });
             }
-            cur = nxt;
         }
         __syncthreads();
     }
     if (AGG) agg_commit(agg, ctrl);
-    if constexpr (PAIRS) warp_chunk_commit(wc, sink, blockIdx.x * kJoinWarps + threadIdx.x / kWarp);
+    if constexpr (PAIRS) warp_chunk_commit(wc, sink, first_warp + blockIdx.x * kJoinWarps + threadIdx.x / kWarp);
 }
 
+// Launches of one join; counts the warps launched (each writes a warp record
+// of the pairs sink).
 template <typename KeyT>
-size_t join_smem(bool stage) {
-    return (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes + (stage ? sizeof(Stage<kJoinStage>) : 0);
-}
+struct JoinLaunch {
+    static constexpr int kAll = 1 << 20;  // as many CTAs per SM as fit
+    const JoinIn<KeyT>& a;
+    const JoinOut& out;
+    const PairSink& sink;
+    Ctrl* ctrl;
+    const DevInfo& di;
+    cudaStream_t stream;
+    uint32_t warps;
+
+    template <int MODE, bool POS, int KIND>
+    cudaError_t run(int most_per_sm) {
+        auto kern = phj_join_kernel<KeyT, MODE, POS, KIND>;
+        const size_t smem =
+            KIND == kDirect ? ((size_t)4 << a.sbits) + 16
+                            : (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
+                                  (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kJoinThreads, smem) != cudaSuccess ||
+            per_sm < 1)
+            per_sm = 1;
+        if (per_sm > most_per_sm) per_sm = most_per_sm;
+        uint32_t grid = (uint32_t)(di.sms * per_sm);
+        const uint32_t room = (kMaxOutWarps - warps) / kJoinWarps;  // warp records left
+        // (a direct launch leaves records for the second one)
+        const uint32_t keep = KIND == kDirect ? room / 4 : 0;
+        if (grid > room - keep) grid = room - keep;
+        kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, warps, ctrl);
+        warps += grid * kJoinWarps;
+        return cudaGetLastError();
+    }
+};
 
 template <typename KeyT>
 cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut& out, Ctrl* ctrl,
@@ -523,23 +655,14 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     a.P = 1u << (plan.bits1 + (passes == 2 ? plan.bits2 : 0));
     const bool pairs = !out.aggregate && out.bidx && out.pidx && out.b.n == 0 && out.p.n == 0 && !out.b.rowmap &&
                        !out.p.rowmap;
+    a.bcap = plan.direct ? 0xFFFFFFFFu : kBuildCap;
+    a.pcap = plan.direct ? kDirectProbeChunk : kProbeChunk;
+    a.pbits = plan.bits1 + (passes == 2 ? plan.bits2 : 0);
+    a.sbits = plan.kbits - a.pbits > 1 ? plan.kbits - a.pbits : 1;
     // the sum with carried payloads has its own kernel (phj_sum.cu)
-    if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, out, ctrl, di, stream, nb, np);
-    auto kern = out.aggregate ? phj_join_kernel<KeyT, true, false, false>
-                : pairs       ? phj_join_kernel<KeyT, false, true, false>
-                : plan.gftr   ? phj_join_kernel<KeyT, false, false, true>
-                              : phj_join_kernel<KeyT, false, false, false>;
+    if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, plan.direct, out, ctrl, di, stream, nb, np);
     // reads every partitioned (key', row) of both sides once, writes the matches
     ProfScope ps("phj_join", (double)(sizeof(KeyT) + sizeof(uint32_t)) * (double)(nb + np), stream, match_bytes(out));
-    const size_t smem = join_smem<KeyT>(!pairs && !out.aggregate);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kJoinThreads, smem) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    uint32_t grid = (uint32_t)(di.sms * per_sm);
-    if (grid > kMaxOutWarps / kJoinWarps) grid = kMaxOutWarps / kJoinWarps;  // warp records of the pairs sink
     PairSink sink{};
     if (pairs) {
         sink.bidx = out.bidx;
@@ -550,9 +673,31 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
         sink.cursor = &ctrl->cursor;
         sink.rec = static_cast<ChunkRec*>(s.rec);
     }
-    kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, ctrl);
-    if ((e = cudaGetLastError()) != cudaSuccess || !pairs) return e;
-    return chunk_fix_run(sink, grid * kJoinWarps, s.fix, &ctrl->err, di, stream);
+    a.redo = s.redo;
+    JoinLaunch<KeyT> l{a, out, sink, ctrl, di, stream, 0};
+    cudaError_t e;
+    if constexpr (sizeof(KeyT) == 4) {
+        if (plan.direct) {
+            e = out.aggregate ? l.template run<kSum, false, kDirect>(l.kAll)
+                : pairs       ? l.template run<kPairs, false, kDirect>(l.kAll)
+                : plan.gftr   ? l.template run<kColumns, true, kDirect>(l.kAll)
+                              : l.template run<kColumns, false, kDirect>(l.kAll);
+            // the items whose build keys repeat (most often none)
+            if (e == cudaSuccess)
+                e = out.aggregate ? l.template run<kSum, false, kRedo>(1)
+                    : pairs       ? l.template run<kPairs, false, kRedo>(1)
+                    : plan.gftr   ? l.template run<kColumns, true, kRedo>(1)
+                                  : l.template run<kColumns, false, kRedo>(1);
+            if (e != cudaSuccess || !pairs) return e;
+            return chunk_fix_run(sink, l.warps, s.fix, &ctrl->err, di, stream);
+        }
+    }
+    e = out.aggregate ? l.template run<kSum, false, kHash>(l.kAll)
+        : pairs       ? l.template run<kPairs, false, kHash>(l.kAll)
+        : plan.gftr   ? l.template run<kColumns, true, kHash>(l.kAll)
+                      : l.template run<kColumns, false, kHash>(l.kAll);
+    if (e != cudaSuccess || !pairs) return e;
+    return chunk_fix_run(sink, l.warps, s.fix, &ctrl->err, di, stream);
 }
 
 }  // namespace
@@ -570,6 +715,7 @@ PhjScratch phj_layout(Carve& c, int64_t nb, int64_t np, const PlanDev& plan) {
     s.ovf[0] = c.take<uint32_t>((size_t)kMaxOutWarps * kOutChunk);
     s.ovf[1] = c.take<uint32_t>((size_t)kMaxOutWarps * kOutChunk);
     s.fix = chunk_fix_layout(c);
+    s.redo = c.take<unsigned long long>(P + (size_t)np / kDirectProbeChunk + 1);
     return s;
 }
 
@@ -593,8 +739,9 @@ cudaError_t phj_run(const JoinArgs& a, const PlanDev& plan, const PhjScratch& s,
     const uint32_t P = 1u << (plan.bits1 + (passes == 2 ? plan.bits2 : 0));
     {
         ProfScope ps("phj_items", 32.0 * P, stream, 0.0, 2);
-        items_count_kernel<<<(P + 255) / 256, 256, 0, stream>>>(s.side[0].part_start, s.side[1].part_start,
-                                                               P, s.item_prefix);
+        items_count_kernel<<<(P + 255) / 256, 256, 0, stream>>>(
+            s.side[0].part_start, s.side[1].part_start, P, plan.direct ? 0xFFFFFFFFu : kBuildCap,
+            plan.direct ? kDirectProbeChunk : kProbeChunk, s.item_prefix);
         items_scan_kernel<<<1, 1024, 0, stream>>>(s.item_prefix, P, ctrl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -15,6 +15,17 @@ constexpr int kJoinThreads = EIGER_JOIN_THREADS;
 constexpr uint32_t kBuildCap = EIGER_BUILD_CAP;      // build rows per shared-memory table
 constexpr uint32_t kProbeChunk = EIGER_PROBE_CHUNK;  // probe rows per work item, at most
 
+// Direct-addressed tables: the partition's bits and the kbits - pbits bits
+// below them name a mixed key completely, so those low bits are its slot and no
+// key is stored or compared. Used while the slots are few enough
+// (kDirectBits) and the build rows fill at least an eighth of them.
+constexpr int kDirectBits = 14;     // 4-byte slots: 64 KB, three CTAs per SM
+constexpr int kDirectSumBits = 13;  // 12-byte slots: 96 KB beside the sum's row stages
+constexpr uint32_t kDirectProbeChunk = 65536;  // probe rows per work item then: one table serves more
+__device__ __forceinline__ uint32_t direct_slot(uint32_t k, int pbits, int sbits) {
+    return (k << pbits) >> (32 - sbits);
+}
+
 template <typename KeyT>
 struct JoinIn {
     const KeyT* bkey;
@@ -25,7 +36,14 @@ struct JoinIn {
     const uint32_t* pstart;
     const unsigned long long* item_prefix;
     uint32_t P;
+    uint32_t bcap, pcap;  // build and probe rows per work item, at most
+    int pbits, sbits;     // partition bits; direct-addressed tables: bits of the slot below them
+    unsigned long long* redo;  // direct-addressed tables: the items left to hash tables
 };
+
+__host__ __device__ __forceinline__ uint32_t chunks_of(uint32_t rows, uint32_t cap) {
+    return rows / cap + (rows % cap != 0);
+}
 
 // A work item's rows: partition p's build chunk [bs0, bs0 + bn) and probe chunk
 // [ps0, ps0 + pn). The chunks of a partition are balanced (sizes differ by at
@@ -38,8 +56,7 @@ template <typename KeyT>
 __device__ __forceinline__ ItemRows item_rows(const JoinIn<KeyT>& a, unsigned long long item, uint32_t p) {
     const uint32_t b0 = a.bstart[p], bsz = a.bstart[p + 1] - b0;
     const uint32_t p0 = a.pstart[p], psz = a.pstart[p + 1] - p0;
-    const uint32_t npc = (psz + kProbeChunk - 1) / kProbeChunk;
-    const uint32_t nbc = (bsz + kBuildCap - 1) / kBuildCap;
+    const uint32_t npc = chunks_of(psz, a.pcap), nbc = chunks_of(bsz, a.bcap);
     const uint32_t local = (uint32_t)(item - a.item_prefix[p]);  // < items of one partition
     const uint32_t bc = local / npc, pc = local - bc * npc;
     ItemRows r;
@@ -99,7 +116,7 @@ __device__ __forceinline__ uint32_t find_partition(const unsigned long long* __r
 // The fused sum over positions (phj_sum.cu): out.b.src[0] and out.p.src[0] are
 // the carried payload columns, indexed like the keys of `a`.
 template <typename KeyT>
-cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
+cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
                            cudaStream_t stream, int64_t nb, int64_t np);
 
 }  // namespace eiger

@@ -6,15 +6,17 @@
 // b_i + q_j, taken probe row by probe row. Everything is modulo 2^64, so the
 // order of the additions does not matter.
 //
-// The rows arrive through the CTA's stream (stream.cuh), two CTAs per SM. What
-// bounds it is shared memory, not the row streams: about 29 shared-memory
-// wavefronts per 32 probe rows (the key group's 16-byte loads at random
-// groups, the sum's 8-byte loads at random slots) keep its pipe 87 % busy.
-// Measured on GB300, 150M x 600M int32 keys, int64 payloads (16-bit
-// partitions): 6.76 ms when every match gathered both payloads from global
-// memory by position, 4.76 ms with the sums in the table, rows in registers
-// one round ahead and one slot per probe, 3.92 ms as it is; 8M x 30M 64-bit
-// keys of six rows each: 2.79 -> 0.21 ms (the multiplicity no longer counts).
+// The rows arrive through the CTA's stream (stream.cuh). Hash tables, two CTAs
+// per SM, are bound by shared memory: about 29 wavefronts per 32 probe rows (the
+// key group's 16-byte loads at random groups, the sum's 8-byte loads at random
+// slots) keep its pipe 87 % busy. Direct-addressed tables need about 11 and run
+// near the row streams' rate (5.3 TB/s with 2^12 slots). Measured on GB300,
+// 150M x 600M dense int32 keys, int64 payloads: 6.76 ms when every match
+// gathered both payloads from global memory by position, 4.76 ms with the sums
+// in hash tables, rows in registers one round ahead and one slot per probe,
+// 3.92 ms streamed with key groups (3.46 ms on mixed keys), 1.71 ms direct with
+// 2^12 slots, 1.91 ms with 2^13 (whose partitions take 1.9 ms less to make);
+// 8M x 30M 64-bit keys of six rows each: 2.79 -> 0.21 ms.
 #include "emit.cuh"
 #include "kernels.cuh"
 #include "phj.cuh"
@@ -24,8 +26,6 @@ namespace eiger {
 
 namespace {
 
-constexpr int kConsumers = kJoinThreads;
-constexpr int kSumThreads = kConsumers + kStreamWarps * kWarp;
 constexpr int kStages = 2;
 
 // Slots of {key, sum as two 32-bit halves, rows beyond the first}. The all-ones
@@ -52,8 +52,9 @@ struct SumTable {
         key[i] = kEmpty;
         more[i] = 0;
     }
+    template <int THREADS>
     __device__ void clear(uint32_t tsize) {
-        for (uint32_t i = threadIdx.x; i < tsize; i += kConsumers) clear_slot(i);
+        for (uint32_t i = threadIdx.x; i < tsize; i += THREADS) clear_slot(i);
         if (threadIdx.x == 0) clear_slot(kSlots);
     }
     using Group = KeyGroup<KeyT>;
@@ -97,26 +98,58 @@ struct SumTable {
     }
 };
 
-template <typename KeyT, typename PayT>
-struct SumStream : Stream<2, kStages, 4, 4096 / sizeof(KeyT), ItemRows> {
+// Direct-addressed form (phj.cuh): slot -> {sum, rows}. No key is stored, no
+// search is made, and a key's further rows need no other treatment.
+struct SumDirect {
+    uint32_t* lo;
+    uint32_t* hi;
+    uint32_t* rows;
+    int pbits, sbits;
+    static __host__ __device__ size_t bytes(int sbits) { return (((size_t)1 << sbits) * 3 * 4 + 15) / 16 * 16; }
+    __device__ void bind(unsigned char* smem, int pb, int sb) {
+        lo = reinterpret_cast<uint32_t*>(smem);
+        hi = lo + (1u << sb);
+        rows = hi + (1u << sb);
+        pbits = pb;
+        sbits = sb;
+    }
+    template <int THREADS>
+    __device__ void clear() {
+        uint4* p = reinterpret_cast<uint4*>(lo);
+        const uint32_t n = (uint32_t)(bytes(sbits) / 16);
+        for (uint32_t i = threadIdx.x; i < n; i += THREADS) p[i] = make_uint4(0, 0, 0, 0);
+    }
+    __device__ void add(uint32_t k, uint64_t v) {
+        const uint32_t s = direct_slot(k, pbits, sbits), l = (uint32_t)v;
+        const uint32_t old = atomicAdd(lo + s, l);
+        const uint32_t h = (uint32_t)(v >> 32) + (old + l < l ? 1u : 0u);
+        if (h) atomicAdd(hi + s, h);
+        atomicAdd(rows + s, 1u);
+    }
+};
+
+template <typename KeyT, typename PayT, bool DIRECT, int CONS>
+struct SumStream : Stream<2, kStages, 4, DIRECT ? 2 * CONS : 4096 / sizeof(KeyT), ItemRows> {
     static constexpr size_t kBytes = kStages * (SumStream::col_bytes(sizeof(KeyT)) + SumStream::col_bytes(sizeof(PayT)));
 };
 
-template <typename KeyT, typename PayT>
-__global__ void __launch_bounds__(kSumThreads, 2)
+// CONS consumer threads (plus the stream's two warps): 512, two CTAs per SM, or
+// 960 over a table that only one CTA per SM has room for.
+template <typename KeyT, typename PayT, bool DIRECT, int CONS>
+__global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
     phj_sum_kernel(JoinIn<KeyT> a, const PayT* __restrict__ bpay, const PayT* __restrict__ ppay, Ctrl* ctrl) {
-    using S = SumStream<KeyT, PayT>;
+    using S = SumStream<KeyT, PayT, DIRECT, CONS>;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ typename S::Shared s_stream;
     S st;
     st.w[0] = sizeof(KeyT);
     st.w[1] = sizeof(PayT);
-    st.setup(&s_stream, smem + SumTable<KeyT>::kBytes, kConsumers / kWarp);
+    st.setup(&s_stream, smem + (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT>::kBytes), CONS / kWarp);
     constexpr uint32_t kStageRows = S::kRows;
     typename S::ItemPos q;
     const int warp = threadIdx.x / kWarp;
 
-    if (warp == kConsumers / kWarp) {  // scheduler
+    if (warp == CONS / kWarp) {  // scheduler
         const unsigned long long nitems = ctrl->nitems;
         for (;;) {
             unsigned long long item = 0;
@@ -131,7 +164,7 @@ __global__ void __launch_bounds__(kSumThreads, 2)
         return;
     }
     typename S::StagePos sp;
-    if (warp == kConsumers / kWarp + 1) {  // producer
+    if (warp == CONS / kWarp + 1) {  // producer
         if (lane_id() == 0) {
             bool ok = true;
             while (ok) {
@@ -155,88 +188,125 @@ __global__ void __launch_bounds__(kSumThreads, 2)
     }
 
     SumTable<KeyT> tab;
-    tab.bind(smem);
+    SumDirect dir;
+    if constexpr (DIRECT)
+        dir.bind(smem, a.pbits, a.sbits);
+    else
+        tab.bind(smem);
     AggState agg{0ull, 0ull};
     bool dead = false;
+    // Every row of n streamed rows: f(key, payload), two rows of a thread at a
+    // time; the warp is brought together after each pair.
+    auto rows_of = [&](const KeyT* kp, const PayT* vp, uint32_t n, auto&& f) {
+        for (uint32_t base = 0; base < n; base += kStageRows) {
+            if (!dead && !st.wait(&s_stream.full[sp.i], sp.phase)) dead = true;
+            const KeyT* k = st.template rows<KeyT>(sp, 0, reinterpret_cast<const char*>(kp), base);
+            const PayT* v = st.template rows<PayT>(sp, 1, reinterpret_cast<const char*>(vp), base);
+            const uint32_t len = dead ? 0u : min(n - base, kStageRows);
+            f(k, v, len);
+            st.release(sp);
+        }
+    };
     for (;;) {
         if (!st.wait(&s_stream.ifull[q.i], q.phase)) dead = true;
-        ItemRows it = s_stream.item[q.i];
+        const ItemRows it = s_stream.item[q.i];
         __syncwarp();
         if (lane_id() == 0) mbar_arrive(&s_stream.iempty[q.i]);
         q.next();
         // (every consumer has left the previous item's table here)
-        if (consumers_or<kConsumers>(dead) || it.bn == 0) break;
-        uint32_t tsize = (3 * it.bn + 3) & ~3u;  // load 1/3 while that fits
-        if (tsize < 64) tsize = 64;
-        if (tsize > SumTable<KeyT>::kSlots) tsize = SumTable<KeyT>::kSlots;
-        tab.clear(tsize);
-        consumers_sync<kConsumers>();
-        int dup = 0;
-        for (uint32_t base = 0; base < it.bn; base += kStageRows) {
-            if (!dead && !st.wait(&s_stream.full[sp.i], sp.phase)) dead = true;
-            const KeyT* k = st.template rows<KeyT>(sp, 0, reinterpret_cast<const char*>(a.bkey + it.bs0), base);
-            const PayT* v = st.template rows<PayT>(sp, 1, reinterpret_cast<const char*>(bpay + it.bs0), base);
-            const uint32_t len = dead ? 0u : min(it.bn - base, kStageRows);
-            for (uint32_t i = threadIdx.x; i < len; i += kConsumers) {
-                const int r = tab.add(k[i], (uint64_t)(int64_t)v[i], tsize);
-                if (r < 0) atomicOr(&ctrl->err, kErrTableFull);
-                dup |= r;
-            }
-            st.release(sp);
-        }
-        const bool unique = !consumers_or<kConsumers>(dup != 0);
-        for (uint32_t base = 0; base < it.pn; base += kStageRows) {
-            if (!dead && !st.wait(&s_stream.full[sp.i], sp.phase)) dead = true;
-            const KeyT* k = st.template rows<KeyT>(sp, 0, reinterpret_cast<const char*>(a.pkey + it.ps0), base);
-            const PayT* v = st.template rows<PayT>(sp, 1, reinterpret_cast<const char*>(ppay + it.ps0), base);
-            const uint32_t len = dead ? 0u : min(it.pn - base, kStageRows);
+        if (consumers_or<CONS>(dead) || it.bn == 0) break;
+        if constexpr (DIRECT) {
+            dir.template clear<CONS>();
+            consumers_sync<CONS>();
+            rows_of(a.bkey + it.bs0, bpay + it.bs0, it.bn, [&](const KeyT* k, const PayT* v, uint32_t len) {
+                for (uint32_t i = threadIdx.x; i < len; i += CONS) dir.add((uint32_t)k[i], (uint64_t)(int64_t)v[i]);
+            });
+            consumers_sync<CONS>();
+            rows_of(a.pkey + it.ps0, ppay + it.ps0, it.pn, [&](const KeyT* k, const PayT* v, uint32_t len) {
 #pragma unroll 2
-            for (uint32_t i = threadIdx.x; i < len; i += kConsumers) {
-                const uint32_t s = tab.find(k[i], tsize);
-                if (s == ~0u) continue;
-                const uint2 bs = tab.sum[s];
-                const uint64_t b = ((uint64_t)bs.y << 32) | bs.x;
-                const uint64_t q8 = (uint64_t)(int64_t)v[i];
-                const uint32_t rows = unique ? 1u : 1u + tab.more[s];
-                agg.sum += b + (unique ? q8 : rows * q8);
-                agg.count += rows;
-            }
-            st.release(sp);
+                for (uint32_t i = threadIdx.x; i < len; i += CONS) {
+                    const uint32_t s = direct_slot((uint32_t)k[i], a.pbits, a.sbits);
+                    const uint32_t rows = dir.rows[s];
+                    // an empty slot adds sum 0 and rows 0
+                    agg.sum += (((uint64_t)dir.hi[s] << 32) | dir.lo[s]) + rows * (uint64_t)(int64_t)v[i];
+                    agg.count += rows;
+                }
+            });
+        } else {
+            uint32_t tsize = (3 * it.bn + 3) & ~3u;  // load 1/3 while that fits
+            if (tsize < 64) tsize = 64;
+            if (tsize > SumTable<KeyT>::kSlots) tsize = SumTable<KeyT>::kSlots;
+            tab.template clear<CONS>(tsize);
+            consumers_sync<CONS>();
+            int dup = 0;
+            rows_of(a.bkey + it.bs0, bpay + it.bs0, it.bn, [&](const KeyT* k, const PayT* v, uint32_t len) {
+                for (uint32_t i = threadIdx.x; i < len; i += CONS) {
+                    const int r = tab.add(k[i], (uint64_t)(int64_t)v[i], tsize);
+                    if (r < 0) atomicOr(&ctrl->err, kErrTableFull);
+                    dup |= r;
+                }
+            });
+            const bool unique = !consumers_or<CONS>(dup != 0);
+            rows_of(a.pkey + it.ps0, ppay + it.ps0, it.pn, [&](const KeyT* k, const PayT* v, uint32_t len) {
+#pragma unroll 2
+                for (uint32_t i = threadIdx.x; i < len; i += CONS) {
+                    const uint32_t s = tab.find(k[i], tsize);
+                    if (s == ~0u) continue;
+                    const uint2 bs = tab.sum[s];
+                    const uint64_t b = ((uint64_t)bs.y << 32) | bs.x;
+                    const uint64_t q8 = (uint64_t)(int64_t)v[i];
+                    const uint32_t rows = unique ? 1u : 1u + tab.more[s];
+                    agg.sum += b + (unique ? q8 : rows * q8);
+                    agg.count += rows;
+                }
+            });
         }
     }
     if (dead && lane_id() == 0) atomicOr(&ctrl->err, kErrInternal);
     agg_commit(agg, ctrl);
 }
 
-template <typename KeyT, typename PayT>
+template <typename KeyT, typename PayT, bool DIRECT, int CONS>
 cudaError_t launch_sum(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, const DevInfo& di, cudaStream_t stream,
                        int64_t nb, int64_t np) {
-    auto kern = phj_sum_kernel<KeyT, PayT>;
-    const size_t smem = SumTable<KeyT>::kBytes + SumStream<KeyT, PayT>::kBytes;
+    auto kern = phj_sum_kernel<KeyT, PayT, DIRECT, CONS>;
+    const size_t smem = (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT>::kBytes) + SumStream<KeyT, PayT, DIRECT, CONS>::kBytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
+    constexpr int kThreads = CONS + kStreamWarps * kWarp;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSumThreads, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     // keys and payloads of both sides, each read once
     ProfScope ps("phj_sum", (double)(sizeof(KeyT) + sizeof(PayT)) * (double)(nb + np), stream);
-    kern<<<di.sms * per_sm, kSumThreads, smem, stream>>>(a, static_cast<const PayT*>(out.b.src[0]),
-                                                        static_cast<const PayT*>(out.p.src[0]), ctrl);
+    kern<<<di.sms * per_sm, kThreads, smem, stream>>>(a, static_cast<const PayT*>(out.b.src[0]),
+                                                     static_cast<const PayT*>(out.p.src[0]), ctrl);
     return cudaGetLastError();
+}
+
+template <typename KeyT, typename PayT>
+cudaError_t launch_sum_for(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
+                           cudaStream_t stream, int64_t nb, int64_t np) {
+    if constexpr (sizeof(KeyT) == 4) {
+        if (direct)
+            return a.sbits <= 12 ? launch_sum<KeyT, PayT, true, 512>(a, out, ctrl, di, stream, nb, np)
+                                 : launch_sum<KeyT, PayT, true, 960>(a, out, ctrl, di, stream, nb, np);
+    }
+    return launch_sum<KeyT, PayT, false, 512>(a, out, ctrl, di, stream, nb, np);
 }
 
 }  // namespace
 
 template <typename KeyT>
-cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
+cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
                            cudaStream_t stream, int64_t nb, int64_t np) {
-    return out.b.bytes[0] == 4 ? launch_sum<KeyT, int32_t>(a, out, ctrl, di, stream, nb, np)
-                               : launch_sum<KeyT, int64_t>(a, out, ctrl, di, stream, nb, np);
+    return out.b.bytes[0] == 4 ? launch_sum_for<KeyT, int32_t>(a, direct, out, ctrl, di, stream, nb, np)
+                               : launch_sum_for<KeyT, int64_t>(a, direct, out, ctrl, di, stream, nb, np);
 }
 
-template cudaError_t phj_sum_launch<uint32_t>(const JoinIn<uint32_t>&, const JoinOut&, Ctrl*, const DevInfo&,
+template cudaError_t phj_sum_launch<uint32_t>(const JoinIn<uint32_t>&, int, const JoinOut&, Ctrl*, const DevInfo&,
                                               cudaStream_t, int64_t, int64_t);
-template cudaError_t phj_sum_launch<uint64_t>(const JoinIn<uint64_t>&, const JoinOut&, Ctrl*, const DevInfo&,
+template cudaError_t phj_sum_launch<uint64_t>(const JoinIn<uint64_t>&, int, const JoinOut&, Ctrl*, const DevInfo&,
                                               cudaStream_t, int64_t, int64_t);
 
 }  // namespace eiger
