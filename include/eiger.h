@@ -174,8 +174,10 @@ eiger_status eiger_join_workspace(int64_t nb, int64_t np, eiger_dtype dtype, eig
  *          d_out_*pay output is requested (gather by tuple ID, Sec. 3.2 GFUR).
  * variant: EIGER_AUTO runs eiger_stats on the build keys, then eiger_plan,
  *          then the chosen variant; where the build keys are dense and distinct
- *          (32-bit keys over a span of at most 8 nb) a partitioned plan gets
- *          fewer radix bits (tables of up to 2^14 direct-addressed slots).
+ *          (32-bit keys over a span of at most 8 nb), a partitioned plan gives
+ *          way to NPHJ while 4 bytes per key of the span and the build columns
+ *          fit 7/8 of L2, and else gets fewer radix bits (direct-addressed
+ *          tables of up to 2^14 slots).
  *          NPHJ/PHJ1/PHJ2 also profile the build keys (narrowing and the probe
  *          range test need min/max) and take their knobs from `knobs` when
  *          non-NULL (bits1/bits2/narrow/load_factor), else from the planner.

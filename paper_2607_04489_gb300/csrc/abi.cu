@@ -473,6 +473,25 @@ bool dense_keys(int dtype, bool narrow, int64_t nb, const eiger_stats_t* bst) {
            (double)nb * 8.0 >= (double)(1ull << mix_bits(key32, bst->min, bst->max));
 }
 
+// Whether AUTO takes the non-partitioned join in place of a partitioned plan:
+// dense keys, whose direct-addressed table (nphj.cu), with the build columns
+// that are gathered beside it, stays in L2. Measured on GB300 (ms, NPHJ /
+// partitioned): pairs of 2^24 x 2^26 rows (64 MB) 0.89 / 1.44, 2^24.5 x 2^26.5
+// (95 MB) 1.37 / 1.87, 2^25 x 2^27 (134 MB) 2.34 / 2.49; two 4-byte columns a
+// side, 5M x 100M (60 MB) 1.81 / 2.78, 10M x 120M (120 MB) 3.40 / 3.37, 16M x
+// 100M (192 MB) 4.11 / 3.01; 8-byte sums, 8M x 60M (96 MB) 0.89 / 1.29, 16M x
+// 60M (192 MB) 1.53 / 1.43. A caller who asks for carried columns keeps the
+// partitioned plan.
+bool dense_nphj(const JoinCall& c, const eiger_stats_t* bst, const eiger_plan_t& p) {
+    if (p.variant != EIGER_PHJ1 && p.variant != EIGER_PHJ2) return false;
+    if (c.materialize == EIGER_GFTR || !dense_keys(c.dtype, p.narrow, c.nb, bst)) return false;
+    const uint64_t words = (uint64_t)bst->max - (uint64_t)bst->min + 1;
+    if (words > 2ull * nphj_slots(c.nb, 0.5f)) return false;  // see run_join: the hash table would be the smaller one
+    double bytes = 4.0 * (double)words;
+    for (int q = 0; q < c.out.b.n; ++q) bytes += (double)c.out.b.bytes[q] * (double)c.nb;
+    return bytes <= 0.875 * (double)l2_bytes_or_default();
+}
+
 // AUTO's radix bits where direct-addressed tables serve (see direct_tables):
 // a table of 2^kDirectBits slots (2^kDirectSumBits of the sum's larger ones)
 // holds several times the rows of a hash table,
@@ -572,8 +591,12 @@ eiger_status run_join(const JoinCall& c) {
         s = resolve_plan(c, adaptive ? &bst : nullptr, &pub);
         if (s != EIGER_OK) return s;
         // a partitioned plan for a probe side at least twice the build side
-        // looks at a probe sample first: heavy skew favours the NPHJ
-        if (c.variant == EIGER_AUTO && !c.knobs &&
+        // looks at a probe sample first: heavy skew favours the NPHJ (as a
+        // dense build side that stays in L2 does anyway)
+        if (c.variant == EIGER_AUTO && !c.knobs && dense_nphj(c, &bst, pub)) {
+            pub.variant = EIGER_NPHJ;
+            pub.bits1 = pub.bits2 = 0;
+        } else if (c.variant == EIGER_AUTO && !c.knobs &&
             wants_probe_sample(pub, c.nb, c.np, c.dtype, narrowable(c.dtype, c.nb, bst.min, bst.max))) {
             static thread_local eiger_stats_t pst;
             const int64_t ns = c.np < kProbeSampleRows ? c.np : kProbeSampleRows;
@@ -608,6 +631,9 @@ eiger_status run_join(const JoinCall& c) {
     if (fault && std::strcmp(fault, "table_full") == 0 &&
         (pd.variant == EIGER_NPHJ || pd.variant == EIGER_STATIC))
         ns.slots = 64;
+    // direct-addressed where the span takes no more memory than the hash table
+    ns.direct = pd.variant == EIGER_NPHJ && pd.key32 &&
+                (uint64_t)bst.max - (uint64_t)bst.min < 2ull * ns.slots;
 
     EIGER_CUDA(cudaMemsetAsync(lay.ctrl, 0, sizeof(Ctrl), c.stream), "control block reset");
     const JoinArgs a{c.bkeys, c.nb, c.pkeys, c.np};

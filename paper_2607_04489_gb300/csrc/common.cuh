@@ -223,6 +223,12 @@ __device__ __forceinline__ ulonglong2 ld_keep2(const ulonglong2* a, uint64_t pol
     return v;
 }
 
+__device__ __forceinline__ uint32_t ld_keep(const uint32_t* a, uint64_t pol) {
+    uint32_t v;
+    asm volatile("ld.global.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(pol));
+    return v;
+}
+
 // ---------------------------------------------------------------- TMA bulk copies
 
 // Shared-memory address of a generic pointer into shared memory.

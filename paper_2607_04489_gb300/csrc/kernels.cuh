@@ -93,6 +93,8 @@ struct NphjScratch {
     void* table;
     unsigned long long slots;  // power of two
     int slot_bytes;            // 8 (packed 32-bit key + idx) or 16 (64-bit key, idx)
+    uint32_t* next = nullptr;  // [nb] direct-addressed form: further rows of a key
+    int direct = 0;            // table is head[span + 1] (32-bit keys; at most 2 * slots words)
 };
 
 unsigned long long nphj_slots(int64_t nb, float load_factor);

@@ -115,7 +115,7 @@ extern "C" eiger_status eiger_join_static_noalloc(eiger_dtype dtype, const void*
     eiger_status s = scratch_address(&base);
     if (s != EIGER_OK) return s;
     Ctrl* ctrl = static_cast<Ctrl*>(base);
-    NphjScratch ns;
+    NphjScratch ns{};
     ns.table = static_cast<unsigned char*>(base) + kCtrlBytes;
     ns.slots = slots;
     ns.slot_bytes = slot_bytes;

@@ -235,95 +235,7 @@ __device__ __forceinline__ void load_round(RoundRegs<KeyT, N>& r, const KeyT* __
     }
 }
 
-constexpr uint32_t kHole = 0xFFFFFFFFu;  // stage position without a match
-
 constexpr int kJoinWarps = kJoinThreads / kWarp;
-
-// Block-collective: writes a round's matches (b[j] != kHole) with their columns.
-// Ballots rank every match within its (row j, warp) group, one scan over the
-// group counts places the groups, one global atomic reserves the round's
-// output. Each column is then read for all rows of a thread before any of them
-// is written (one memory round trip per column and round; row by row the
-// gathers of 8 rows x 4 columns had waited for one another). s_grp alternates
-// between two halves by round, so no barrier follows the writes.
-template <int kN>
-__device__ __forceinline__ void flush_columns(const uint32_t (&b)[kN], const uint32_t (&p)[kN], uint32_t* s_grp,
-                                              unsigned long long* s_base, const JoinOut& out, Ctrl* ctrl) {
-    const unsigned lane = lane_id();
-    const int w = threadIdx.x / kWarp;
-    constexpr int kGroups = kN * kJoinWarps;
-    unsigned rank[kN];
-#pragma unroll
-    for (int j = 0; j < kN; ++j) {
-        const unsigned m = __ballot_sync(0xffffffffu, b[j] != kHole);
-        rank[j] = __popc(m & lanemask_lt());
-        if (lane == 0) s_grp[j * kJoinWarps + w] = __popc(m);
-    }
-    __syncthreads();
-    if (w == 0) {
-        constexpr int kPer = (kGroups + kWarp - 1) / kWarp;
-        uint32_t v[kPer], local = 0;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int e = lane * kPer + i;
-            v[i] = e < kGroups ? s_grp[e] : 0u;
-            local += v[i];
-        }
-        uint32_t x = local;
-#pragma unroll
-        for (int o = 1; o < kWarp; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if ((int)lane >= o) x += y;
-        }
-        uint32_t run = x - local;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const int e = lane * kPer + i;
-            if (e < kGroups) s_grp[e] = run;
-            run += v[i];
-        }
-        if (lane == kWarp - 1) *s_base = x ? atomicAdd(&ctrl->cursor, (unsigned long long)x) : 0ull;
-    }
-    __syncthreads();
-    const unsigned long long base = *s_base;
-    const unsigned long long room = out.capacity > base ? out.capacity - base : 0ull;
-    uint32_t pos[kN];  // offset from base, or kHole
-#pragma unroll
-    for (int j = 0; j < kN; ++j) {
-        pos[j] = s_grp[j * kJoinWarps + w] + rank[j];
-        if (b[j] == kHole || pos[j] >= room) pos[j] = kHole;
-    }
-    auto index = [&](uint32_t* dst, const uint32_t* map, const uint32_t(&row)[kN]) {
-        uint32_t v[kN];
-#pragma unroll
-        for (int j = 0; j < kN; ++j)
-            if (pos[j] != kHole) v[j] = map ? __ldg(map + row[j]) : row[j];
-#pragma unroll
-        for (int j = 0; j < kN; ++j)
-            if (pos[j] != kHole) __stcs(dst + base + pos[j], v[j]);
-    };
-    auto column = [&](const ColSide& cs, int c, const uint32_t(&row)[kN]) {
-        if (cs.bytes[c] == 4) {
-            index(static_cast<uint32_t*>(cs.dst[c]), static_cast<const uint32_t*>(cs.src[c]), row);
-        } else {
-            const uint2* src = static_cast<const uint2*>(cs.src[c]);
-            uint2* dst = static_cast<uint2*>(cs.dst[c]);
-            uint2 v[kN];
-#pragma unroll
-            for (int j = 0; j < kN; ++j)
-                if (pos[j] != kHole) v[j] = __ldg(src + row[j]);
-#pragma unroll
-            for (int j = 0; j < kN; ++j)
-                if (pos[j] != kHole) __stcs(dst + base + pos[j], v[j]);
-        }
-    };
-    if (out.bidx) index(out.bidx, out.b.rowmap, b);
-    if (out.pidx) index(out.pidx, out.p.rowmap, p);
-#pragma unroll 1
-    for (int c = 0; c < out.b.n; ++c) column(out.b, c, b);
-#pragma unroll 1
-    for (int c = 0; c < out.p.n; ++c) column(out.p, c, p);
-}
 
 // kHash: one hash table per item. kDirect: direct-addressed tables (32-bit
 // keys), slot -> build row; an item whose build keys repeat (a slot taken twice)
@@ -442,7 +354,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
                     }
             } else {
                 const uint32_t h = flushes++ & 1;
-                flush_columns<kN>(brow, cur.id, s_grp[h], &s_base[h], out, ctrl);
+                flush_matches<kN, kJoinThreads>(brow, cur.id, s_grp[h], &s_base[h], out, &ctrl->cursor);
             }
         };
 
