@@ -85,16 +85,22 @@ __global__ void __launch_bounds__(256) store_to_host_kernel(uint32_t* __restrict
 
 }  // namespace
 
+// The calling thread's staging buffer as the device sees it, or nullptr.
+void* host_stage_device(size_t bytes) {
+    void* st = host_stage(bytes);
+    void* dev = nullptr;
+    if (st && cudaHostGetDevicePointer(&dev, st, 0) != cudaSuccess) {
+        cudaGetLastError();
+        dev = nullptr;
+    }
+    return dev;
+}
+
 // Small result from device memory to `dst` on `stream`, then a synchronisation
 // of the stream: stored by a kernel into the mapped staging buffer when it
 // exists (bytes a multiple of 4), else copied by cudaMemcpyAsync.
 cudaError_t readback_sync(void* dst, const void* src, size_t bytes, cudaStream_t stream) {
-    void* st = bytes % 4 == 0 ? host_stage(bytes) : nullptr;
-    void* st_dev = nullptr;
-    if (st && cudaHostGetDevicePointer(&st_dev, st, 0) != cudaSuccess) {
-        cudaGetLastError();
-        st_dev = nullptr;
-    }
+    void* st_dev = bytes % 4 == 0 ? host_stage_device(bytes) : nullptr;
     cudaError_t e;
     if (st_dev) {
         store_to_host_kernel<<<1, 256, 0, stream>>>(static_cast<uint32_t*>(st_dev), static_cast<const uint32_t*>(src),
@@ -104,7 +110,7 @@ cudaError_t readback_sync(void* dst, const void* src, size_t bytes, cudaStream_t
         e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    if (e == cudaSuccess && st_dev) std::memcpy(dst, st, bytes);
+    if (e == cudaSuccess && st_dev) std::memcpy(dst, host_stage(bytes), bytes);
     return e;
 }
 
@@ -178,8 +184,10 @@ size_t l2_bytes_or_default() {
 
 bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 
+// Statistics of a column. The registers are read back only when want_regs (the
+// joins need the estimate alone, which the counts of the ranks give).
 eiger_status run_stats(const void* keys, int64_t n, int dtype, const StatsScratch& ss,
-                       cudaStream_t stream, eiger_stats_t* out) {
+                       cudaStream_t stream, eiger_stats_t* out, bool want_regs) {
     out->n = n;
     if (n == 0) {
         out->min = INT64_MAX;
@@ -188,15 +196,24 @@ eiger_status run_stats(const void* keys, int64_t n, int dtype, const StatsScratc
         out->estimate = 0.0;
         return EIGER_OK;
     }
-    EIGER_CUDA(stats_launch(keys, n, dtype, ss, stream), "statistics kernels");
-    static thread_local StatsDev host;
-    EIGER_CUDA(readback_sync(&host, ss.out, sizeof(StatsDev), stream), "statistics readback");
-    out->min = host.mn;
-    out->max = host.mx;
-    std::memcpy(out->hll, host.regs, sizeof out->hll);
-    for (int j = 0; j < kHllM; ++j)
-        if (out->hll[j] > kRhoMax) return fail(EIGER_ERR_INTERNAL, "register %d holds %d", j, out->hll[j]);
-    out->estimate = hll_estimate(out->hll);
+    static_assert(sizeof(StatsDev) <= kStageBytes, "the statistics fit the staging buffer");
+    static thread_local StatsDev copy;
+    StatsDev* mapped = static_cast<StatsDev*>(host_stage_device(sizeof(StatsDev)));
+    EIGER_CUDA(stats_launch(keys, n, dtype, ss, mapped, want_regs, stream), "statistics kernels");
+    const StatsDev* host = &copy;
+    if (mapped) {
+        EIGER_CUDA(cudaStreamSynchronize(stream), "statistics synchronise");
+        host = static_cast<const StatsDev*>(host_stage(sizeof(StatsDev)));
+    } else {
+        EIGER_CUDA(readback_sync(&copy, ss.out, sizeof(StatsDev), stream), "statistics readback");
+    }
+    out->min = host->mn;
+    out->max = host->mx;
+    uint32_t regs = 0;
+    for (int r = 0; r <= kRhoMax; ++r) regs += host->hist[r];
+    if (regs != kHllM) return fail(EIGER_ERR_INTERNAL, "%u of %d registers hold a rank", regs, kHllM);
+    if (want_regs) std::memcpy(out->hll, host->regs, sizeof out->hll);
+    out->estimate = hll_estimate_counts(host->hist);
     return EIGER_OK;
 }
 
@@ -535,7 +552,7 @@ eiger_status learned_plan(const JoinCall& c, const eiger_stats_t& bst, const Lay
     *chosen = false;
     static thread_local eiger_stats_t pst;
     const int64_t nps = c.np < kProbeSample ? c.np : kProbeSample;
-    eiger_status s = run_stats(c.pkeys, nps, c.dtype, lay.stats, c.stream, &pst);
+    eiger_status s = run_stats(c.pkeys, nps, c.dtype, lay.stats, c.stream, &pst, false);
     if (s != EIGER_OK) return s;
     float f[EIGER_MLP_IN];
     compute_features(&bst, &pst, c.nb, c.np, c.dtype, l2_bytes_or_default(), f);
@@ -575,7 +592,7 @@ eiger_status run_join(const JoinCall& c) {
     static thread_local eiger_stats_t bst;
     const bool adaptive = c.variant != EIGER_STATIC;
     if (adaptive) {
-        s = run_stats(c.bkeys, c.nb, c.dtype, lay.stats, c.stream, &bst);
+        s = run_stats(c.bkeys, c.nb, c.dtype, lay.stats, c.stream, &bst, false);
         if (s != EIGER_OK) return s;
     }
     eiger_plan_t pub;
@@ -600,7 +617,7 @@ eiger_status run_join(const JoinCall& c) {
             wants_probe_sample(pub, c.nb, c.np, c.dtype, narrowable(c.dtype, c.nb, bst.min, bst.max))) {
             static thread_local eiger_stats_t pst;
             const int64_t ns = c.np < kProbeSampleRows ? c.np : kProbeSampleRows;
-            s = run_stats(c.pkeys, ns, c.dtype, lay.stats, c.stream, &pst);
+            s = run_stats(c.pkeys, ns, c.dtype, lay.stats, c.stream, &pst, false);
             if (s != EIGER_OK) return s;
             s = resolve_plan(c, &bst, &pub, pst.estimate / (double)ns);
             if (s != EIGER_OK) return s;
@@ -777,7 +794,7 @@ eiger_status eiger_stats(const void* d_keys, int64_t n, eiger_dtype dtype, eiger
     StatsScratch ss = stats_layout(c);
     if (n > 0 && (c.off > ws_bytes || !d_workspace))
         return fail(EIGER_ERR_WORKSPACE, "workspace %zu bytes < %zu needed", ws_bytes, c.off);
-    return run_stats(d_keys, n, dtype, ss, static_cast<cudaStream_t>(stream), out);
+    return run_stats(d_keys, n, dtype, ss, static_cast<cudaStream_t>(stream), out, true);
 }
 
 eiger_status eiger_plan(const eiger_stats_t* build, const eiger_stats_t* probe, int64_t nb, int64_t np,
@@ -1051,7 +1068,7 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
     if (lay.fixed_end > ws_bytes)
         return fail(EIGER_ERR_WORKSPACE, "workspace %zu bytes < %zu needed", ws_bytes, lay.fixed_end);
     static thread_local eiger_stats_t kst;
-    s = run_stats(d_keys, n, dtype, lay.stats, st, &kst);
+    s = run_stats(d_keys, n, dtype, lay.stats, st, &kst, false);
     if (s != EIGER_OK) return s;
 
     eiger_groupby_plan_t pub{};

@@ -43,9 +43,13 @@ cudaError_t join_side(cudaStream_t main, cudaStream_t side);
 
 constexpr int kStatsMaxGrid = 512;
 
+constexpr int kRankBins = 64;
+
 struct StatsDev {
     int64_t mn;
     int64_t mx;
+    uint32_t hist[kRankBins];  // registers per rank
+    uint32_t ticket, pad;
     uint32_t regs[kHllM / 4];  // register bytes, 4 per word, little-endian order
 };
 
@@ -56,7 +60,9 @@ struct StatsScratch {
 };
 
 StatsScratch stats_layout(Carve& c);
-cudaError_t stats_launch(const void* keys, int64_t n, int dtype, const StatsScratch& s,
+// Results into *s.out, and into *host (mapped host memory, or nullptr): min, max
+// and the rank counts, the registers too when want_regs.
+cudaError_t stats_launch(const void* keys, int64_t n, int dtype, const StatsScratch& s, StatsDev* host, bool want_regs,
                          cudaStream_t stream);
 
 // ------------------------------------------------------------------ plans

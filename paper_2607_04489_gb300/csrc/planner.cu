@@ -123,15 +123,13 @@ eiger_plan_t plan_rules(int variant, int64_t nb, int64_t np, int dtype, bool nar
 }
 
 // HyperLogLog estimate (Flajolet et al. 2007, with HyperLogLog++'s 64-bit hash:
-// no large-range correction) from the dense registers: the raw estimate
+// no large-range correction) from the counts of the registers' ranks: the raw estimate
 // alpha_m m^2 / sum_j 2^-reg[j], replaced by linear counting m ln(m / V) when V
 // registers are still zero and the raw estimate is at most 2.5 m. The harmonic
 // sum is accumulated exactly as an integer count of 2^-kRhoMax units, so the
 // only rounding is the final fp64 expression, evaluated in a fixed order.
-double hll_estimate(const uint8_t* regs) {
+double hll_estimate_counts(const uint32_t* hist) {
     constexpr int kRho = 64 - EIGER_HLL_P + 1;  // largest rank
-    uint32_t hist[kRho + 1] = {0};
-    for (int j = 0; j < EIGER_HLL_M; ++j) hist[regs[j] <= kRho ? regs[j] : kRho] += 1;
     unsigned __int128 units = 0;
     for (int r = 0; r <= kRho; ++r) units += (unsigned __int128)hist[r] << (kRho - r);
     const double m = (double)EIGER_HLL_M;
