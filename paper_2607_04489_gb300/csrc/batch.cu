@@ -7,14 +7,18 @@
 // table each), build items and probe items (`chunk` rows each). The items of
 // all joins form one sequence, pulled by a persistent grid with an atomic
 // counter, in stages: stage s holds the clear items of join s, then the build
-// items of join s-1, then the probe items of join s-2. A build item waits
-// (bounded) until all clear items of its join are done, a probe item until
-// all build rows of its join are in. So a table is cleared just before it is
-// filled (its lines are still in L2), and a join's probes start one stage
-// after its builds, with the next join's builds in between to absorb the
-// wait. No wait can deadlock: every item waits only on items earlier in the
-// sequence, items are claimed in order, waiting items never hold anything an
-// earlier item needs, and the grid is no larger than what is resident at once.
+// items of join s - L, then the probe items of join s - 2L. A build item waits
+// (bounded) until all clear items of its join are done, a probe item until all
+// build rows of its join are in. The lag L puts kLagGrids grids of items
+// between them, so that a claimed item finds its predecessors done instead of
+// running beside it, and is small enough that the tables of the joins in
+// between stay in L2 (kLagBytes). Measured, L = 1 against the lag: 4096 int32
+// joins of 2^U(6, 16) rows 3403 -> 2275 us, 1024 of 2^U(10, 17) 2184 -> 1508,
+// 256 of 2^U(10, 20) 2994 -> 2625; int64 joins, which are bound by their
+// 16-byte slots, 1749 -> 1728 and, 512 of 2^U(10, 17), 2989 -> 2680. No wait
+// can deadlock: every item waits only on items earlier in the sequence, items
+// are claimed in order, waiting items never hold anything an earlier item
+// needs, and the grid is no larger than what is resident at once.
 // Matches go through the CTA stage to join j's own outputs, reserved on its
 // own cursor (d_counts[j]).
 //
@@ -58,10 +62,13 @@ struct BatchCtrl {
     unsigned long long next_solo;   // small joins' items (probe chunks)
     unsigned long long total_solo;
     unsigned int err;
-    unsigned int pad;
+    int lag;                        // stages between a join's clear, build and probe items
 };
 
 constexpr int kSetupThreads = 1024;
+constexpr int kMaxLag = 128;
+constexpr float kLagGrids = 3.0f;                // grids of items between dependent ones
+constexpr float kLagBytes = 64.0f * (1 << 20);  // tables between a join's clear and its builds
 constexpr uint32_t kWaitLimit = 1u << 22;  // polls (with back-off) before giving up
 
 struct alignas(16) WideSlot {
@@ -70,8 +77,8 @@ struct alignas(16) WideSlot {
 };
 
 // One block. Pass 1: per-join slots, item counts and table offsets (prefix
-// sum of slots). Pass 2: item counts of the stages (clear items of join s,
-// build items of join s-1, probe items of join s-2) and their prefix sums.
+// sum of slots). Pass 2: the lag, item counts of the stages (clear items of join
+// s, build items of join s - L, probe items of join s - 2L) and their prefix sums.
 __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long long v, unsigned long long* s_w,
                                                                 unsigned long long* total) {
     const unsigned lane = lane_id();
@@ -102,23 +109,25 @@ __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long lo
 
 __global__ void __launch_bounds__(kSetupThreads)
     batch_setup_kernel(const eiger_join_desc* __restrict__ descs, int k, int chunk, float load,
-                       long long small_rows, uint32_t solo_max, unsigned long long max_slots,
+                       long long small_rows, uint32_t solo_max, unsigned long long max_slots, int grid,
+                       int slot_bytes,
                        BatchMeta* __restrict__ meta,
                        unsigned long long* __restrict__ stage_prefix, unsigned* __restrict__ built,
                        unsigned* __restrict__ cleared, unsigned* __restrict__ dup, long long* __restrict__ counts,
                        unsigned long long* __restrict__ solo_prefix, BatchCtrl* __restrict__ bc, int* status) {
     __shared__ unsigned long long s_w[kSetupThreads / kWarp];
-    unsigned long long slot_carry = 0, item_carry = 0, solo_carry = 0, total;
+    unsigned long long slot_carry = 0, item_carry = 0, solo_carry = 0, my_work = 0, total;
     for (int base = 0; base < k; base += kSetupThreads) {
         const int j = base + threadIdx.x;
-        unsigned long long slots = 0, solo_items = 0;
+        unsigned long long slots = 0, solo_items = 0, work = 0;
         if (j < k) {
             const long long nb = descs[j].nb, np = descs[j].np;
             BatchMeta m{};
             if (nb > 0 && np > 0) {
-                const double want = (double)nb / (double)load;
+                // the smallest power of two with sl >= nb / load, at least 64,
+                // without FP64 (1/64 rate): sl * load is exact in a float
                 unsigned long long sl = 64;
-                while ((double)sl < want) sl <<= 1;
+                while ((long long)((float)sl * load) < nb && sl < (1ull << 62)) sl <<= 1;
                 if (nb <= small_rows) {
                     // whole per probe chunk, table in shared memory (load at
                     // most 1/2 at the cap: small_rows <= solo_max / 2)
@@ -130,6 +139,7 @@ __global__ void __launch_bounds__(kSetupThreads)
                     m.nci = (uint32_t)((sl + kClearSlots - 1) / kClearSlots);
                     m.nbi = (uint32_t)((nb + chunk - 1) / chunk);
                     m.npi = (uint32_t)((np + chunk - 1) / chunk);
+                    work = (unsigned long long)m.nci + m.nbi + m.npi;
                 }
             }
             meta[j] = m;
@@ -144,17 +154,28 @@ __global__ void __launch_bounds__(kSetupThreads)
         const unsigned long long soff = solo_carry + block_excl_scan64(solo_items, s_w, &total);
         if (j < k) solo_prefix[j] = soff;
         solo_carry += total;
+        my_work += work;
     }
+    block_excl_scan64(my_work, s_w, &total);
+    const unsigned long long work_carry = total;
     __syncthreads();
     __threadfence_block();
-    const int nstages = k + 2;
+    // grids of items between dependent ones, the tables in between bounded
+    int lag = 1;
+    if (work_carry) {
+        const float want = kLagGrids * (float)grid * (float)k / (float)work_carry;
+        const float most = kLagBytes * (float)k / ((float)slot_carry * (float)slot_bytes + 1.0f);
+        const float l = fminf(want, most);
+        lag = l < 1.0f ? 1 : l > (float)kMaxLag ? kMaxLag : (int)(l + 0.5f);
+    }
+    const int nstages = k + 2 * lag;
     for (int base = 0; base < nstages; base += kSetupThreads) {
         const int st = base + threadIdx.x;
         unsigned long long items = 0;
         if (st < nstages) {
             if (st < k) items += meta[st].nci;
-            if (st >= 1 && st - 1 < k) items += meta[st - 1].nbi;
-            if (st >= 2) items += meta[st - 2].npi;
+            if (st >= lag && st - lag < k) items += meta[st - lag].nbi;
+            if (st >= 2 * lag) items += meta[st - 2 * lag].npi;
         }
         const unsigned long long off = item_carry + block_excl_scan64(items, s_w, &total);
         if (st < nstages) stage_prefix[st] = off;
@@ -166,6 +187,7 @@ __global__ void __launch_bounds__(kSetupThreads)
         bc->next_item = 0;
         bc->next_solo = 0;
         bc->err = 0;
+        bc->lag = lag;
         bc->total_slots = slot_carry;
         if (slot_carry > max_slots) {  // tables do not fit: run nothing, report
             bc->total_items = 0;
@@ -357,8 +379,13 @@ __device__ __forceinline__ void probe_rows(const unsigned char* tab, uint32_t ma
     stage_flush<false, kStage>(st, out, cursor);
 }
 
+// Bound by latency (each row is a dependent chain of key, slot and stage, each
+// item a chain of rounds), so by the rows in flight: 64 warps per SM, at 32
+// registers, take 2283 us for 4096 joins of 2^U(6, 16) rows where 48 warps at
+// 40 registers take 3301. Four rows per thread in flight with items claimed
+// ahead needs 40 registers and spills: 4553 us.
 template <typename InKey, int THREADS>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, 2048 / THREADS)
     batch_join_kernel(const eiger_join_desc* __restrict__ descs, int k, const BatchMeta* __restrict__ meta,
                       const unsigned long long* __restrict__ stage_prefix, unsigned char* __restrict__ tables,
                       unsigned* __restrict__ built, unsigned* __restrict__ cleared, unsigned* __restrict__ dup,
@@ -375,13 +402,14 @@ __global__ void __launch_bounds__(THREADS)
     AggState agg{0ull, 0ull};
     if (threadIdx.x == 0) st.count = 0;
     const unsigned long long total = bc->total_items;
+    const int lag = bc->lag;
 
     for (;;) {
         if (threadIdx.x < kWarp) {
             unsigned long long it = 0;
             if (lane == 0) it = atomicAdd(&bc->next_item, 1ull);
             it = __shfl_sync(0xffffffffu, it, 0);
-            const int sg = it < total ? find_join(stage_prefix, k + 2, it) : 0;
+            const int sg = it < total ? find_join(stage_prefix, k + 2 * lag, it) : 0;
             if (lane == 0) {
                 s_item = it;
                 s_stage = sg;
@@ -392,18 +420,18 @@ __global__ void __launch_bounds__(THREADS)
         const int sg = s_stage;
         if (item >= total) break;
         // decode: the clear items of join sg, then the build items of join
-        // sg - 1, then the probe items of join sg - 2
+        // sg - lag, then the probe items of join sg - 2 lag
         unsigned long long local = item - stage_prefix[sg];
         int kind = 0, j = sg;
         if (sg < k && local < meta[sg].nci) {
             kind = 0;
         } else {
             if (sg < k) local -= meta[sg].nci;
-            j = sg - 1;
+            j = sg - lag;
             kind = 1;
             if (!(j >= 0 && j < k && local < meta[j].nbi)) {
                 if (j >= 0 && j < k) local -= meta[j].nbi;
-                j = sg - 2;
+                j = sg - 2 * lag;
                 kind = 2;
             }
         }
@@ -493,7 +521,10 @@ __global__ void __launch_bounds__(THREADS)
 // of join j's build rows, and probes chunk c against it. No item waits on
 // another, so the grid may be any size.
 template <typename InKey, int THREADS>
-__global__ void __launch_bounds__(THREADS)
+// 64 warps per SM for 32-bit keys (16,384 joins of 2^U(6, 11) rows: 387 us, at
+// 48 warps 446, at 32 580); 64-bit keys do better with twice the registers
+// (4096 joins of 2^U(7, 11): 158 us against 174).
+__global__ void __launch_bounds__(THREADS, (sizeof(InKey) == 8 ? 1024 : 2048) / THREADS)
     batch_small_kernel(const eiger_join_desc* __restrict__ descs, int k, const BatchMeta* __restrict__ meta,
                        const unsigned long long* __restrict__ solo_prefix, long long* __restrict__ counts,
                        BatchCtrl* bc, int chunk) {
@@ -606,7 +637,7 @@ BatchLayout batch_layout(Carve& c, int k, unsigned long long total_slots, int sl
     BatchLayout L;
     L.ctrl = c.take<unsigned char>(sizeof(BatchCtrl));
     L.meta = c.take<unsigned char>(sizeof(BatchMeta) * (size_t)(k > 0 ? k : 1));
-    L.item_prefix = c.take<unsigned long long>((size_t)k + 3);  // stage prefix sums
+    L.item_prefix = c.take<unsigned long long>((size_t)k + 2 * kMaxLag + 1);  // stage prefix sums
     L.solo_prefix = c.take<unsigned long long>((size_t)k + 1);  // small joins' item prefix sums
     L.built = c.take<unsigned>((size_t)(k > 0 ? k : 1));
     L.cleared = c.take<unsigned>((size_t)(k > 0 ? k : 1));
@@ -628,7 +659,8 @@ cudaError_t batch_run(const eiger_join_desc* d_descs, int k, int dtype, const ei
         batch_setup_kernel<<<1, kSetupThreads, 0, stream>>>(d_descs, k, knobs.chunk_rows, knobs.load_factor,
                                                             (long long)knobs.small_rows,
                                                             (uint32_t)(kSoloBytes / (dtype == EIGER_I32 ? 8 : 16)),
-                                                            L.table_slots, meta, L.item_prefix, L.built,
+                                                            L.table_slots, di.sms * (2048 / knobs.block_threads),
+                                                            dtype == EIGER_I32 ? 8 : 16, meta, L.item_prefix, L.built,
                                                             L.cleared, L.dup, d_counts, L.solo_prefix, bc,
                                                             d_status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

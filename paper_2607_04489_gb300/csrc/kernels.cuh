@@ -285,7 +285,7 @@ eiger_plan_t class_plan(int cls);
 struct BatchLayout {
     unsigned char* ctrl;
     unsigned char* meta;
-    unsigned long long* item_prefix;  // [k + 3] item prefix of the k + 2 stages
+    unsigned long long* item_prefix;  // item prefix of the stages (k + twice the lag of batch.cu)
     unsigned long long* solo_prefix;  // [k + 1] item prefix of the small joins
     unsigned* built;                  // [k] build rows inserted per join
     unsigned* cleared;                // [k] clear items done per join
