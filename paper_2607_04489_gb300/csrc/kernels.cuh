@@ -131,8 +131,8 @@ struct PartSide {
     uint32_t* idx[2];    // matching tuple-ID buffers
     void* col[2][kMaxCols];  // GFTR: ping-pong copies of the carried payload columns
     uint32_t* counts;    // per-(tile, digit) counts, scanned in place
-    uint32_t* block_sums;
-    uint32_t* total;     // [2] kept rows after pass 1 / pass 2
+    uint32_t* block_sums;  // of the scan
+    uint32_t* total;     // [4] kept rows after pass 1 / pass 2, pass-2 tiles, chunks scanned
     SegInfo* segs;       // pass-2 segments (pass-1 partitions)
     Tile* tiles;         // pass-2 tiles
     uint32_t* part_start;  // [P + 1] final partition starts

@@ -63,6 +63,7 @@ struct PartPass {
     int bits;
     int kbits;               // hash partitioning: bits of the key mix
     uint32_t* counts;
+    uint32_t* scan_done;     // chunks the scan has summed; the histogram clears it
     const Tile* tiles;       // nullptr: pass-1 tiling of [0, n)
     const uint32_t* ntiles_dev;
     uint32_t ntiles_fixed;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(kPartThreads) part_hist_kernel(PartPass<InKey,
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t nd = 1u << a.bits;
     uint32_t* s_cnt2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd]
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.scan_done = 0u;
     const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, align_up(16 + 2 * (size_t)nd * 4, 16), false);
     __syncthreads();
     const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
@@ -900,99 +902,133 @@ struct ScanLen {
     }
 };
 
-__device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t* s_warp) {
+// Exclusive scan of a warp's sums: returns the prefix of `v`, the warp's total
+// in *total.
+__device__ __forceinline__ uint32_t warp_exscan(uint32_t v, uint32_t* total) {
+    uint32_t x = v;
 #pragma unroll
-    for (int o = kWarp / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane_id() == 0) s_warp[threadIdx.x / kWarp] = v;
-    __syncthreads();
-    uint32_t t = 0;
-    for (int w = 0; w < (int)(blockDim.x / kWarp); ++w) t += s_warp[w];
-    return t;
+    for (int o = 1; o < kWarp; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if ((int)lane_id() >= o) x += y;
+    }
+    *total = __shfl_sync(0xffffffffu, x, kWarp - 1);
+    return x - v;
 }
 
+// The prefix of this warp's `mine` among the CTA's warps; *total: their sum.
+__device__ __forceinline__ uint32_t warps_exscan(uint32_t mine, uint32_t* s_warp, uint32_t* total) {
+    constexpr int kWarps = kScanThreads / kWarp;
+    const int warp = threadIdx.x / kWarp;
+    if (lane_id() == 0) s_warp[warp] = mine;
+    __syncthreads();
+    const uint32_t v = lane_id() < kWarps ? s_warp[lane_id()] : 0u;
+    *total = __reduce_add_sync(0xffffffffu, v);
+    return __reduce_add_sync(0xffffffffu, (int)lane_id() < warp ? v : 0u);
+}
+
+// A thread's entries of a chunk of m: kScanItems / 4 words of 16 bytes, a warp's
+// words side by side (entries at or past m read as 0).
+constexpr int kScanVec = kScanItems / 4;
+static_assert(kScanItems % 4 == 0 && kScanThreads / kWarp <= kWarp, "layout of a chunk");
+
+__device__ __forceinline__ uint32_t scan_first() {
+    return (threadIdx.x / kWarp) * (kWarp * kScanItems) + lane_id() * 4;
+}
+
+__device__ __forceinline__ void scan_load(const uint32_t* p, uint32_t m, uint4 (&v)[kScanVec]) {
+#pragma unroll
+    for (int r = 0; r < kScanVec; ++r) {
+        const uint32_t i = scan_first() + r * (kWarp * 4);
+        if (i + 4 <= m) {
+            v[r] = *reinterpret_cast<const uint4*>(p + i);
+        } else {
+            v[r].x = i < m ? p[i] : 0u;
+            v[r].y = i + 1 < m ? p[i + 1] : 0u;
+            v[r].z = i + 2 < m ? p[i + 2] : 0u;
+            v[r].w = 0u;
+        }
+    }
+}
+
+// Scan of the counts in two launches: chunk sums, whose prefixes the CTA that
+// finishes last computes (no CTA waits for another), then the chunks in place.
+// Bound by reading the counts twice, the second time mostly from L2. 146,484
+// tiles x 256 digits: 242 -> 76 us; 4,883 tiles x 64: 24.5 -> 12.3 us, against
+// three launches with strided shared-memory access. One launch, with the
+// scatter adding the chunk prefixes as it loads the offsets, takes 51 and 8 us
+// but costs the scatters that carry columns 4 % (3253 -> 3426 us), in registers.
 __global__ void __launch_bounds__(kScanThreads)
-    scan_reduce_kernel(const uint32_t* __restrict__ data, ScanLen L, uint32_t* __restrict__ block_sums) {
+    scan_sums_kernel(const uint32_t* __restrict__ data, ScanLen L, uint32_t* sums, uint32_t* done, uint32_t* total) {
     __shared__ uint32_t s_warp[kScanThreads / kWarp];
+    __shared__ uint32_t s_last;
     const size_t len = L.get();
     const size_t beg = (size_t)blockIdx.x * kScanChunk;
-    uint32_t v = 0;
-    for (size_t i = beg + threadIdx.x; i < beg + kScanChunk && i < len; i += blockDim.x) v += data[i];
-    v = block_sum(v, s_warp);
-    if (threadIdx.x == 0) block_sums[blockIdx.x] = v;
-}
-
-// One block: exclusive scan of block_sums[0, nblocks) in place; *total = sum.
-__global__ void __launch_bounds__(1024)
-    scan_blocksums_kernel(uint32_t* __restrict__ block_sums, uint32_t nblocks, uint32_t* total) {
-    __shared__ uint32_t s_in[1024];
-    __shared__ uint32_t s_out[1024];
-    __shared__ uint32_t s_warp[1024 / kWarp];
+    if (len == 0 && blockIdx.x == 0 && threadIdx.x == 0) *total = 0u;
+    if (beg >= len) return;
+    uint4 v[kScanVec];
+    scan_load(data + beg, (uint32_t)(len - beg < (size_t)kScanChunk ? len - beg : (size_t)kScanChunk), v);
+    uint32_t mine = 0, chunk;
+#pragma unroll
+    for (int r = 0; r < kScanVec; ++r) mine += v[r].x + v[r].y + v[r].z + v[r].w;
+    warps_exscan(__reduce_add_sync(0xffffffffu, mine), s_warp, &chunk);
+    const uint32_t nchunks = (uint32_t)((len + kScanChunk - 1) / kScanChunk);
+    if (threadIdx.x == 0) {
+        sums[blockIdx.x] = chunk;
+        __threadfence();
+        s_last = atomicAdd(done, 1u) + 1 == nchunks;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
     uint32_t carry = 0;
-    for (uint32_t base = 0; base < nblocks; base += 1024) {
+    for (uint32_t base = 0; base < nchunks; base += kScanThreads) {
         const uint32_t i = base + threadIdx.x;
-        s_in[threadIdx.x] = i < nblocks ? block_sums[i] : 0u;
-        __syncthreads();
-        const uint32_t m = nblocks - base < 1024u ? nblocks - base : 1024u;
-        const uint32_t t = block_scan_smem(s_in, s_out, m, s_warp);
-        __syncthreads();
-        if (i < nblocks) block_sums[i] = s_out[threadIdx.x] + carry;
+        uint32_t wt, t;
+        const uint32_t x = warp_exscan(i < nchunks ? __ldcg(sums + i) : 0u, &wt);
+        const uint32_t w = warps_exscan(wt, s_warp, &t);
+        if (i < nchunks) sums[i] = carry + w + x;
         carry += t;
-        __syncthreads();
+        __syncthreads();  // s_warp is read
     }
     if (threadIdx.x == 0) *total = carry;
 }
 
 __global__ void __launch_bounds__(kScanThreads)
-    scan_apply_kernel(uint32_t* __restrict__ data, ScanLen L, const uint32_t* __restrict__ block_sums,
+    scan_apply_kernel(uint32_t* __restrict__ data, ScanLen L, const uint32_t* __restrict__ sums,
                       const uint32_t* __restrict__ total) {
-    __shared__ uint32_t s_buf[kScanChunk];
     __shared__ uint32_t s_warp[kScanThreads / kWarp];
     const size_t len = L.get();
     const size_t beg = (size_t)blockIdx.x * kScanChunk;
     if (beg >= len) return;
     const uint32_t m = (uint32_t)(len - beg < (size_t)kScanChunk ? len - beg : (size_t)kScanChunk);
-    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) s_buf[i] = data[beg + i];
-    __syncthreads();
-    // per-thread run of kScanItems consecutive entries
-    const uint32_t lo = threadIdx.x * kScanItems;
-    uint32_t local = 0;
+    uint32_t* p = data + beg;
+    uint4 v[kScanVec];
+    scan_load(p, m, v);
+    uint32_t pre[kScanVec], mine = 0, chunk;
 #pragma unroll
-    for (int j = 0; j < kScanItems; ++j)
-        if (lo + j < m) local += s_buf[lo + j];
-    uint32_t x = local;
-    const unsigned lane = lane_id();
-#pragma unroll
-    for (int o = 1; o < kWarp; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if ((int)lane >= o) x += y;
+    for (int r = 0; r < kScanVec; ++r) {
+        uint32_t t;
+        pre[r] = mine + warp_exscan(v[r].x + v[r].y + v[r].z + v[r].w, &t);
+        mine += t;
     }
-    const int warp = threadIdx.x / kWarp;
-    if ((int)lane == kWarp - 1) s_warp[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        uint32_t v = s_warp[lane < kScanThreads / kWarp ? lane : 0];
-        if (lane >= kScanThreads / kWarp) v = 0;
+    const uint32_t before = sums[blockIdx.x] + warps_exscan(mine, s_warp, &chunk);
 #pragma unroll
-        for (int o = 1; o < kWarp; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-            if ((int)lane >= o) v += y;
-        }
-        if (lane < kScanThreads / kWarp) s_warp[lane] = v;
-    }
-    __syncthreads();
-    uint32_t prefix = block_sums[blockIdx.x] + (warp ? s_warp[warp - 1] : 0u) + x - local;
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        if (lo + j < m) {
-            const uint32_t v = s_buf[lo + j];
-            s_buf[lo + j] = prefix;
-            prefix += v;
+    for (int r = 0; r < kScanVec; ++r) {
+        const uint32_t i = scan_first() + r * (kWarp * 4);
+        uint4 o;
+        o.x = before + pre[r];
+        o.y = o.x + v[r].x;
+        o.z = o.y + v[r].y;
+        o.w = o.z + v[r].z;
+        if (i + 4 <= m) {
+            *reinterpret_cast<uint4*>(p + i) = o;
+        } else {
+            if (i < m) p[i] = o.x;
+            if (i + 1 < m) p[i + 1] = o.y;
+            if (i + 2 < m) p[i + 2] = o.z;
         }
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) data[beg + i] = s_buf[i];
-    if (threadIdx.x == 0 && beg + m == len) data[len] = *total;  // the end of the last run
+    if (threadIdx.x == 0 && beg + m == len) p[m] = *total;  // the end of the last run
 }
 
 // ------------------------------------------------------------ pass-2 tiling
@@ -1097,12 +1133,11 @@ int occupancy_grid(K kern, int threads, size_t smem, const DevInfo& di, size_t w
     return (int)(g < 1 ? 1 : g);
 }
 
-cudaError_t scan_counts(uint32_t* counts, ScanLen L, size_t max_len, uint32_t* block_sums,
+cudaError_t scan_counts(uint32_t* counts, ScanLen L, size_t max_len, uint32_t* block_sums, uint32_t* done,
                         uint32_t* total, cudaStream_t stream) {
     const uint32_t nblocks = (uint32_t)((max_len + kScanChunk - 1) / kScanChunk);
     const uint32_t g = nblocks ? nblocks : 1;
-    scan_reduce_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums);
-    scan_blocksums_kernel<<<1, 1024, 0, stream>>>(block_sums, g, total);
+    scan_sums_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums, done, total);
     scan_apply_kernel<<<g, kScanThreads, 0, stream>>>(counts, L, block_sums, total);
     return cudaGetLastError();
 }
@@ -1122,6 +1157,7 @@ template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
 cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& s, uint32_t* total,
                      unsigned* err, const DevInfo& di, cudaStream_t stream, const char* side_name, int pass_no) {
     cudaError_t e;
+    a.scan_done = s.total + 3;
     const size_t hsmem = hist_smem_bytes<InKey, KeyT, FIRST>(a.bits);
     // The first batch of carried columns is staged beside the keys when no
     // tuple IDs travel and two CTAs still fit an SM (2^28 rows, two 4-byte
@@ -1157,8 +1193,9 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
     ScanLen L{max_tiles << a.bits, a.tiles ? a.ntiles_dev : nullptr, a.bits};
     {
         snprintf(name, sizeof name, "%s_scan.p%d.%s", kind, pass_no, side_name);
-        ProfScope ps(name, 12.0 * (double)(max_tiles << a.bits), stream, 0.0, 3);
-        if ((e = scan_counts(a.counts, L, max_tiles << a.bits, s.block_sums, total, stream)) != cudaSuccess)
+        ProfScope ps(name, 12.0 * (double)(max_tiles << a.bits), stream, 0.0, 2);
+        if ((e = scan_counts(a.counts, L, max_tiles << a.bits, s.block_sums, a.scan_done, total, stream)) !=
+            cudaSuccess)
             return e;
     }
     snprintf(name, sizeof name, "%s_scatter.p%d.%s", kind, pass_no, side_name);
