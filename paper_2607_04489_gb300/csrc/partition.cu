@@ -269,24 +269,31 @@ __device__ __forceinline__ void issue_tile(const TileRing<InKey, KeyT, FIRST>& r
     }
 }
 
-// Decodes element e of the current tile: applies the range test, the narrowing
-// and (hash partitioning) the mix in pass 1. Returns false for a dropped row.
+// Decodes an input key: applies the range test, the narrowing and (hash
+// partitioning) the mix in pass 1. Returns false for a dropped row.
 template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
-__device__ __forceinline__ bool tile_key(const PartPass<InKey, KeyT>& a,
-                                         const typename PassIn<InKey, KeyT, FIRST>::E* kbuf, uint32_t e,
-                                         KeyT& k) {
+__device__ __forceinline__ bool decode_key(const PartPass<InKey, KeyT>& a,
+                                           typename PassIn<InKey, KeyT, FIRST>::E in, KeyT& k) {
     if constexpr (FIRST) {
         // offset from the build minimum; a key outside [min, max] has one
         // beyond the span (compared in the input's width)
         using U = typename std::conditional<sizeof(InKey) == 4, uint32_t, uint64_t>::type;
-        const U d = (U)kbuf[e] - (U)a.offset;
+        const U d = (U)in - (U)a.offset;
         if (d > (U)a.span) return false;
         k = (KeyT)d;
         if constexpr (!SORTM) k = KeyCodec<KeyT>::mix(k, a.kbits);
     } else {
-        k = kbuf[e];
+        k = in;
     }
     return true;
+}
+
+// Element e of the current tile, decoded.
+template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
+__device__ __forceinline__ bool tile_key(const PartPass<InKey, KeyT>& a,
+                                         const typename PassIn<InKey, KeyT, FIRST>::E* kbuf, uint32_t e,
+                                         KeyT& k) {
+    return decode_key<InKey, KeyT, FIRST, SORTM>(a, kbuf[e], k);
 }
 
 template <typename InKey, typename KeyT, bool FIRST>
@@ -315,56 +322,109 @@ __device__ void ring_abort(const TileRing<InKey, KeyT, FIRST>& r, int other, uin
     }
 }
 
-template <typename InKey, typename KeyT, bool FIRST>
-__host__ __device__ constexpr size_t hist_smem_bytes(int bits) {
-    return align_up(16 + 2 * ((size_t)1 << bits) * sizeof(uint32_t), 16) +
-           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(false);
+constexpr int kHistThreads = 256;
+constexpr int kHistWarps = kHistThreads / kWarp;
+constexpr int kHistPad = 4;  // words behind a warp's counters: a tile's counts lie in other banks than its neighbours'
+constexpr int kHistLoads = 4;  // 16-byte loads in flight per lane
+
+constexpr size_t hist_smem_bytes(int bits) {
+    return kHistWarps * (((size_t)1 << bits) + kHistPad) * sizeof(uint32_t);
 }
 
-// Two CTA barriers per tile: the digit counters are double-buffered by tile
-// parity, so the next tile's counting starts while slower threads still store
-// this tile's counts.
+// Warp-collective: counts elements [beg, end) of the pass's input by digit into
+// the warp's counters. The 16-byte words inside are loaded whole, the elements
+// before and behind them one by one.
 template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
-__global__ void __launch_bounds__(kPartThreads) part_hist_kernel(PartPass<InKey, KeyT> a, unsigned* err) {
-    using Ring = TileRing<InKey, KeyT, FIRST>;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t nd = 1u << a.bits;
-    uint32_t* s_cnt2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd]
-    if (blockIdx.x == 0 && threadIdx.x == 0) *a.scan_done = 0u;
-    const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, align_up(16 + 2 * (size_t)nd * 4, 16), false);
-    __syncthreads();
-    const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
-    uint32_t t = blockIdx.x;
-    Tile d_next{};  // warp 0: descriptor of the next tile to issue, loaded one tile early
-    if (threadIdx.x < kWarp) {
-        if (t < ntiles) ring.template issue<false>(a, get_tile(a, t), 0);
-        if (t + gridDim.x < ntiles) d_next = get_tile(a, t + gridDim.x);
+__device__ __forceinline__ void warp_count(const PartPass<InKey, KeyT>& a,
+                                           const typename PassIn<InKey, KeyT, FIRST>::E* src, uint32_t n,
+                                           uint32_t* cnt) {
+    using E = typename PassIn<InKey, KeyT, FIRST>::E;
+    constexpr uint32_t V = 16 / sizeof(E);
+    const uint32_t lane = lane_id();
+    const auto count = [&](E e) {
+        KeyT k;
+        if (decode_key<InKey, KeyT, FIRST, SORTM>(a, e, k)) atomicAdd(&cnt[digit_of(k, a.dshift, a.dmask)], 1u);
+    };
+    uint32_t head = (V - lead_of(src)) % V;
+    if (head > n) head = n;
+    const uint32_t nv = (n - head) / V, tail = head + nv * V;
+    if (lane < head) count(src[lane]);
+    if (tail + lane < n) count(src[tail + lane]);
+    const uint4* v = reinterpret_cast<const uint4*>(src + head);
+    for (uint32_t base = lane; base < nv; base += kWarp * kHistLoads) {
+        union {
+            uint4 w;
+            E e[V];
+        } x[kHistLoads];
+#pragma unroll
+        for (int j = 0; j < kHistLoads; ++j)
+            if (base + j * kWarp < nv) x[j].w = __ldg(v + base + j * kWarp);
+#pragma unroll
+        for (int j = 0; j < kHistLoads; ++j)
+            if (base + j * kWarp < nv) {
+#pragma unroll
+                for (uint32_t q = 0; q < V; ++q) count(x[j].e[q]);
+            }
     }
-    for (uint32_t it = 0; t < ntiles; t += gridDim.x, ++it) {
-        const int b = it & 1;
-        const uint32_t tn = t + gridDim.x;
-        if (threadIdx.x < kWarp && tn < ntiles) {
-            ring.template issue<false>(a, d_next, b ^ 1);
-            if (tn + gridDim.x < ntiles) d_next = get_tile(a, tn + gridDim.x);
-        }
-        uint32_t* s_cnt = s_cnt2 + b * nd;
-        for (uint32_t d = threadIdx.x; d < nd; d += blockDim.x) s_cnt[d] = 0;
-        const Tile tl = get_tile(a, t);
-        const bool ok = mbar_wait(&ring.bar[b], (it >> 1) & 1);
-        if (__syncthreads_or(!ok)) {
-            ring_abort(ring, b ^ 1, ((it + 1) >> 1) & 1, tn < ntiles, err);
-            return;
-        }
-        const auto* kbuf = ring.keys(b) + lead_of(Ring::key_src(a, tl.start));
-#pragma unroll 4
-        for (uint32_t e = threadIdx.x; e < tl.len; e += kPartThreads) {
-            KeyT k;
-            if (tile_key<InKey, KeyT, FIRST, SORTM>(a, kbuf, e, k))
-                atomicAdd(&s_cnt[digit_of(k, a.dshift, a.dmask)], 1u);
+}
+
+// Digit counts of every tile. A warp takes a tile (with `split`, an eighth of
+// one, for inputs of few tiles) and counts it into shared memory of its own, so
+// nothing waits inside a tile; the CTA then stores the counts of its eight
+// neighbouring tiles together, a 32-byte sector per digit. Bound by
+// instructions (about fifteen per row in pass 1, with the mix, and seven in
+// pass 2) and the shared-memory atomics. Against a CTA per 4096-row tile fed by
+// bulk copies, two barriers and a store of lone counts per tile: 600M 32-bit
+// keys 750 -> 484 us (7 bits, pass 1) and 556 -> 352 us (8 bits, pass 2); 60M
+// 64-bit keys, 12 bits, 622 -> 310 us; 20M 64-bit keys, near HBM already,
+// 41 -> 42 us. Five CTAs per SM: four cost 4 %, six no less.
+template <typename InKey, typename KeyT, bool FIRST, bool SORTM>
+__global__ void __launch_bounds__(kHistThreads, 5) part_hist_kernel(PartPass<InKey, KeyT> a, bool split) {
+    using Ring = TileRing<InKey, KeyT, FIRST>;
+    extern __shared__ __align__(16) uint32_t s_hist[];
+    __shared__ size_t s_index[kHistWarps];     // of the tile's count of digit 0
+    __shared__ uint32_t s_stride[kHistWarps];  // from one digit to the next; 0: no tile
+    const uint32_t nd = 1u << a.bits, lane = lane_id(), w = threadIdx.x / kWarp;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.scan_done = 0u;
+    uint32_t* cnt = s_hist + w * (nd + kHistPad);
+    const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
+    const uint32_t per = split ? 1u : (uint32_t)kHistWarps;  // tiles per CTA and round
+    for (uint32_t t0 = blockIdx.x * per; t0 < ntiles; t0 += gridDim.x * per) {
+        const uint32_t t = split ? t0 : t0 + w;
+        for (uint32_t d = lane; d < nd; d += kWarp) cnt[d] = 0;
+        __syncwarp();
+        if (t < ntiles) {
+            const Tile tl = get_tile(a, t);
+            uint32_t beg = 0, end = tl.len;
+            if (split) {
+                beg = w * (kPartTile / kHistWarps);
+                end = beg + kPartTile / kHistWarps < tl.len ? beg + kPartTile / kHistWarps : tl.len;
+            }
+            if (beg < end)
+                warp_count<InKey, KeyT, FIRST, SORTM>(a, Ring::key_src(a, tl.start) + beg, end - beg, cnt);
+            if (lane == 0) {
+                s_index[w] = count_index(tl, t, 0, a.bits);
+                s_stride[w] = tl.ntiles_seg;
+            }
+        } else if (lane == 0) {
+            s_stride[w] = 0;
         }
         __syncthreads();
-        for (uint32_t d = threadIdx.x; d < nd; d += blockDim.x)
-            a.counts[count_index(tl, t, d, a.bits)] = s_cnt[d];
+        if (split) {
+            for (uint32_t d = threadIdx.x; d < nd; d += kHistThreads) {
+                uint32_t c = 0;
+#pragma unroll
+                for (int q = 0; q < kHistWarps; ++q) c += s_hist[q * (nd + kHistPad) + d];
+                a.counts[s_index[0] + (size_t)d * s_stride[0]] = c;
+            }
+        } else {
+            const uint32_t q = threadIdx.x % kHistWarps;
+            const size_t at = s_index[q], stride = s_stride[q];
+            if (stride)
+                for (uint32_t d = threadIdx.x / kHistWarps; d < nd; d += kHistThreads / kHistWarps)
+                    a.counts[at + d * stride] = s_hist[q * (nd + kHistPad) + d];
+        }
+        __syncthreads();
     }
 }
 
@@ -1158,7 +1218,7 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
                      unsigned* err, const DevInfo& di, cudaStream_t stream, const char* side_name, int pass_no) {
     cudaError_t e;
     a.scan_done = s.total + 3;
-    const size_t hsmem = hist_smem_bytes<InKey, KeyT, FIRST>(a.bits);
+    const size_t hsmem = hist_smem_bytes(a.bits);
     // The first batch of carried columns is staged beside the keys when no
     // tuple IDs travel and two CTAs still fit an SM (2^28 rows, two 4-byte
     // columns, 6 bits: 1.58 against 1.72 ms); not in a first pass of 8 bits or
@@ -1187,7 +1247,12 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
     {
         snprintf(name, sizeof name, "%s_hist.p%d.%s", kind, pass_no, side_name);
         ProfScope ps(name, n * in_key, stream);
-        hist<<<occupancy_grid(hist, kPartThreads, hsmem, di, max_tiles), kPartThreads, hsmem, stream>>>(a, err);
+        // fewer tiles than about two warps' worth of the chip: a CTA per tile,
+        // or the last wave of whole tiles is nearly empty (4,883 tiles of 64-bit
+        // keys: 42 us split, 53 whole; 12,208 of 32-bit keys: 122 split, 88 whole)
+        const bool split = max_tiles < (size_t)di.sms * 64;
+        const size_t work = split ? max_tiles : (max_tiles + kHistWarps - 1) / kHistWarps;
+        hist<<<occupancy_grid(hist, kHistThreads, hsmem, di, work), kHistThreads, hsmem, stream>>>(a, split);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     ScanLen L{max_tiles << a.bits, a.tiles ? a.ntiles_dev : nullptr, a.bits};
