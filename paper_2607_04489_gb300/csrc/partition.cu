@@ -163,10 +163,11 @@ struct TileRing {
     using P = PassIn<InKey, KeyT, FIRST>;
     using E = typename P::E;
     uint64_t* bar;          // [2]
-    unsigned char* buf[2];  // keys, then (later passes) rows
+    unsigned char* buf;     // [2] of `stride` bytes: keys, then (later passes) rows
+    uint32_t stride;
 
-    __device__ E* keys(int b) const { return reinterpret_cast<E*>(buf[b]); }
-    __device__ uint32_t* rows(int b) const { return reinterpret_cast<uint32_t*>(buf[b] + P::kKeyBytes); }
+    __device__ E* keys(int b) const { return reinterpret_cast<E*>(buf + b * stride); }
+    __device__ uint32_t* rows(int b) const { return reinterpret_cast<uint32_t*>(buf + b * stride + P::kKeyBytes); }
 
     __device__ static const E* key_src(const PartPass<InKey, KeyT>& a, uint32_t start) {
         if constexpr (FIRST)
@@ -279,9 +280,9 @@ __device__ __forceinline__ bool decode_key(const PartPass<InKey, KeyT>& a,
         // beyond the span (compared in the input's width)
         using U = typename std::conditional<sizeof(InKey) == 4, uint32_t, uint64_t>::type;
         const U d = (U)in - (U)a.offset;
-        if (d > (U)a.span) return false;
         k = (KeyT)d;
         if constexpr (!SORTM) k = KeyCodec<KeyT>::mix(k, a.kbits);
+        return d <= (U)a.span;
     } else {
         k = in;
     }
@@ -301,8 +302,8 @@ __device__ __forceinline__ TileRing<InKey, KeyT, FIRST> ring_setup(unsigned char
     using P = PassIn<InKey, KeyT, FIRST>;
     TileRing<InKey, KeyT, FIRST> r;
     r.bar = reinterpret_cast<uint64_t*>(smem);
-    r.buf[0] = smem + off;
-    r.buf[1] = smem + off + P::buf_bytes(rows);
+    r.buf = smem + off;
+    r.stride = (uint32_t)P::buf_bytes(rows);
     if (threadIdx.x == 0) {
         mbar_init(&r.bar[0], 1);
         mbar_init(&r.bar[1], 1);
@@ -428,6 +429,18 @@ __global__ void __launch_bounds__(kHistThreads, 5) part_hist_kernel(PartPass<InK
     }
 }
 
+// A dropped row (outside the range, or behind a short tile) counts under a digit
+// of its lane's own and is staged behind the tile, where nothing is read: the loops
+// over a thread's rows then have no branches.
+constexpr uint32_t kDropped = kPartTile;     // its stage position
+constexpr uint32_t kStageRows = kPartTile + 8;
+constexpr uint32_t kPosPad = kWarp;          // words behind the digits' positions: the dropped rows' counters
+
+// Words of the digit positions and offsets of two tiles.
+__host__ __device__ constexpr size_t scatter_counters(int bits) {
+    return 4 * ((size_t)1 << bits) + 2 * kPosPad;
+}
+
 // Ring and stage of the hash scatter: keys, with tuple IDs beside them (pass 1:
 // as 16-bit rows of the tile), and a batch of carried columns (8 bytes per
 // row), apart from the keys or in their place.
@@ -435,8 +448,8 @@ template <typename InKey, typename KeyT, bool FIRST>
 __host__ __device__ constexpr size_t scatter_smem_bytes(int bits, bool rows, bool cols, bool col_apart) {
     const size_t key_stage = sizeof(KeyT) + (rows ? (FIRST ? 2 : 4) : 0);
     const size_t stage = !cols ? key_stage : col_apart ? key_stage + 8 : key_stage > 8 ? key_stage : 8;
-    return align_up(16 + 4 * ((size_t)1 << bits) * sizeof(uint32_t), 16) +
-           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(rows) + (size_t)kPartTile * stage;
+    return align_up(16 + scatter_counters(bits) * sizeof(uint32_t), 16) +
+           2 * PassIn<InKey, KeyT, FIRST>::buf_bytes(rows) + (size_t)kStageRows * stage;
 }
 
 // Shared memory that lets two CTAs of a kernel share an SM.
@@ -491,13 +504,14 @@ __device__ __forceinline__ int batch_end(const ColCarry& cc, int c) {
 // registers (issued before the barrier that precedes their staging), staged at
 // their tile positions, and written to the output positions g of the stage
 // entries. v[0], v[1]: the halves of an 8-byte value, or two 4-byte columns.
-__device__ __forceinline__ void load_batch(const ColCarry& cc, int c, int ce, const Tile& tl,
-                                           uint32_t (&v)[2][kPartItems]) {
+template <bool FULL>
+__device__ __forceinline__ void load_batch_rows(const ColCarry& cc, int c, int ce, const Tile& tl,
+                                                uint32_t (&v)[2][kPartItems]) {
     if (cc.bytes[c] == 8) {
         const uint2* src = static_cast<const uint2*>(cc.in[c]) + tl.start + threadIdx.x;
 #pragma unroll
         for (int j = 0; j < kPartItems; ++j)
-            if (j * kPartThreads + threadIdx.x < tl.len) {
+            if (FULL || j * kPartThreads + threadIdx.x < tl.len) {
                 const uint2 x = __ldcs(src + j * kPartThreads);
                 v[0][j] = x.x;
                 v[1][j] = x.y;
@@ -508,12 +522,20 @@ __device__ __forceinline__ void load_batch(const ColCarry& cc, int c, int ce, co
     const uint32_t* s1 = static_cast<const uint32_t*>(cc.in[ce - 1]) + tl.start + threadIdx.x;
 #pragma unroll
     for (int j = 0; j < kPartItems; ++j)
-        if (j * kPartThreads + threadIdx.x < tl.len) v[0][j] = __ldcs(s0 + j * kPartThreads);
+        if (FULL || j * kPartThreads + threadIdx.x < tl.len) v[0][j] = __ldcs(s0 + j * kPartThreads);
     if (ce - c == 2) {
 #pragma unroll
         for (int j = 0; j < kPartItems; ++j)
-            if (j * kPartThreads + threadIdx.x < tl.len) v[1][j] = __ldcs(s1 + j * kPartThreads);
+            if (FULL || j * kPartThreads + threadIdx.x < tl.len) v[1][j] = __ldcs(s1 + j * kPartThreads);
     }
+}
+
+__device__ __forceinline__ void load_batch(const ColCarry& cc, int c, int ce, const Tile& tl,
+                                           uint32_t (&v)[2][kPartItems]) {
+    if (tl.len == (uint32_t)kPartTile)
+        load_batch_rows<true>(cc, c, ce, tl, v);
+    else
+        load_batch_rows<false>(cc, c, ce, tl, v);
 }
 
 __device__ __forceinline__ void stage_batch(const ColCarry& cc, int c, int ce, const uint32_t (&pos)[kPartItems],
@@ -521,44 +543,46 @@ __device__ __forceinline__ void stage_batch(const ColCarry& cc, int c, int ce, c
     if (cc.bytes[c] == 8) {
         uint2* s = reinterpret_cast<uint2*>(stage);
 #pragma unroll
-        for (int j = 0; j < kPartItems; ++j)
-            if (pos[j] != kNoDigit) s[pos[j]] = make_uint2(v[0][j], v[1][j]);
+        for (int j = 0; j < kPartItems; ++j) s[pos[j]] = make_uint2(v[0][j], v[1][j]);
         return;
     }
     uint32_t* s = reinterpret_cast<uint32_t*>(stage);
 #pragma unroll
-    for (int j = 0; j < kPartItems; ++j)
-        if (pos[j] != kNoDigit) s[pos[j]] = v[0][j];
+    for (int j = 0; j < kPartItems; ++j) s[pos[j]] = v[0][j];
     if (ce - c == 2) {
-        s += kPartTile;
+        s += kStageRows;
 #pragma unroll
-        for (int j = 0; j < kPartItems; ++j)
-            if (pos[j] != kNoDigit) s[pos[j]] = v[1][j];
+        for (int j = 0; j < kPartItems; ++j) s[pos[j]] = v[1][j];
+    }
+}
+
+template <bool FULL>
+__device__ __forceinline__ void write_batch_rows(const ColCarry& cc, int c, int ce, const uint32_t (&g)[kPartItems],
+                                                 uint32_t nk, const unsigned char* stage) {
+    if (cc.bytes[c] == 8) {
+        const uint2* s = reinterpret_cast<const uint2*>(stage) + threadIdx.x;
+        uint2* dst = static_cast<uint2*>(cc.out[c]);
+#pragma unroll
+        for (int i = 0; i < kPartItems; ++i)
+            if (FULL || i * kPartThreads + threadIdx.x < nk) dst[g[i]] = s[i * kPartThreads];
+        return;
+    }
+    const uint32_t* s = reinterpret_cast<const uint32_t*>(stage) + threadIdx.x;
+#pragma unroll 1
+    for (; c < ce; ++c, s += kStageRows) {
+        uint32_t* dst = static_cast<uint32_t*>(cc.out[c]);
+#pragma unroll
+        for (int i = 0; i < kPartItems; ++i)
+            if (FULL || i * kPartThreads + threadIdx.x < nk) dst[g[i]] = s[i * kPartThreads];
     }
 }
 
 __device__ __forceinline__ void write_batch(const ColCarry& cc, int c, int ce, const uint32_t (&g)[kPartItems],
                                             uint32_t nk, const unsigned char* stage) {
-    if (cc.bytes[c] == 8) {
-        const uint2* s = reinterpret_cast<const uint2*>(stage);
-        uint2* dst = static_cast<uint2*>(cc.out[c]);
-#pragma unroll
-        for (int i = 0; i < kPartItems; ++i) {
-            const uint32_t q = i * kPartThreads + threadIdx.x;
-            if (q < nk) dst[g[i]] = s[q];
-        }
-        return;
-    }
-    const uint32_t* s = reinterpret_cast<const uint32_t*>(stage);
-#pragma unroll 1
-    for (; c < ce; ++c, s += kPartTile) {
-        uint32_t* dst = static_cast<uint32_t*>(cc.out[c]);
-#pragma unroll
-        for (int i = 0; i < kPartItems; ++i) {
-            const uint32_t q = i * kPartThreads + threadIdx.x;
-            if (q < nk) dst[g[i]] = s[q];
-        }
-    }
+    if (nk == (uint32_t)kPartTile)
+        write_batch_rows<true>(cc, c, ce, g, nk, stage);
+    else
+        write_batch_rows<false>(cc, c, ce, g, nk, stage);
 }
 
 // One thread: asks L2 to fetch the carried columns of tile `tl`, a tile ahead
@@ -658,14 +682,19 @@ struct TileDigits {
 // pass 1; the global positions of a thread's rows are computed once and serve
 // the tuple IDs and every carried column.
 //
-// What bounds it: shared-memory wavefronts (about 22 per 32 rows with one
-// 8-byte column: the rank atomics, and staging at random positions) and issue
-// slots, each near 60 %, with DRAM at 55 %; it had taken about 38 (the rank's
-// start looked up per use, a digit array beside the keys) and eight barriers
-// per tile. Measured on GB300: 20M random 64-bit keys, 5 + 6 bits, 164 + 174 ->
-// 88 + 125 us; 28M narrowed keys, 6 + 6 bits, 138 + 130 -> 105 + 106 us; 2^28
-// rows with two 4-byte columns, 6 + 6 bits, 2.13 + 1.93 -> 1.60 + 1.60 ms; 30M
-// 64-bit keys with a 4-byte column, 6 + 6 bits, 322 + 297 -> 226 + 184 us.
+// What bounds it: the output runs, short pieces of as many places as there are
+// digits (DRAM moves 4.5 to 5.4 TB/s, of 6.8 for a copy), and close behind them
+// shared-memory wavefronts, about 22 per 32 rows with one 8-byte column: the
+// rank atomics, and staging at random positions. It had taken about 38 (the
+// rank's start looked up per use, a digit array beside the keys) and eight
+// barriers per tile; then issue slots (126 instructions per 32 rows: a branch
+// per row and step, ring buffers behind an indexed array in local memory, spills).
+// Measured on GB300, first written -> two barriers -> without branches: 2^28
+// rows with two 4-byte columns, 6 + 6 bits, 2.13 + 1.93 -> 1.60 + 1.60 -> 1.39 +
+// 1.35 ms; 30M 64-bit keys with a 4-byte column, 6 + 6 bits, 322 + 297 -> 229 +
+// 186 -> 142 + 143 us; 20M random 64-bit keys with tuple IDs, 5 + 6 bits, 164 +
+// 174 -> 90 + 125 -> 86 + 115 us; 600M 32-bit keys with an 8-byte column, 7 + 8
+// bits, 3.68 + 3.25 -> 2.65 + 3.19 ms.
 //
 // At most 64 registers: two CTAs per SM wherever shared memory allows.
 template <typename InKey, typename KeyT, bool FIRST, int DPT, bool COLS>
@@ -676,16 +705,16 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
     __shared__ uint32_t s_wtot[kPartWarps];
     const uint32_t nd = 1u << a.bits;
     const bool rows = a.out_idx != nullptr;  // tuple IDs travel with the keys
-    uint32_t* s_pos2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd]
-    uint32_t* s_goff2 = s_pos2 + 2 * nd;                        // [2][nd]
-    const size_t ring_off = align_up(16 + 4 * (size_t)nd * 4, 16);
+    uint32_t* s_pos2 = reinterpret_cast<uint32_t*>(smem + 16);  // [2][nd + kPosPad]
+    uint32_t* s_goff2 = s_pos2 + 2 * (nd + kPosPad);            // [2][nd]
+    const size_t ring_off = align_up(16 + scatter_counters(a.bits) * 4, 16);
     const Ring ring = ring_setup<InKey, KeyT, FIRST>(smem, ring_off, rows);
     KeyT* s_key = reinterpret_cast<KeyT*>(smem + ring_off + 2 * P::buf_bytes(rows));
     static_assert(kPartTile <= 65536, "a row of a tile fits 16 bits");
     using RowT = typename std::conditional<FIRST, uint16_t, uint32_t>::type;  // pass 1: row in the tile
-    RowT* s_idx = reinterpret_cast<RowT*>(s_key + kPartTile);
+    RowT* s_idx = reinterpret_cast<RowT*>(s_key + kStageRows);
     unsigned char* col_stage =
-        reinterpret_cast<unsigned char*>(s_key) + (a.col_apart ? (size_t)kPartTile * sizeof(KeyT) : 0);
+        reinterpret_cast<unsigned char*>(s_key) + (a.col_apart ? (size_t)kStageRows * sizeof(KeyT) : 0);
     __syncthreads();
 
     const uint32_t ntiles = a.tiles ? *a.ntiles_dev : a.ntiles_fixed;
@@ -712,7 +741,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
         if (threadIdx.x < kWarp && more) issue_tile(ring, a, tl_next, b ^ 1);
         if constexpr (COLS)
             if (threadIdx.x == kWarp && more) prefetch_columns(a.cc, tl_next);
-        uint32_t* s_pos = s_pos2 + b * nd;
+        uint32_t* s_pos = s_pos2 + b * (nd + kPosPad);
         const uint32_t* s_goff = s_goff2 + b * nd;
         int c = 0, ce = 0;
         uint32_t val[2][kPartItems];  // a batch of column values of this thread's tile rows
@@ -722,7 +751,7 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
         }
         const bool ok = mbar_wait(&ring.bar[b], (it >> 1) & 1);
         const auto* kbuf = ring.keys(b) + lead_of(Ring::key_src(a, tl.start));
-        uint32_t pos[kPartItems];  // tile position, or kNoDigit for a dropped row
+        uint32_t pos[kPartItems];  // tile position, kDropped for a dropped row
         if (ok) {
             const uint32_t* rbuf = nullptr;
             if constexpr (!FIRST)
@@ -730,16 +759,16 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
             KeyT kk[kPartItems];
 #pragma unroll
             for (int j = 0; j < kPartItems; ++j) {
+                // (behind a short tile the ring buffer is read as it lies)
                 const uint32_t e = j * kPartThreads + threadIdx.x;
-                pos[j] = kNoDigit;
-                if (e < tl.len && tile_key<InKey, KeyT, FIRST, false>(a, kbuf, e, kk[j])) pos[j] = 0;
+                const bool in = decode_key<InKey, KeyT, FIRST, false>(a, kbuf[e], kk[j]);
+                const bool kept = in & (e < tl.len);
+                const uint32_t d = kept ? digit_of(kk[j], a.dshift, a.dmask) : nd + lane_id();
+                pos[j] = atomicAdd(&s_pos[d], 1u);
+                if (!kept) pos[j] = kDropped;
             }
 #pragma unroll
-            for (int j = 0; j < kPartItems; ++j)
-                if (pos[j] != kNoDigit) pos[j] = atomicAdd(&s_pos[digit_of(kk[j], a.dshift, a.dmask)], 1u);
-#pragma unroll
             for (int j = 0; j < kPartItems; ++j) {
-                if (pos[j] == kNoDigit) continue;
                 s_key[pos[j]] = kk[j];
                 if (rows) {
                     const uint32_t e = j * kPartThreads + threadIdx.x;
@@ -762,23 +791,29 @@ __global__ void __launch_bounds__(kPartThreads, 2) part_scatter_kernel(PartPass<
         uint32_t nk_next = 0;
         Tile tl_after{};
         if (more) {
-            nk_next = dg.place(s_wtot, s_pos2 + (b ^ 1) * nd, s_goff2 + (b ^ 1) * nd, a.bits);
+            nk_next = dg.place(s_wtot, s_pos2 + (b ^ 1) * (nd + kPosPad), s_goff2 + (b ^ 1) * nd, a.bits);
             if (tn + gridDim.x < ntiles) {
                 tl_after = get_tile(a, tn + gridDim.x);
                 dg.load(a.counts, tl_after, tn + gridDim.x, a.bits);
             }
         }
         uint32_t g[kPartItems];  // output positions of stage entries tid, tid + threads, ...
+        const auto write_keys = [&](auto full) {
 #pragma unroll
-        for (int i = 0; i < kPartItems; ++i) {
-            const uint32_t q = i * kPartThreads + threadIdx.x;
-            if (q < nk) {
-                const KeyT k = s_key[q];
-                g[i] = s_goff[digit_of(k, a.dshift, a.dmask)] + q;
-                a.out_key[g[i]] = k;
-                if (rows) a.out_idx[g[i]] = (FIRST ? tl.start : 0u) + s_idx[q];
+            for (int i = 0; i < kPartItems; ++i) {
+                const uint32_t q = i * kPartThreads + threadIdx.x;
+                if (decltype(full)::value || q < nk) {
+                    const KeyT k = s_key[q];
+                    g[i] = s_goff[digit_of(k, a.dshift, a.dmask)] + q;
+                    a.out_key[g[i]] = k;
+                    if (rows) a.out_idx[g[i]] = (FIRST ? tl.start : 0u) + s_idx[q];
+                }
             }
-        }
+        };
+        if (nk == (uint32_t)kPartTile)
+            write_keys(std::true_type{});
+        else
+            write_keys(std::false_type{});
         if constexpr (COLS) {
             if (a.col_apart) {
                 write_batch(a.cc, c, ce, g, nk, col_stage);
