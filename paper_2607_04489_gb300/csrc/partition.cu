@@ -496,7 +496,7 @@ __device__ __forceinline__ void carry_column(const V* __restrict__ src, V* __res
 // Carried columns travel in batches of at most 8 bytes per row: one 8-byte
 // column, or one or two 4-byte ones. Returns the first column after the batch
 // that starts at c.
-__device__ __forceinline__ int batch_end(const ColCarry& cc, int c) {
+__host__ __device__ __forceinline__ int batch_end(const ColCarry& cc, int c) {
     return c + 1 < cc.n && cc.bytes[c] == 4 && cc.bytes[c + 1] == 4 ? c + 2 : c + 1;
 }
 
@@ -1254,12 +1254,18 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
     cudaError_t e;
     a.scan_done = s.total + 3;
     const size_t hsmem = hist_smem_bytes(a.bits);
-    // The first batch of carried columns is staged beside the keys when no
-    // tuple IDs travel and two CTAs still fit an SM (2^28 rows, two 4-byte
-    // columns, 6 bits: 1.58 against 1.72 ms); not in a first pass of 8 bits or
-    // more, whose 2 x 256 output runs lie in as many pages at large sizes (600M
-    // rows, an 8-byte column: 5.4 against 4.7 ms; 3.3 ms with 7 bits).
-    a.col_apart = !SORTM && a.cc.n && !a.out_idx && (!FIRST || a.bits <= 7) &&
+    // The first batch of carried columns is staged beside the keys, and written
+    // with them, when no tuple IDs travel, two CTAs still fit an SM, and the
+    // digits' runs of the keys and of the batch lie in at most 256 places; over
+    // more, keys and columns do better one after the other. Apart against
+    // after, 600M rows with an 8-byte column: 7 bits (256 places) 2.65 against
+    // 3.00 ms in pass 1 and 2.58 against 2.68 in pass 2, 8 bits (512) 3.83
+    // against 3.23 and 3.20 against 2.80; 2^28 rows with two 4-byte columns: 6
+    // bits (192) 1.34 against 1.30 and 1.34 against 1.36, 7 bits (384) 1.78
+    // against 1.39 and 1.52 against 1.41; 120M rows, 5 and 6 bits: 0.54 against
+    // 0.58 and 0.57 against 0.58.
+    const int places = a.cc.n ? 1 + batch_end(a.cc, 0) : 1;
+    a.col_apart = !SORTM && a.cc.n && !a.out_idx && ((size_t)places << a.bits) <= 256 &&
                   scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits, false, true, true) <= kTwoPerSm;
     const size_t ssmem = SORTM ? sort_scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits)
                                : scatter_smem_bytes<InKey, KeyT, FIRST>(a.bits, a.out_idx != nullptr, a.cc.n > 0, a.col_apart);
