@@ -493,11 +493,11 @@ bool dense_keys(int dtype, bool narrow, int64_t nb, const eiger_stats_t* bst) {
 // Whether AUTO takes the non-partitioned join in place of a partitioned plan:
 // dense keys, whose direct-addressed table (nphj.cu), with the build columns
 // that are gathered beside it, stays in L2. Measured on GB300 (ms, NPHJ /
-// partitioned): pairs of 2^24 x 2^26 rows (64 MB) 0.89 / 1.44, 2^24.5 x 2^26.5
-// (95 MB) 1.37 / 1.87, 2^25 x 2^27 (134 MB) 2.34 / 2.49; two 4-byte columns a
-// side, 5M x 100M (60 MB) 1.81 / 2.78, 10M x 120M (120 MB) 3.40 / 3.37, 16M x
-// 100M (192 MB) 4.11 / 3.01; 8-byte sums, 8M x 60M (96 MB) 0.89 / 1.29, 16M x
-// 60M (192 MB) 1.53 / 1.43. A caller who asks for carried columns keeps the
+// partitioned): pairs of 2^24 x 2^26 rows (64 MB) 0.82 / 1.21, 2^24.75 x 2^26.75
+// (113 MB) 1.68 / 1.91, 2^25 x 2^27 (134 MB) 2.21 / 2.12; two 4-byte columns a
+// side, 5M x 100M (60 MB) 1.79 / 2.42, 7M x 120M (84 MB) 2.52 / 2.85, 10M x 120M
+// (120 MB) 3.43 / 2.89; 8-byte sums, 8M x 60M (96 MB) 0.92 / 1.03, 12M x 60M
+// (144 MB) 1.29 / 1.12. A caller who asks for carried columns keeps the
 // partitioned plan.
 bool dense_nphj(const JoinCall& c, const eiger_stats_t* bst, const eiger_plan_t& p) {
     if (p.variant != EIGER_PHJ1 && p.variant != EIGER_PHJ2) return false;

@@ -1,7 +1,7 @@
 // Compaction of the per-warp output runs of a chunked join launch (the pairs
 // of the partitioned join): see chunks.cuh.
 //
-// With R positions reserved (the cursor, a multiple of kOutChunk) and H holes
+// With R positions reserved (the cursor, a multiple of the run length) and H holes
 // (the unfilled tails of the warps' last runs), the match count is C = R - H.
 // Every hole below C is matched with one filled position at or above C, and
 // the pair stored there moves into the hole:
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kFixThreads) chunk_fix_plan_kernel(PairSink s,
     unsigned long long h = 0;
     for (uint32_t w = threadIdx.x; w < W; w += kFixThreads) {
         const ChunkRec r = s.rec[w];
-        if (r.base != ~0ull) h += kOutChunk - r.used;
+        if (r.base != ~0ull) h += s.run - r.used;
     }
 #pragma unroll
     for (int o = kWarp / 2; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kFixThreads) chunk_fix_plan_kernel(PairSink s,
         }
         return;
     }
-    const unsigned long long c0 = C / kOutChunk;
-    const uint32_t nab = (uint32_t)(R / kOutChunk - c0);  // runs at or above C: at most W
+    const unsigned long long c0 = C / s.run;
+    const uint32_t nab = (uint32_t)(R / s.run - c0);  // runs at or above C: at most W
     if (nab > W + 1) {
         if (threadIdx.x == 0) {
             atomicOr(err, kErrInternal);
@@ -92,18 +92,18 @@ __global__ void __launch_bounds__(kFixThreads) chunk_fix_plan_kernel(PairSink s,
         }
         return;
     }
-    for (uint32_t i = threadIdx.x; i < nab; i += kFixThreads) f.used_above[i] = kOutChunk;
+    for (uint32_t i = threadIdx.x; i < nab; i += kFixThreads) f.used_above[i] = s.run;
     __syncthreads();
     for (uint32_t w = threadIdx.x; w < W; w += kFixThreads) {
         const ChunkRec r = s.rec[w];
-        if (r.base != ~0ull && r.base >= c0 * kOutChunk) f.used_above[r.base / kOutChunk - c0] = r.used;
+        if (r.base != ~0ull && r.base >= c0 * s.run) f.used_above[r.base / s.run - c0] = r.used;
     }
     __syncthreads();
     // filled positions of run i inside [C, R): a run's filled part is its prefix
     const unsigned long long va = block_exscan(
         nab,
         [&](uint32_t i) -> unsigned long long {
-            const unsigned long long st = (c0 + i) * kOutChunk;
+            const unsigned long long st = (c0 + i) * s.run;
             const unsigned long long lo = st > C ? st : C;
             const unsigned long long hi = st + f.used_above[i];
             return hi > lo ? hi - lo : 0ull;
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kFixThreads) chunk_fix_plan_kernel(PairSink s,
             const ChunkRec r = s.rec[w];
             if (r.base == ~0ull || r.base >= C) return 0ull;
             const unsigned long long hs = r.base + r.used;
-            const unsigned long long he = r.base + kOutChunk < C ? r.base + kOutChunk : C;
+            const unsigned long long he = r.base + s.run < C ? r.base + s.run : C;
             return he > hs ? he - hs : 0ull;
         },
         f.hb_pref, s_warp);
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(256) chunk_fix_move_kernel(PairSink s, uint32_
         for (uint32_t kb = k0; kb < k1; kb += kWarp) {
             // one binary search per 32 positions (lane 0), then each lane
             // steps forward from there: 32 consecutive positions span at most
-            // a few runs, as a full run holds kOutChunk of them
+            // a few runs, as a full run holds 256 or more of them
             if (lane == 0) {
                 uint32_t lo = run, hi = nab;
                 while (hi - lo > 1) {
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(256) chunk_fix_move_kernel(PairSink s, uint32_
             if (k >= k1) continue;
             uint32_t lo = run;
             while (lo + 1 < nab && f.va_pref[lo + 1] <= k) ++lo;
-            const unsigned long long st = (c0 + lo) * kOutChunk;
+            const unsigned long long st = (c0 + lo) * s.run;
             const unsigned long long src = (st > C ? st : C) + (k - f.va_pref[lo]);
             const unsigned long long dst = r.base + r.used + (k - k0);
             uint32_t b, p;

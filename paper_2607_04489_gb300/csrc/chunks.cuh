@@ -1,6 +1,6 @@
 // Barrier-free output of index pairs through per-warp chunks.
 //
-// Every warp owns a run of kOutChunk consecutive output positions, reserved
+// Every warp owns a run of PairSink::run consecutive output positions, reserved
 // with one global atomic on the output cursor, and fills it in order with its
 // matches (ballot, rank, store: no shared memory, no CTA barrier). When the
 // run is used up the warp reserves the next one. At kernel end every warp
@@ -10,7 +10,7 @@
 // chunks_fix moves the matches stored at or above the final match count C into
 // the holes below C, so the pairs are dense in [0, C) again and the cursor
 // holds C. Reserved positions at or above the caller's capacity go to an
-// overflow area of the workspace (kMaxOutWarps x kOutChunk pairs), never to
+// overflow area of the workspace (kMaxOutWarps x kMaxRun pairs), never to
 // the caller's arrays; when C exceeds the capacity the call reports the count
 // only and nothing is moved.
 #pragma once
@@ -19,11 +19,16 @@
 
 namespace eiger {
 
-// Positions per warp reservation. Longer runs leave more holes to fill behind
-// the join, shorter ones more atomics on the one cursor, which pass at about
-// one per nanosecond: 134M pairs take 749 + 76 us (join + compaction) at 512,
-// 745 + 55 at 256, 1267 + 45 at 128; 20M pairs 289 + 47, 281 + 37, 279 + 29.
-constexpr uint32_t kOutChunk = 256;
+// Positions per warp reservation (PairSink::run). Longer runs leave more holes
+// to fill behind the join, shorter ones more atomics on the one cursor, which
+// pass at about one every two nanoseconds under load. Hash tables take 256:
+// 134M pairs 749 + 76 us (join + compaction) at 512, 745 + 55 at 256, 1267 + 45
+// at 128; 20M pairs 289 + 47, 281 + 37, 279 + 29. Direct-addressed tables emit
+// faster and take 512: 134M pairs of 30M build rows 1002 + 45 us at 256, 565 +
+// 68 at 512, 598 + 115 at 1024.
+constexpr uint32_t kHashRun = 256;
+constexpr uint32_t kDirectRun = 512;
+constexpr uint32_t kMaxRun = 512;
 constexpr uint32_t kMaxOutWarps = 10240;  // warps of one chunked launch (grid x warps per CTA)
 
 struct ChunkRec {
@@ -38,9 +43,10 @@ struct PairSink {
     uint32_t* bidx;
     uint32_t* pidx;
     unsigned long long capacity;
-    uint32_t* ovf_b;  // [kMaxOutWarps * kOutChunk]
+    uint32_t run;     // positions per reservation, at most kMaxRun
+    uint32_t* ovf_b;  // [kMaxOutWarps * kMaxRun]
     uint32_t* ovf_p;
-    unsigned long long* cursor;  // positions reserved so far (a multiple of kOutChunk)
+    unsigned long long* cursor;  // positions reserved so far (a multiple of run)
     ChunkRec* rec;               // [kMaxOutWarps]
 };
 
@@ -48,9 +54,9 @@ struct PairSink {
 struct WarpChunk {
     unsigned long long base;
     uint32_t used;
-    __device__ __forceinline__ void init() {
+    __device__ __forceinline__ void init(uint32_t run) {
         base = ~0ull;
-        used = kOutChunk;
+        used = run;  // no room: the first match reserves
     }
 };
 
@@ -58,7 +64,7 @@ __device__ __forceinline__ void sink_store(const PairSink& s, unsigned long long
     if (pos < s.capacity) {
         __stcs(s.bidx + pos, b);
         __stcs(s.pidx + pos, p);
-    } else if (pos - s.capacity < (unsigned long long)kMaxOutWarps * kOutChunk) {
+    } else if (pos - s.capacity < (unsigned long long)kMaxOutWarps * kMaxRun) {
         s.ovf_b[pos - s.capacity] = b;
         s.ovf_p[pos - s.capacity] = p;
     }
@@ -70,11 +76,11 @@ __device__ __forceinline__ void warp_emit(WarpChunk& wc, const PairSink& s, bool
     if (mask == 0) return;
     const uint32_t n = __popc(mask);
     const uint32_t rank = __popc(mask & lanemask_lt());
-    const uint32_t room = kOutChunk - wc.used;
+    const uint32_t room = s.run - wc.used;
     unsigned long long pos = wc.base + wc.used + rank;
     if (n > room) {  // warp-uniform: the run is used up, reserve the next one
         unsigned long long nb = 0;
-        if (lane_id() == 0) nb = atomicAdd(s.cursor, (unsigned long long)kOutChunk);
+        if (lane_id() == 0) nb = atomicAdd(s.cursor, (unsigned long long)s.run);
         nb = __shfl_sync(0xffffffffu, nb, 0);
         if (rank >= room) pos = nb + (rank - room);
         wc.base = nb;
