@@ -112,7 +112,8 @@ def barrier(world: int):
 # Source files that define each timed kernel (its own translation unit and the
 # headers it includes); recorded ncu counters stay valid while these hash the same.
 KERNEL_SOURCES = {
-    "phj_join": ("phj.cu", "chunks.cuh", "emit.cuh", "common.cuh", "kernels.cuh"),
+    "phj_join": ("phj.cu", "phj.cuh", "keygroup.cuh", "chunks.cuh", "emit.cuh", "common.cuh", "kernels.cuh"),
+    "phj_sum": ("phj_sum.cu", "phj.cuh", "keygroup.cuh", "stream.cuh", "emit.cuh", "common.cuh", "kernels.cuh"),
     "part_scatter": ("partition.cu", "common.cuh", "kernels.cuh"),
     "part_hist": ("partition.cu", "common.cuh", "kernels.cuh"),
 }
