@@ -1092,8 +1092,8 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
         // kGbPartRows rows: atomics on L2 lines cost more per row than a pass
         // over the rows, above all on hot groups, but take three launches
         // instead of ten (int32, 25000 groups, SUM and MAX, ms HASH /
-        // PARTITION: 2M rows 0.19 / 0.24, 20M 0.63 / 0.52, 50M 1.49 / 0.93;
-        // 100M rows over 100000 skewed groups 14.4 / 2.7).
+        // PARTITION: 2M rows 0.17 / 0.22, 20M 0.59 / 0.46, 50M 1.41 / 0.79;
+        // 100M rows over 100000 skewed groups 5.6 / 1.5).
         const double table = (double)hash_slots * (keyb + 8.0 * aggs->n);
         const bool in_l2 = table <= (double)l2_bytes_or_default() / 2;
         v = gb_hash_slots(est, ga, pub.narrow != 0) || (in_l2 && n < kGbPartRows) ? EIGER_GB_HASH : EIGER_GB_PARTITION;

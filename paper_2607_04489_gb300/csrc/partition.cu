@@ -373,8 +373,8 @@ __device__ __forceinline__ void warp_count(const PartPass<InKey, KeyT>& a,
 // one, for inputs of few tiles) and counts it into shared memory of its own, so
 // nothing waits inside a tile; the CTA then stores the counts of its eight
 // neighbouring tiles together, a 32-byte sector per digit. Bound by
-// instructions (about fifteen per row in pass 1, with the mix, and seven in
-// pass 2) and the shared-memory atomics. Against a CTA per 4096-row tile fed by
+// instructions (21 per 32 rows in pass 1, with the mix; 7 in pass 2, which
+// reads at 0.77 of DRAM's rate) and the shared-memory atomics. Against a CTA per 4096-row tile fed by
 // bulk copies, two barriers and a store of lone counts per tile: 600M 32-bit
 // keys 750 -> 484 us (7 bits, pass 1) and 556 -> 352 us (8 bits, pass 2); 60M
 // 64-bit keys, 12 bits, 622 -> 310 us; 20M 64-bit keys, near HBM already,
@@ -687,8 +687,9 @@ struct TileDigits {
 // shared-memory wavefronts, about 22 per 32 rows with one 8-byte column: the
 // rank atomics, and staging at random positions. It had taken about 38 (the
 // rank's start looked up per use, a digit array beside the keys) and eight
-// barriers per tile; then issue slots (126 instructions per 32 rows: a branch
-// per row and step, ring buffers behind an indexed array in local memory, spills).
+// barriers per tile; then issue slots (126 and 100 instructions per 32 rows
+// in passes 1 and 2: a branch per row and step, ring buffers behind an indexed
+// array in local memory, spills; now 90 and 65).
 // Measured on GB300, first written -> two barriers -> without branches: 2^28
 // rows with two 4-byte columns, 6 + 6 bits, 2.13 + 1.93 -> 1.60 + 1.60 -> 1.39 +
 // 1.35 ms; 30M 64-bit keys with a 4-byte column, 6 + 6 bits, 322 + 297 -> 229 +
