@@ -474,20 +474,23 @@ eiger_status resolve_materialize(const JoinCall& c, const eiger_stats_t* bst, ei
 // Whether the partitioned join of this plan addresses its tables by the key
 // bits below the partition's: 32-bit keys, few enough slots, and at least an
 // eighth of them filled. Matches (pairs, columns) also need build keys that
-// hardly repeat, since a repeated one sends its item back to hash tables; the
-// carried sum takes repeated keys as they are.
-bool direct_tables(const PlanDev& d, int64_t nb, bool distinct, bool carried_sum) {
+// hardly repeat, since the chains of a table hold few repeats and an item with
+// more goes back to hash tables (2^25 x 2^27 rows with 1 % repeated, pairs and two
+// 4-byte columns a side: 2.4 and 5.1 ms, 17.4 and 39.2 when any repeat sent its
+// item there; 2.2 and 3.9 without repeats; 8 % repeated, hash tables for all: 3.1
+// and 7.1); the carried sum takes repeated keys as they are.
+bool direct_tables(const PlanDev& d, int64_t nb, double estimate, bool carried_sum) {
     if (!d.key32 || (d.variant != EIGER_PHJ1 && d.variant != EIGER_PHJ2)) return false;
     const int slots = d.kbits - d.bits1 - (d.variant == EIGER_PHJ2 ? d.bits2 : 0);
-    return slots <= (carried_sum ? kDirectSumBits : kDirectBits) && (distinct || carried_sum) && (double)nb * 8.0 >= (double)(1ull << d.kbits);
+    return slots <= (carried_sum ? kDirectSumBits : kDirectBits) && (double)nb * 8.0 >= (double)(1ull << d.kbits) &&
+           (carried_sum || (hardly_repeated(estimate, nb) && nb <= kDirectMaxRows));
 }
 
-// Whether the build keys suit direct-addressed tables for matches or sums alike:
-// 32-bit, hardly repeated, at least an eighth of the span's power of two.
+// Whether the build keys are dense: 32-bit, and at least an eighth of the span's
+// power of two rows.
 bool dense_keys(int dtype, bool narrow, int64_t nb, const eiger_stats_t* bst) {
     const bool key32 = dtype == EIGER_I32 || narrow;
-    return key32 && distinct_keys(bst->estimate, nb) &&
-           (double)nb * 8.0 >= (double)(1ull << mix_bits(key32, bst->min, bst->max));
+    return key32 && (double)nb * 8.0 >= (double)(1ull << mix_bits(key32, bst->min, bst->max));
 }
 
 // Whether AUTO takes the non-partitioned join in place of a partitioned plan:
@@ -501,7 +504,8 @@ bool dense_keys(int dtype, bool narrow, int64_t nb, const eiger_stats_t* bst) {
 // partitioned plan.
 bool dense_nphj(const JoinCall& c, const eiger_stats_t* bst, const eiger_plan_t& p) {
     if (p.variant != EIGER_PHJ1 && p.variant != EIGER_PHJ2) return false;
-    if (c.materialize == EIGER_GFTR || !dense_keys(c.dtype, p.narrow, c.nb, bst)) return false;
+    if (c.materialize == EIGER_GFTR || !dense_keys(c.dtype, p.narrow, c.nb, bst) || !distinct_keys(bst->estimate, c.nb))
+        return false;
     const uint64_t words = (uint64_t)bst->max - (uint64_t)bst->min + 1;
     if (words > 2ull * nphj_slots(c.nb, 0.5f)) return false;  // see run_join: the hash table would be the smaller one
     double bytes = 4.0 * (double)words;
@@ -516,9 +520,13 @@ bool dense_nphj(const JoinCall& c, const eiger_stats_t* bst, const eiger_plan_t&
 // that the items of one partition each still fill the chip evenly. Pass 1 gets
 // the smaller half: its output runs, two arrays of 2^bits1 of them, lie in that
 // many pages (2^27 x 2^29, 7 + 8 bits: pass 1 2.6 ms; 8 + 8: 4.6 ms).
+// A carried sum takes repeats as they are, but distinct keys it must be that the
+// rules sized the partitions for; matches must hardly repeat (direct_tables).
 void dense_bits(eiger_plan_t* p, int dtype, int64_t nb, const eiger_stats_t* bst, bool sum) {
     if (p->variant != EIGER_PHJ1 && p->variant != EIGER_PHJ2) return;
     if (!dense_keys(dtype, p->narrow, nb, bst)) return;
+    const bool carried = sum && p->materialize == EIGER_GFTR;
+    if (!(carried ? distinct_keys(bst->estimate, nb) : hardly_repeated(bst->estimate, nb))) return;
     const int kbits = mix_bits(true, bst->min, bst->max);
     const int now = p->bits1 + (p->variant == EIGER_PHJ2 ? p->bits2 : 0);
     int B = kbits - (sum ? kDirectSumBits : kDirectBits);
@@ -623,9 +631,9 @@ eiger_status run_join(const JoinCall& c) {
             if (s != EIGER_OK) return s;
         }
     }
-    if (c.variant == EIGER_AUTO && !c.knobs && !chosen) dense_bits(&pub, c.dtype, c.nb, &bst, c.out.aggregate != 0);
     s = resolve_materialize(c, adaptive ? &bst : nullptr, &pub);
     if (s != EIGER_OK) return s;
+    if (c.variant == EIGER_AUTO && !c.knobs && !chosen) dense_bits(&pub, c.dtype, c.nb, &bst, c.out.aggregate != 0);
     if (c.plan_used) *c.plan_used = pub;
 
     *c.out_count = 0;
@@ -634,7 +642,7 @@ eiger_status run_join(const JoinCall& c) {
 
     PlanDev pd = to_dev(pub, c.dtype, adaptive ? &bst : nullptr);
     set_carry(pd, c.out, pub.materialize);
-    pd.direct = adaptive && direct_tables(pd, c.nb, distinct_keys(bst.estimate, c.nb), pd.gftr && c.out.aggregate);
+    pd.direct = adaptive && direct_tables(pd, c.nb, bst.estimate, pd.gftr && c.out.aggregate);
     NphjScratch ns{};
     PhjScratch ps{};
     SmjScratch ms{};

@@ -91,6 +91,15 @@ __device__ __forceinline__ void warp_emit(WarpChunk& wc, const PairSink& s, bool
     if (has) sink_store(s, pos, b, p);
 }
 
+// Takes up the run that a warp of an earlier launch of this join left off.
+__device__ __forceinline__ void warp_chunk_resume(WarpChunk& wc, const PairSink& s, uint32_t gwarp) {
+    const ChunkRec r = s.rec[gwarp];
+    if (r.base != ~0ull) {
+        wc.base = r.base;
+        wc.used = r.used;
+    }
+}
+
 // Lane 0 records the warp's last run; `gwarp` < kMaxOutWarps.
 __device__ __forceinline__ void warp_chunk_commit(const WarpChunk& wc, const PairSink& s, uint32_t gwarp) {
     if (lane_id() == 0) {

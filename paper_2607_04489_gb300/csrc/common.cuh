@@ -146,13 +146,15 @@ struct Ctrl {
     unsigned long long sum;        // aggregate mode: sum of payload pairs mod 2^64
     unsigned long long next_item;  // PHJ work-item dispenser
     unsigned long long nitems;     // PHJ work items
-    unsigned long long next_redo;  // PHJ: dispenser and number of the items a direct-addressed
-    unsigned long long nredo;      // launch left to hash tables
+    unsigned long long next_redo;  // PHJ: dispenser of the pieces, and number of the items and pieces,
+    unsigned long long nredo;      // a direct-addressed launch left to hash tables (phj.cuh)
     unsigned int err;              // kErr* flags
     unsigned int ntiles2[2];       // pass-2 tile count per side (build, probe)
     unsigned int kept[2];          // rows kept by the range test per side
     unsigned int dup;              // non-partitioned build: a key was inserted twice
-    unsigned int pad[2];
+    unsigned int nchained;         // PHJ: items left to direct-addressed tables with chains, and
+    unsigned int pad;
+    unsigned long long next_chained;  // their dispenser
 };
 
 // Payload columns per side a wide join can materialise.

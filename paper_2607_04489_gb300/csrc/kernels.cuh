@@ -161,7 +161,8 @@ struct PhjScratch {
     void* rec;
     uint32_t* ovf[2];
     ChunkFix fix;
-    unsigned long long* redo;  // items a direct-addressed launch leaves to hash tables
+    unsigned long long* redo;  // items that direct-addressed launches leave to hash tables
+    uint32_t* chained;         // items that the first of them leaves to one with chains
 };
 
 PhjScratch phj_layout(Carve& c, int64_t nb, int64_t np, const PlanDev& plan);

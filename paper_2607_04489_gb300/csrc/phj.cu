@@ -14,7 +14,7 @@
 // shared-memory CAS, then streams the probe chunk, walking linear-probe chains;
 // or, where the build keys are dense and distinct, fills a direct-addressed
 // table (phj.cuh) that takes the whole build partition and reads one word per
-// probe row.
+// probe row (further launches take the partitions with repeated keys, see JoinKind).
 // Index pairs leave through per-warp output runs (chunks.cuh), so the probe
 // loop has no CTA barrier; columns through one CTA reservation per round, column
 // by column; the matches of repeated build keys through the CTA stage
@@ -24,6 +24,10 @@
 // per probe row (28M rows of dense keys: 0.23 ms with hash tables, 0.17 ms);
 // columns wait on the gathers of the build side's values (114M rows, two 4-byte
 // columns a side: 1.79 ms row by row through hash tables and the stage, 1.29 ms).
+// Equal build keys in a hash table are inserted past one another by reads: 2^25 x
+// 2^27 rows with one key on 5 % of the build rows, 57 -> 28 ms.
+#include <algorithm>
+
 #include "chunks.cuh"
 #include "emit.cuh"
 #include "kernels.cuh"
@@ -156,6 +160,12 @@ struct SmemTable<uint32_t> {
         if (prev == kEmptySlot) return 1;
         return (uint32_t)(prev >> 32) == k ? -1 : 0;
     }
+    // whether slot s is taken (dup: by key k)
+    __device__ bool taken(uint32_t s, uint32_t k, int& dup) const {
+        const unsigned long long v = *(volatile unsigned long long*)(slot + s);
+        if (v != kEmptySlot && (uint32_t)(v >> 32) == k) dup = 1;
+        return v != kEmptySlot;
+    }
     // the aligned pair of slots starting at even slot s
     __device__ ulonglong2 pair(uint32_t s) const { return *reinterpret_cast<const ulonglong2*>(slot + s); }
     // 0: empty (chain ends), 1: occupied, other key, 2: match
@@ -187,6 +197,7 @@ struct SmemTable<uint64_t> {
         key[s] = k;
         return 1;
     }
+    __device__ bool taken(uint32_t s, uint64_t, int&) const { return *(volatile uint32_t*)(row + s) != kEmptyRow; }
     // After every insert has completed: 1 when an occupied slot of this
     // thread's share finds its own key earlier in its probe chain, i.e. the
     // table holds a key twice. Linear probing leaves no empty slot between a
@@ -237,18 +248,29 @@ __device__ __forceinline__ void load_round(RoundRegs<KeyT, N>& r, const KeyT* __
 
 constexpr int kJoinWarps = kJoinThreads / kWarp;
 
-// kHash: one hash table per item. kDirect: direct-addressed tables (32-bit
-// keys), slot -> build row; an item whose build keys repeat (a slot taken twice)
-// is left to a second launch. kRedo: those items, through hash tables of
-// kBuildCap build rows each.
-enum JoinKind { kHash, kDirect, kRedo };
+// kHash: one hash table per item. The rest for dense, hardly repeated 32-bit
+// build keys, one launch after the other:
+// kDirect: direct-addressed tables, slot -> build row. An item whose build keys
+// repeat (a slot taken twice) is left to the next launch.
+// kChained: such items, the further rows of a key in chains (phj.cuh); one with
+// more than the chains hold is left to the last launch. Chains in the first
+// launch, for all items, cost unique keys their registers (2^25 x 2^27 rows:
+// pairs 2163 -> 2254 us, two columns a side 3908 -> 4196).
+// kRedo: those, through hash tables, each piece of at most kBuildCap build rows an
+// item of its own, so that one heavily repeated key (a default value) spreads
+// over the chip.
+enum JoinKind { kHash, kDirect, kChained, kRedo };
+
+// Bytes of a direct-addressed table, a multiple of 16.
+__host__ __device__ constexpr size_t direct_table_bytes(int sbits) { return ((size_t)4 << sbits) / 16 * 16 + 16; }
 
 template <typename KeyT, int MODE, bool POS, int KIND>
 __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
-    phj_join_kernel(JoinIn<KeyT> a, const __grid_constant__ JoinOut out, PairSink sink, uint32_t first_warp,
-                    Ctrl* ctrl) {
+    phj_join_kernel(JoinIn<KeyT> a, const __grid_constant__ JoinOut out, PairSink sink, Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool PAIRS = MODE == kPairs, AGG = MODE == kSum;
+    constexpr bool kSlots = KIND == kDirect || KIND == kChained;  // direct-addressed
+    constexpr bool kLater = KIND == kChained || KIND == kRedo;    // goes on with an earlier launch's output runs
     // the stage follows the table in dynamic shared memory; index pairs and
     // aggregates use none, so none is allocated for them (shared memory left
     // unreserved serves as L1 cache, which the payload gathers of the
@@ -259,31 +281,57 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
     __shared__ uint32_t s_grp[2][MODE == kColumns ? kN * kJoinWarps : 1];
     __shared__ unsigned long long s_base[2];
     __shared__ unsigned long long s_next_item;
-    __shared__ uint32_t s_next_part;
+    __shared__ unsigned long long s_item;
+    __shared__ uint32_t s_next_part, s_piece, s_chained;
     SmemTable<KeyT> tab;
     tab.bind(smem);
     uint32_t* dtab = reinterpret_cast<uint32_t*>(smem);
-    if (MODE == kColumns && KIND != kDirect && threadIdx.x == 0) st.count = 0;
+    ChainEntry* chain = reinterpret_cast<ChainEntry*>(smem + direct_table_bytes(a.sbits));
+    // (without items left to it, a later launch leaves the warp records as they are)
+    const unsigned long long left = KIND == kRedo ? ctrl->nredo : KIND == kChained ? ctrl->nchained : 0ull;
+    if (kLater && left == 0) return;
+    if (MODE == kColumns && !kSlots && threadIdx.x == 0) st.count = 0;
     AggState agg{0ull, 0ull};
+    const uint32_t gwarp = blockIdx.x * kJoinWarps + threadIdx.x / kWarp;
     WarpChunk wc;
     wc.init(sink.run);
+    if (PAIRS && kLater) warp_chunk_resume(wc, sink, gwarp);
     uint32_t flushes = 0;
-    const unsigned long long nitems = KIND == kRedo ? ctrl->nredo : ctrl->nitems;
-    unsigned long long* const next = KIND == kRedo ? &ctrl->next_redo : &ctrl->next_item;
-    auto item_of = [&](unsigned long long i) { return KIND == kRedo ? a.redo[i] : i; };
+    const unsigned long long nitems = KIND == kRedo      ? left & ((1ull << kRedoPieceBits) - 1)
+                                      : KIND == kChained ? left
+                                                         : ctrl->nitems;
+    unsigned long long* const next = KIND == kRedo      ? &ctrl->next_redo
+                                     : KIND == kChained ? &ctrl->next_chained
+                                                        : &ctrl->next_item;
 
     // Work items are claimed one ahead: the claim for the next item is issued
     // when an item starts, and its partition is looked up by warp 0 after the
     // build, so neither round trip sits between two items.
+    auto look_up = [&](unsigned long long claim) {  // warp 0
+        unsigned long long item = claim;
+        uint32_t piece = 0, p = 0;
+        if (claim < nitems) {
+            if constexpr (KIND == kRedo) {
+                const uint32_t e = warp_last_le((uint32_t)(left >> kRedoPieceBits), claim,
+                                                [&](uint32_t i) { return a.redo[i] >> kRedoItemBits; });
+                piece = (uint32_t)(claim - (a.redo[e] >> kRedoItemBits));
+                item = a.redo[e] & ((1ull << kRedoItemBits) - 1);
+            }
+            if (KIND == kChained) item = a.chained[claim];
+            p = find_partition(a.item_prefix, a.P, item);
+        }
+        if (threadIdx.x == 0) {
+            s_next_item = claim;
+            s_next_part = p;
+            if (kLater) s_item = item;
+            if (KIND == kRedo) s_piece = piece;
+        }
+        return p;
+    };
     if (threadIdx.x < kWarp) {
         unsigned long long it0 = 0;
         if (threadIdx.x == 0) it0 = atomicAdd(next, 1ull);
-        it0 = __shfl_sync(0xffffffffu, it0, 0);
-        const uint32_t p0 = it0 < nitems ? find_partition(a.item_prefix, a.P, item_of(it0)) : 0u;
-        if (threadIdx.x == 0) {
-            s_next_item = it0;
-            s_next_part = p0;
-        }
+        look_up(__shfl_sync(0xffffffffu, it0, 0));
     }
     __syncthreads();
 
@@ -291,11 +339,18 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         const unsigned long long cur_item = s_next_item;
         const uint32_t p = s_next_part;
         if (cur_item >= nitems) break;
-        const unsigned long long item = item_of(cur_item);
+        const unsigned long long item = kLater ? s_item : cur_item;
         unsigned long long claim = 0;
         if (threadIdx.x == 0) claim = atomicAdd(next, 1ull);
 
-        const ItemRows ir = item_rows(a, item, p);
+        ItemRows ir = item_rows(a, item, p);
+        if constexpr (KIND == kRedo) {  // the piece's share of the build rows
+            const uint32_t pieces = chunks_of(ir.bn, kBuildCap);
+            const uint32_t lo = (uint32_t)((unsigned long long)s_piece * ir.bn / pieces);
+            const uint32_t hi = (uint32_t)((unsigned long long)(s_piece + 1) * ir.bn / pieces);
+            ir.bs0 += lo;
+            ir.bn = hi - lo;
+        }
         const uint32_t bn = ir.bn, pn = ir.pn;
         const KeyT* bkey = a.bkey + ir.bs0;
         const uint32_t* bidx = a.bidx + ir.bs0;
@@ -306,8 +361,8 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         // Issue the first build and probe loads before clearing the table, so
         // their latency overlaps the clear.
         RoundRegs<KeyT, kN> cur, nxt;
-        load_round<POS>(nxt, bkey, bidx, 0, KIND == kRedo ? min(bn, kBuildCap) : bn, bpos0);
-        if (KIND != kDirect) load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
+        load_round<POS>(nxt, bkey, bidx, 0, bn, bpos0);
+        if (!kSlots) load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
 
         // Looks up the next item while the probes run, and asks L2 for the
         // start of its partition's build rows and its first probe round, so
@@ -315,11 +370,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         auto next_item = [&] {
             if (threadIdx.x >= kWarp) return;
             const unsigned long long cl = __shfl_sync(0xffffffffu, claim, 0);
-            const uint32_t pn2 = cl < nitems ? find_partition(a.item_prefix, a.P, item_of(cl)) : 0u;
-            if (threadIdx.x == 0) {
-                s_next_item = cl;
-                s_next_part = pn2;
-            }
+            const uint32_t pn2 = look_up(cl);
             if (cl < nitems) {
                 const uint32_t nb0 = a.bstart[pn2], nbn = min(a.bstart[pn2 + 1] - nb0, kBuildCap);
                 const uint32_t np0 = a.pstart[pn2], npn = min(a.pstart[pn2 + 1] - np0, kRound);
@@ -358,17 +409,21 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
             }
         };
 
-        if constexpr (KIND == kDirect) {
+        if constexpr (kSlots) {
             const uint32_t slots = 1u << a.sbits;
+            // more build rows than slots and chains together hold: no use trying
+            const bool over = KIND == kDirect && bn > slots + kChainMax;
             uint4* d4 = reinterpret_cast<uint4*>(dtab);
-            for (uint32_t i = threadIdx.x; i < slots / 4 + 1; i += kJoinThreads)
-                d4[i] = make_uint4(kHole, kHole, kHole, kHole);
+            if (!over)
+                for (uint32_t i = threadIdx.x; i < slots / 4 + 1; i += kJoinThreads)
+                    d4[i] = make_uint4(kHole, kHole, kHole, kHole);
+            if (KIND == kChained && threadIdx.x == 0) s_chained = 0;
             __syncthreads();
             int dup = 0;
             // Build rows a round ahead (a partition's build takes several);
             // behind the last round, the first probe rows. 10M x 120M rows with
             // two columns a side: 1285 -> 1187 us.
-            for (uint32_t bb = 0; bb < bn; bb += kRound) {
+            for (uint32_t bb = 0; bb < bn && !over; bb += kRound) {
                 const bool more = bb + kRound < bn;
                 if (more)
                     load_round<POS>(cur, bkey, bidx, bb + kRound, bn, bpos0);
@@ -376,36 +431,68 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
                     load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
 #pragma unroll
                 for (int j = 0; j < kN; ++j)
-                    if (bb + j * kJoinThreads + threadIdx.x < bn)
-                        dup |= atomicExch(dtab + direct_slot(nxt.k[j], a.pbits, a.sbits), nxt.id[j]) != kHole;
+                    if (bb + j * kJoinThreads + threadIdx.x < bn) {
+                        const uint32_t s = direct_slot(nxt.k[j], a.pbits, a.sbits);
+                        const uint32_t old = atomicExch(dtab + s, nxt.id[j]);
+                        if constexpr (KIND == kDirect) {
+                            dup |= old != kHole;
+                        } else if (old != kHole) {  // a repeated key: its earlier row leaves the slot
+                            const uint32_t e = atomicAdd(&s_chained, 1u);
+                            if (e < kChainMax) chain[e] = ChainEntry{old, s};
+                        }
+                    }
                 if (more) nxt = cur;
             }
             const bool repeats = __syncthreads_or(dup) != 0;
+            const uint32_t chained = KIND == kChained ? s_chained : 0u;
             next_item();
-            if (repeats) {
-                if (threadIdx.x == 0) a.redo[atomicAdd(&ctrl->nredo, 1ull)] = item;
+            if (over || chained > kChainMax) {
+                if (threadIdx.x == 0) {
+                    const unsigned long long at =
+                        atomicAdd(&ctrl->nredo, (1ull << kRedoPieceBits) | chunks_of(bn, kBuildCap));
+                    a.redo[at >> kRedoPieceBits] = redo_entry(at & ((1ull << kRedoPieceBits) - 1), item);
+                }
+            } else if (repeats) {
+                if (threadIdx.x == 0) a.chained[atomicAdd(&ctrl->nchained, 1u)] = (uint32_t)item;
             } else {
+                if constexpr (KIND == kChained) {  // hang the displaced rows before the rows that stayed
+                    for (uint32_t e = threadIdx.x; e < chained; e += kJoinThreads)
+                        chain[e].next = atomicExch(dtab + chain[e].next, kChainTop - e);
+                    __syncthreads();
+                }
                 probe_rounds([&](uint32_t base) {
-                    uint32_t brow[kN];
+                    uint32_t at[kN];
 #pragma unroll
                     for (int j = 0; j < kN; ++j)
-                        brow[j] = base + j * kJoinThreads + threadIdx.x < pn
-                                      ? dtab[direct_slot(cur.k[j], a.pbits, a.sbits)]
-                                      : kHole;
-                    emit_round(brow);
+                        at[j] = base + j * kJoinThreads + threadIdx.x < pn
+                                    ? dtab[direct_slot(cur.k[j], a.pbits, a.sbits)]
+                                    : kHole;
+                    if constexpr (KIND == kDirect) {
+                        emit_round(at);
+                    } else {  // every row's first match, then their second ones, and so on
+                        bool more;
+                        do {
+                            more = false;
+                            uint32_t brow[kN];
+#pragma unroll
+                            for (int j = 0; j < kN; ++j) {
+                                brow[j] = at[j];
+                                const uint32_t e = kChainTop - at[j];
+                                at[j] = kHole;
+                                if (e < kChainMax) {
+                                    brow[j] = chain[e].row;
+                                    at[j] = chain[e].next;
+                                    more = true;
+                                }
+                            }
+                            emit_round(brow);
+                        } while (MODE == kColumns ? __syncthreads_or(more) : __any_sync(0xffffffffu, more));
+                    }
                 });
             }
-        }
-        // hash tables: the whole build chunk, or kBuildCap of its rows at a time
-        if constexpr (KIND != kDirect) for (uint32_t b0 = 0; b0 < bn; b0 += KIND == kRedo ? kBuildCap : bn) {
-            const uint32_t hn = KIND == kRedo ? min(bn - b0, kBuildCap) : bn;
-            if (KIND == kRedo && b0) {  // the registers hold other rows by now
-                __syncthreads();
-                load_round<POS>(nxt, bkey + b0, bidx + b0, 0, hn, bpos0 + b0);
-                load_round<POS>(cur, pkey, pidx, 0, pn, ppos0);
-            }
+        } else {  // hash tables
             // about three slots per build row (load <= 1/3), at most kTableMax
-            uint32_t tsize = (3 * hn + 31) & ~31u;
+            uint32_t tsize = (3 * bn + 31) & ~31u;
             if (tsize < 64) tsize = 64;
             if (tsize > kTableMax) tsize = kTableMax;
             tab.clear_all(tsize);
@@ -413,21 +500,25 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
             // Build. An insert that meets its own key proves a duplicate in this
             // chunk; without one, every probe key has at most one match here.
             int dup = 0;
-            for (uint32_t bb = 0; bb < hn; bb += kRound) {
-                if (bb) load_round<POS>(nxt, bkey + b0, bidx + b0, bb, hn, bpos0 + b0);
+            for (uint32_t bb = 0; bb < bn; bb += kRound) {
+                if (bb) load_round<POS>(nxt, bkey, bidx, bb, bn, bpos0);
 #pragma unroll
                 for (int j = 0; j < kN; ++j) {
-                    if (bb + j * kJoinThreads + threadIdx.x < hn) {
+                    if (bb + j * kJoinThreads + threadIdx.x < bn) {
                         uint32_t s = home_slot(nxt.k[j], tsize);
-                        for (uint32_t step = 0;; ++step) {
+                        for (uint32_t step = 0;;) {
                             const int r = tab.insert(s, nxt.k[j], nxt.id[j]);
                             if (r > 0) break;
                             if (r < 0) dup = 1;
-                            if (step + 1 == tsize) {
+                            // past the taken slots by reads: the rows of one
+                            // key would all queue for each slot's atomic
+                            do {
+                                s = next_slot(s, tsize);
+                            } while (++step < tsize && tab.taken(s, nxt.k[j], dup));
+                            if (step >= tsize) {
                                 atomicOr(&ctrl->err, kErrTableFull);
                                 break;
                             }
-                            s = next_slot(s, tsize);
                         }
                     }
                     __syncwarp();
@@ -438,7 +529,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
                 dup = tab.has_equal_keys(tsize);
             }
             const bool unique = __syncthreads_or(dup) == 0;
-            if (b0 == 0) next_item();
+            next_item();
             if (unique) {
                 // Fast path: stop at the first match, no collectives per step.
                 probe_rounds([&](uint32_t base) {
@@ -518,45 +609,47 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         __syncthreads();
     }
     if (AGG) agg_commit(agg, ctrl);
-    if constexpr (PAIRS) warp_chunk_commit(wc, sink, first_warp + blockIdx.x * kJoinWarps + threadIdx.x / kWarp);
+    if constexpr (PAIRS) warp_chunk_commit(wc, sink, gwarp);
 }
 
-// Launches of one join; counts the warps launched (each writes a warp record
-// of the pairs sink).
+// Launches of one join, as many CTAs per SM as fit. Each warp writes a record of
+// the pairs sink; a later launch is no larger than the one before it, so that its
+// warps go on with that one's runs.
 template <typename KeyT>
 struct JoinLaunch {
-    static constexpr int kAll = 1 << 20;  // as many CTAs per SM as fit
     const JoinIn<KeyT>& a;
     const JoinOut& out;
     const PairSink& sink;
     Ctrl* ctrl;
     const DevInfo& di;
     cudaStream_t stream;
-    uint32_t warps;
+    uint32_t grid = kMaxOutWarps / kJoinWarps;
 
     template <int MODE, bool POS, int KIND>
-    cudaError_t run(int most_per_sm) {
+    cudaError_t run() {
         auto kern = phj_join_kernel<KeyT, MODE, POS, KIND>;
-        const size_t smem =
-            KIND == kDirect ? ((size_t)4 << a.sbits) + 16
-                            : (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
-                                  (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0);
+        const size_t smem = KIND == kDirect    ? direct_table_bytes(a.sbits)
+                            : KIND == kChained ? direct_table_bytes(a.sbits) + kChainMax * sizeof(ChainEntry)
+                                               : (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
+                                                     (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0);
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kJoinThreads, smem) != cudaSuccess ||
             per_sm < 1)
             per_sm = 1;
-        if (per_sm > most_per_sm) per_sm = most_per_sm;
-        uint32_t grid = (uint32_t)(di.sms * per_sm);
-        const uint32_t room = (kMaxOutWarps - warps) / kJoinWarps;  // warp records left
-        // (a direct launch leaves records for the second one)
-        const uint32_t keep = KIND == kDirect ? room / 4 : 0;
-        if (grid > room - keep) grid = room - keep;
-        kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, warps, ctrl);
-        warps += grid * kJoinWarps;
+        grid = std::min(grid, (uint32_t)(di.sms * per_sm));
+        kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, ctrl);
         return cudaGetLastError();
     }
+    template <int KIND>
+    cudaError_t run_as(bool pairs, int gftr) {
+        return out.aggregate ? run<kSum, false, KIND>()
+               : pairs       ? run<kPairs, false, KIND>()
+               : gftr        ? run<kColumns, true, KIND>()
+                             : run<kColumns, false, KIND>();
+    }
+    uint32_t warps() const { return grid * kJoinWarps; }  // of the last launch
 };
 
 template <typename KeyT>
@@ -595,30 +688,22 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
         sink.rec = static_cast<ChunkRec*>(s.rec);
     }
     a.redo = s.redo;
-    JoinLaunch<KeyT> l{a, out, sink, ctrl, di, stream, 0};
+    a.chained = s.chained;
+    JoinLaunch<KeyT> l{a, out, sink, ctrl, di, stream};
     cudaError_t e;
     if constexpr (sizeof(KeyT) == 4) {
         if (plan.direct) {
-            e = out.aggregate ? l.template run<kSum, false, kDirect>(l.kAll)
-                : pairs       ? l.template run<kPairs, false, kDirect>(l.kAll)
-                : plan.gftr   ? l.template run<kColumns, true, kDirect>(l.kAll)
-                              : l.template run<kColumns, false, kDirect>(l.kAll);
-            // the items whose build keys repeat (most often none)
-            if (e == cudaSuccess)
-                e = out.aggregate ? l.template run<kSum, false, kRedo>(1)
-                    : pairs       ? l.template run<kPairs, false, kRedo>(1)
-                    : plan.gftr   ? l.template run<kColumns, true, kRedo>(1)
-                                  : l.template run<kColumns, false, kRedo>(1);
+            e = l.template run_as<kDirect>(pairs, plan.gftr);
+            const uint32_t warps = l.warps();
+            if (e == cudaSuccess) e = l.template run_as<kChained>(pairs, plan.gftr);
+            if (e == cudaSuccess) e = l.template run_as<kRedo>(pairs, plan.gftr);
             if (e != cudaSuccess || !pairs) return e;
-            return chunk_fix_run(sink, l.warps, s.fix, &ctrl->err, di, stream);
+            return chunk_fix_run(sink, warps, s.fix, &ctrl->err, di, stream);
         }
     }
-    e = out.aggregate ? l.template run<kSum, false, kHash>(l.kAll)
-        : pairs       ? l.template run<kPairs, false, kHash>(l.kAll)
-        : plan.gftr   ? l.template run<kColumns, true, kHash>(l.kAll)
-                      : l.template run<kColumns, false, kHash>(l.kAll);
+    e = l.template run_as<kHash>(pairs, plan.gftr);
     if (e != cudaSuccess || !pairs) return e;
-    return chunk_fix_run(sink, l.warps, s.fix, &ctrl->err, di, stream);
+    return chunk_fix_run(sink, l.warps(), s.fix, &ctrl->err, di, stream);
 }
 
 }  // namespace
@@ -637,6 +722,7 @@ PhjScratch phj_layout(Carve& c, int64_t nb, int64_t np, const PlanDev& plan) {
     s.ovf[1] = c.take<uint32_t>((size_t)kMaxOutWarps * kMaxRun);
     s.fix = chunk_fix_layout(c);
     s.redo = c.take<unsigned long long>(P + (size_t)np / kDirectProbeChunk + 1);
+    s.chained = c.take<uint32_t>(P + (size_t)np / kDirectProbeChunk + 1);
     return s;
 }
 

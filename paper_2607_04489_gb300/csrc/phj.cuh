@@ -19,7 +19,18 @@ constexpr uint32_t kProbeChunk = EIGER_PROBE_CHUNK;  // probe rows per work item
 // below them name a mixed key completely, so those low bits are its slot and no
 // key is stored or compared. Used while the slots are few enough
 // (kDirectBits) and the build rows fill at least an eighth of them.
-constexpr int kDirectBits = 14;     // 4-byte slots: 64 KB, three CTAs per SM
+//
+// A further row of a key that is already in the table goes to a chain entry of
+// the item (in a launch for such items): the slot then holds the entry's code instead of a row, the entry its
+// row and what the slot held before (a row or another code). Codes are the
+// kChainMax words below kHole, so rows stay below them (kDirectMaxRows).
+constexpr int kDirectBits = 14;     // 4-byte slots: 64 KB, and 8 KB of chains: three CTAs per SM
+constexpr uint32_t kChainMax = 1024;              // further rows of repeated keys an item holds
+constexpr uint32_t kChainTop = 0xFFFFFFFEu;       // code of entry e: kChainTop - e
+constexpr int64_t kDirectMaxRows = (int64_t)kChainTop - (kChainMax - 1);  // build rows, for matches
+struct ChainEntry {
+    uint32_t row, next;
+};
 constexpr int kDirectSumBits = 13;  // 12-byte slots: 96 KB beside the sum's row stages
 constexpr uint32_t kDirectProbeChunk = 65536;  // probe rows per work item then: one table serves more
 __device__ __forceinline__ uint32_t direct_slot(uint32_t k, int pbits, int sbits) {
@@ -38,8 +49,18 @@ struct JoinIn {
     uint32_t P;
     uint32_t bcap, pcap;  // build and probe rows per work item, at most
     int pbits, sbits;     // partition bits; direct-addressed tables: bits of the slot below them
-    unsigned long long* redo;  // direct-addressed tables: the items left to hash tables
+    unsigned long long* redo;  // direct-addressed tables: the items left to hash tables (redo_entry)
+    uint32_t* chained;         // and, before those, to tables with chains
 };
+
+// Items that direct-addressed launches leave to hash tables, cut into pieces of
+// at most kBuildCap build rows. Ctrl::nredo counts the items (upper 24 bits) and
+// their pieces (lower 40) in one atomic, so the list is in the order of its
+// items' first pieces; an entry holds an item's first piece and the item.
+constexpr int kRedoItemBits = 24, kRedoPieceBits = 40;
+__host__ __device__ __forceinline__ unsigned long long redo_entry(unsigned long long first, unsigned long long item) {
+    return (first << kRedoItemBits) | item;
+}
 
 __host__ __device__ __forceinline__ uint32_t chunks_of(uint32_t rows, uint32_t cap) {
     return rows / cap + (rows % cap != 0);
@@ -94,23 +115,29 @@ __device__ __forceinline__ void prefetch_rows_l2(const KeyT* key, const uint32_t
     }
 }
 
-// Warp-collective: the last partition p in [0, P) with prefix[p] <= item
-// (prefix is non-decreasing, prefix[0] = 0). Each step tests 32 evenly spaced
-// pivots at once, so 2^15 partitions take three dependent loads.
-__device__ __forceinline__ uint32_t find_partition(const unsigned long long* __restrict__ prefix,
-                                                   uint32_t P, unsigned long long item) {
+// Warp-collective: the last i in [0, n) with value(i) <= x (value is
+// non-decreasing, value(0) <= x). Each step tests 32 evenly spaced pivots at
+// once, so 2^15 entries take three dependent loads.
+template <typename F>
+__device__ __forceinline__ uint32_t warp_last_le(uint32_t n, unsigned long long x, F value) {
     const unsigned lane = lane_id();
-    uint32_t lo = 0, hi = P;
+    uint32_t lo = 0, hi = n;
     while (hi - lo > 1) {
         const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
         const uint32_t piv = lo + lane * step;
-        const bool le = piv < hi && prefix[piv] <= item;
+        const bool le = piv < hi && value(piv) <= x;
         const unsigned m = __ballot_sync(0xffffffffu, le);
         const uint32_t last = 31 - __clz(m);  // lane 0 always qualifies
         lo = lo + last * step;
         hi = lo + step < hi ? lo + step : hi;
     }
     return lo;
+}
+
+// Warp-collective: the partition of a work item (prefix[0] = 0).
+__device__ __forceinline__ uint32_t find_partition(const unsigned long long* __restrict__ prefix,
+                                                   uint32_t P, unsigned long long item) {
+    return warp_last_le(P, item, [&](uint32_t i) { return prefix[i]; });
 }
 
 // The fused sum over positions (phj_sum.cu): out.b.src[0] and out.p.src[0] are

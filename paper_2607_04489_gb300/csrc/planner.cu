@@ -50,6 +50,10 @@ constexpr int64_t kTargetRowsDistinctLarge = 4096;  // ... from kLargeBuild buil
 constexpr int64_t kLargeBuild = 1ll << 27;
 static_assert(kTargetRowsDistinctLarge < EIGER_BUILD_CAP, "an average partition fits one table");
 constexpr double kDistinctFraction = 0.9;  // estimate / rows above which the keys count as distinct
+// ... above which direct-addressed tables take a partition's repeats: with 3 % of
+// the rows of a full table of 2^14 slots, and as much again for the estimate's
+// error (0.8 % standard), about 1000 rows go to its chains (kChainMax, phj.cuh)
+constexpr double kHardlyRepeated = 0.97;
 constexpr int kOnePassBits = 8;
 constexpr double kSkewHeavy = 0.1;     // probe sample distinct fraction: heavy skew
 constexpr double kSkewModerate = 0.5;  // ... moderate skew
@@ -58,6 +62,10 @@ constexpr int kMaxTotalBits = 20;
 
 bool distinct_keys(double estimate, int64_t nb) {
     return nb > 0 && estimate >= kDistinctFraction * (double)nb;
+}
+
+bool hardly_repeated(double estimate, int64_t nb) {
+    return nb > 0 && estimate >= kHardlyRepeated * (double)nb;
 }
 
 int phj_total_bits(int64_t nb, bool distinct) {

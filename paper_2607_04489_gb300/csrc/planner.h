@@ -32,6 +32,9 @@ bool wants_probe_sample(const eiger_plan_t& rules_plan, int64_t nb, int64_t np, 
 // Rows of the probe sample the rules profile (the first rows of the column).
 constexpr int64_t kProbeSampleRows = 1 << 20;
 
+// Whether so few build rows repeat a key that direct-addressed tables take them.
+bool hardly_repeated(double estimate, int64_t nb);
+
 // HyperLogLog estimate from the counts of the 2^14 dense registers' ranks, 0..51
 // (Sec. 4.1).
 double hll_estimate_counts(const uint32_t* hist);
