@@ -7,7 +7,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
+#include <set>
 #include <string>
+#include <utility>
 
 #include "kernels.cuh"
 #include "phj.cuh"
@@ -43,6 +45,22 @@ cudaError_t current_device_info(DevInfo* out) {
     }
     *out = d;
     return cudaSuccess;
+}
+
+cudaError_t allow_smem(const void* kern) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    DevInfo di;
+    cudaError_t e = current_device_info(&di);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({kern, di.dev})) return cudaSuccess;
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             di.smem_optin - (int)fa.sharedSizeBytes);
+    if (e == cudaSuccess) done.insert({kern, di.dev});
+    return e;
 }
 
 namespace {

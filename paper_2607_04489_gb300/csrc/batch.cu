@@ -611,19 +611,11 @@ cudaError_t launch_batch(const eiger_join_desc* d_descs, int k, const BatchLayou
         if (e != cudaSuccess || !small) return e;
     }
     auto skern = batch_small_kernel<InKey, THREADS>;
-    // kSoloBytes plus the static stage: more than the 48 KB a launch gets
-    // without opting in. Set once per device, so that later calls, which may
-    // be recorded into a CUDA graph, make no attribute call.
-    constexpr int kDevSlots = 64;
-    static bool opted_in[kDevSlots] = {};
-    const bool cached = di.dev >= 0 && di.dev < kDevSlots;
-    cudaError_t e;
-    if (!(cached && opted_in[di.dev])) {
-        if ((e = cudaFuncSetAttribute(skern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSoloBytes)) !=
-            cudaSuccess)
-            return e;
-        if (cached) opted_in[di.dev] = true;
-    }
+    // kSoloBytes plus the static stage are more than the 48 KB a launch gets
+    // without opting in (no attribute call after the first run on a device: a
+    // later one may be recorded into a CUDA graph)
+    cudaError_t e = allow_smem(skern);
+    if (e != cudaSuccess) return e;
     ProfScope ps("batch_small", 0.0, stream);
     skern<<<resident_grid(skern, THREADS, kSoloBytes, di), THREADS, kSoloBytes, stream>>>(
         d_descs, k, reinterpret_cast<const BatchMeta*>(L.meta), L.solo_prefix, d_counts,

@@ -374,4 +374,14 @@ struct DevInfo {
 // Cached properties of the current device; returns cudaSuccess or the error.
 cudaError_t current_device_info(DevInfo* out);
 
+// Lets launches of `kern` on the current device take as much dynamic shared memory
+// as its static use leaves. Once per kernel and device, and always the same size:
+// the limit is state of the function, shared by all host threads, so that a size
+// set for one launch could be another thread's before the launch is made.
+cudaError_t allow_smem(const void* kern);
+template <typename K>
+cudaError_t allow_smem(K* kern) {
+    return allow_smem(reinterpret_cast<const void*>(kern));
+}
+
 }  // namespace eiger

@@ -787,8 +787,7 @@ cudaError_t gb_hash_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
                     : s.n == 2 ? (w8 ? gb_hash_smem_kernel<InKey, KeyT, 2, true> : gb_hash_smem_kernel<InKey, KeyT, 2, false>)
                                : (w8 ? gb_hash_smem_kernel<InKey, KeyT, 4, true> : gb_hash_smem_kernel<InKey, KeyT, 4, false>);
         const CtaLayout l = hash_cta_layout<KeyT>(s, plan.smem_slots);
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l.bytes)) != cudaSuccess)
-            return e;
+        if ((e = allow_smem(kern)) != cudaSuccess) return e;
         // a table that leaves room for a second CTA runs 512 threads each, a
         // larger one 1024; no more CTAs than rounds of rows
         const int threads = l.bytes <= kGbHalfSm ? 512 : 1024;
@@ -881,8 +880,7 @@ cudaError_t gb_part_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch&
                 : s.n == 2 ? (w8 ? gb_part_kernel<KeyT, 2, true> : gb_part_kernel<KeyT, 2, false>)
                            : (w8 ? gb_part_kernel<KeyT, 4, true> : gb_part_kernel<KeyT, 4, false>);
     const size_t smem = in.layout.bytes;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(kern)) != cudaSuccess) return e;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGbThreads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;

@@ -1213,12 +1213,6 @@ __global__ void part_start_kernel(const uint32_t* __restrict__ counts, int passe
 }
 
 template <typename K>
-cudaError_t set_smem(K kern, size_t bytes) {
-    if (bytes <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
-template <typename K>
 int occupancy_grid(K kern, int threads, size_t smem, const DevInfo& di, size_t work) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess ||
@@ -1277,8 +1271,7 @@ cudaError_t run_pass(PartPass<InKey, KeyT> a, size_t max_tiles, const PartSide& 
                               : part_scatter_kernel<InKey, KeyT, FIRST, 1, false>)
                     : (a.cc.n ? part_scatter_kernel<InKey, KeyT, FIRST, kGoffPerThread, true>
                               : part_scatter_kernel<InKey, KeyT, FIRST, kGoffPerThread, false>);
-    if ((e = set_smem(hist, hsmem)) != cudaSuccess) return e;
-    if ((e = set_smem(scat, ssmem)) != cudaSuccess) return e;
+    if ((e = allow_smem(hist)) != cudaSuccess || (e = allow_smem(scat)) != cudaSuccess) return e;
     const double n = (double)a.n;
     const double in_key = FIRST ? (double)sizeof(InKey) : (double)sizeof(KeyT);
     const double row = a.out_idx ? (double)sizeof(uint32_t) : 0.0;  // tuple IDs, when the side keeps them

@@ -632,7 +632,7 @@ struct JoinLaunch {
                             : KIND == kChained ? direct_table_bytes(a.sbits) + kChainMax * sizeof(ChainEntry)
                                                : (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
                                                      (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kJoinThreads, smem) != cudaSuccess ||

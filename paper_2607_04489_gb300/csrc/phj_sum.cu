@@ -271,7 +271,7 @@ cudaError_t launch_sum(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, co
                        int64_t nb, int64_t np) {
     auto kern = phj_sum_kernel<KeyT, PayT, DIRECT, CONS>;
     const size_t smem = (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT>::kBytes) + SumStream<KeyT, PayT, DIRECT, CONS>::kBytes;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     constexpr int kThreads = CONS + kStreamWarps * kWarp;
     int per_sm = 0;

@@ -269,17 +269,6 @@ __global__ void __launch_bounds__(kMergeThreads)
     if (s_last && host && threadIdx.x < kRankBins) host->hist[threadIdx.x] = __ldcg(&out->hist[threadIdx.x]);
 }
 
-template <typename K>
-cudaError_t configure_partial(int dev) {
-    static bool done[64] = {};
-    if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(stats_partial_kernel<K>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kHllM * (int)sizeof(uint32_t));
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = true;
-    return e;
-}
-
 }  // namespace
 
 StatsScratch stats_layout(Carve& c) {
@@ -302,7 +291,8 @@ cudaError_t stats_launch(const void* keys, int64_t n, int dtype, const StatsScra
     const size_t smem = kHllM * sizeof(uint32_t);
     const double kb = dtype == 0 ? 4.0 : 8.0;
     {
-        if ((e = dtype == 0 ? configure_partial<int32_t>(di.dev) : configure_partial<int64_t>(di.dev)) != cudaSuccess)
+        if ((e = dtype == 0 ? allow_smem(stats_partial_kernel<int32_t>) : allow_smem(stats_partial_kernel<int64_t>)) !=
+            cudaSuccess)
             return e;
         ProfScope ps("stats_partial", kb * n, stream);
         if (dtype == 0)
