@@ -47,7 +47,7 @@ cudaError_t current_device_info(DevInfo* out) {
     return cudaSuccess;
 }
 
-cudaError_t allow_smem(const void* kern) {
+cudaError_t allow_smem(const void* kern, size_t most) {
     static std::mutex mu;
     static std::set<std::pair<const void*, int>> done;
     DevInfo di;
@@ -55,10 +55,12 @@ cudaError_t allow_smem(const void* kern) {
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lock(mu);
     if (done.count({kern, di.dev})) return cudaSuccess;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             di.smem_optin - (int)fa.sharedSizeBytes);
+    if (most == 0) {
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+        most = (size_t)di.smem_optin - fa.sharedSizeBytes;
+    }
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e == cudaSuccess) done.insert({kern, di.dev});
     return e;
 }

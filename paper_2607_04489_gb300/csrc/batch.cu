@@ -614,7 +614,7 @@ cudaError_t launch_batch(const eiger_join_desc* d_descs, int k, const BatchLayou
     // kSoloBytes plus the static stage are more than the 48 KB a launch gets
     // without opting in (no attribute call after the first run on a device: a
     // later one may be recorded into a CUDA graph)
-    cudaError_t e = allow_smem(skern);
+    cudaError_t e = allow_smem(skern, kSoloBytes);
     if (e != cudaSuccess) return e;
     ProfScope ps("batch_small", 0.0, stream);
     skern<<<resident_grid(skern, THREADS, kSoloBytes, di), THREADS, kSoloBytes, stream>>>(

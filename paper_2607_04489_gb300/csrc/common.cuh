@@ -374,14 +374,15 @@ struct DevInfo {
 // Cached properties of the current device; returns cudaSuccess or the error.
 cudaError_t current_device_info(DevInfo* out);
 
-// Lets launches of `kern` on the current device take as much dynamic shared memory
-// as its static use leaves. Once per kernel and device, and always the same size:
-// the limit is state of the function, shared by all host threads, so that a size
-// set for one launch could be another thread's before the launch is made.
-cudaError_t allow_smem(const void* kern);
+// Lets launches of `kern` on the current device take up to `most` bytes of dynamic
+// shared memory (0: as much as its static use leaves). Once per kernel and device,
+// with what its largest call needs: the limit is state of the function, shared by
+// all host threads, so that a size set for one launch could be another thread's
+// before the launch is made.
+cudaError_t allow_smem(const void* kern, size_t most);
 template <typename K>
-cudaError_t allow_smem(K* kern) {
-    return allow_smem(reinterpret_cast<const void*>(kern));
+cudaError_t allow_smem(K* kern, size_t most = 0) {
+    return allow_smem(reinterpret_cast<const void*>(kern), most);
 }
 
 }  // namespace eiger

@@ -238,7 +238,7 @@ cudaError_t launch_smj(const SmjScratch& s, const PlanDev& plan, const JoinOut& 
                 : plan.gftr   ? smj_join_kernel<KeyT, false, true>
                               : smj_join_kernel<KeyT, false, false>;
     const size_t smem = smj_smem<KeyT>();
-    if ((e = allow_smem(kern)) != cudaSuccess) return e;
+    if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSmjThreads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;

@@ -291,8 +291,8 @@ cudaError_t stats_launch(const void* keys, int64_t n, int dtype, const StatsScra
     const size_t smem = kHllM * sizeof(uint32_t);
     const double kb = dtype == 0 ? 4.0 : 8.0;
     {
-        if ((e = dtype == 0 ? allow_smem(stats_partial_kernel<int32_t>) : allow_smem(stats_partial_kernel<int64_t>)) !=
-            cudaSuccess)
+        if ((e = dtype == 0 ? allow_smem(stats_partial_kernel<int32_t>, smem)
+                            : allow_smem(stats_partial_kernel<int64_t>, smem)) != cudaSuccess)
             return e;
         ProfScope ps("stats_partial", kb * n, stream);
         if (dtype == 0)
