@@ -2,6 +2,7 @@
 // workspace carving, the statistics -> plan -> variant pipeline, and the
 // mapping of CUDA and device-side errors to statuses.
 #include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -1165,7 +1166,10 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
         if (pd.variant == EIGER_GB_HASH)
             pd.smem_slots = gb_hash_slots(est, ga, pd.key32);
         else
-            pd.part_slots = gb_part_slots(est / (double)(1ll << (pub.bits1 + pub.bits2)));
+            // sized from the estimate at first; a retry shows that it was too
+            // low, or one partition overfull, and takes the largest tables (the
+            // same ratio again over four times the partitions gained nothing)
+            pd.part_slots = gb_part_slots(attempt > 1 ? HUGE_VAL : est / (double)(1ll << (pub.bits1 + pub.bits2)));
         Carve c = carve;
         const GbScratch sc = gb_layout(c, n, pd, cb, nc);
         if (c.off > ws_bytes)

@@ -57,16 +57,18 @@ __device__ __forceinline__ uint32_t next_group(uint32_t s, uint32_t slots) {
 }
 
 // Slot of k in keys[0, slots), claimed if new (`fresh`), searched from the
-// group at `base`; ~0u when the table is full. A lost race for a slot reads
-// the group again (at most `slots` times in all).
+// group at `base`; ~0u when the table is full (every group walked once). A lost
+// race for a slot reads its group again (at most kN times a group: its slots
+// fill up).
 template <typename KeyT>
 __device__ __forceinline__ uint32_t claim_slot(KeyT* keys, uint32_t slots, KeyT k, uint32_t base, bool& fresh) {
-    for (uint32_t step = 0; step <= 2 * slots; ++step) {
+    for (uint32_t left = slots / KeyGroup<KeyT>::kN; left > 0;) {
         KeyGroup<KeyT> g;
         g.load(keys + base);
         const uint32_t i = g.first_or_empty(k);
         if (i == KeyGroup<KeyT>::kN) {
             base = next_group<KeyT>(base, slots);
+            --left;
             continue;
         }
         const KeyT cur = cas_smem(keys + base + i, ~KeyT(0), k);
