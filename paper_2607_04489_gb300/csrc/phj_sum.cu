@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
         if (lane_id() == 0) mbar_arrive(&s_stream.iempty[q.i]);
         q.next();
         // (every consumer has left the previous item's table here)
-        if (consumers_or<CONS>(dead) || it.bn == 0) break;
+        if (consumers_stop<CONS>(dead, it.bn == 0, &ctrl->err)) break;
         if constexpr (DIRECT) {
             dir.template clear<CONS>();
             consumers_sync<CONS>();
@@ -262,7 +262,6 @@ __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
             });
         }
     }
-    if (dead && lane_id() == 0) atomicOr(&ctrl->err, kErrInternal);
     agg_commit(agg, ctrl);
 }
 

@@ -16,7 +16,7 @@
 //
 // Every wait is bounded: when one runs out, the CTA's abort flag goes up, all
 // other waits return at once, and the consumers leave together at the end of
-// their item.
+// their item (consumers_stop).
 #pragma once
 
 #include "common.cuh"
@@ -172,6 +172,16 @@ __device__ __forceinline__ bool consumers_or(bool v) {
         : "r"((uint32_t)v), "n"(THREADS)
         : "memory");
     return r != 0;
+}
+
+// Every consumer together, between two items: whether to leave, after the `last`
+// item or because some thread's wait ran out (lanes of a warp may differ), which
+// raises kErrInternal in *err.
+template <int THREADS>
+__device__ __forceinline__ bool consumers_stop(bool dead, bool last, unsigned* err) {
+    const bool failed = consumers_or<THREADS>(dead);
+    if (failed && threadIdx.x == 0) atomicOr(err, kErrInternal);
+    return failed || last;
 }
 
 }  // namespace eiger
