@@ -668,7 +668,7 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     a.P = 1u << (plan.bits1 + (passes == 2 ? plan.bits2 : 0));
     const bool pairs = !out.aggregate && out.bidx && out.pidx && out.b.n == 0 && out.p.n == 0 && !out.b.rowmap &&
                        !out.p.rowmap;
-    a.bcap = plan.direct ? 0xFFFFFFFFu : kBuildCap;
+    a.bcap = build_chunk(plan.direct, out.aggregate && plan.gftr);
     a.pcap = plan.direct ? kDirectProbeChunk : kProbeChunk;
     a.pbits = plan.bits1 + (passes == 2 ? plan.bits2 : 0);
     a.sbits = plan.kbits - a.pbits > 1 ? plan.kbits - a.pbits : 1;
@@ -747,7 +747,7 @@ cudaError_t phj_run(const JoinArgs& a, const PlanDev& plan, const PhjScratch& s,
     {
         ProfScope ps("phj_items", 32.0 * P, stream, 0.0, 2);
         items_count_kernel<<<(P + 255) / 256, 256, 0, stream>>>(
-            s.side[0].part_start, s.side[1].part_start, P, plan.direct ? 0xFFFFFFFFu : kBuildCap,
+            s.side[0].part_start, s.side[1].part_start, P, build_chunk(plan.direct, out.aggregate && plan.gftr),
             plan.direct ? kDirectProbeChunk : kProbeChunk, s.item_prefix);
         items_scan_kernel<<<1, 1024, 0, stream>>>(s.item_prefix, P, ctrl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

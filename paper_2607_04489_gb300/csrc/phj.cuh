@@ -33,6 +33,12 @@ struct ChainEntry {
 };
 constexpr int kDirectSumBits = 13;  // 12-byte slots: 96 KB beside the sum's row stages
 constexpr uint32_t kDirectProbeChunk = 65536;  // probe rows per work item then: one table serves more
+// Build rows per work item of the direct sum, at most: a table takes any number of
+// rows, but with few keys a partition has many rows for one CTA, all on a few slots
+// (2^24 rows of two keys: 5.96 ms by one CTA a key, 0.16 in chunks).
+// The items of a partition's chunks add up. Beyond twice the probe chunk, more
+// build rows save little of the probe rows read again per chunk.
+constexpr uint32_t kDirectSumChunk = 2 * kDirectProbeChunk;
 __device__ __forceinline__ uint32_t direct_slot(uint32_t k, int pbits, int sbits) {
     return (k << pbits) >> (32 - sbits);
 }
@@ -88,6 +94,12 @@ __device__ __forceinline__ ItemRows item_rows(const JoinIn<KeyT>& a, unsigned lo
     r.ps0 = p0 + p_lo;
     r.pn = (uint32_t)((unsigned long long)(pc + 1) * psz / npc) - p_lo;
     return r;
+}
+
+// Build rows per work item of a join (a partition's at most this many at a time);
+// the pieces of an item of direct matches are its later launch's business.
+inline uint32_t build_chunk(int direct, bool carried_sum) {
+    return !direct ? kBuildCap : carried_sum ? kDirectSumChunk : 0xFFFFFFFFu;
 }
 
 __device__ __forceinline__ uint32_t slot_hash(uint32_t k) { return k * 0x9E3779B1u; }
