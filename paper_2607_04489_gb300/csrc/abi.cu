@@ -667,7 +667,12 @@ eiger_status run_join(const JoinCall& c) {
     NphjScratch ns{};
     PhjScratch ps{};
     SmjScratch ms{};
-    const size_t need = variant_bytes(carve, c.nb, c.np, pd, &ns, &ps, &ms);
+    size_t need = variant_bytes(carve, c.nb, c.np, pd, &ns, &ps, &ms);
+    // a workspace without room for the direct-addressed form's chains still holds the hash table
+    if (pd.variant == EIGER_NPHJ && need > c.ws_bytes) {
+        need = ns.hash_end;
+        ns.next = nullptr;
+    }
     if (need > c.ws_bytes)
         return fail(EIGER_ERR_WORKSPACE, "workspace %zu bytes < %zu needed for this plan", c.ws_bytes, need);
     // Host-side fault injection for tests: EIGER_FAULT=table_full shrinks the
@@ -678,7 +683,7 @@ eiger_status run_join(const JoinCall& c) {
         (pd.variant == EIGER_NPHJ || pd.variant == EIGER_STATIC))
         ns.slots = 64;
     // direct-addressed where the span takes no more memory than the hash table
-    ns.direct = pd.variant == EIGER_NPHJ && pd.key32 &&
+    ns.direct = pd.variant == EIGER_NPHJ && pd.key32 && ns.next &&
                 (uint64_t)bst.max - (uint64_t)bst.min < 2ull * ns.slots;
 
     EIGER_CUDA(cudaMemsetAsync(lay.ctrl, 0, sizeof(Ctrl), c.stream), "control block reset");

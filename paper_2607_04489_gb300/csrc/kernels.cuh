@@ -99,6 +99,7 @@ struct NphjScratch {
     void* table;
     unsigned long long slots;  // power of two
     int slot_bytes;            // 8 (packed 32-bit key + idx) or 16 (64-bit key, idx)
+    size_t hash_end = 0;       // workspace that the hash table needs; behind it:
     uint32_t* next = nullptr;  // [nb] direct-addressed form: further rows of a key
     int direct = 0;            // table is head[span + 1] (32-bit keys; at most 2 * slots words)
 };

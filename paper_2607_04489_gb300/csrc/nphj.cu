@@ -415,6 +415,7 @@ NphjScratch nphj_layout(Carve& c, int64_t nb, const PlanDev& plan) {
     s.slots = nphj_slots(nb, plan.load_factor);
     s.slot_bytes = plan.key32 ? 8 : 16;
     s.table = c.take<unsigned char>(s.slots * (size_t)s.slot_bytes);
+    s.hash_end = c.off;
     s.next = plan.key32 && plan.variant != EIGER_STATIC ? c.take<uint32_t>((size_t)nb) : nullptr;
     return s;
 }

@@ -70,3 +70,22 @@ def test_direct_addressed_nphj(eiger, oracle_mod, dt, kind, nb, np_):
     np.testing.assert_array_equal(w.probe_cols[0].cpu().numpy(), pc[p])
     s, c, _ = eiger.join_sum(tb, torch.from_numpy(bc).cuda(), tp, torch.from_numpy(pc).cuda(), variant="nphj")
     assert (s, c) == oracle_mod.join_sum(bk, bc, pk, pc)
+
+
+def test_workspace_of_the_hash_table_alone(eiger, oracle_mod):
+    """4 bytes per build row less than the query says, all that the hash table
+    needs: the join runs; one page less: refused."""
+    rng = np.random.default_rng(5)
+    nb = 100_000
+    bk, pk = rng.permutation(nb).astype(np.int32), rng.integers(-10, nb + 10, size=nb).astype(np.int32)
+    _, _, n = oracle_mod.join(bk, pk)
+    tb, tp = torch.from_numpy(bk).cuda(), torch.from_numpy(pk).cuda()
+    query = eiger.join_workspace(nb, nb, eiger.I32, "nphj")
+    ob, op = (torch.empty(nb, dtype=torch.int32, device="cuda") for _ in range(2))
+    for less, status in ((0, eiger.OK), (4 * nb, eiger.OK), (4 * nb + 4096, eiger.ERR_WORKSPACE)):
+        ws = torch.empty(query - less, dtype=torch.uint8, device="cuda")
+        st, cnt, _ = eiger.join_into(tb, tp, variant="nphj", out_bidx=ob, out_pidx=op, capacity=nb, workspace=ws)
+        assert st == status
+        if st == eiger.OK:
+            assert cnt == n and bool((tb[ob[:n].long()] == tp[op[:n].long()]).all())
+            assert torch.unique(op[:n]).numel() == n
