@@ -623,6 +623,7 @@ struct JoinLaunch {
     Ctrl* ctrl;
     const DevInfo& di;
     cudaStream_t stream;
+    double bytes;  // of the first launch, but for the matches
     uint32_t grid = kMaxOutWarps / kJoinWarps;
 
     template <int MODE, bool POS, int KIND>
@@ -639,6 +640,9 @@ struct JoinLaunch {
             per_sm < 1)
             per_sm = 1;
         grid = std::min(grid, (uint32_t)(di.sms * per_sm));
+        constexpr bool kFirst = KIND == kHash || KIND == kDirect;
+        ProfScope ps(kFirst ? "phj_join" : KIND == kChained ? "phj_join.chained" : "phj_join.redo", kFirst ? bytes : 0.0,
+                     stream, kFirst ? match_bytes(out) : 0.0);
         kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, ctrl);
         return cudaGetLastError();
     }
@@ -674,8 +678,6 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     a.sbits = plan.kbits - a.pbits > 1 ? plan.kbits - a.pbits : 1;
     // the sum with carried payloads has its own kernel (phj_sum.cu)
     if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, plan.direct, out, ctrl, di, stream, nb, np);
-    // reads every partitioned (key', row) of both sides once, writes the matches
-    ProfScope ps("phj_join", (double)(sizeof(KeyT) + sizeof(uint32_t)) * (double)(nb + np), stream, match_bytes(out));
     PairSink sink{};
     sink.run = plan.direct ? kDirectRun : kHashRun;
     if (pairs) {
@@ -689,7 +691,9 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     }
     a.redo = s.redo;
     a.chained = s.chained;
-    JoinLaunch<KeyT> l{a, out, sink, ctrl, di, stream};
+    // reads every partitioned (key', row) of both sides once, writes the matches
+    const double bytes = (double)(sizeof(KeyT) + sizeof(uint32_t)) * (double)(nb + np);
+    JoinLaunch<KeyT> l{a, out, sink, ctrl, di, stream, bytes};
     cudaError_t e;
     if constexpr (sizeof(KeyT) == 4) {
         if (plan.direct) {
