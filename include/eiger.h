@@ -105,7 +105,9 @@ typedef struct {
     int64_t key_max;     /* the library; ignored on input)                           */
     int32_t materialize; /* EIGER_GFUR or EIGER_GFTR: how payloads were gathered
                             (filled in by the library; ignored on input)             */
-    int32_t reserved;
+    int32_t direct;      /* 1: the build tables were direct-addressed by the key (dense
+                            32-bit keys), not hashed (filled in by the library; ignored
+                            on input)                                                */
 } eiger_plan_t;
 
 /*
@@ -173,11 +175,15 @@ eiger_status eiger_join_workspace(int64_t nb, int64_t np, eiger_dtype dtype, eig
  *          row; NULL when absent). They are read only when the matching
  *          d_out_*pay output is requested (gather by tuple ID, Sec. 3.2 GFUR).
  * variant: EIGER_AUTO runs eiger_stats on the build keys, then eiger_plan,
- *          then the chosen variant; where the build keys are dense and distinct
- *          (32-bit keys over a span of at most 8 nb), a partitioned plan gives
- *          way to NPHJ while 4 bytes per key of the span and the build columns
- *          fit 7/8 of L2, and else gets fewer radix bits (direct-addressed
- *          tables of up to 2^14 slots).
+ *          then the chosen variant. Where the build keys are dense (32-bit keys
+ *          whose span, rounded up to a power of two, is at most 8 nb) and
+ *          distinct (estimate >= 0.9 nb), a partitioned plan gives way to NPHJ
+ *          while 4 bytes per key of the span and the build columns fit 7/8 of L2
+ *          and the span is at most two words per slot of the hash table (load
+ *          1/2); else, for sums of carried payloads or where the estimate is at
+ *          least 0.97 nb, it gets fewer radix bits (direct-addressed tables of up
+ *          to 2^14 slots, 2^13 for sums). eiger_plan knows neither the columns nor
+ *          these rules: plan_used tells what ran.
  *          NPHJ/PHJ1/PHJ2 also profile the build keys (narrowing and the probe
  *          range test need min/max) and take their knobs from `knobs` when
  *          non-NULL (bits1/bits2/narrow/load_factor), else from the planner.
@@ -516,12 +522,12 @@ eiger_status eiger_join_static_noalloc(eiger_dtype dtype, const void* d_bkeys, i
                                        uint32_t* d_out_pidx, int64_t capacity, int64_t* out_count,
                                        void* stream);
 
-/* One timed stage (one kernel launch, or the three of a scan) of the last
-   call (see eiger_profile). */
+/* One timed stage (one kernel launch, or the two of a scan, of the work items or
+   of a pairs compaction) of the last call (see eiger_profile). */
 typedef struct {
     char name[32];    /* stage name, e.g. "part_scatter.p1.probe"              */
     float ms;         /* device time between CUDA events around the stage     */
-    int32_t launches; /* kernels the stage launched (1, or 3 for a scan)      */
+    int32_t launches; /* kernels the stage launched (1 or 2)                  */
     double bytes;     /* algorithmic bytes the stage must move (reads of its
                          inputs plus writes of its outputs, no re-reads)      */
 } eiger_stage_t;

@@ -437,6 +437,7 @@ eiger_status resolve_plan(const JoinCall& c, const eiger_stats_t* bst, eiger_pla
     if (s != EIGER_OK) return s;
     pub->key_min = bst->min;
     pub->key_max = bst->max;
+    pub->direct = 0;  // (run_join fills it in)
     if (pub->variant == EIGER_SMJ) sort_passes(pub);
     return EIGER_OK;
 }
@@ -685,6 +686,7 @@ eiger_status run_join(const JoinCall& c) {
     // direct-addressed where the span takes no more memory than the hash table
     ns.direct = pd.variant == EIGER_NPHJ && pd.key32 && ns.next &&
                 (uint64_t)bst.max - (uint64_t)bst.min < 2ull * ns.slots;
+    if (c.plan_used) c.plan_used->direct = pd.variant == EIGER_NPHJ ? ns.direct : pd.direct;
 
     EIGER_CUDA(cudaMemsetAsync(lay.ctrl, 0, sizeof(Ctrl), c.stream), "control block reset");
     const JoinArgs a{c.bkeys, c.nb, c.pkeys, c.np};

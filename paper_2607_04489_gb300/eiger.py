@@ -75,7 +75,7 @@ class PlanT(ctypes.Structure):
                 ("narrow", ctypes.c_int32), ("load_factor", ctypes.c_float),
                 ("selector", ctypes.c_int32), ("key_min", ctypes.c_int64),
                 ("key_max", ctypes.c_int64), ("materialize", ctypes.c_int32),
-                ("reserved", ctypes.c_int32)]
+                ("direct", ctypes.c_int32)]
 
 
 MAX_AGGS = 4
@@ -155,12 +155,13 @@ class Plan:
     key_min: int = 0
     key_max: int = 0
     materialize: str = "gfur"
+    direct: int = 0  # 1: direct-addressed build tables (filled in)
 
     @classmethod
     def from_c(cls, p: PlanT) -> "Plan":
         return cls(VARIANT_NAMES.get(p.variant, str(p.variant)), p.bits1, p.bits2, p.narrow,
                    p.load_factor, p.selector, p.key_min, p.key_max,
-                   MATERIALIZE_NAMES.get(p.materialize, str(p.materialize)))
+                   MATERIALIZE_NAMES.get(p.materialize, str(p.materialize)), p.direct)
 
     def to_c(self) -> PlanT:
         p = PlanT()

@@ -1,12 +1,13 @@
 """The partitioned join's direct-addressed tables (dense, hardly repeated 32-bit
 build keys) against the oracle, in every output mode.
 
-Plans put the slots of a partition at the largest table, one bit below it and
-at a handful; a span one past a power of two and an eighth-full span set the
-density limits. A few repeated build keys send their partitions (larger than one
-hash table) through the second launch beside partitions that stay direct, and a
-hot probe key cuts its partition's probe side into several items. Pairs and
-columns are compared after the canonical sort, sums exactly.
+Plans put the slots of a partition above the largest table (hash tables then), at
+it, one bit below it and at a handful; a span one past a power of two and an
+eighth-full span set the density limits. A few repeated build keys send their
+partitions (larger than one hash table) through the later launches beside
+partitions that stay in the first, and a hot probe key cuts its partition's probe
+side into several items. plan_used says which tables ran. Pairs and columns are
+compared after the canonical sort, sums exactly.
 """
 
 import numpy as np
@@ -56,7 +57,7 @@ def _canon(b, p, *cols):
 
 
 @pytest.mark.parametrize("kind", ["dense", "sparse", "repeats", "tiny"])
-@pytest.mark.parametrize("bits", [(2, 0), (2, 1), (5, 6)])
+@pytest.mark.parametrize("bits", [(2, 0), (2, 1), (4, 0), (5, 6)])
 def test_direct_addressed_joins(eiger, oracle_mod, kind, bits):
     rng = np.random.default_rng(len(kind) + 10 * sum(bits))
     bk, pk = _input(kind, rng)
@@ -65,9 +66,12 @@ def test_direct_addressed_joins(eiger, oracle_mod, kind, bits):
     tb, tp = torch.from_numpy(bk).cuda(), torch.from_numpy(pk).cuda()
     eb, ep, n = oracle_mod.join(bk, pk)
 
+    kbits = max(2, (int(bk.max()) - int(bk.min())).bit_length())
+    direct = 1 if kbits - sum(bits) <= 14 else 0  # slots; at most 2^13 for the carried sum
+
     r = eiger.join(tb, tp, variant=variant, knobs=knobs)
     b, p = _canon(r.build_idx, r.probe_idx)
-    assert r.count == n
+    assert r.count == n and r.plan.direct == direct
     np.testing.assert_array_equal(p, ep)
     np.testing.assert_array_equal(b, eb)
 
@@ -77,13 +81,14 @@ def test_direct_addressed_joins(eiger, oracle_mod, kind, bits):
         w = eiger.join_wide(tb, tp, [torch.from_numpy(c).cuda() for c in bcols],
                             [torch.from_numpy(c).cuda() for c in pcols], variant=variant, knobs=knobs, materialize=mat)
         b, p, b0, b1, p0, p1 = _canon(w.build_idx, w.probe_idx, *w.build_cols, *w.probe_cols)
-        assert w.count == n and w.plan.materialize == mat
+        assert w.count == n and w.plan.materialize == mat and w.plan.direct == direct
         np.testing.assert_array_equal(p, ep)
         np.testing.assert_array_equal(b, eb)
         for got, want in ((b0, bcols[0][b]), (b1, bcols[1][b]), (p0, pcols[0][p]), (p1, pcols[1][p])):
             np.testing.assert_array_equal(got, want)
-        s, c, _ = eiger.join_sum(tb, torch.from_numpy(bcols[1]).cuda(), tp, torch.from_numpy(pcols[0]).cuda(),
-                                 variant=variant, knobs=knobs, materialize=mat)
+        s, c, plan = eiger.join_sum(tb, torch.from_numpy(bcols[1]).cuda(), tp, torch.from_numpy(pcols[0]).cuda(),
+                                    variant=variant, knobs=knobs, materialize=mat)
+        assert plan.direct == (direct if mat == "gfur" else 1 if kbits - sum(bits) <= 13 else 0)
         assert (s, c) == oracle_mod.join_sum(bk, bcols[1], pk, pcols[0])
 
 
@@ -101,3 +106,48 @@ def test_direct_addressed_join_capacity(eiger, oracle_mod):
                                      workspace=ws)
         assert cnt == n and st == (eiger.OK if cap == n else eiger.ERR_CAPACITY)
         assert bool((ob[cap:] == -7).all()) and bool((op[cap:] == -7).all())
+
+
+@pytest.mark.parametrize("span_bits,direct", [(18, 1), (19, 0)])
+@pytest.mark.parametrize("mode", ["pairs", "columns", "gfur", "gftr"])
+def test_density_limit(eiger, span_bits, direct, mode):
+    """2^15 build rows: direct-addressed over a span of an eighth's density, 2^18
+    keys, and no more over one key further (2^18 + 1, which counts as 2^19)."""
+    rng = np.random.default_rng(span_bits)
+    nb, top = 1 << 15, (1 << 18) - (1 if span_bits == 18 else 0)
+    bk = np.append(rng.choice(np.arange(1, top), size=nb - 2, replace=False), [0, top]).astype(np.int32)
+    tb = torch.from_numpy(bk).cuda()
+    pay = torch.ones(nb, dtype=torch.int32, device="cuda")
+    bits = 6 if mode == "gftr" else 5
+    knobs = eiger.Plan("phj1", bits, 0, 1)
+    if mode == "pairs":
+        r = eiger.join(tb, tb, variant="phj1", knobs=knobs)
+    elif mode == "columns":
+        r = eiger.join_wide(tb, tb, [pay], [pay], variant="phj1", knobs=knobs)
+    else:
+        s, c, plan = eiger.join_sum(tb, pay, tb, pay, variant="phj1", knobs=knobs, materialize=mode)
+        assert (s, c, plan.direct) == (2 * nb, nb, direct)
+        return
+    assert r.count == nb and r.plan.direct == direct
+    assert bool((r.build_idx == r.probe_idx).all())
+
+
+def test_auto_takes_the_dense_plans(eiger):
+    """AUTO on dense keys: NPHJ while the table stays in L2, partitions of up to
+    2^14 slots (2^13 for carried sums) beyond; on as many sparse keys neither."""
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    for log2nb, variant in ((23, "nphj"), (26, "phj2")):
+        nb = 1 << log2nb
+        bk = torch.randperm(nb, generator=gen, device="cuda").to(torch.int32)
+        pk = bk[:nb // 2].contiguous()
+        r = eiger.join(bk, pk)
+        assert r.count == pk.numel() and (r.plan.variant, r.plan.direct) == (variant, 1)
+        if variant == "phj2":
+            assert r.plan.bits1 + r.plan.bits2 == log2nb - 14
+            s = eiger.join_sum(bk, bk, pk, pk, materialize="gftr")[2]
+            assert (s.variant, s.direct, s.bits1 + s.bits2) == ("phj2", 1, log2nb - 13)
+        del r
+        sparse = (bk * 31).contiguous() if log2nb == 26 else (bk * 400).contiguous()
+        r = eiger.join(sparse, sparse[:1000].contiguous())
+        assert r.count == 1000 and (r.plan.variant, r.plan.direct) == ("phj2", 0)
+        del r

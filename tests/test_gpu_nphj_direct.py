@@ -60,7 +60,15 @@ def test_direct_addressed_nphj(eiger, oracle_mod, dt, kind, nb, np_):
     pc = rng.integers(-2**62, 2**62, size=np_)
     w = eiger.join_wide(tb, tp, [torch.from_numpy(bc).cuda()], [torch.from_numpy(pc).cuda()], variant="nphj")
     r = eiger.join(tb, tp, variant="nphj")
+    span = int(bk.max()) - int(bk.min())
+    slots = 64
+    while slots < 2 * nb:
+        slots *= 2
+    direct = 1 if span < 2 * slots else 0
+    if nb > 1:  # (one row has no span)
+        assert direct == {"last": 1, "past": 0}.get(kind, direct)
     for x in (r, w):
+        assert x.plan.direct == direct
         b, p = (t.cpu().numpy().astype(np.int64) & 0xFFFFFFFF for t in (x.build_idx, x.probe_idx))
         o = np.lexsort((b, p))
         assert x.count == n and x.plan.variant == "nphj"
@@ -68,8 +76,8 @@ def test_direct_addressed_nphj(eiger, oracle_mod, dt, kind, nb, np_):
         np.testing.assert_array_equal(b[o], eb)
     np.testing.assert_array_equal(w.build_cols[0].cpu().numpy(), bc[b])
     np.testing.assert_array_equal(w.probe_cols[0].cpu().numpy(), pc[p])
-    s, c, _ = eiger.join_sum(tb, torch.from_numpy(bc).cuda(), tp, torch.from_numpy(pc).cuda(), variant="nphj")
-    assert (s, c) == oracle_mod.join_sum(bk, bc, pk, pc)
+    s, c, plan = eiger.join_sum(tb, torch.from_numpy(bc).cuda(), tp, torch.from_numpy(pc).cuda(), variant="nphj")
+    assert plan.direct == direct and (s, c) == oracle_mod.join_sum(bk, bc, pk, pc)
 
 
 def test_workspace_of_the_hash_table_alone(eiger, oracle_mod):
@@ -84,8 +92,9 @@ def test_workspace_of_the_hash_table_alone(eiger, oracle_mod):
     ob, op = (torch.empty(nb, dtype=torch.int32, device="cuda") for _ in range(2))
     for less, status in ((0, eiger.OK), (4 * nb, eiger.OK), (4 * nb + 4096, eiger.ERR_WORKSPACE)):
         ws = torch.empty(query - less, dtype=torch.uint8, device="cuda")
-        st, cnt, _ = eiger.join_into(tb, tp, variant="nphj", out_bidx=ob, out_pidx=op, capacity=nb, workspace=ws)
+        st, cnt, plan = eiger.join_into(tb, tp, variant="nphj", out_bidx=ob, out_pidx=op, capacity=nb, workspace=ws)
         assert st == status
         if st == eiger.OK:
+            assert plan.direct == (1 if less == 0 else 0)
             assert cnt == n and bool((tb[ob[:n].long()] == tp[op[:n].long()]).all())
             assert torch.unique(op[:n]).numel() == n

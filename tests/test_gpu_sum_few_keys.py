@@ -42,7 +42,7 @@ def test_few_keys(eiger, nb, keys, pay):
         count += rb * rp
     knobs = eiger.Plan("phj1", 1, 0, 1)
     s, c, plan = eiger.join_sum(bk, bp, pk, pp, variant="phj1", knobs=knobs, materialize="gftr")
-    assert (s, c) == (_mod64(total), count)
+    assert (s, c, plan.direct) == (_mod64(total), count, 1)
 
 
 def test_few_keys_spread_over_the_chip(eiger):
