@@ -204,18 +204,7 @@ __global__ void __launch_bounds__(kSetupThreads)
 // Warp-collective: the stage whose items contain `item` (last s with prefix[s] <= item).
 __device__ __forceinline__ int find_join(const unsigned long long* __restrict__ prefix, int k,
                                          unsigned long long item) {
-    const unsigned lane = lane_id();
-    int lo = 0, hi = k;
-    while (hi - lo > 1) {
-        const int step = (hi - lo + kWarp - 1) / kWarp;
-        const int piv = lo + (int)lane * step;
-        const bool le = piv < hi && prefix[piv] <= item;
-        const unsigned m = __ballot_sync(0xffffffffu, le);
-        const int last = 31 - __clz(m);
-        lo = lo + last * step;
-        hi = lo + step < hi ? lo + step : hi;
-    }
-    return lo;
+    return (int)warp_last_le((uint32_t)k, item, [&](uint32_t i) { return prefix[i]; });
 }
 
 // Table words: a global table is read through L2 (other CTAs wrote it), a

@@ -192,6 +192,25 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+// Warp-collective: the last i in [0, n) with value(i) <= x (value is
+// non-decreasing, value(0) <= x). Each step tests 32 evenly spaced pivots at
+// once, so 2^15 entries take three dependent loads.
+template <typename F>
+__device__ __forceinline__ uint32_t warp_last_le(uint32_t n, unsigned long long x, F value) {
+    const unsigned lane = lane_id();
+    uint32_t lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
+        const uint32_t piv = lo + lane * step;
+        const bool le = piv < hi && value(piv) <= x;
+        const unsigned m = __ballot_sync(0xffffffffu, le);
+        const uint32_t last = 31 - __clz(m);  // lane 0 always qualifies
+        lo = lo + last * step;
+        hi = lo + step < hi ? lo + step : hi;
+    }
+    return lo;
+}
+
 __device__ __forceinline__ int64_t read_pay(const void* p, int bytes, uint32_t i) {
     return bytes == 4 ? (int64_t)((const int32_t*)p)[i] : ((const int64_t*)p)[i];
 }
@@ -321,13 +340,6 @@ __device__ __forceinline__ uint32_t tile_copy_plan(const E* first, uint32_t len,
     body_lo = lo;
     body_hi = hi;
     return (hi - lo) * (uint32_t)sizeof(E);
-}
-
-template <typename E>
-__device__ __forceinline__ void tile_copy_edges(E* dst, const E* first, uint32_t len, uint32_t lead,
-                                                uint32_t body_lo, uint32_t body_hi) {
-    for (uint32_t e = 0; e < body_lo; ++e) dst[lead + e] = first[e];
-    for (uint32_t e = body_hi; e < len; ++e) dst[lead + e] = first[e];
 }
 
 template <typename E>

@@ -99,11 +99,6 @@ __device__ __forceinline__ long long agg_value(const AggSpec& s, int a, uint32_t
                            : __ldcs(static_cast<const long long*>(s.vals[a]) + row);
 }
 
-__device__ __forceinline__ uint32_t cas_key(uint32_t* p, uint32_t expect, uint32_t v) { return atomicCAS(p, expect, v); }
-__device__ __forceinline__ uint64_t cas_key(uint64_t* p, uint64_t expect, uint64_t v) {
-    return atomicCAS(reinterpret_cast<unsigned long long*>(p), (unsigned long long)expect, (unsigned long long)v);
-}
-
 // ------------------------------------------------------------------ hash variant
 
 template <typename KeyT>
@@ -621,22 +616,6 @@ __global__ void __launch_bounds__(1024)
     }
 }
 
-// Warp-collective: the partition of work item `item` (last p with prefix[p] <= item).
-__device__ __forceinline__ uint32_t find_item_part(const unsigned long long* __restrict__ prefix, uint32_t P,
-                                                   unsigned long long item) {
-    const unsigned lane = lane_id();
-    uint32_t lo = 0, hi = P;
-    while (hi - lo > 1) {
-        const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
-        const uint32_t piv = lo + lane * step;
-        const bool le = piv < hi && prefix[piv] <= item;
-        const unsigned m = __ballot_sync(0xffffffffu, le);
-        lo = lo + (31 - __clz(m)) * step;
-        hi = lo + step < hi ? lo + step : hi;
-    }
-    return lo;
-}
-
 // A persistent grid takes work items (a partition's chunk of rows) from a
 // global counter and aggregates each in a shared-memory table. A partition
 // that is one item writes its groups out directly; the items of a larger
@@ -663,7 +642,8 @@ __global__ void __launch_bounds__(kGbThreads, 2)
             unsigned long long it = 0;
             if (threadIdx.x == 0) it = atomicAdd(&ctrl->next_item, 1ull);
             it = __shfl_sync(0xffffffffu, it, 0);
-            const uint32_t p = it < nitems ? find_item_part(a.item_prefix, a.P, it) : 0u;
+            const uint32_t p =
+                it < nitems ? warp_last_le(a.P, it, [&](uint32_t i) { return a.item_prefix[i]; }) : 0u;
             if (threadIdx.x == 0) {
                 s_item = it;
                 s_part = p;

@@ -1,14 +1,15 @@
-// Key arrays of shared-memory hash tables (phj_sum.cu, groupby.cu).
+// Key arrays of hash tables in shared memory (phj_sum.cu, groupby.cu); cas_key
+// claims slots in global memory too.
 #pragma once
 
 #include "common.cuh"
 
 namespace eiger {
 
-__device__ __forceinline__ uint32_t cas_smem(uint32_t* p, uint32_t expect, uint32_t v) {
+__device__ __forceinline__ uint32_t cas_key(uint32_t* p, uint32_t expect, uint32_t v) {
     return atomicCAS(p, expect, v);
 }
-__device__ __forceinline__ uint64_t cas_smem(uint64_t* p, uint64_t expect, uint64_t v) {
+__device__ __forceinline__ uint64_t cas_key(uint64_t* p, uint64_t expect, uint64_t v) {
     return atomicCAS(reinterpret_cast<unsigned long long*>(p), (unsigned long long)expect, (unsigned long long)v);
 }
 
@@ -71,7 +72,7 @@ __device__ __forceinline__ uint32_t claim_slot(KeyT* keys, uint32_t slots, KeyT 
             --left;
             continue;
         }
-        const KeyT cur = cas_smem(keys + base + i, ~KeyT(0), k);
+        const KeyT cur = cas_key(keys + base + i, ~KeyT(0), k);
         fresh = cur == ~KeyT(0);
         if (fresh || cur == k) return base + i;
     }

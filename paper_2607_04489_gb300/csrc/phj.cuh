@@ -127,25 +127,6 @@ __device__ __forceinline__ void prefetch_rows_l2(const KeyT* key, const uint32_t
     }
 }
 
-// Warp-collective: the last i in [0, n) with value(i) <= x (value is
-// non-decreasing, value(0) <= x). Each step tests 32 evenly spaced pivots at
-// once, so 2^15 entries take three dependent loads.
-template <typename F>
-__device__ __forceinline__ uint32_t warp_last_le(uint32_t n, unsigned long long x, F value) {
-    const unsigned lane = lane_id();
-    uint32_t lo = 0, hi = n;
-    while (hi - lo > 1) {
-        const uint32_t step = (hi - lo + kWarp - 1) / kWarp;
-        const uint32_t piv = lo + lane * step;
-        const bool le = piv < hi && value(piv) <= x;
-        const unsigned m = __ballot_sync(0xffffffffu, le);
-        const uint32_t last = 31 - __clz(m);  // lane 0 always qualifies
-        lo = lo + last * step;
-        hi = lo + step < hi ? lo + step : hi;
-    }
-    return lo;
-}
-
 // Warp-collective: the partition of a work item (prefix[0] = 0).
 __device__ __forceinline__ uint32_t find_partition(const unsigned long long* __restrict__ prefix,
                                                    uint32_t P, unsigned long long item) {

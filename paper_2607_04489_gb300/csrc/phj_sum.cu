@@ -68,7 +68,7 @@ struct SumTable {
         bool again;
         if (k == kEmpty) {
             s = kSlots;
-            again = cas_smem(key + s, kEmpty, KeyT(0)) != kEmpty;
+            again = cas_key(key + s, kEmpty, KeyT(0)) != kEmpty;
         } else {
             bool fresh = false;
             s = claim_slot(key, tsize, k, home(k, tsize), fresh);
