@@ -152,7 +152,8 @@ eiger_status eiger_stats(const void* d_keys, int64_t n, eiger_dtype dtype, eiger
  *          build->estimate >= 0.9 nb, i.e. the keys are distinct; 4096 for
  *          distinct keys from 2^27 rows up), in one pass up to 8 bits, else in
  *          two passes with an odd count's extra bit in the second; narrow = 1
- *          when the build range spans < 2^32.
+ *          when the build range spans < 2^32. On dense distinct keys AUTO goes on
+ *          from this plan by the columns it has (see eiger_join).
  * Errors: INVALID_ARG.
  */
 eiger_status eiger_plan(const eiger_stats_t* build, const eiger_stats_t* probe, int64_t nb,
@@ -353,8 +354,8 @@ eiger_status eiger_groupby_workspace(int64_t n, eiger_dtype dtype, const eiger_a
  *          one pass up to 8 bits (10 below 2^25 rows), else two (knobs may set
  *          bits1/bits2).
  * If a table overflows (an estimate far too low, or caller knobs too small)
- * the plan is enlarged and the group-by re-run; plan_used->attempts counts the
- * runs. Groups are written in unspecified order: d_out_keys (dtype, nullable
+ * the plan is enlarged (4x the slots; two more bits and the largest partition
+ * tables) and the group-by re-run; plan_used->attempts counts the runs. Groups are written in unspecified order: d_out_keys (dtype, nullable
  * when capacity is 0) and aggs->out[a]; *out_groups receives the number of
  * groups. Capacity rules as eiger_join (EIGER_ERR_CAPACITY with the required
  * count). Synchronises `stream`.

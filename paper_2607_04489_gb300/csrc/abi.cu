@@ -536,12 +536,12 @@ bool dense_nphj(const JoinCall& c, const eiger_stats_t* bst, const eiger_plan_t&
 }
 
 // AUTO's radix bits where direct-addressed tables serve (see direct_tables):
-// a table of 2^kDirectBits slots (2^kDirectSumBits of the sum's larger ones)
-// holds several times the rows of a hash table,
-// so fewer partitions do, and no more than the rules' plan. At least 2^11, so
-// that the items of one partition each still fill the chip evenly. Pass 1 gets
-// the smaller half: its output runs, two arrays of 2^bits1 of them, lie in that
-// many pages (2^27 x 2^29, 7 + 8 bits: pass 1 2.6 ms; 8 + 8: 4.6 ms).
+// a table of 2^kDirectBits slots (2^kDirectSumBits of the sum's larger ones) holds
+// several times the rows of a hash table, so fewer partitions do, and no more than
+// the rules' plan. At least 2^11, so that the items of one partition each still
+// fill the chip evenly. Pass 1 gets the smaller half: its output runs, two arrays
+// of 2^bits1 of them, lie in that many pages (2^27 x 2^29, 7 + 8 bits: pass 1 2.6
+// ms; 8 + 8: 4.6 ms).
 // A carried sum takes repeats as they are, but distinct keys it must be that the
 // rules sized the partitions for; matches must hardly repeat (direct_tables).
 void dense_bits(eiger_plan_t* p, int dtype, int64_t nb, const eiger_stats_t* bst, bool sum) {
@@ -988,8 +988,13 @@ unsigned long long pow2_at_least(double x) {
 unsigned long long gb_max_slots(int64_t n) { return pow2_at_least(2.0 * (double)(n > 0 ? n : 1)); }
 
 // One pass while its digits leave the tiles runs of some length and its output
-// pages stay few: always up to 8 bits, up to 10 below 2^25 rows (5M rows, 10
-// bits: one pass; 2^28 rows, 10 bits: 8.7 ms against 3.4 ms for 5 + 5), else two.
+// pages stay few: always up to 8 bits, up to 10 below 2^25 rows, else two.
+// Group-bys of SUM and MAX, ms in one pass / in two, int32 keys and int64 ones:
+// 9 bits, 2^24 rows 0.46 / 0.52 and 0.59 / 0.65, 2^25 0.89 / 0.94 and 1.12 / 1.14,
+// 2^26 1.74 / 1.54 and 2.06 / 2.00, 2^27 3.52 / 2.62 and 3.97 / 3.50; 10 bits, 2^22
+// 0.30 / 0.33 and 0.33 / 0.34, 2^24 0.57 / 0.54 and 0.76 / 0.66, 2^25 0.98 / 0.83 and
+// 1.37 / 1.06. One line for both: at 10 bits two passes are ahead from 2^23 to
+// 2^24 rows on, at 9 from 2^26.
 void gb_split_bits(int B, int64_t n, int32_t* b1, int32_t* b2) {
     if (B <= 8 || (B <= 10 && n < (1ll << 25))) {
         *b1 = B;

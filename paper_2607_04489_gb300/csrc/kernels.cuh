@@ -261,7 +261,7 @@ struct GbScratch {
 uint32_t gb_hash_slots(double groups, const GbAggs& aggs, bool key32);
 // Slots of a partition's table for an estimated number of groups per partition
 // (load about 1/4; 2^28 rows, 2^22 groups, load 4/9 -> 2/7: 2.06 -> 1.43 ms),
-// capped.
+// capped (a retry takes the cap).
 uint32_t gb_part_slots(double groups);
 GbScratch gb_layout(Carve& c, int64_t n, const GbPlanDev& plan, const int* col_bytes, int ncols);
 cudaError_t gb_run(const GbArgs& g, const GbPlanDev& plan, const GbScratch& s, const GbAggs& aggs, void* out_keys,

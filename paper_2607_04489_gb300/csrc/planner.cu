@@ -26,7 +26,8 @@
 //    (2^24: 1.81 against 1.72 ms);
 //  - except under heavy probe skew: when a probe sample of 2^20 rows holds
 //    fewer than kSkewHeavy distinct keys per row (Zipf theta ~1.5 gives
-//    0.014), or fewer than kSkewModerate with the NPHJ table within 4x the
+//    0.014), or fewer than kSkewModerate with the NPHJ's hash table (also
+//    where dense keys take a smaller, direct-addressed one) within 4x the
 //    L2 cache (theta ~1 gives 0.22-0.45), and the probe side is at least
 //    twice the build side, 32-bit keys go to the NPHJ: hot keys keep their
 //    slots in cache, while the partitioned join funnels them through one
