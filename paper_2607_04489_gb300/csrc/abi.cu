@@ -496,10 +496,10 @@ eiger_status resolve_materialize(const JoinCall& c, const eiger_stats_t* bst, ei
 // Whether the partitioned join of this plan addresses its tables by the key
 // bits below the partition's: 32-bit keys, few enough slots, and at least an
 // eighth of them filled. Matches (pairs, columns) also need build keys that
-// hardly repeat, since the chains of a table hold few repeats and an item with
-// more goes back to hash tables (2^25 x 2^27 rows with 1 % repeated, pairs and two
+// hardly repeat, since the chains of a table hold few repeats and the probe rows
+// of an item with more are read again for every 4096 of its build rows (2^25 x 2^27 rows with 1 % repeated, pairs and two
 // 4-byte columns a side: 2.4 and 5.1 ms, 17.4 and 39.2 when any repeat sent its
-// item there; 2.2 and 3.9 without repeats; 8 % repeated, hash tables for all: 3.1
+// item to hash tables; 2.2 and 3.9 without repeats; 8 % repeated, hash tables for all: 3.1
 // and 7.1); the carried sum takes repeated keys as they are.
 bool direct_tables(const PlanDev& d, int64_t nb, double estimate, bool carried_sum) {
     if (!d.key32 || (d.variant != EIGER_PHJ1 && d.variant != EIGER_PHJ2)) return false;

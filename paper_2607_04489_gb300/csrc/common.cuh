@@ -147,7 +147,7 @@ struct Ctrl {
     unsigned long long next_item;  // PHJ work-item dispenser
     unsigned long long nitems;     // PHJ work items
     unsigned long long next_redo;  // PHJ: dispenser of the pieces, and number of the items and pieces,
-    unsigned long long nredo;      // a direct-addressed launch left to hash tables (phj.cuh)
+    unsigned long long nredo;      // of direct-addressed items with many repeats (phj.cuh)
     unsigned int err;              // kErr* flags
     unsigned int ntiles2[2];       // pass-2 tile count per side (build, probe)
     unsigned int kept[2];          // rows kept by the range test per side

@@ -162,8 +162,8 @@ struct PhjScratch {
     void* rec;
     uint32_t* ovf[2];
     ChunkFix fix;
-    unsigned long long* redo;  // items that direct-addressed launches leave to hash tables
-    uint32_t* chained;         // items that the first of them leaves to one with chains
+    unsigned long long* redo;  // items whose build rows a direct-addressed launch takes in pieces
+    uint32_t* chained;         // items that the first such launch leaves to one with chains
 };
 
 PhjScratch phj_layout(Carve& c, int64_t nb, int64_t np, const PlanDev& plan);

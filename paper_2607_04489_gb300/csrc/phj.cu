@@ -14,7 +14,7 @@
 // shared-memory CAS, then streams the probe chunk, walking linear-probe chains;
 // or, where the build keys are dense and distinct, fills a direct-addressed
 // table (phj.cuh) that takes the whole build partition and reads one word per
-// probe row (further launches take the partitions with repeated keys, see JoinKind).
+// probe row (later launches take the partitions with repeated keys, see JoinKind).
 // Index pairs leave through per-warp output runs (chunks.cuh), so the probe
 // loop has no CTA barrier; columns through one CTA reservation per round, column
 // by column; the matches of repeated build keys through the CTA stage
@@ -256,21 +256,51 @@ constexpr int kJoinWarps = kJoinThreads / kWarp;
 // more than the chains hold is left to the last launch. Chains in the first
 // launch, for all items, cost unique keys their registers (2^25 x 2^27 rows:
 // pairs 2163 -> 2254 us, two columns a side 3908 -> 4196).
-// kRedo: those, through hash tables, each piece of at most kBuildCap build rows an
-// item of its own, so that one heavily repeated key (a default value) spreads
-// over the chip.
-enum JoinKind { kHash, kDirect, kChained, kRedo };
+// kPieces: those, each piece of at most kPieceRows build rows an item of its own
+// with chains for all of them, so that one heavily repeated key (a default value)
+// spreads over the chip and no other key meets its rows (2^25 x 2^27 rows, one key
+// on 2 % of the build rows, pairs: 180 ms with hash tables, whose equal keys half
+// of the probes walked, 2.2 ms; two columns a side 127 and 4.3).
+enum JoinKind { kHash, kDirect, kChained, kPieces };
 
 // Bytes of a direct-addressed table, a multiple of 16.
 __host__ __device__ constexpr size_t direct_table_bytes(int sbits) { return ((size_t)4 << sbits) / 16 * 16 + 16; }
+
+// Warp-collective: the rest of the chains at[j] of probe rows id[j], with their
+// columns. One reservation for the warp, then each lane walks its chains.
+template <int N, uint32_t CHAINS>
+__device__ __forceinline__ void emit_chains(const uint32_t (&at)[N], const uint32_t (&id)[N], const ChainEntry* chain,
+                                            const JoinOut& out, unsigned long long* cursor) {
+    auto next = [&](uint32_t v) { return kChainTop - v < CHAINS ? chain[kChainTop - v].next : kHole; };
+    uint32_t count = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        for (uint32_t v = at[j]; v != kHole; v = next(v)) ++count;
+    __syncwarp();
+    uint32_t x = count;
+#pragma unroll
+    for (int o = 1; o < kWarp; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if ((int)lane_id() >= o) x += y;
+    }
+    unsigned long long base = 0;
+    if (lane_id() == kWarp - 1 && x) base = atomicAdd(cursor, (unsigned long long)x);
+    unsigned long long pos = __shfl_sync(0xffffffffu, base, kWarp - 1) + x - count;
+#pragma unroll
+    for (int j = 0; j < N; ++j)
+        for (uint32_t v = at[j]; v != kHole; v = next(v))
+            write_match(out, pos++, kChainTop - v < CHAINS ? chain[kChainTop - v].row : v, id[j]);
+    __syncwarp();
+}
 
 template <typename KeyT, int MODE, bool POS, int KIND>
 __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
     phj_join_kernel(JoinIn<KeyT> a, const __grid_constant__ JoinOut out, PairSink sink, Ctrl* ctrl) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool PAIRS = MODE == kPairs, AGG = MODE == kSum;
-    constexpr bool kSlots = KIND == kDirect || KIND == kChained;  // direct-addressed
-    constexpr bool kLater = KIND == kChained || KIND == kRedo;    // goes on with an earlier launch's output runs
+    constexpr bool kSlots = KIND != kHash;                // direct-addressed
+    constexpr bool kLater = kSlots && KIND != kDirect;    // goes on with an earlier launch's output runs
+    constexpr uint32_t kChains = KIND == kPieces ? kPieceRows : kChainMax;
     // the stage follows the table in dynamic shared memory; index pairs and
     // aggregates use none, so none is allocated for them (shared memory left
     // unreserved serves as L1 cache, which the payload gathers of the
@@ -288,7 +318,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
     uint32_t* dtab = reinterpret_cast<uint32_t*>(smem);
     ChainEntry* chain = reinterpret_cast<ChainEntry*>(smem + direct_table_bytes(a.sbits));
     // (without items left to it, a later launch leaves the warp records as they are)
-    const unsigned long long left = KIND == kRedo ? ctrl->nredo : KIND == kChained ? ctrl->nchained : 0ull;
+    const unsigned long long left = KIND == kPieces ? ctrl->nredo : KIND == kChained ? ctrl->nchained : 0ull;
     if (kLater && left == 0) return;
     if (MODE == kColumns && !kSlots && threadIdx.x == 0) st.count = 0;
     AggState agg{0ull, 0ull};
@@ -297,10 +327,10 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
     wc.init(sink.run);
     if (PAIRS && kLater) warp_chunk_resume(wc, sink, gwarp);
     uint32_t flushes = 0;
-    const unsigned long long nitems = KIND == kRedo      ? left & ((1ull << kRedoPieceBits) - 1)
+    const unsigned long long nitems = KIND == kPieces      ? left & ((1ull << kRedoPieceBits) - 1)
                                       : KIND == kChained ? left
                                                          : ctrl->nitems;
-    unsigned long long* const next = KIND == kRedo      ? &ctrl->next_redo
+    unsigned long long* const next = KIND == kPieces      ? &ctrl->next_redo
                                      : KIND == kChained ? &ctrl->next_chained
                                                         : &ctrl->next_item;
 
@@ -311,7 +341,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         unsigned long long item = claim;
         uint32_t piece = 0, p = 0;
         if (claim < nitems) {
-            if constexpr (KIND == kRedo) {
+            if constexpr (KIND == kPieces) {
                 const uint32_t e = warp_last_le((uint32_t)(left >> kRedoPieceBits), claim,
                                                 [&](uint32_t i) { return a.redo[i] >> kRedoItemBits; });
                 piece = (uint32_t)(claim - (a.redo[e] >> kRedoItemBits));
@@ -324,7 +354,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
             s_next_item = claim;
             s_next_part = p;
             if (kLater) s_item = item;
-            if (KIND == kRedo) s_piece = piece;
+            if (KIND == kPieces) s_piece = piece;
         }
         return p;
     };
@@ -344,8 +374,8 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
         if (threadIdx.x == 0) claim = atomicAdd(next, 1ull);
 
         ItemRows ir = item_rows(a, item, p);
-        if constexpr (KIND == kRedo) {  // the piece's share of the build rows
-            const uint32_t pieces = chunks_of(ir.bn, kBuildCap);
+        if constexpr (KIND == kPieces) {  // the piece's share of the build rows
+            const uint32_t pieces = chunks_of(ir.bn, kPieceRows);
             const uint32_t lo = (uint32_t)((unsigned long long)s_piece * ir.bn / pieces);
             const uint32_t hi = (uint32_t)((unsigned long long)(s_piece + 1) * ir.bn / pieces);
             ir.bs0 += lo;
@@ -417,7 +447,7 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
             if (!over)
                 for (uint32_t i = threadIdx.x; i < slots / 4 + 1; i += kJoinThreads)
                     d4[i] = make_uint4(kHole, kHole, kHole, kHole);
-            if (KIND == kChained && threadIdx.x == 0) s_chained = 0;
+            if (kLater && threadIdx.x == 0) s_chained = 0;
             __syncthreads();
             int dup = 0;
             // Build rows a round ahead (a partition's build takes several);
@@ -438,24 +468,24 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
                             dup |= old != kHole;
                         } else if (old != kHole) {  // a repeated key: its earlier row leaves the slot
                             const uint32_t e = atomicAdd(&s_chained, 1u);
-                            if (e < kChainMax) chain[e] = ChainEntry{old, s};
+                            if (e < kChains) chain[e] = ChainEntry{old, s};
                         }
                     }
                 if (more) nxt = cur;
             }
             const bool repeats = __syncthreads_or(dup) != 0;
-            const uint32_t chained = KIND == kChained ? s_chained : 0u;
+            const uint32_t chained = kLater ? s_chained : 0u;
             next_item();
-            if (over || chained > kChainMax) {
+            if (over || chained > kChains) {  // (never a piece)
                 if (threadIdx.x == 0) {
                     const unsigned long long at =
-                        atomicAdd(&ctrl->nredo, (1ull << kRedoPieceBits) | chunks_of(bn, kBuildCap));
+                        atomicAdd(&ctrl->nredo, (1ull << kRedoPieceBits) | chunks_of(bn, kPieceRows));
                     a.redo[at >> kRedoPieceBits] = redo_entry(at & ((1ull << kRedoPieceBits) - 1), item);
                 }
             } else if (repeats) {
                 if (threadIdx.x == 0) a.chained[atomicAdd(&ctrl->nchained, 1u)] = (uint32_t)item;
             } else {
-                if constexpr (KIND == kChained) {  // hang the displaced rows before the rows that stayed
+                if constexpr (kLater) {  // hang the displaced rows before the rows that stayed
                     for (uint32_t e = threadIdx.x; e < chained; e += kJoinThreads)
                         chain[e].next = atomicExch(dtab + chain[e].next, kChainTop - e);
                     __syncthreads();
@@ -470,23 +500,31 @@ __global__ void __launch_bounds__(kJoinThreads, (Rows<KeyT, MODE>::kMinBlocks))
                     if constexpr (KIND == kDirect) {
                         emit_round(at);
                     } else {  // every row's first match, then their second ones, and so on
-                        bool more;
-                        do {
-                            more = false;
+                        for (int level = 0;; ++level) {
+                            bool more = false;
                             uint32_t brow[kN];
 #pragma unroll
                             for (int j = 0; j < kN; ++j) {
                                 brow[j] = at[j];
                                 const uint32_t e = kChainTop - at[j];
                                 at[j] = kHole;
-                                if (e < kChainMax) {
+                                if (e < kChains) {
                                     brow[j] = chain[e].row;
                                     at[j] = chain[e].next;
                                     more = true;
                                 }
                             }
                             emit_round(brow);
-                        } while (MODE == kColumns ? __syncthreads_or(more) : __any_sync(0xffffffffu, more));
+                            if constexpr (MODE == kColumns) {
+                                if (!__syncthreads_or(more)) break;
+                                if (level == 1) {  // third matches and on are few, or all of a few rows
+                                    emit_chains<kN, kChains>(at, cur.id, chain, out, &ctrl->cursor);
+                                    break;
+                                }
+                            } else {
+                                if (!__any_sync(0xffffffffu, more)) break;
+                            }
+                        }
                     }
                 });
             }
@@ -629,10 +667,12 @@ struct JoinLaunch {
     template <int MODE, bool POS, int KIND>
     cudaError_t run() {
         auto kern = phj_join_kernel<KeyT, MODE, POS, KIND>;
-        const size_t smem = KIND == kDirect    ? direct_table_bytes(a.sbits)
-                            : KIND == kChained ? direct_table_bytes(a.sbits) + kChainMax * sizeof(ChainEntry)
-                                               : (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
-                                                     (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0);
+        const size_t smem = KIND == kHash ? (size_t)kTableMax * SmemTable<KeyT>::kSlotBytes +
+                                                (MODE == kColumns ? sizeof(Stage<kJoinStage>) : 0)
+                                          : direct_table_bytes(a.sbits) +
+                                                (KIND == kChained  ? kChainMax
+                                                 : KIND == kPieces ? kPieceRows
+                                                                   : 0) * sizeof(ChainEntry);
         cudaError_t e = allow_smem(kern);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
@@ -641,7 +681,7 @@ struct JoinLaunch {
             per_sm = 1;
         grid = std::min(grid, (uint32_t)(di.sms * per_sm));
         constexpr bool kFirst = KIND == kHash || KIND == kDirect;
-        ProfScope ps(kFirst ? "phj_join" : KIND == kChained ? "phj_join.chained" : "phj_join.redo", kFirst ? bytes : 0.0,
+        ProfScope ps(kFirst ? "phj_join" : KIND == kChained ? "phj_join.chained" : "phj_join.pieces", kFirst ? bytes : 0.0,
                      stream, kFirst ? match_bytes(out) : 0.0);
         kern<<<grid, kJoinThreads, smem, stream>>>(a, out, sink, ctrl);
         return cudaGetLastError();
@@ -700,7 +740,7 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
             e = l.template run_as<kDirect>(pairs, plan.gftr);
             const uint32_t warps = l.warps();
             if (e == cudaSuccess) e = l.template run_as<kChained>(pairs, plan.gftr);
-            if (e == cudaSuccess) e = l.template run_as<kRedo>(pairs, plan.gftr);
+            if (e == cudaSuccess) e = l.template run_as<kPieces>(pairs, plan.gftr);
             if (e != cudaSuccess || !pairs) return e;
             return chunk_fix_run(sink, warps, s.fix, &ctrl->err, di, stream);
         }

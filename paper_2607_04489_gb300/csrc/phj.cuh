@@ -21,13 +21,15 @@ constexpr uint32_t kProbeChunk = EIGER_PROBE_CHUNK;  // probe rows per work item
 // (kDirectBits) and the build rows fill at least an eighth of them.
 //
 // A further row of a key that is already in the table goes to a chain entry of
-// the item (in a launch for such items): the slot then holds the entry's code instead of a row, the entry its
-// row and what the slot held before (a row or another code). Codes are the
-// kChainMax words below kHole, so rows stay below them (kDirectMaxRows).
+// the item (in a launch for such items): the slot then holds the entry's code
+// instead of a row, the entry its row and what the slot held before (a row or
+// another code). Codes are the kPieceRows words below kHole, so rows stay below
+// them (kDirectMaxRows).
 constexpr int kDirectBits = 14;     // 4-byte slots: 64 KB, and 8 KB of chains: three CTAs per SM
 constexpr uint32_t kChainMax = 1024;              // further rows of repeated keys an item holds
+constexpr uint32_t kPieceRows = 4096;             // build rows of a piece of an item with more: all may be chained
 constexpr uint32_t kChainTop = 0xFFFFFFFEu;       // code of entry e: kChainTop - e
-constexpr int64_t kDirectMaxRows = (int64_t)kChainTop - (kChainMax - 1);  // build rows, for matches
+constexpr int64_t kDirectMaxRows = (int64_t)kChainTop - (kPieceRows - 1);  // build rows, for matches
 struct ChainEntry {
     uint32_t row, next;
 };
@@ -55,12 +57,12 @@ struct JoinIn {
     uint32_t P;
     uint32_t bcap, pcap;  // build and probe rows per work item, at most
     int pbits, sbits;     // partition bits; direct-addressed tables: bits of the slot below them
-    unsigned long long* redo;  // direct-addressed tables: the items left to hash tables (redo_entry)
-    uint32_t* chained;         // and, before those, to tables with chains
+    uint32_t* chained;         // direct-addressed tables: the items left to tables with chains
+    unsigned long long* redo;  // and those with too many repeats for these, left to pieces (redo_entry)
 };
 
-// Items that direct-addressed launches leave to hash tables, cut into pieces of
-// at most kBuildCap build rows. Ctrl::nredo counts the items (upper 24 bits) and
+// Items with more repeats than their chains hold, cut into pieces of at most
+// kPieceRows build rows. Ctrl::nredo counts the items (upper 24 bits) and
 // their pieces (lower 40) in one atomic, so the list is in the order of its
 // items' first pieces; an entry holds an item's first piece and the item.
 constexpr int kRedoItemBits = 24, kRedoPieceBits = 40;

@@ -1,7 +1,7 @@
 """Repeated build keys in the partitioned join's direct-addressed tables.
 
 An item whose keys repeat goes to a launch whose tables chain up to 1024 further
-rows; one with more goes to hash tables in pieces of at most 4608 build rows. The
+rows; one with more goes to another in pieces of at most 4096 build rows. The
 cases lie on each side of both limits, against the oracle in every output mode,
 and the time of a column with a few repeats is held against the unique column's.
 """
@@ -119,3 +119,18 @@ def test_few_repeats_cost_little(eiger, cols):
     rep = bk.clone()
     rep[: nb // 100] = rep[nb // 2: nb // 2 + nb // 100]
     assert _join_ms(eiger, rep, pk, cols) < 2.5 * _join_ms(eiger, bk, pk, cols)
+
+
+@pytest.mark.parametrize("cols", [False, True])
+def test_default_key_costs_little(eiger, cols):
+    """One key on 2 % of the build rows that no probe row asks for: the join's
+    kernels take no more than 4 times what they take on unique keys (its rows on one
+    CTA, or in hash tables whose equal keys the probes walk: tens)."""
+    nb, np_ = 1 << 23, 1 << 25
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    bk = torch.randperm(nb, generator=gen, device="cuda").to(torch.int32)
+    pk = torch.randint(0, nb, (np_,), generator=gen, device="cuda").to(torch.int32)
+    pk += (pk == 777).to(torch.int32)
+    rep = bk.clone()
+    rep[: nb // 50] = 777
+    assert _join_ms(eiger, rep, pk, cols) < 4 * _join_ms(eiger, bk, pk, cols)
