@@ -488,7 +488,8 @@ eiger_status eiger_class_plan(int32_t cls, eiger_plan_t* out);
  * Makes EIGER_AUTO (with knobs == NULL) choose the plan with the network:
  * d_params (device, caller-owned, kept until the next call) and per-feature
  * normalisation x' = (x - mean) / scale (host arrays of 12, copied). The join
- * then also profiles a probe sample. d_params == NULL restores the rules.
+ * then also profiles a probe sample. The network's class replaces the rules' plan,
+ * the adjustments for dense keys included (see eiger_join). d_params == NULL restores the rules.
  * Process-wide setting. Errors: INVALID_ARG.
  */
 eiger_status eiger_selector_set(const float* d_params, const float* h_feature_mean,
