@@ -665,6 +665,7 @@ eiger_status run_join(const JoinCall& c) {
     PlanDev pd = to_dev(pub, c.dtype, adaptive ? &bst : nullptr);
     set_carry(pd, c.out, pub.materialize);
     pd.direct = adaptive && direct_tables(pd, c.nb, bst.estimate, pd.gftr && c.out.aggregate);
+    pd.distinct = adaptive ? std::min(1.0, bst.estimate / (double)c.nb) : 1.0;
     NphjScratch ns{};
     PhjScratch ps{};
     SmjScratch ms{};

@@ -75,6 +75,7 @@ struct PlanDev {
     int key32;        // keys carried as 32-bit values (int32, or int64 narrowed)
     int kbits;        // hash partitioning: bits of the key mix (key32: of the build span; else 64)
     int direct;       // partitioned join: direct-addressed tables (phj.cuh)
+    double distinct;  // partitioned join: estimated share of distinct build keys, at most 1
     float load_factor;
     int dtype;        // 0 int32, 1 int64
     KeyRange range;   // build range (probe range test) and encoding offset

@@ -717,7 +717,7 @@ cudaError_t launch_join(const PhjScratch& s, const PlanDev& plan, const JoinOut&
     a.pbits = plan.bits1 + (passes == 2 ? plan.bits2 : 0);
     a.sbits = plan.kbits - a.pbits > 1 ? plan.kbits - a.pbits : 1;
     // the sum with carried payloads has its own kernel (phj_sum.cu)
-    if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, plan.direct, out, ctrl, di, stream, nb, np);
+    if (out.aggregate && plan.gftr) return phj_sum_launch<KeyT>(a, plan.direct, plan.distinct, out, ctrl, di, stream, nb, np);
     PairSink sink{};
     sink.run = plan.direct ? kDirectRun : kHashRun;
     if (pairs) {

@@ -136,9 +136,10 @@ __device__ __forceinline__ uint32_t find_partition(const unsigned long long* __r
 }
 
 // The fused sum over positions (phj_sum.cu): out.b.src[0] and out.p.src[0] are
-// the carried payload columns, indexed like the keys of `a`.
+// the carried payload columns, indexed like the keys of `a`; distinct: the
+// estimated share of the build rows that differ in their key.
 template <typename KeyT>
-cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
-                           cudaStream_t stream, int64_t nb, int64_t np);
+cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, double distinct, const JoinOut& out, Ctrl* ctrl,
+                           const DevInfo& di, cudaStream_t stream, int64_t nb, int64_t np);
 
 }  // namespace eiger

@@ -7,7 +7,7 @@
 // order of the additions does not matter.
 //
 // The rows arrive through the CTA's stream (stream.cuh). Hash tables, two CTAs
-// per SM, are bound by shared memory: about 29 wavefronts per 32 probe rows (the
+// per SM (one over full partitions, see big_tables), are bound by shared memory: about 29 wavefronts per 32 probe rows (the
 // key group's 16-byte loads at random groups, the sum's 8-byte loads at random
 // slots) keep its pipe 87 % busy. Direct-addressed tables need about 11 and run
 // near the row streams' rate (5.3 TB/s with 2^12 slots). Measured on GB300,
@@ -17,6 +17,9 @@
 // 3.92 ms streamed with key groups (3.46 ms on mixed keys), 1.71 ms direct with
 // 2^12 slots, 1.91 ms with 2^13 (whose partitions take 1.9 ms less to make);
 // 8M x 30M 64-bit keys of six rows each: 2.79 -> 0.21 ms.
+#include <algorithm>
+#include <cmath>
+
 #include "emit.cuh"
 #include "kernels.cuh"
 #include "phj.cuh"
@@ -31,10 +34,11 @@ constexpr int kStages = 2;
 // Slots of {key, sum as two 32-bit halves, rows beyond the first}. The all-ones
 // key is the empty pattern; that key itself lives in the extra slot kSlots,
 // whose key word turns 0 when it is taken.
-template <typename KeyT>
+template <typename KeyT, bool BIG>
 struct SumTable {
-    // More than a full build chunk, and two CTAs' tables and rings fit an SM.
-    static constexpr uint32_t kSlots = sizeof(KeyT) == 4 ? 4864 : 4640;
+    // More than a full build chunk, and two CTAs' tables and rings fit an SM; or,
+    // BIG, twice that for one CTA per SM (see big_tables).
+    static constexpr uint32_t kSlots = (sizeof(KeyT) == 4 ? 4864 : 4640) * (BIG ? 2 : 1);
     static_assert(kSlots > kBuildCap && kSlots % 4 == 0, "a full build chunk leaves empty slots");
     static constexpr uint32_t kAll = kSlots + 4;  // arrays stay 16-byte aligned
     static constexpr size_t kBytes = kAll * (8 + sizeof(KeyT) + 4);
@@ -135,6 +139,8 @@ struct SumStream : Stream<2, kStages, 4, DIRECT ? 2 * CONS : 4096 / sizeof(KeyT)
 
 // CONS consumer threads (plus the stream's two warps): 512, two CTAs per SM, or
 // 960 over a table that only one CTA per SM has room for.
+template <int CONS>
+constexpr bool kBig = CONS > 512;
 template <typename KeyT, typename PayT, bool DIRECT, int CONS>
 __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
     phj_sum_kernel(JoinIn<KeyT> a, const PayT* __restrict__ bpay, const PayT* __restrict__ ppay, Ctrl* ctrl) {
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
     S st;
     st.w[0] = sizeof(KeyT);
     st.w[1] = sizeof(PayT);
-    st.setup(&s_stream, smem + (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT>::kBytes), CONS / kWarp);
+    st.setup(&s_stream, smem + (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT, kBig<CONS>>::kBytes), CONS / kWarp);
     constexpr uint32_t kStageRows = S::kRows;
     typename S::ItemPos q;
     const int warp = threadIdx.x / kWarp;
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
         return;
     }
 
-    SumTable<KeyT> tab;
+    SumTable<KeyT, kBig<CONS>> tab;
     SumDirect dir;
     if constexpr (DIRECT)
         dir.bind(smem, a.pbits, a.sbits);
@@ -235,7 +241,7 @@ __global__ void __launch_bounds__(CONS + kStreamWarps* kWarp, 1024 / CONS)
         } else {
             uint32_t tsize = (3 * it.bn + 3) & ~3u;  // load 1/3 while that fits
             if (tsize < 64) tsize = 64;
-            if (tsize > SumTable<KeyT>::kSlots) tsize = SumTable<KeyT>::kSlots;
+            if (tsize > SumTable<KeyT, kBig<CONS>>::kSlots) tsize = SumTable<KeyT, kBig<CONS>>::kSlots;
             tab.template clear<CONS>(tsize);
             consumers_sync<CONS>();
             int dup = 0;
@@ -269,7 +275,7 @@ template <typename KeyT, typename PayT, bool DIRECT, int CONS>
 cudaError_t launch_sum(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, const DevInfo& di, cudaStream_t stream,
                        int64_t nb, int64_t np) {
     auto kern = phj_sum_kernel<KeyT, PayT, DIRECT, CONS>;
-    const size_t smem = (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT>::kBytes) + SumStream<KeyT, PayT, DIRECT, CONS>::kBytes;
+    const size_t smem = (DIRECT ? SumDirect::bytes(a.sbits) : SumTable<KeyT, kBig<CONS>>::kBytes) + SumStream<KeyT, PayT, DIRECT, CONS>::kBytes;
     cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     constexpr int kThreads = CONS + kStreamWarps * kWarp;
@@ -283,29 +289,45 @@ cudaError_t launch_sum(const JoinIn<KeyT>& a, const JoinOut& out, Ctrl* ctrl, co
     return cudaGetLastError();
 }
 
+// Whether hash tables want the larger form: where the distinct keys of an ordinary
+// work item fill more than about two thirds of the smaller one's slots, whose
+// searches then grow long. 2^20 to 2^22 distinct keys in 1024 partitions, four probe
+// rows a key, int64 payloads, us in the smaller / larger form: 32-bit keys, 2816
+// rows a partition 119 / 135, 3328 162 / 164, 3584 197 / 172, 4096 379 / 203, 4500
+// 1024 / 236, 8192 (two items) 1809 / 682; 64-bit ones 2816 170 / 180, 3072 223 / 195,
+// 4096 1034 / 270, 4500 6058 / 326, 8192 5729 / 944. The items of a partition hold
+// some rows of most of its repeated keys.
+template <typename KeyT>
+bool big_tables(const JoinIn<KeyT>& a, int64_t nb, double distinct) {
+    const double rows = (double)nb / a.P, items = std::max(1.0, std::ceil(rows / kBuildCap));
+    const double keys = distinct * rows * (1.0 - std::pow(1.0 - 1.0 / items, 1.0 / std::max(distinct, 1e-9)));
+    return keys > (sizeof(KeyT) == 4 ? 3300.0 : 2900.0);
+}
+
 template <typename KeyT, typename PayT>
-cudaError_t launch_sum_for(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
+cudaError_t launch_sum_for(const JoinIn<KeyT>& a, int direct, double distinct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
                            cudaStream_t stream, int64_t nb, int64_t np) {
     if constexpr (sizeof(KeyT) == 4) {
         if (direct)
             return a.sbits <= 12 ? launch_sum<KeyT, PayT, true, 512>(a, out, ctrl, di, stream, nb, np)
                                  : launch_sum<KeyT, PayT, true, 960>(a, out, ctrl, di, stream, nb, np);
     }
-    return launch_sum<KeyT, PayT, false, 512>(a, out, ctrl, di, stream, nb, np);
+    return big_tables(a, nb, distinct) ? launch_sum<KeyT, PayT, false, 960>(a, out, ctrl, di, stream, nb, np)
+                                       : launch_sum<KeyT, PayT, false, 512>(a, out, ctrl, di, stream, nb, np);
 }
 
 }  // namespace
 
 template <typename KeyT>
-cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, const JoinOut& out, Ctrl* ctrl, const DevInfo& di,
-                           cudaStream_t stream, int64_t nb, int64_t np) {
-    return out.b.bytes[0] == 4 ? launch_sum_for<KeyT, int32_t>(a, direct, out, ctrl, di, stream, nb, np)
-                               : launch_sum_for<KeyT, int64_t>(a, direct, out, ctrl, di, stream, nb, np);
+cudaError_t phj_sum_launch(const JoinIn<KeyT>& a, int direct, double distinct, const JoinOut& out, Ctrl* ctrl,
+                           const DevInfo& di, cudaStream_t stream, int64_t nb, int64_t np) {
+    return out.b.bytes[0] == 4 ? launch_sum_for<KeyT, int32_t>(a, direct, distinct, out, ctrl, di, stream, nb, np)
+                               : launch_sum_for<KeyT, int64_t>(a, direct, distinct, out, ctrl, di, stream, nb, np);
 }
 
-template cudaError_t phj_sum_launch<uint32_t>(const JoinIn<uint32_t>&, int, const JoinOut&, Ctrl*, const DevInfo&,
-                                              cudaStream_t, int64_t, int64_t);
-template cudaError_t phj_sum_launch<uint64_t>(const JoinIn<uint64_t>&, int, const JoinOut&, Ctrl*, const DevInfo&,
-                                              cudaStream_t, int64_t, int64_t);
+template cudaError_t phj_sum_launch<uint32_t>(const JoinIn<uint32_t>&, int, double, const JoinOut&, Ctrl*,
+                                              const DevInfo&, cudaStream_t, int64_t, int64_t);
+template cudaError_t phj_sum_launch<uint64_t>(const JoinIn<uint64_t>&, int, double, const JoinOut&, Ctrl*,
+                                              const DevInfo&, cudaStream_t, int64_t, int64_t);
 
 }  // namespace eiger
