@@ -346,8 +346,9 @@ eiger_status eiger_groupby_workspace(int64_t n, eiger_dtype dtype, const eiger_a
  * Profiles the keys (min/max, HyperLogLog++; Sec. 4.1), narrows them to
  * uint32 offsets when their span allows (Sec. 4.3), then runs:
  *   EIGER_GB_AUTO: HASH when a table of the estimated groups fits a CTA's
- *          shared memory, or below 2^24 rows when a table of 2.5x the estimate
- *          fits in half of the L2 cache; else PARTITION;
+ *          shared memory, or below 2^24 rows (without aggregates: at any size)
+ *          when a table of 2.5x the estimate fits in half of the L2 cache; else
+ *          PARTITION;
  *   EIGER_GB_HASH: slots = the power of two >= 2.5x the estimate (knobs may
  *          set table_slots);
  *   EIGER_GB_PARTITION: 2^B partitions with B = ceil(log2(estimate / 1024)),

@@ -1130,15 +1130,20 @@ eiger_status eiger_groupby(eiger_dtype dtype, const void* d_keys, int64_t n, con
     int v = variant;
     if (v == EIGER_GB_AUTO) {
         // HASH while its CTA tables fit shared memory. Beyond that its global
-        // table must fit half of L2, and is only the better one for fewer than
-        // kGbPartRows rows: atomics on L2 lines cost more per row than a pass
-        // over the rows, above all on hot groups, but take three launches
-        // instead of ten (int32, 25000 groups, SUM and MAX, ms HASH /
-        // PARTITION: 2M rows 0.17 / 0.22, 20M 0.59 / 0.46, 50M 1.41 / 0.79;
-        // 100M rows over 100000 skewed groups 5.6 / 1.5).
+        // table must fit half of L2, and with aggregates is only the better one
+        // for fewer than kGbPartRows rows: atomics on L2 lines cost more per row
+        // than a pass over the rows, above all on hot groups, but take three
+        // launches instead of ten (int32, 25000 groups, SUM and MAX, ms HASH /
+        // PARTITION: 2M rows 0.17 / 0.22, 20M 0.59 / 0.46, 50M 1.41 / 0.79; 100M rows
+        // over 100000 skewed groups 5.6 / 1.5). Keys alone are read, hardly ever
+        // written: HASH at any size (2^25 rows, 300000 groups, int32 0.38 / 0.62 and
+        // 0.32 / 0.60 under Zipf 1, int64 0.44 / 0.84). The line is drawn for skew: over
+        // even groups a single aggregate of 64-bit keys would do better by HASH (2^26
+        // rows, 300000 groups, SUM 1.18 / 1.69, but 3.33 / 1.60 under Zipf 1).
         const double table = (double)hash_slots * (keyb + 8.0 * aggs->n);
         const bool in_l2 = table <= (double)l2_bytes_or_default() / 2;
-        v = gb_hash_slots(est, ga, pub.narrow != 0) || (in_l2 && n < kGbPartRows) ? EIGER_GB_HASH : EIGER_GB_PARTITION;
+        v = gb_hash_slots(est, ga, pub.narrow != 0) || (in_l2 && (n < kGbPartRows || ga.n == 0)) ? EIGER_GB_HASH
+                                                                                                   : EIGER_GB_PARTITION;
     }
     pub.variant = v;
     pub.selector = knobs ? 2 : 0;
